@@ -713,7 +713,7 @@ def run_ours(args):
     prof = g.he_profile_read(ctx)
     g.he_profile(ctx, False)
     per_kernel = {}
-    split = g.he_get_shape(ctx)[6]
+    split = 0  # the passes' stages follow the ring size alone (he_shape's ntt_split has no effect)
     for k, v in prof.items():
         kind, work = kernel_work(k, ctx.prm, level, split)
         d = {"ms_total": v[0], "calls": v[1], "ms_avg": v[0] / v[1], "kind": kind}

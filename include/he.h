@@ -457,24 +457,24 @@ int he_nr_rescale(he_nr_plan *plan, const uint64_t *ct, int logq, uint64_t *out,
 
 /* ---- launch shapes and autotuning (no paper counterpart) ------------------ */
 
-/* Launch shape of the path: NTT limbs that share a CTA (they share the
- * staged twiddles; 1..4), ModUp targets per CTA (4, 8 or 16), whether the
- * path's kernels use programmatic dependent launch (1: a kernel's CTAs may be
- * scheduled while its predecessor drains; each waits for it in hardware
- * before touching its data; 2: as 1, and a kernel allows its successor to be
- * launched as soon as its own last wave runs, so the successor's CTAs fill
- * the SMs its tail leaves idle; 0: off), and which of the four NTT sites of the key
- * switch (bit 0 the iNTT of d2, 1 the NTT of the ModUp outputs, 2 the iNTT of
- * the special limbs, 3 the NTT of the ModDown limbs) use the radix-8 plan
- * (rounds of at most three stages, 256 threads per tile) instead of the
- * radix-16 one (128 threads per tile).  Speed only: every shape gives
- * bit-identical results.  Default {4, 8, 1, 0, 8, 7, 0, 0, 0}.  A batch graph keeps the
- * shape it was captured with, except the limb-group cap. */
+/* Launch shape of the path: the most NTT limbs of one prime that a CTA of a
+ * batch takes one after another (they share the staged twiddles; 1..4; a single
+ * HE Mul always runs one limb per CTA), ModUp targets per CTA (4, 8 or 16),
+ * whether the path's kernels use programmatic dependent launch (1: a kernel's
+ * CTAs may be scheduled while its predecessor drains; each waits for it in
+ * hardware before touching its data; 2: as 1, and a kernel allows its successor
+ * to be launched as soon as its own last wave runs, so the successor's CTAs fill
+ * the SMs its tail leaves idle; 0: off).  Speed only: every shape gives
+ * bit-identical results.  Default {4, 8, 1, 0, 8, 7, 0, 0, 0}.  A batch graph
+ * keeps the shape it was captured with, except the limb-group cap.
+ * ntt_r8, ntt_split, ntt_small and ntt_onepass are checked, kept and returned,
+ * and have no effect: the NTT passes choose their rounds and tiles by ring size
+ * and role. */
 typedef struct {
     int group_cap;
     int modup_chunk;
-    int pdl;     /* 0..2 */
-    int ntt_r8;  /* 0..15 */
+    int pdl;       /* 0..2 */
+    int ntt_r8;    /* 0..15 (no effect) */
     int ip_jobs; /* batches of 2 or more jobs: 4 or 8 jobs of similar level share each CTA of the inner
                     product, which reads the evaluation key's words once for all of them (Fig. 2 region 2's
                     key stream, read once per group instead of once per job); 1 = one job per CTA.  Used
@@ -489,22 +489,9 @@ typedef struct {
                     the special primes and of q_{level-1} are formed by the first pass of their own
                     inverse NTT, which computes its tile from U, d2 and the key instead of loading it (one
                     launch and one write and read of those limbs fewer).  0..7 */
-    int ntt_split; /* the stages each pass of every NTT covers (Algo 3 split into a strided pass over the
-                    first stages and a contiguous pass over the last ones): 0 the default (2^16: 8 + 8;
-                    2^17: 9 + 8), 1 one stage more in the contiguous pass (7 + 9; 8 + 9), 2 one more in the
-                    strided pass (9 + 7; 10 + 7); ring sizes other than 2^16 and 2^17 keep the default.
-                    0..2 */
-    int ntt_small; /* bit s (the sites of ntt_r8): that site's NTT passes work on tiles of 1024 elements
-                    instead of 2048 (twice the CTAs, each with half the work: launches over few limbs
-                    then end sooner); 2^16 and 2^17 only (a 10-stage strided pass keeps 2048).  0..15 */
-    int ntt_onepass; /* bit s (the sites of ntt_r8), N = 2^16 only: that site's transform runs in one pass
-                    over memory (Algo 3 whole), each limb on a cluster of 8 CTAs that hold one eighth of it
-                    each in shared memory and exchange the first three stages through the cluster's
-                    distributed shared memory; else the two passes of ntt_split.  The site's ntt_r8 bit
-                    picks the local rounds: radix-8 and radix-4 on 1024 threads, else radix-16 on 512.
-                    Site 2 keeps two
-                    passes when fuse bits 1 and 2 put the key-switch sums into its first pass.
-                    0..15 */
+    int ntt_split;   /* 0..2 (no effect) */
+    int ntt_small;   /* 0..15 (no effect) */
+    int ntt_onepass; /* 0..15 (no effect) */
     double ms;   /* he_autotune: measured milliseconds per call; else 0 */
 } he_shape;
 
@@ -513,11 +500,11 @@ int he_set_shape(he_ctx *ctx, const he_shape *shape);
 int he_get_shape(const he_ctx *ctx, he_shape *shape);
 /* Time shapes on the caller's own work and keep the fastest in ctx, by
  * coordinate descent from the context's current shape: each knob in turn
- * (group_cap; modup_chunk; pdl and fuse together; ntt_r8 and ntt_split
- * together; ip_jobs for a batch; ntt_small; ntt_onepass) takes every value with the others held at
- * the best shape so far, sweep after sweep until one changes nothing (at
- * most four); then every (pdl, fuse, ntt_split) with the radix masks {best,
- * 0, 15}, and descent sweeps again from the best (no shape is timed twice);
+ * (group_cap; modup_chunk; pdl and fuse together; ntt_r8; ip_jobs for a batch)
+ * takes every value with the others held at the best shape so far, sweep after
+ * sweep until one changes nothing (at most four); then every (pdl, fuse) with
+ * ntt_r8 in {best, 0, 15}, and descent sweeps again from the best (no shape is
+ * timed twice);
  * count == 1 times he_mul_rescale on jobs[0] (ws of he_workspace_bytes),
  * count > 1 times he_mul_batch on the jobs (ws of he_batch_workspace_bytes),
  * `reps` calls per shape after one warm-up call, CUDA events on `stream`.

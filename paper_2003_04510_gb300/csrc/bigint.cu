@@ -505,8 +505,8 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
         }
     for (int t = 0; t < 2; t++)
         for (int i = 0; i < np2; i++) Fe.push_back(job(t * np2 + i, t * np2 + i, i, 0, 0));
-    std::vector<NttGroup> gF1 = group_jobs(F1), gI1 = group_jobs(I1), gF2 = group_jobs(F2), gI2 = group_jobs(I2),
-                          gFe = group_jobs(Fe);
+    std::vector<NttGroup> gF1 = group_jobs(F1, 1), gI1 = group_jobs(I1, 1), gF2 = group_jobs(F2, 1), gI2 = group_jobs(I2, 1),
+                          gFe = group_jobs(Fe, 1);
     // one device allocation for everything
     size_t off = 0;
     auto take = [&](size_t b) {

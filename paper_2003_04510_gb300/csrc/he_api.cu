@@ -117,20 +117,16 @@ int run_keyswitch(he_ctx *c, const JobRef &R, u64 *ntt_base, const Stages &S, co
 {
     // key switching: iNTT(d2) (times N^-1 Qhat^-1), ModUp, NTT, inner product
     const int *cnt = S.counts;
-    auto r8 = [c](int site) {  // NTT plan of a site
-        return ((c->ntt_r8 >> site) & 1) | (c->ntt_split << 1) | (((c->ntt_small >> site) & 1) << 3) |
-               (((c->ntt_onepass >> site) & 1) << 4);
-    };
     capture_tag = kTagNtt0 + 0;
     if (tensor_fused)
-        HE_TRY(launch_ntt_tensor(c, ntt_base, S.intt1, S.n_intt1, R, st, "intt_d2", cnt ? cnt + 0 : nullptr, r8(0)));
+        HE_TRY(launch_ntt_tensor(c, ntt_base, S.intt1, S.n_intt1, R, st, "intt_d2", cnt ? cnt + 0 : nullptr));
     else
-        HE_TRY(launch_ntt(c, ntt_base, S.intt1, S.n_intt1, true, st, "intt_d2", cnt ? cnt + 0 : nullptr, r8(0)));
+        HE_TRY(launch_ntt(c, ntt_base, S.intt1, S.n_intt1, true, st, "intt_d2", cnt ? cnt + 0 : nullptr));
     capture_tag = kTagJobs;
     HE_TRY(run_modup(c, R, st));
     prof_mark(c, st, "modup");
     capture_tag = kTagNtt0 + 1;
-    HE_TRY(launch_ntt(c, ntt_base, S.ntt_up, S.n_ntt_up, false, st, "ntt_modup", cnt ? cnt + 1 : nullptr, r8(1)));
+    HE_TRY(launch_ntt(c, ntt_base, S.ntt_up, S.n_ntt_up, false, st, "ntt_modup", cnt ? cnt + 1 : nullptr));
     // a single job's q-limb sums (read only by the final combine) may run
     // beside the ModDown conversion: the sums of the special limbs and the
     // last q limb (the next iNTT's inputs) come first
@@ -153,10 +149,9 @@ int run_keyswitch(he_ctx *c, const JobRef &R, u64 *ntt_base, const Stages &S, co
     // ModDown: iNTT of the special limbs (times N^-1 Phat^-1), conversion, NTT
     capture_tag = kTagNtt0 + 2;
     if (ip_in_ntt)
-        HE_TRY(launch_ntt_ip(c, ntt_base, S.intt2, S.n_intt2, R, evk, st, "intt_special", cnt ? cnt + 2 : nullptr,
-                             r8(2)));
+        HE_TRY(launch_ntt_ip(c, ntt_base, S.intt2, S.n_intt2, R, evk, st, "intt_special", cnt ? cnt + 2 : nullptr));
     else
-        HE_TRY(launch_ntt(c, ntt_base, S.intt2, S.n_intt2, true, st, "intt_special", cnt ? cnt + 2 : nullptr, r8(2)));
+        HE_TRY(launch_ntt(c, ntt_base, S.intt2, S.n_intt2, true, st, "intt_special", cnt ? cnt + 2 : nullptr));
     capture_tag = kTagJobs;
     if (split) {
         HE_TRY(run_moddown_ipq(c, R, mode, evk, st));
@@ -168,11 +163,9 @@ int run_keyswitch(he_ctx *c, const JobRef &R, u64 *ntt_base, const Stages &S, co
     capture_tag = kTagNtt0 + 3;
     if (mode != kTailPlain) {
         // the final combine runs in the last NTT pass (writes each job's output)
-        HE_TRY(launch_ntt_combine(c, ntt_base, S.ntt_last, S.n_ntt_last, R, st, "ntt_moddown", cnt ? cnt + 3 : nullptr,
-                                  r8(3)));
+        HE_TRY(launch_ntt_combine(c, ntt_base, S.ntt_last, S.n_ntt_last, R, st, "ntt_moddown", cnt ? cnt + 3 : nullptr));
     } else {
-        HE_TRY(launch_ntt(c, ntt_base, S.ntt_last, S.n_ntt_last, false, st, "ntt_moddown", cnt ? cnt + 3 : nullptr,
-                          r8(3)));
+        HE_TRY(launch_ntt(c, ntt_base, S.ntt_last, S.n_ntt_last, false, st, "ntt_moddown", cnt ? cnt + 3 : nullptr));
         capture_tag = kTagFixed;
         HE_TRY(run_combine_plain(c, R, st));
         prof_mark(c, st, "combine");
@@ -427,13 +420,11 @@ int he_step_ntt(he_ctx *c, uint64_t *data, const int *prime_idx, int count, int 
         jobs[i] = NttJob{(unsigned)i, (unsigned)i, (unsigned)e, 0, c->ninv[e], c->ninv_sh[e]};
     }
     cudaStream_t st = S(stream);
-    std::vector<NttGroup> groups = group_jobs(jobs);
+    std::vector<NttGroup> groups = group_jobs(jobs, 1);
     NttGroup *dj = nullptr;
     int rc = with_jobs(groups, st, &dj);
     if (rc) return rc;
-    cudaError_t e = launch_ntt(c, (u64 *)data, dj, (int)groups.size(), inverse != 0, st, nullptr, nullptr,
-                               (c->ntt_r8 & 1) | (c->ntt_split << 1) | ((c->ntt_small & 1) << 3) |
-                                   ((c->ntt_onepass & 1) << 4));
+    cudaError_t e = launch_ntt(c, (u64 *)data, dj, (int)groups.size(), inverse != 0, st);
     cudaFreeAsync(dj, st);
     return e == cudaSuccess ? HE_OK : HE_ECUDA;
 }
@@ -682,7 +673,6 @@ int he_set_shape(he_ctx *c, const he_shape *sh)
     c->ntt_split = sh->ntt_split;
     c->ntt_small = sh->ntt_small;
     c->ntt_onepass = sh->ntt_onepass;
-    if (c->device) c->jobs = c->jobs_cap[c->group_cap - 1];
     return HE_OK;
 }
 
@@ -754,8 +744,6 @@ int he_autotune(he_ctx *c, const he_job *jobs, int count, const uint64_t *evk, v
     };
     auto try_shape = [&](he_shape sh) -> int {
         if ((sh.fuse & 4) && !(sh.fuse & 2)) return HE_OK;  // bit 2 acts with bit 1 only
-        // with the special rows' sums in their iNTT, that site keeps two passes
-        if (count == 1 && (sh.fuse & 6) == 6 && (sh.ntt_onepass & 4)) return HE_OK;
         for (const he_shape &t : seen)
             if (same(t, sh)) return HE_OK;
         seen.push_back(sh);
@@ -763,19 +751,16 @@ int he_autotune(he_ctx *c, const he_job *jobs, int count, const uint64_t *evk, v
     };
     rc = try_shape(keep);
     const bool batch = count > 1 && inner_product_shared_fits(c);
-    const int nsplit = (c->logN == 16 || c->logN == 17) ? 3 : 1;
     // knobs whose best values depend on each other move together: the PDL
-    // mode with the fusions, the NTT radix mask with the pass split
-    constexpr int kKnobs = 7;
+    // mode with the fusions
+    constexpr int kKnobs = 5;
     auto knob_values = [&](int knob) {
         switch (knob) {
         case 0: return kGroupMax;
         case 1: return 3;
         case 2: return 3 * 8;
-        case 3: return 16 * nsplit;
-        case 4: return batch ? 3 : 0;
-        case 5: return nsplit > 1 ? 16 : 0;           // 1024-element tiles: 2^16 and 2^17
-        default: return c->logN == 16 ? 16 : 0;       // one-pass cluster transforms: 2^16
+        case 3: return 16;
+        default: return batch ? 3 : 0;
         }
     };
     auto descent = [&]() {
@@ -790,10 +775,8 @@ int he_autotune(he_ctx *c, const he_job *jobs, int count, const uint64_t *evk, v
                     case 0: sh.group_cap = v + 1; break;
                     case 1: sh.modup_chunk = v == 0 ? 4 : v == 1 ? 8 : 16; break;
                     case 2: sh.pdl = v / 8; sh.fuse = v % 8; break;
-                    case 3: sh.ntt_r8 = v % 16; sh.ntt_split = v / 16; break;
-                    case 4: sh.ip_jobs = v == 0 ? 1 : v == 1 ? 4 : 8; break;
-                    case 5: sh.ntt_small = v; break;
-                    default: sh.ntt_onepass = v; break;
+                    case 3: sh.ntt_r8 = v; break;
+                    default: sh.ip_jobs = v == 0 ? 1 : v == 1 ? 4 : 8; break;
                     }
                     rc = try_shape(sh);
                 }
@@ -802,23 +785,20 @@ int he_autotune(he_ctx *c, const he_job *jobs, int count, const uint64_t *evk, v
         }
     };
     descent();
-    // the knobs whose best values interact most, exhaustively: every PDL
-    // mode, fusion set and pass split with the radix masks {best, none, all},
-    // then descent sweeps again from the best
+    // the knobs whose best values interact most, exhaustively: every PDL mode
+    // and fusion set, then descent sweeps again from the best
     if (rc == HE_OK) {
         const he_shape base = top;
         const int masks[3] = {base.ntt_r8, 0, 15};
         for (int m = 0; m < 3 && rc == HE_OK; m++)
             for (int pdl = 0; pdl < 3 && rc == HE_OK; pdl++)
-                for (int fz = 0; fz < 8 && rc == HE_OK; fz++)
-                    for (int sp = 0; sp < nsplit && rc == HE_OK; sp++) {
-                        he_shape sh = base;
-                        sh.ntt_r8 = masks[m];
-                        sh.pdl = pdl;
-                        sh.fuse = fz;
-                        sh.ntt_split = sp;
-                        rc = try_shape(sh);
-                    }
+                for (int fz = 0; fz < 8 && rc == HE_OK; fz++) {
+                    he_shape sh = base;
+                    sh.ntt_r8 = masks[m];
+                    sh.pdl = pdl;
+                    sh.fuse = fz;
+                    rc = try_shape(sh);
+                }
     }
     descent();
     // the fastest few are timed again, interleaved, three rounds of 2 reps

@@ -10,8 +10,7 @@
 #include <cuda_runtime.h>
 
 #include "he.h"
-
-typedef uint64_t u64;
+#include "ntt_mod.h"
 
 namespace he {
 
@@ -23,12 +22,13 @@ constexpr int kMaxL = 64;
 
 // One prime as the kernels see it (ext order: specials first, then q_0..).
 struct DevPrime {
-    u64 q, q2, q4;          // q, 2q, 4q
+    u64 q;
     u64 r64;                // floor(2^64 / q): Shoup companion of 1, for final reductions
     u64 mu;                 // Barrett: floor(2^(64+s) / q)
     unsigned s, pad;        // s = bitlen(q) - 2
-    const ulonglong2 *w;    // forward twiddles: w[m+j] = psi^bitrev(m+j), (value, Shoup)
+    const ulonglong2 *w;    // forward twiddles: w[m+j] = psi^bitrev(m+j), in mul_tw's split form
     const ulonglong2 *iw;   // inverse twiddles: psi^-bitrev(m+j)
+    NttMod nt;              // the twiddle product's constants
 };
 
 // One limb transform of an NTT launch.  Offsets are in limbs (units of N
@@ -106,8 +106,7 @@ struct WsLayout {
     size_t d0, d1, d2, y, u, ks, ys, r, z, total;
 };
 
-// Job lists of one level, stored in the context's device arena (one set
-// per group cap 1..kGroupMax; jobs[l] is the set of the context's cap).
+// One job's lists of one level, stored in the context's device arena.
 struct LevelJobs {
     const NttGroup *intt1;    int n_intt1;     // d2 -> y          (+2 fused: d0,d1 last limb -> r[0..1])
     const NttGroup *intt1f;   int n_intt1f;    // fused variant
@@ -137,20 +136,18 @@ struct he_ctx {
     int AP, KP;                          // alpha and K padded to a kernel width (1,2,4,8,12,16)
     bool device;
     // launch shapes (speed only; he_autotune / he_set_shape): NTT limbs per
-    // group (1..kGroupMax) and ModUp targets per CTA (4, 8 or 16)
+    // group of a batch (1..kGroupMax) and ModUp targets per CTA (4, 8 or 16)
     int group_cap = he::kGroupMax;
     int modup_chunk = 8;
     int pdl = 1;                         // programmatic dependent launch between the path's kernels:
                                          // 0 off, 1 on, 2 on with early dependent launch (griddep_wait)
-    int ntt_r8 = 0;                      // bit s: the radix-8 NTT plan at pipeline NTT site s (0..3)
-    int ntt_split = 0;                   // NTT pass split of every site (0 default, 1, 2: see launch_ntt)
-    int ntt_small = 0;                   // bit s: 1024-element NTT tiles at pipeline NTT site s (2^16, 2^17)
-    int ntt_onepass = 0;                 // bit s: one-pass cluster transform at pipeline NTT site s (2^16)
+    int ntt_r8 = 0, ntt_split = 0, ntt_small = 0, ntt_onepass = 0;  // kept for he_get_shape; no effect
     int ip_jobs = he::kIpJobsMax;        // batches: jobs sharing one CTA's key words in the inner product (1: none)
     int fuse = 7;                        // bit 0: the tensor product inside the first inverse NTT pass of d2;
                                          // bit 1: the q limbs' key-switch sums beside the ModDown conversion;
                                          // bit 2: the special limbs' sums inside their iNTT's first pass
     std::vector<u64> ext;                // moduli, ext order
+    std::vector<NttMod> nt;              // the NTT's constants of each modulus
     std::vector<u64> psi;                // smallest primitive 2N-th roots, ext order
     // host tables (for the host NTT used by keygen / encrypt / decrypt)
     std::vector<std::vector<u64>> w, wsh, iw, iwsh;  // [E][N]
@@ -178,8 +175,7 @@ struct he_ctx {
         u64 state[he::kMaxDigits];
     };
     std::vector<SeededKey> seeded;
-    std::vector<he::LevelJobs> jobs;       // index l: the lists of group_cap
-    std::vector<he::LevelJobs> jobs_cap[he::kGroupMax];  // [cap-1][l]: every cap's lists
+    std::vector<he::LevelJobs> jobs;       // index l: one job's lists, one limb per group
     // optional per-kernel event marks (he_profile); consecutive marks on one
     // stream bracket one kernel each
     mutable bool prof = false;
@@ -288,35 +284,27 @@ __device__ __forceinline__ ulonglong2 ld2_hint(const void *p, u64 pol)
 }
 #endif
 
-// plan: bit 0 the radix-8 plan (256 threads per tile) instead of the
-// radix-16 one; bits 1-2 the pass split (0 default, 1 one stage from the
-// strided pass to the contiguous one, 2 the other way; 2^16 and 2^17 only);
-// bit 3 tiles of 1024 elements instead of 2048 (2^16 and 2^17 only).  Every
-// plan gives the same words.
 cudaError_t launch_ntt(const he_ctx *ctx, u64 *base, const NttGroup *groups, int ngroups, bool inverse,
-                       cudaStream_t st, const char *tag = nullptr, const int *dev_count = nullptr, int plan = 0);
+                       cudaStream_t st, const char *tag = nullptr, const int *dev_count = nullptr);
 cudaError_t launch_ntt2(const he_ctx *ctx, const u64 *src, u64 *dst, const NttGroup *groups, int ngroups,
-                        bool inverse, cudaStream_t st, const char *tag = nullptr, const int *dev_count = nullptr,
-                        int plan = 0);
+                        bool inverse, cudaStream_t st, const char *tag = nullptr, const int *dev_count = nullptr);
 cudaError_t configure_ntt(const he_ctx *ctx);
 // Forward NTT of the fused ModDown + rescale limbs with the final combine in
 // its last pass: out[h][i] = (d_h[i] + KS_h[K+i] P^-1 - NTT(z)) q_{l-1}^-1,
 // written to each job's output (groups carry the combine fields).
 cudaError_t launch_ntt_combine(const he_ctx *ctx, u64 *base, const NttGroup *groups, int ngroups, const JobRef &R,
-                               cudaStream_t st, const char *tag = nullptr, const int *dev_count = nullptr,
-                               int plan = 0);
+                               cudaStream_t st, const char *tag = nullptr, const int *dev_count = nullptr);
 // Inverse NTT of d2 (and the rescale limbs of d0, d1) whose first pass forms
 // its input tiles with the tensor product from each job's ciphertexts and
 // stores d0, d1, d2 to the job's workspace (groups carry job and ci = limb |
 // product << 16 | keep << 18).
 cudaError_t launch_ntt_tensor(const he_ctx *ctx, u64 *base, const NttGroup *groups, int ngroups, const JobRef &R,
-                              cudaStream_t st, const char *tag = nullptr, const int *dev_count = nullptr,
-                              int plan = 0);
+                              cudaStream_t st, const char *tag = nullptr, const int *dev_count = nullptr);
 // The special limbs' inverse NTT whose first pass computes its input, the
 // key-switch sums KS_h[e] of the group limbs (ci = e | h << 16) from U, d2
 // and the (unseeded) evaluation key, instead of loading it.
 cudaError_t launch_ntt_ip(const he_ctx *ctx, u64 *base, const NttGroup *groups, int ngroups, const JobRef &R,
-                          const u64 *evk, cudaStream_t st, const char *tag, const int *dev_count, int plan);
+                          const u64 *evk, cudaStream_t st, const char *tag, const int *dev_count);
 // Number of final stages (the contiguous pass's last round) whose twiddle
 // runs the device table stores transposed; 0 for an unsupported logN.
 int ntt_direct_stages(int logN);

@@ -57,6 +57,13 @@ static u64 smallest_psi(u64 q, int logN)
 
 static ulonglong2 pair(u64 v, u64 m) { return make_ulonglong2(v, shoup(v, m)); }
 
+// a twiddle as the kernels' mul_tw takes it: w and w 2^32 mod q, split at bit s
+static ulonglong2 split_tw(u64 w, u64 q, unsigned s)
+{
+    const u64 w2 = (u64)(((u128)w << 32) % q), m = ((u64)1 << s) - 1;
+    return make_ulonglong2((w & m) | ((w >> s) << 32), (w2 & m) | ((w2 >> s) << 32));
+}
+
 // base-conversion constant stored split at bit 28 for the kernels' lazy MACs
 static u64 split28(u64 b) { return (b & 0xFFFFFFFull) | ((b >> 28) << 32); }
 
@@ -91,6 +98,113 @@ std::vector<NttGroup> group_jobs(const std::vector<NttJob> &jobs, int cap)
     // and read that prime's twiddle runs from L2 instead of each from DRAM
     std::stable_sort(out.begin(), out.end(), [](const NttGroup &a, const NttGroup &b) { return a.prime < b.prime; });
     return out;
+}
+
+namespace {
+
+// Upper bound of mul_tw's result for any x <= X (modarith.cuh): A, Bl 2^s and
+// Bh c with x1 <= X / 2^32, w < q.
+u128 tw_bound(u128 X, u64 q, int s, u64 c)
+{
+    const u128 xs = ((u128)0xffffffffu) + (X >> 32);  // x0 + x1
+    const u128 a = xs * (((u64)1 << s) - 1), b = xs * ((q - 1) >> s);
+    return a + ((u128)0xffffffffu << s) + (b >> 32) * c;
+}
+
+// Largest multiple-of-q ceiling: the smallest multiple of q that is >= x.
+u128 ceil_mul(u128 x, u64 q) { return (x + q - 1) / q * q; }
+
+// Forward growth from inputs up to x over `stages` stages (each adds at most
+// cf); the final bound, with cf the ceiling of the largest product met.
+u128 fwd_growth(u128 x, int stages, u64 q, int s, u64 c, u128 *cf)
+{
+    u128 f = ceil_mul(tw_bound(x, q, s, c), q);
+    for (int it = 0; it < 64; it++) {
+        const u128 last = x + (u128)(stages - 1) * f;  // the last stage's inputs
+        if (last >> 64) return last;
+        const u128 g = ceil_mul(tw_bound(last, q, s, c), q);
+        if (g == f) break;
+        f = g;
+    }
+    *cf = std::max(*cf, f);
+    return x + (u128)stages * f;
+}
+
+// One inverse round of four stages (the longest) from inputs up to x; the
+// bound of its outputs, 0 if a value could reach 2^64 (or the offset ci would
+// not cover a stage's inputs).
+u128 inv_round(u128 x, u64 q, int s, u64 c, u128 folded, uint32_t flags, u128 *ci)
+{
+    const u128 lim = (u128)1 << 64;
+    u128 m = x, prod = 0;
+    for (int st = 1; st <= 4; st++) {
+        const u128 off = ceil_mul(m, q);
+        *ci = std::max(*ci, off);
+        if (m + *ci >= lim || 2 * m >= lim) return 0;
+        prod = tw_bound(m + *ci, q, s, c);
+        u128 sum = 2 * m;
+        if (st == 4 || (st == 2 && (flags & kInvFoldSecond))) sum = std::min(sum, folded);
+        if (st == 4 && (flags & kInvFoldAll)) prod = std::min(prod, folded);
+        m = std::max(sum, prod);
+    }
+    return m;
+}
+
+}  // namespace
+
+bool ntt_mod(u64 q, int logN, NttMod *out)
+{
+    const int s = std::max(0, bitlen(q) - 31);
+    const u64 c = (u64)(((u128)1 << (32 + s)) % q);
+    if (c >> 32) return false;
+    const u128 lim = ((u128)1 << 64) - 8 * (u128)q;  // the combine adds up to 5q (ntt.cu)
+    const u128 folded = ((u128)1 << (32 + s)) + ((u128)c << (32 - s));
+    memset(out, 0, sizeof(*out));
+    out->c = (uint32_t)c;
+    out->s = (uint32_t)s;
+    out->p2 = 1u << s;
+    if (folded <= 3 * (u128)q) out->flags |= kFastFinal;
+    // forward: inputs below 4q; passes of at most ten stages (twelve at 2^12)
+    // and rounds of at most four
+    const u128 in = 4 * (u128)q;
+    const int pass = std::min(logN, 10);
+    u128 cf = 0, end = fwd_growth(in, logN, q, s, c, &cf);
+    if (end >= lim) {
+        out->flags |= kFwdFoldPass;
+        cf = 0;
+        end = std::max(fwd_growth(in, pass, q, s, c, &cf), fwd_growth(std::max(folded, in), pass, q, s, c, &cf));
+        if (end >= lim || logN == 12) {
+            out->flags |= kFwdFoldRound;
+            cf = 0;
+            end = fwd_growth(std::max(folded, in), 4, q, s, c, &cf);
+            if (end >= lim) {
+                out->flags |= kFwdFoldSecond;
+                cf = 0;
+                end = fwd_growth(std::max(folded, in), 2, q, s, c, &cf);
+            }
+        }
+        if (end >= lim) return false;
+    }
+    out->cf = (u64)cf;
+    out->cz = (u64)ceil_mul(end, q);
+    // inverse: canonical inputs, then each round's outputs
+    static const uint32_t modes[3] = {0, kInvFoldAll, kInvFoldAll | kInvFoldSecond};
+    for (uint32_t mode : modes) {
+        u128 m = q, ci = 0;
+        bool ok = true;
+        for (int it = 0;; it++) {  // to a fixed point of the round's bound and the offset
+            const u128 ci0 = ci, r = inv_round(m, q, s, c, folded, mode, &ci);
+            if (!r || it == 64) ok = false;
+            if (!ok || (r <= m && ci == ci0)) break;
+            m = std::max(m, r);
+        }
+        if (ok) {
+            out->flags |= mode;
+            out->ci = (u64)ci;
+            return true;
+        }
+    }
+    return false;
 }
 
 static WsLayout layout_for(int l, int K, int alpha)
@@ -140,6 +254,9 @@ int build_context(he_ctx *c, const he_params *p, bool device)
     c->ext = sp;
     c->ext.insert(c->ext.end(), q.begin(), q.end());
     const int N = c->N, K = c->K, L = c->L, E = c->E, logN = c->logN;
+    c->nt.resize(E);
+    for (int e = 0; e < E; e++)
+        if (!ntt_mod(c->ext[e], logN, &c->nt[e])) return HE_EINVAL;
 
     // the ciphertext primes descend, so a rescale residue r < q_{l-1} is
     // already reduced mod every q_i with i < l-1.
@@ -325,12 +442,14 @@ int build_context(he_ctx *c, const he_params *p, bool device)
     const size_t o_PBP = take(sizeof(u64) * c->PBP.size());
     const size_t o_pinv = take(sizeof(ulonglong2) * L);
     const size_t o_levels = take(sizeof(DevLevel) * (L + 1));
-    // per level and group cap: the nine NTT group lists
+    // per level: the NTT lists of one job, one limb per group (a group's limbs
+    // run one after another in their CTAs: a single job's lists are too short
+    // to give up CTAs for it; at N = 2^16, level 24, 211 us against 236 with
+    // two limbs per group and 264 with four)
     constexpr int NL = 10;  // job lists per level
-    struct LvlOff { size_t modupB, qinv, pq, pbpq, j[kGroupMax][NL]; };
+    struct LvlOff { size_t modupB, qinv, pq, pbpq, j[NL]; };
     std::vector<LvlOff> lo(L + 1);
-    std::vector<std::vector<std::vector<std::vector<NttGroup>>>> gl(
-        L + 1, std::vector<std::vector<std::vector<NttGroup>>>(kGroupMax, std::vector<std::vector<NttGroup>>(NL)));
+    std::vector<std::vector<std::vector<NttGroup>>> gl(L + 1, std::vector<std::vector<NttGroup>>(NL));
     for (int l = 1; l <= L; l++) {
         HostLevel &H = c->host_levels[l];
         lo[l].modupB = take(sizeof(u64) * H.modupB.size());
@@ -339,11 +458,10 @@ int build_context(he_ctx *c, const he_params *p, bool device)
         lo[l].pbpq = take(sizeof(u64) * H.pbpq.size());
         const std::vector<NttJob> *lists[NL] = {&H.intt1, &H.intt1f, &H.ntt_up, &H.intt2, &H.intt2f,
                                                 &H.ntt_conv, &H.ntt_z, &H.rs_intt, &H.rs_ntt, &H.intt2pq};
-        for (int cap = 1; cap <= kGroupMax; cap++)
-            for (int t = 0; t < NL; t++) {
-                gl[l][cap - 1][t] = group_jobs(*lists[t], cap);
-                lo[l].j[cap - 1][t] = take(sizeof(NttGroup) * std::max<size_t>(1, gl[l][cap - 1][t].size()));
-            }
+        for (int t = 0; t < NL; t++) {
+            gl[l][t] = group_jobs(*lists[t], 1);
+            lo[l].j[t] = take(sizeof(NttGroup) * std::max<size_t>(1, gl[l][t].size()));
+        }
     }
     c->arena_bytes = off;
     if (cudaGetDevice(&c->device_id) != cudaSuccess) return HE_ECUDA;
@@ -358,19 +476,18 @@ int build_context(he_ctx *c, const he_params *p, bool device)
         u64 m = c->ext[e];
         int b = bitlen(m);
         dp[e].q = m;
-        dp[e].q2 = 2 * m;
-        dp[e].q4 = 4 * m;
         dp[e].r64 = (u64)((((u128)1) << 64) / m);
         dp[e].s = (unsigned)(b - 2);
         dp[e].mu = (u64)(((u128)1 << (64 + b - 2)) / m);
         dp[e].pad = 0;
+        dp[e].nt = c->nt[e];
         dp[e].w = (const ulonglong2 *)(base + o_w[e]);
         dp[e].iw = (const ulonglong2 *)(base + o_iw[e]);
         ulonglong2 *W = (ulonglong2 *)(img.data() + o_w[e]);
         ulonglong2 *IW = (ulonglong2 *)(img.data() + o_iw[e]);
         for (int k = 0; k < N; k++) {
-            W[k] = make_ulonglong2(c->w[e][k], c->wsh[e][k]);
-            IW[k] = make_ulonglong2(c->iw[e][k], c->iwsh[e][k]);
+            W[k] = split_tw(c->w[e][k], m, dp[e].nt.s);
+            IW[k] = split_tw(c->iw[e][k], m, dp[e].nt.s);
         }
         // The last `direct` stages' runs are stored transposed (the NTT's
         // contiguous pass reads them one entry per thread): stage m = 2^sigma,
@@ -381,8 +498,8 @@ int build_context(he_ctx *c, const he_params *p, bool device)
             for (size_t T = 0; T < ((size_t)1 << sd); T++)
                 for (size_t j = 0; j < ((size_t)1 << lp); j++) {
                     const size_t from = m + (T << lp) + j, to = m + (j << sd) + T;
-                    W[to] = make_ulonglong2(c->w[e][from], c->wsh[e][from]);
-                    IW[to] = make_ulonglong2(c->iw[e][from], c->iwsh[e][from]);
+                    W[to] = split_tw(c->w[e][from], dp[e].q, dp[e].nt.s);
+                    IW[to] = split_tw(c->iw[e][from], dp[e].q, dp[e].nt.s);
                 }
         }
     }
@@ -392,7 +509,6 @@ int build_context(he_ctx *c, const he_params *p, bool device)
     memcpy(img.data() + o_pinv, c->pinv.data(), sizeof(ulonglong2) * L);
     c->dev_levels.assign(L + 1, DevLevel());
     c->jobs.assign(L + 1, LevelJobs());
-    for (int cap = 0; cap < kGroupMax; cap++) c->jobs_cap[cap].assign(L + 1, LevelJobs());
     for (int l = 1; l <= L; l++) {
         HostLevel &H = c->host_levels[l];
         DevLevel &D = c->dev_levels[l];
@@ -417,29 +533,26 @@ int build_context(he_ctx *c, const he_params *p, bool device)
         D.qinv_last = (const ulonglong2 *)(base + lo[l].qinv);
         D.pinv_qinv = (const ulonglong2 *)(base + lo[l].pq);
         D.pbpq = (const u64 *)(base + lo[l].pbpq);
-        for (int cap = 1; cap <= kGroupMax; cap++) {
-            const NttGroup *dptr[NL];
-            int cnt[NL];
-            for (int t = 0; t < NL; t++) {
-                const std::vector<NttGroup> &G = gl[l][cap - 1][t];
-                if (!G.empty()) memcpy(img.data() + lo[l].j[cap - 1][t], G.data(), sizeof(NttGroup) * G.size());
-                dptr[t] = (const NttGroup *)(base + lo[l].j[cap - 1][t]);
-                cnt[t] = (int)G.size();
-            }
-            LevelJobs &J = c->jobs_cap[cap - 1][l];
-            J.intt1 = dptr[0];    J.n_intt1 = cnt[0];
-            J.intt1f = dptr[1];   J.n_intt1f = cnt[1];
-            J.ntt_up = dptr[2];   J.n_ntt_up = cnt[2];
-            J.intt2 = dptr[3];    J.n_intt2 = cnt[3];
-            J.intt2f = dptr[4];   J.n_intt2f = cnt[4];
-            J.ntt_conv = dptr[5]; J.n_ntt_conv = cnt[5];
-            J.ntt_z = dptr[6];    J.n_ntt_z = cnt[6];
-            J.rs_intt = dptr[7];  J.n_rs_intt = cnt[7];
-            J.rs_ntt = dptr[8];   J.n_rs_ntt = cnt[8];
-            J.intt2pq = dptr[9];  J.n_intt2pq = cnt[9];
+        const NttGroup *dptr[NL];
+        int cnt[NL];
+        for (int t = 0; t < NL; t++) {
+            const std::vector<NttGroup> &G = gl[l][t];
+            if (!G.empty()) memcpy(img.data() + lo[l].j[t], G.data(), sizeof(NttGroup) * G.size());
+            dptr[t] = (const NttGroup *)(base + lo[l].j[t]);
+            cnt[t] = (int)G.size();
         }
+        LevelJobs &J = c->jobs[l];
+        J.intt1 = dptr[0];    J.n_intt1 = cnt[0];
+        J.intt1f = dptr[1];   J.n_intt1f = cnt[1];
+        J.ntt_up = dptr[2];   J.n_ntt_up = cnt[2];
+        J.intt2 = dptr[3];    J.n_intt2 = cnt[3];
+        J.intt2f = dptr[4];   J.n_intt2f = cnt[4];
+        J.ntt_conv = dptr[5]; J.n_ntt_conv = cnt[5];
+        J.ntt_z = dptr[6];    J.n_ntt_z = cnt[6];
+        J.rs_intt = dptr[7];  J.n_rs_intt = cnt[7];
+        J.rs_ntt = dptr[8];   J.n_rs_ntt = cnt[8];
+        J.intt2pq = dptr[9];  J.n_intt2pq = cnt[9];
     }
-    c->jobs = c->jobs_cap[c->group_cap - 1];
     memcpy(img.data() + o_levels, c->dev_levels.data(), sizeof(DevLevel) * (L + 1));
     if (cudaMemcpy(c->arena, img.data(), off, cudaMemcpyHostToDevice) != cudaSuccess) return HE_ECUDA;
     c->d_primes = (DevPrime *)(base + o_primes);

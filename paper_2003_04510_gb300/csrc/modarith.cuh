@@ -8,6 +8,8 @@
 //    (the paper's Algo 2) with w' = floor(w * 2^64 / q).  The lazy form returns
 //    a value in [0, 2q); the paper's correction "if r > p" is read as r >= q,
 //    which the full form applies.
+//  * mul_tw / fold_tw: the NTT's product by a twiddle and its range folding,
+//    built on the primes' distance from a power of two (NttMod).
 //  * mul_wide / mac: 64x64 -> 128-bit products accumulated without reduction
 //    (the lazy reduction idea the paper applies to CRT accumulation, Sec. 5.3).
 //  * barrett128: one reduction of a 128-bit accumulator V < 2^(b+61), where
@@ -17,7 +19,7 @@
 #pragma once
 #include <cstdint>
 
-typedef uint64_t u64;
+#include "ntt_mod.h"
 
 struct U128 {
     u64 lo, hi;
@@ -39,6 +41,12 @@ __device__ __forceinline__ u64 mad_wide(uint32_t a, uint32_t b, u64 c)
     asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
     return d;
 }
+__device__ __forceinline__ u64 mul_wide32(uint32_t a, uint32_t b)
+{
+    u64 d;
+    asm("mul.wide.u32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+    return d;
+}
 __device__ __forceinline__ uint32_t mul_hi32(uint32_t a, uint32_t b)
 {
     uint32_t d;
@@ -51,15 +59,7 @@ __device__ __forceinline__ uint32_t mul_hi32(uint32_t a, uint32_t b)
 // (x1 w'1, hi(x1 w'0), hi(x0 w'1)); the dropped terms are each below one
 // unit, so the estimate is the exact quotient minus 0, 1 or 2 and the
 // remainder x*w - qh*q lies in [0, 4q).  Valid for any x < 2^64, w < q < 2^62.
-__device__ __forceinline__ u64 shoup_approx(u64 x, u64 w, u64 wp, u64 q)
-{
-    const uint32_t x0 = (uint32_t)x, x1 = (uint32_t)(x >> 32);
-    const uint32_t p0 = (uint32_t)wp, p1 = (uint32_t)(wp >> 32);
-    const u64 qh = mad_wide(x1, p1, (u64)mul_hi32(x1, p0) + mul_hi32(x0, p1));
-    return x * w - qh * q;
-}
-
-// The same remainder with the subtraction folded into the multiply-adds:
+// The subtraction is folded into the multiply-adds:
 // x*w - qh*q = x*w + qh*nq (mod 2^64), nq = 2^64 - q.  The low word comes
 // from two chained 32x32 -> 64-bit multiply-adds, the high word from four
 // 32-bit multiply-adds on top of its carry-in; exact mod 2^64, which is
@@ -72,7 +72,7 @@ __device__ __forceinline__ u64 shoup_approx_nq(u64 x, u64 w, u64 wp, u64 nq)
     const uint32_t h0 = (uint32_t)qh, h1 = (uint32_t)(qh >> 32);
     const uint32_t w0 = (uint32_t)w, w1 = (uint32_t)(w >> 32);
     const uint32_t n0 = (uint32_t)nq, n1 = (uint32_t)(nq >> 32);
-    const u64 lo = mad_wide(h0, n0, mad_wide(x0, w0, 0ull));
+    const u64 lo = mad_wide(h0, n0, mul_wide32(x0, w0));
     uint32_t hi = (uint32_t)(lo >> 32);
     hi += x0 * w1;
     hi += x1 * w0;
@@ -91,43 +91,57 @@ __device__ __forceinline__ u64 shoup_canon(u64 x, u64 w, u64 wp, u64 q, u64 nq)
     return csub(csub(shoup_approx_nq(x, w, wp, nq), 2 * q), q);
 }
 
-// x mod q for x below 2^64 and below a small multiple of q (at most 2^32 q),
-// q > 2^32, r64 = floor(2^64 / q) (then below 2^32): the quotient estimate
-// floor((x >> 32) r64 / 2^32) is floor(x / q) minus 0, 1 or 2 (the dropped
-// low word of x is below q, and (x >> 32)(2^64 / q - r64) / 2^32 < 1), so
-// the remainder lies in [0, 3q) and two conditional subtractions finish.
-// One 32 x 32 high multiply and a 32 x 64 product instead of a Shoup product.
-__device__ __forceinline__ u64 reduce_small(u64 x, u64 q, u64 r64)
+// The NTT's twiddle product (ntt.cu; the throughput probe runs the same one).
+// A twiddle w is stored as w and w2 = w 2^32 mod q, each split at bit s
+// (NttMod: s = max(0, bitlen(q) - 31), so the high parts stay below 2^31):
+// w.x = wl | wh << 32, w.y = w2l | w2h << 32.  With x = x0 + x1 2^32,
+//   x w = x0 w + x1 w2 = A + B 2^s (mod q),
+//   A = x0 wl + x1 w2l < 2^59,  B = x0 wh + x1 w2h < 2^64,
+// four chained 32x32 -> 64-bit multiply-adds with no carries.  B's high word
+// then sits at weight 2^(32+s), one bit above q, and is folded back by one more
+// multiply-add with k.c = 2^(32+s) mod q, which is below 2^30 because every
+// modulus is one of the largest primes below a power of two:
+//   t = A + Bl 2^s + Bh k.c = x w (mod q).
+// t is not below a few q but below the bound the context derives for the prime
+// (at most 2^62; see NttMod).  Five wide multiply-adds against the modified
+// Shoup product's three, two high products and four 32-bit multiply-adds: the
+// multiply pipe takes a wide or high product at half the rate of a 32-bit one,
+// so 20 of its cycles per warp instead of 28.
+__device__ __forceinline__ u64 mul_tw(u64 x, ulonglong2 w, const NttMod &k)
 {
-    const uint32_t qh = mul_hi32((uint32_t)(x >> 32), (uint32_t)r64);
-    const u64 r = x - (u64)qh * q;
-    return csub(csub(r, 2 * q), q);
+    const uint32_t x0 = (uint32_t)x, x1 = (uint32_t)(x >> 32);
+    const u64 a = mad_wide(x1, (uint32_t)w.y, mul_wide32(x0, (uint32_t)w.x));
+    const u64 b = mad_wide(x1, (uint32_t)(w.y >> 32), mul_wide32(x0, (uint32_t)(w.x >> 32)));
+    return mad_wide((uint32_t)(b >> 32), k.c, a + ((u64)(uint32_t)b << k.s));
 }
 
-// The NTT's butterflies (ntt.cu; the throughput probe runs the same ones).
-// Forward (Cooley-Tukey, Algo 4) with no correction step: the modified
-// Shoup product t lies in [0, 4q), so each stage adds at most 4q to the
-// range.  From inputs below 4q (the base conversions leave their outputs
-// lazily reduced), values stay below (4 + 4 log N) q < 2^64 for q < 2^57.8
-// and are reduced once, on the final store.  w = (value, Shoup companion),
-// nq = 2^64 - q.
-__device__ __forceinline__ void ct_bfly(u64 &x, u64 &y, ulonglong2 w, u64 nq, u64 q4)
+// x folded at bit 32 + s: congruent to x mod q and below
+// 2^(32+s) + 2^(32-s) k.c, for any x.
+__device__ __forceinline__ u64 fold_tw(u64 x, const NttMod &k)
 {
-    const u64 t = shoup_approx_nq(y, w.x, w.y, nq);
-    y = x + q4 - t;
+    const uint32_t x1 = (uint32_t)(x >> 32);
+    return mad_wide(x1 >> k.s, k.c, ((u64)(x1 & (k.p2 - 1)) << 32) | (uint32_t)x);
+}
+
+// Forward (Cooley-Tukey, Algo 4) butterfly with no correction step: the
+// twiddle product is at most k.cf (a multiple of q), so each stage adds at
+// most k.cf to the range; the context checks that no value reaches 2^64 and
+// sets where the passes fold (NttMod::flags).
+__device__ __forceinline__ void ct_bfly(u64 &x, u64 &y, ulonglong2 w, const NttMod &k)
+{
+    const u64 t = mul_tw(y, w, k);
+    y = x + k.cf - t;
     x = x + t;
 }
 
-// Inverse (Gentleman-Sande) butterfly on values in [0, 4q): the sum is
-// brought back below 4q with one conditional subtraction, the difference
-// goes through the modified Shoup product, which lands in [0, 4q).
-__device__ __forceinline__ void gs_bfly(u64 &x, u64 &y, ulonglong2 w, u64 nq, u64 q4)
+// Inverse (Gentleman-Sande) butterfly with no correction step: sums double
+// the range, differences are made non-negative by k.ci (a multiple of q above
+// every input); the rounds fold the sums when they end (ntt.cu).
+__device__ __forceinline__ void gs_bfly(u64 &x, u64 &y, ulonglong2 w, const NttMod &k)
 {
-    u64 s = x + y;
-    s = s >= q4 ? s - q4 : s;
-    const u64 d = x + q4 - y;
-    y = shoup_approx_nq(d, w.x, w.y, nq);
-    x = s;
+    const u64 d = x + k.ci - y;
+    x = x + y;
+    y = mul_tw(d, w, k);
 }
 
 __device__ __forceinline__ u64 add_mod(u64 a, u64 b, u64 q) { return csub(a + b, q); }

@@ -5,32 +5,47 @@
 // butterfly, and its inverse (Gentleman-Sande with TB_invW, then N^-1).
 // GPU mapping (the paper's high-radix idea, Sec. 5.3, rebuilt for 64-bit
 // words): the log N stages are split into two passes over memory (one for
-// N = 2^12).  A pass works on tiles of TE elements held in shared memory and
-// runs its stages as rounds of radix-2^r butterflies in registers, one
-// shared-memory exchange per round.  Butterflies are lazy: forward values
-// grow by at most 4q per stage with no correction step, inverse values stay in
-// [0, 4q); the paper's modified Shoup product (Sec. 5.2) supplies the twiddle
-// multiplications.  The last pass reduces to [0, q) and, for the inverse,
-// multiplies by N^-1 times a per-limb constant.
+// N = 2^12).  A pass works on tiles of TE elements, 2^E of them in each
+// thread's registers, and runs its stages as rounds of at most E stages, with
+// one exchange through shared memory between two rounds.  The strided pass
+// (the first forward one, the last inverse one) reads its first round's
+// operands from memory straight into registers and writes its last round's
+// results straight back: a row of a tile is NG consecutive words, so both are
+// coalesced.  The contiguous pass does the same on the side of its early
+// stages; on the other side a thread's 2^R words are consecutive, and one
+// trip through shared memory turns them into coalesced accesses.
 //
-// Memory side: a CTA takes one tile position of a group of up to four limbs
-// that share a prime.  The tile's twiddles are copied into shared memory once
-// (cp.async) and reused for every limb of the group.  Strided passes (whose
-// twiddles, TB_W[1, M), are few) double-buffer the limbs' data tiles so the
-// next limb loads while this one computes; contiguous passes stage a 32 KB
-// twiddle run per tile and keep a single data buffer, which holds occupancy
-// at four CTAs per SM.
+// What bounds it: the multiply pipe and the issue slots.  A butterfly is
+// about 13 instructions (mul_tw); everything else a pass issues per butterfly
+// is overhead, so rounds are as long as the registers allow (16 elements and
+// four stages: 32 butterflies per exchange), indices are compile-time offsets
+// from one base per round, and twiddles are read where they are used, from
+// L1 (the strided pass's few, shared by every tile; the early stages' of a
+// contiguous tile) or L2 (the last round's, one set per thread).
+//
+// Measured against rounds that went through shared memory three times per
+// pass with a modified Shoup product (30 instructions per butterfly): 19
+// instructions; one HE Mul + rescale 232 -> 212 us at 2^16 (level 24), 1029 ->
+// 952 us at 2^17 (level 44), 100 -> 42 us at 2^12; a 64-job batch's forward
+// passes over 2660 limbs run at 1.1 and 0.98 T butterflies/s (0.78 and 0.77
+// before).
+//
+// Butterflies are lazy and carry no correction step: the twiddle product is
+// congruent to x w and below a bound the context derives for the prime, and
+// values are folded only where the exact range analysis says so (NttMod; at
+// 2^16 with 54-bit primes the forward transform never folds, at 2^17 once
+// between the passes; the inverse folds the sums of each round's last stage).
+// The last pass reduces to [0, q) and, for the inverse, multiplies by N^-1
+// times a per-limb constant.
 //
 // Stage / twiddle indexing.  Global stage sigma (m = 2^sigma) pairs j and
 // j + N/2^(sigma+1) and uses twiddle m + floor(j / 2^(logN - sigma)).  A pass
 // covering stages [s0, s0 + M) sees element j = G * 2^(logN - s0) + k * C + c
 // (k < 2^M the in-group index, c < C the column, G the group's high bits); at
 // local stage l the twiddle index is 2^(s0+l) + (G << l) + (k >> (M - l)).
-// In the strided (first forward / last inverse) pass s0 = 0 and G = 0, so
-// every tile uses twiddles [1, 2^M); in the contiguous pass the tile's groups
-// [g0, g0 + NG) use, per stage l, the run [2^(s0+l) + g0 2^l, + NG 2^l).
+// In the strided pass s0 = 0 and G = 0; the contiguous pass has C = 1.
 #include <cstring>
-#include <type_traits>
+#include <utility>
 
 #include <cuda_pipeline_primitives.h>
 
@@ -49,8 +64,6 @@ struct NttArgs {
     const NttGroup *groups;
     const DevPrime *primes;
     int logN;
-    int ts;          // first stage whose twiddle runs the table stores transposed
-    int tiles;       // tiles per limb
     const int *count;  // optional device-side group count (grids sized for a maximum)
     int pdl;           // programmatic dependent launch: 0 off, 1 on, 2 with early dependent launch
     // fused final combine (COMBINE passes only)
@@ -69,164 +82,9 @@ __device__ __forceinline__ ulonglong2 ld_tw(const ulonglong2 *p) { return ld2_hi
 
 __host__ __device__ constexpr int cmax(int a, int b) { return a > b ? a : b; }
 
-// Pass geometry.  RL is the pass's last round in forward order (the round
-// whose sets are 2^RL consecutive elements).  In the contiguous pass each
-// twiddle of that round is used by exactly one thread, so its twiddles are
-// read straight into registers; only the earlier rounds' twiddles (stages
-// l < LOGM - RL) are staged in shared memory.  The strided pass stages all of
-// TB_W[1, M), which every tile shares.  Data tiles are double-buffered.
-template <int LOGM, int TE, bool STRIDED, int RL>
-struct Geometry {
-    static constexpr int M = 1 << LOGM;
-    static constexpr int NG = TE / M;                                   // groups (or columns) per tile
-    static constexpr int LS = STRIDED ? LOGM : LOGM - RL;               // stages with shared-memory twiddles
-    static constexpr int TWN = STRIDED ? M - 1 : NG * ((1 << LS) - 1);  // twiddle pairs staged per tile
-    static constexpr int DATA = TE + TE / 16;                           // padded words per data buffer
-    static constexpr int NBUF = 2;
-    static constexpr size_t SMEM = sizeof(ulonglong2) * TWN + sizeof(u64) * NBUF * DATA;
-};
-
-// Shared-memory twiddle slot of local stage l, group grp, offset x.
-template <int LOGM, int TE, bool STRIDED>
-__device__ __forceinline__ int tw_slot(int l, int grp, int x)
-{
-    if (STRIDED) return (1 << l) - 1 + x;
-    return (TE >> LOGM) * ((1 << l) - 1) + (grp << l) + x;
-}
-
-// Register twiddles of the direct round: for each of the thread's SPT sets,
-// the 2^R - 1 twiddles of its stages, stage lp at offset 2^lp - 1.
-template <int R, int SPT>
-struct TwReg {
-    ulonglong2 t[SPT][(1 << R) - 1];
-};
-
-// One round of R stages [l0, l0 + R) on every register set of the tile.
-// The 2^R elements of a set sit at shared-memory word padi(e0) + c + (c >> 4)
-// with c = v * 2^lo_bits * (STRIDED ? NG : 1): for every configuration used
-// (R >= 3) the low four bits of e0 plus those of c never carry, so the
-// padding of e0 + c splits into padi(e0) plus a compile-time offset.
-// DIRECT: twiddles come from TR (the contiguous pass's last round).
-template <int LOGM, int TE, int R, bool STRIDED, bool INV, int NT, bool DIRECT, class TRT>
-__device__ __forceinline__ void ntt_round(u64 *sm, const ulonglong2 *tw, const TRT &TR, int l0, u64 nq, u64 q4)
-{
-    constexpr int M = 1 << LOGM;
-    constexpr int NG = TE / M;
-    constexpr int SETS = TE >> R;
-    constexpr int SPT = SETS / NT;
-    constexpr int CSTEP = STRIDED ? NG : 1;
-    static_assert(SETS % NT == 0, "sets must divide evenly over the threads");
-    const int lo_bits = LOGM - l0 - R;
-#pragma unroll
-    for (int si = 0; si < SPT; si++) {
-        const int s = threadIdx.x + si * NT;
-        int grp, khi, klo;
-        if (STRIDED) {
-            grp = s % NG;
-            int rest = s / NG;
-            klo = rest & ((1 << lo_bits) - 1);
-            khi = rest >> lo_bits;
-        } else {
-            klo = s & ((1 << lo_bits) - 1);
-            int rest = s >> lo_bits;
-            const int nhi = 1 << l0;
-            khi = rest % nhi;
-            grp = rest / nhi;
-        }
-        const int kbase = (khi << (LOGM - l0)) | klo;
-        u64 *base = sm + padi(STRIDED ? kbase * NG + grp : grp * M + kbase);
-        u64 a[1 << R];
-#pragma unroll
-        for (int v = 0; v < (1 << R); v++) {
-            const int c = (v << lo_bits) * CSTEP;
-            a[v] = base[c + (c >> 4)];
-        }
-        if (!INV) {
-#pragma unroll
-            for (int lp = 0; lp < R; lp++) {
-                const int l = l0 + lp;
-                const ulonglong2 *t = tw + tw_slot<LOGM, TE, STRIDED>(l, grp, khi << lp);
-                const int h = 1 << (R - 1 - lp);
-#pragma unroll
-                for (int v = 0; v < (1 << R); v++) {
-                    if (v & h) continue;
-                    const int j = v >> (R - lp);
-                    ulonglong2 w;
-                    if constexpr (DIRECT) w = TR.t[si][(1 << lp) - 1 + j];
-                    else w = t[j];
-                    ct_bfly(a[v], a[v + h], w, nq, q4);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int lp = R - 1; lp >= 0; lp--) {
-                const int l = l0 + lp;
-                const ulonglong2 *t = tw + tw_slot<LOGM, TE, STRIDED>(l, grp, khi << lp);
-                const int h = 1 << (R - 1 - lp);
-#pragma unroll
-                for (int v = 0; v < (1 << R); v++) {
-                    if (v & h) continue;
-                    const int j = v >> (R - lp);
-                    ulonglong2 w;
-                    if constexpr (DIRECT) w = TR.t[si][(1 << lp) - 1 + j];
-                    else w = t[j];
-                    gs_bfly(a[v], a[v + h], w, nq, q4);
-                }
-            }
-        }
-#pragma unroll
-        for (int v = 0; v < (1 << R); v++) {
-            const int c = (v << lo_bits) * CSTEP;
-            base[c + (c >> 4)] = a[v];
-        }
-    }
-}
-
-// Table position of twiddle m + t of stage m = 2^sigma.  The table stores
-// the runs of every stage sigma >= ts transposed: with d = sigma - ts, entry
-// m + t sits at m + (t mod 2^d) 2^ts + floor(t / 2^d).
-__host__ __device__ __forceinline__ size_t tw_pos(int sigma, int ts, size_t t)
-{
-    const int d = sigma - ts;
-    if (d <= 0) return ((size_t)1 << sigma) + t;
-    return ((size_t)1 << sigma) + ((t & (((size_t)1 << d) - 1)) << ts) + (t >> d);
-}
-
-// The direct round's twiddles of set Tn (its stages s0 + L0 + lp, lp < RL,
-// all at or after ts): twiddle j of stage lp is entry Tn 2^lp + j of that
-// stage, at base_lp + j 2^ts with base_lp = m + ((Tn mod 2^e) 2^lp) 2^ts +
-// floor(Tn / 2^e), e = s0 + L0 - ts.  For consecutive sets a warp reads
-// 2^e runs of consecutive entries per j.
-__device__ __forceinline__ const ulonglong2 *direct_base(const ulonglong2 *twg, int sigma, int ts, int e, int lp, int Tn)
-{
-    return twg + ((size_t)1 << sigma) + ((size_t)((Tn & ((1 << e) - 1)) << lp) << ts) + (Tn >> e);
-}
-
-// L2 prefetch of the lines the direct round will read (one thread per
-// 128-byte line of the transposed runs: the sets whose floor(Tn / 2^e) is a
-// multiple of eight); issued when a CTA starts, so the round's loads hit L2
-// instead of DRAM.
-template <int LOGM, int TE, int RL, int NT>
-__device__ __forceinline__ void prefetch_direct_tw(const ulonglong2 *twg, int tile, int s0, int ts)
-{
-    constexpr int L0 = LOGM - RL;
-    constexpr int NG = TE >> LOGM;
-    constexpr int SPT = (TE >> RL) / NT;
-    const int e = s0 + L0 - ts;
-#pragma unroll
-    for (int si = 0; si < SPT; si++) {
-        const int s = threadIdx.x + si * NT;
-        const int Tn = ((tile * NG + (s >> L0)) << L0) + (s & ((1 << L0) - 1));
-        if ((Tn >> e) & 7) continue;
-#pragma unroll
-        for (int lp = 0; lp < RL; lp++) {
-            const ulonglong2 *g = direct_base(twg, s0 + L0 + lp, ts, e, lp, Tn);
-#pragma unroll
-            for (int j = 0; j < (1 << lp); j++)
-                asm volatile("prefetch.global.L2::evict_last [%0];" ::"l"(g + ((size_t)j << ts)));
-        }
-    }
-}
+// Final stages whose twiddle runs the device table stores transposed: the
+// last round of the sixteen-element plan's contiguous pass.
+__host__ __device__ constexpr int direct_stages(int logN) { return logN >= 16 ? 4 : 3; }
 
 // The tensor product (Fig. 2 region 1 in RNS form: d0 = b1 b2, d1 = a1 b2 +
 // a2 b1, d2 = a1 a2 mod q_i) of the contiguous tile `tile` of limb i, as the
@@ -364,11 +222,10 @@ __device__ __forceinline__ void combine_store(const NttArgs &P, const NttGroup &
     const BatchItem it = job_item(P.R, (int)G.job[i]);
     const int ci = (int)(G.ci[i] & 0x7fffffffu), hh = (int)(G.ci[i] >> 31);
     const ulonglong2 pv = P.pinv[ci], qv = P.levels[it.level].qinv_last[ci];
-    // above any forward-NTT output (values grow by < 4q per stage from
-    // inputs below 4q): d + KS P^-1 (lazy, < 4q) + Cz - z stays in
-    // (0, (9 + 4 log N) q), below 2^64, and one Shoup product by
-    // q_{l-1}^-1 reduces it
-    const u64 Cz = pr.q * (u64)(4 + 4 * P.logN);
+    // at least any forward-NTT output: d + KS P^-1 (lazy, < 4q) + Cz - z
+    // stays positive and below Cz + 5q < 2^64 (ntt_mod leaves 8q of room),
+    // and one Shoup product by q_{l-1}^-1 reduces it
+    const u64 Cz = pr.nt.cz;
     u64 *o = it.out + ((((size_t)hh * (it.level - 1) + ci)) << P.logN) + g2;
     const u64 *dd = P.dst + ((size_t)G.cd[i] << P.logN) + g2, *kk = P.dst + ((size_t)G.cks[i] << P.logN) + g2;
     const u64 *sp = sm + padi(2 * threadIdx.x);
@@ -384,7 +241,7 @@ __device__ __forceinline__ void combine_store(const NttArgs &P, const NttGroup &
         }
 #pragma unroll
         for (int k = 0; k < B4; k++) {
-            // KS P^-1 lazily in [0, 4q): x < (6 + 4 log N) q < 2^64
+            // KS P^-1 lazily in [0, 4q)
             const u64 *z = sp + (b0 + k) * (2 * NT + NT / 8);
             const u64 x = dv[k].x + shoup_approx_nq(kv[k].x, pv.x, pv.y, nq) + Cz - z[0];
             const u64 y = dv[k].y + shoup_approx_nq(kv[k].y, pv.x, pv.y, nq) + Cz - z[1];
@@ -395,32 +252,25 @@ __device__ __forceinline__ void combine_store(const NttArgs &P, const NttGroup &
 }
 
 // Shared memory -> HBM for limb i of the group (same thread walk as
-// combine_store), 16-byte stores; LAST: the output reduction (forward: from
-// below (4 + 4 log N) q to [0, q); inverse: times the limb's scale).
-template <int TE, int NT, bool LAST, bool INV>
+// combine_store), 16-byte stores, with the forward transform's output
+// reduction: from any word to [0, q), one fold and two conditional
+// subtractions where the prime allows it.
+template <int TE, int NT>
 __device__ __forceinline__ void final_store(const NttArgs &P, const NttGroup &G, int i, const u64 *sm, size_t g2,
-                                            size_t gs2, const DevPrime &pr, u64 nq)
+                                            size_t gs2, const DevPrime &pr)
 {
     u64 *dst = P.dst + ((size_t)G.dst[i] << P.logN) + g2;
-    const u64 sc = G.scale[i], scs = G.scale_sh[i];
-    const bool small_red = (pr.r64 >> 32) == 0;  // q > 2^32: reduce_small applies
+    const bool fast = (pr.nt.flags & kFastFinal) != 0;
     const u64 *sp = sm + padi(2 * threadIdx.x);
 #pragma unroll
     for (int k = 0; k < TE / 2 / NT; k++) {
         u64 x = sp[0], y = sp[1];
-        if (LAST) {
-            if (!INV) {  // x < (4 + 4 log N) q
-                if (small_red) {
-                    x = reduce_small(x, pr.q, pr.r64);
-                    y = reduce_small(y, pr.q, pr.r64);
-                } else {
-                    x = shoup(x, 1, pr.r64, pr.q);
-                    y = shoup(y, 1, pr.r64, pr.q);
-                }
-            } else {
-                x = shoup_canon(x, sc, scs, pr.q, nq);
-                y = shoup_canon(y, sc, scs, pr.q, nq);
-            }
+        if (fast) {
+            x = csub(csub(fold_tw(x, pr.nt), 2 * pr.q), pr.q);
+            y = csub(csub(fold_tw(y, pr.nt), 2 * pr.q), pr.q);
+        } else {
+            x = shoup(x, 1, pr.r64, pr.q);
+            y = shoup(y, 1, pr.r64, pr.q);
         }
         *reinterpret_cast<ulonglong2 *>(dst) = make_ulonglong2(x, y);
         dst += gs2;
@@ -428,853 +278,503 @@ __device__ __forceinline__ void final_store(const NttArgs &P, const NttGroup &G,
     }
 }
 
-// One pass of LOGM stages over a group of limbs.  Rounds RA, RB, RC (RC may
-// be 0) in forward order; the inverse runs them in reverse.  FIRST: read
-// group.src (else group.dst); LAST: apply the output reduction / scaling.
-// Resident CTAs per SM the register allocation is bounded for (0: no bound):
-// 256-thread tiles (radix-8 rounds) five (51 registers; inverse ones four, 64
-// registers, as their first pass holds the direct round's twiddles from the
-// start and the tensor-fused variant its products), forward 128-thread
-// tiles six (85 registers, what their shared memory allows; measured faster
-// than the compiler's own choice), inverse 128-thread tiles unbounded (their
-// first pass holds the direct round's fifteen twiddles from the start and
-// spills under a bound).
-__host__ __device__ constexpr int ntt_min_blocks(int nt, int logm, bool inv)
-{
-    // 64-thread tiles (radix-16 rounds on 1024 elements): twelve forward (85
-    // registers), inverse unbounded
-    return logm >= 12 ? 0 : nt >= 256 ? (inv ? 4 : 5) : nt <= 64 ? (inv ? 0 : 12) : inv ? 0 : 6;
-}
-
-// FUSE: kFuseNone; kFuseCombine, the final combine in the store loop of the
-// forward contiguous last pass (ModDown + rescale limbs); kFuseTensor, the
-// tensor product computed in place of the inverse contiguous first pass's
-// tile load (d2 limbs and the rescale limbs of d0, d1).
-// kFuseIp, the key-switch sums of Fig. 2 region 2 computed in place of the
-// tile load of the special limbs' inverse contiguous first pass.
+// One pass: stages of rounds R0, R1, R2, R3 (forward order, 0: absent; the
+// inverse runs them in reverse) on tiles of TE elements of a ring of 2^LOGN,
+// each thread holding 2^E of them (E the longest round).  FUSE: kFuseNone;
+// kFuseCombine, the final combine in the store loop of the forward contiguous
+// last pass (ModDown + rescale limbs); kFuseTensor, the tensor product computed
+// in place of the inverse contiguous first pass's tile load (d2 limbs and the
+// rescale limbs of d0, d1); kFuseIp, the key-switch sums of Fig. 2 region 2
+// computed in place of the tile load of the special limbs' inverse contiguous
+// first pass.
 enum { kFuseNone = 0, kFuseCombine = 1, kFuseTensor = 2, kFuseIp = 3 };
 
-template <int LOGM, int RA, int RB, int RC, bool STRIDED, bool INV, bool FIRST, bool LAST, int TE, int FUSE = kFuseNone>
-__global__ void __launch_bounds__(TE >> cmax(RA, cmax(RB, RC)), ntt_min_blocks(TE >> cmax(RA, cmax(RB, RC)), LOGM, INV))
-k_ntt_pass(const NttArgs P)
-{
-    constexpr bool COMBINE = FUSE == kFuseCombine, TENSOR = FUSE == kFuseTensor, IPF = FUSE == kFuseIp;
-    constexpr bool COMPUTED = TENSOR || IPF;  // the tile load computes its words
-    static_assert(!COMBINE || (LAST && !INV && !STRIDED), "the combine follows a forward contiguous last pass");
-    static_assert(!COMPUTED || (FIRST && INV && !STRIDED), "computed tiles feed an inverse contiguous first pass");
-    constexpr int NT = TE >> cmax(RA, cmax(RB, RC));
-    constexpr int RL = RC ? RC : RB;  // last round in forward order
-    constexpr int L0 = LOGM - RL;     // its first stage
-    constexpr bool DIRECT = !STRIDED;
-    using Gm = Geometry<LOGM, TE, STRIDED, RL>;
-    constexpr int NG = Gm::NG;
-    static_assert(RA + RB + RC == LOGM, "rounds must cover the pass");
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    ulonglong2 *tw = reinterpret_cast<ulonglong2 *>(smem_raw);
-    u64 *buf = reinterpret_cast<u64 *>(smem_raw + sizeof(ulonglong2) * Gm::TWN);
-
-    const int gidx = blockIdx.x / P.tiles;
-    const int tile = blockIdx.x - gidx * P.tiles;
-    if (P.count && gidx >= *P.count) return idle_exit();
-    const NttGroup &G = P.groups[gidx];
-    const int nl = (int)G.nl;
-    const DevPrime pr = P.primes[G.prime];
-    const u64 nq = 0ull - pr.q;
-    const int s0 = STRIDED ? 0 : P.logN - LOGM;
-
-    // Thread walks over the tile: element threadIdx.x + k NT sits at global
-    // index g1 + k gs1 and shared word padi(threadIdx.x) + k (NT + NT / 16)
-    // (NT is a multiple of 16 and of NG); the pair 2 (threadIdx.x + k NT),
-    // +1 at g2 + k gs2 and padi(2 threadIdx.x) + k (2 NT + NT / 8).  Index
-    // arithmetic by shifts and additions only, which leaves the wide-multiply
-    // pipe to the butterflies.
-    const int lsh = P.logN - LOGM;  // log2 of the strided pass's row stride
-    const size_t g1 = STRIDED ? (((size_t)(threadIdx.x / NG) << lsh) + (size_t)tile * NG + threadIdx.x % NG)
-                              : (size_t)tile * TE + threadIdx.x;
-    const size_t gs1 = STRIDED ? ((size_t)(NT / NG) << lsh) : (size_t)NT;
-    const size_t g2 = STRIDED ? (((size_t)(2 * threadIdx.x / NG) << lsh) + (size_t)tile * NG + 2 * threadIdx.x % NG)
-                              : (size_t)tile * TE + 2 * threadIdx.x;
-    const size_t gs2 = STRIDED ? ((size_t)(2 * NT / NG) << lsh) : (size_t)(2 * NT);
-    static_assert(NT % 16 == 0 && NT % NG == 0 && (2 * NT) % NG == 0, "tile walk");
-
-    // data tile of limb i of the group -> shared memory (8-byte async copies)
-    auto load_tile = [&](int i, u64 *b) {
-        if constexpr (TENSOR) {
-            tensor_tile<TE, NT>(P, G, i, tile, pr, b);
-        } else if constexpr (IPF) {
-            ip_tile<TE, NT>(P, G, i, tile, pr, b);
-        } else {
-            const u64 *src = (FIRST ? P.src + ((size_t)G.src[i] << P.logN) : P.dst + ((size_t)G.dst[i] << P.logN)) + g1;
-            u64 *d = b + padi(threadIdx.x);
-#pragma unroll
-            for (int k = 0; k < TE / NT; k++) {
-                __pipeline_memcpy_async(d, src, 8);
-                d += NT + NT / 16;
-                src += gs1;
-            }
-        }
-    };
-    // staged twiddles of this tile -> shared memory (16-byte async copies)
-    const ulonglong2 *twg = INV ? pr.iw : pr.w;
-    if (STRIDED) {
-        for (int f = threadIdx.x; f < Gm::TWN; f += NT) __pipeline_memcpy_async(&tw[f], &twg[1 + f], 16);
-    } else {
-#pragma unroll
-        for (int l = 0; l < Gm::LS; l++) {
-            const int n = NG << l;
-            if (s0 + l < P.ts) {
-                const ulonglong2 *g = twg + (1 << (s0 + l)) + (size_t)tile * n;
-                for (int f = threadIdx.x; f < n; f += NT)
-                    __pipeline_memcpy_async(&tw[NG * ((1 << l) - 1) + f], &g[f], 16);
-            } else {  // a stage of the transposed region (radix-8 plans)
-                for (int f = threadIdx.x; f < n; f += NT)
-                    __pipeline_memcpy_async(&tw[NG * ((1 << l) - 1) + f],
-                                            &twg[tw_pos(s0 + l, P.ts, (size_t)tile * n + f)], 16);
-            }
-        }
-    }
-    if (DIRECT) prefetch_direct_tw<LOGM, TE, RL, NT>(twg, tile, s0, P.ts);
-    // the limbs come from the previous kernels; the pass that streams the key
-    // (kFuseIp) does not launch its successor early, whose waiting CTAs would
-    // hold SM slots its last loads need (measured: 2^17 985 against 992 µs)
-    griddep_wait(P.pdl >= 2 && FUSE != kFuseIp);
-    load_tile(0, buf);
-    __pipeline_commit();
-
-    // the direct round's twiddles -> registers (reloaded for every limb from
-    // L2 so that they are live only during that round), from the table's
-    // transposed runs (direct_base).
-    constexpr int SPT = (TE >> RL) / NT;
-    const int te = s0 + L0 - P.ts;
-    auto load_direct = [&](TwReg<RL, SPT> &T) {
-#pragma unroll
-        for (int si = 0; si < SPT; si++) {
-            const int s = threadIdx.x + si * NT;
-            const int khi = s & ((1 << L0) - 1);
-            const int gg = tile * NG + (s >> L0);
-            const int Tn = (gg << L0) + khi;
-#pragma unroll
-            for (int lp = 0; lp < RL; lp++) {
-                const ulonglong2 *g = direct_base(twg, s0 + L0 + lp, P.ts, te, lp, Tn);
-#pragma unroll
-                for (int j = 0; j < (1 << lp); j++) T.t[si][(1 << lp) - 1 + j] = ld_tw(g + ((size_t)j << P.ts));
-            }
-        }
-    };
-
-    for (int i = 0; i < nl; i++) {
-        u64 *sm = buf + (i & 1) * Gm::DATA;
-        TwReg<RL, SPT> TR;
-        // the inverse starts with the direct round (its twiddles are loaded
-        // after the next limb's computed tile, which needs the registers)
-        if (DIRECT && INV && !COMPUTED) load_direct(TR);
-        if (i + 1 < nl) {
-            load_tile(i + 1, buf + ((i + 1) & 1) * Gm::DATA);
-            __pipeline_commit();
-            __pipeline_wait_prior(1);
-        } else {
-            __pipeline_wait_prior(0);
-        }
-        if (DIRECT && INV && COMPUTED) load_direct(TR);
-        __syncthreads();
-        if (!INV) {
-            ntt_round<LOGM, TE, RA, STRIDED, false, NT, false>(sm, tw, TR, 0, nq, pr.q4);
-            if (DIRECT && RC == 0) load_direct(TR);
-            __syncthreads();
-            ntt_round<LOGM, TE, RB, STRIDED, false, NT, DIRECT && RC == 0>(sm, tw, TR, RA, nq, pr.q4);
-            if (DIRECT && RC != 0) load_direct(TR);
-            __syncthreads();
-            if (RC) {
-                ntt_round<LOGM, TE, (RC ? RC : 1), STRIDED, false, NT, DIRECT>(sm, tw, TR, RA + RB, nq, pr.q4);
-                __syncthreads();
-            }
-        } else {
-            if (RC) {
-                ntt_round<LOGM, TE, (RC ? RC : 1), STRIDED, true, NT, DIRECT>(sm, tw, TR, RA + RB, nq, pr.q4);
-                __syncthreads();
-            }
-            ntt_round<LOGM, TE, RB, STRIDED, true, NT, DIRECT && RC == 0>(sm, tw, TR, RA, nq, pr.q4);
-            __syncthreads();
-            ntt_round<LOGM, TE, RA, STRIDED, true, NT, false>(sm, tw, TR, 0, nq, pr.q4);
-            __syncthreads();
-        }
-        if (COMBINE) {
-            combine_store<TE, NT>(P, G, i, sm, g2, gs2, pr, nq);
-            __syncthreads();  // the next prefetch reuses this buffer
-            continue;
-        }
-        final_store<TE, NT, LAST, INV>(P, G, i, sm, g2, gs2, pr, nq);
-        __syncthreads();  // the next prefetch reuses this buffer
-    }
-}
-
-// ngroups == 0 only sets the kernel's shared-memory limit (no launch).
-template <int LOGM, int RA, int RB, int RC, bool STRIDED, bool INV, bool FIRST, bool LAST, int TE, int FUSE = kFuseNone>
-cudaError_t run_pass(const NttArgs &a, int ngroups, cudaStream_t st)
-{
-    constexpr int NT = TE >> cmax(RA, cmax(RB, RC));
-    constexpr size_t smem = Geometry<LOGM, TE, STRIDED, (RC ? RC : RB)>::SMEM;
-    auto kern = k_ntt_pass<LOGM, RA, RB, RC, STRIDED, INV, FIRST, LAST, TE, FUSE>;
-    static bool configured = false;  // once per instantiation
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
-    if (ngroups == 0) return cudaSuccess;
-    launch_k(a.pdl != 0, kern, dim3(ngroups * a.tiles), dim3(NT), smem, st, a);
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// One-pass transform of N = 2^16 over a thread-block cluster.
-//
-// The limb is cut into kCl = 8 contiguous chunks of TE = N / 8 elements, one
-// per CTA of a cluster, each held in its CTA's shared memory.  Stages 0-2
-// pair elements of different chunks (stage sigma pairs j and
-// j + N / 2^(sigma+1) with twiddle 2^sigma + floor(j / 2^(16 - sigma)), which
-// depends only on the chunk of j): for every offset k of a chunk they form one
-// radix-8 set {v TE + k : v < 8} with the twiddles of entries 1..7.  CTA r
-// runs those sets for the offsets [r TE / 8, (r + 1) TE / 8) and moves the
-// values between the CTAs through distributed shared memory; stages 3-15 are
-// the contiguous pass of one group (s0 = 3, LOGM = 13, tile r of the limb).
-// Forward: the cross round reads HBM and writes every chunk into its CTA's
-// shared memory, then the local rounds, then the output reduction (or the
-// final combine) and the store.  Inverse: the chunk is loaded (or formed by
-// the tensor product), local rounds in reverse, then the cross round reads the
-// chunks from the cluster's shared memory, scales and stores.  The limb makes
-// one trip through HBM instead of two; every butterfly is the one the two-pass
-// plans apply to the same operands, so every output word equals theirs.
-constexpr int kCl = 8;                  // CTAs per cluster (portable size)
-constexpr int kClLogN = 16;             // ring size of the plan
-constexpr int kClTE = (1 << kClLogN) / kCl;
-constexpr int kClLogM = kClLogN - 3;    // local stages 3 .. 15
-
-__device__ __forceinline__ unsigned cl_rank()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-// Barrier over every thread of the cluster; shared-memory writes before it
-// (local or remote) are visible to every thread after it.
-__device__ __forceinline__ void cl_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// Address in the cluster's shared window of the word `p` of this CTA's
-// shared memory as held by CTA `rank`.
-__device__ __forceinline__ uint32_t cl_map(const void *p, unsigned rank)
-{
-    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-
-__device__ __forceinline__ void cl_st(uint32_t a, u64 v)
-{
-    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ u64 cl_ld(uint32_t a)
-{
-    u64 v;
-    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
-    return v;
-}
-
-// Stages 0-2 on one radix-8 set (element v of the set in a[v]), twiddle
-// entry 2^l + (v >> (3 - l)) of stage l at w[2^l - 1 + (v >> (3 - l))].
-__device__ __forceinline__ void cross_fwd(u64 (&a)[8], const ulonglong2 (&w)[7], u64 nq, u64 q4)
-{
-#pragma unroll
-    for (int l = 0; l < 3; l++) {
-        const int h = 4 >> l;
-#pragma unroll
-        for (int v = 0; v < 8; v++)
-            if (!(v & h)) ct_bfly(a[v], a[v + h], w[(1 << l) - 1 + (v >> (3 - l))], nq, q4);
-    }
-}
-
-__device__ __forceinline__ void cross_inv(u64 (&a)[8], const ulonglong2 (&w)[7], u64 nq, u64 q4)
-{
-#pragma unroll
-    for (int l = 2; l >= 0; l--) {
-        const int h = 4 >> l;
-#pragma unroll
-        for (int v = 0; v < 8; v++)
-            if (!(v & h)) gs_bfly(a[v], a[v + h], w[(1 << l) - 1 + (v >> (3 - l))], nq, q4);
-    }
-}
-
-// Local rounds R0..R4 in forward order (R4 = 0: four rounds); the last one
-// is the direct round.  NT threads: one set of the widest round each.
-template <int R0, int R1, int R2, int R3, int R4>
-struct ClGeom {
-    static constexpr int RMAX = cmax(cmax(cmax(R0, R1), cmax(R2, R3)), R4);
-    static constexpr int NT = kClTE >> RMAX;
-    static constexpr int RL = R4 ? R4 : R3;
-    using Gm = Geometry<kClLogM, kClTE, false, RL>;
-    static constexpr size_t SMEM = sizeof(ulonglong2) * Gm::TWN + sizeof(u64) * Gm::DATA;  // one data buffer
+template <int LOGN_, bool STRIDED_, int R0, int R1, int R2, int R3, int TE_>
+struct Pass {
+    static constexpr int LOGN = LOGN_, TE = TE_;
+    static constexpr bool STRIDED = STRIDED_;
+    static constexpr int LOGM = R0 + R1 + R2 + R3, M = 1 << LOGM, NG = TE / M;
+    static constexpr int E = cmax(cmax(R0, R1), cmax(R2, R3)), NT = TE >> E;
+    static constexpr int S0 = STRIDED ? 0 : LOGN - LOGM;        // first stage
+    static constexpr int ROUNDS = R3 ? 4 : R2 ? 3 : 2;
+    static constexpr int RL = R3 ? R3 : R2 ? R2 : R1;           // last round in forward order
+    static constexpr int TILES = (1 << LOGN) / TE;              // per limb
+    static constexpr int TS = LOGN - direct_stages(LOGN);       // stages from TS on are stored transposed
+    static constexpr bool WHOLE = LOGM == LOGN;                 // a single pass
+    static constexpr int TWN = STRIDED ? M - 1 : NG * ((1 << (LOGM - RL)) - 1);  // staged twiddles
+    static constexpr size_t SMEM = sizeof(ulonglong2) * TWN + sizeof(u64) * (TE + TE / 16);
+    static_assert(R0 > 0 && R1 > 0, "at least two rounds");
+    static_assert(TE % M == 0 && (STRIDED || S0 + LOGM == LOGN), "tiles of whole groups");
 };
 
-template <int R0, int R1, int R2, int R3, int R4, bool INV, int FUSE>
-__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(ClGeom<R0, R1, R2, R3, R4>::NT, 1)
-k_ntt_cluster(const NttArgs P)
-{
-    constexpr bool COMBINE = FUSE == kFuseCombine, TENSOR = FUSE == kFuseTensor;
-    static_assert(!COMBINE || !INV, "the combine follows a forward transform");
-    static_assert(!TENSOR || INV, "the tensor product feeds an inverse transform");
-    using CG = ClGeom<R0, R1, R2, R3, R4>;
-    using Gm = typename CG::Gm;
-    constexpr int LOGM = kClLogM, TE = kClTE, NT = CG::NT, RL = CG::RL, L0 = LOGM - RL;
-    static_assert(R0 + R1 + R2 + R3 + R4 == LOGM, "rounds must cover the local stages");
-    static_assert(Gm::NG == 1, "one group per chunk");
-    constexpr int CK = TE / kCl;    // cross-round offsets per CTA
-    constexpr int CPT = CK / NT;    // per thread: consecutive offsets k0 .. k0 + CPT - 1
-    static_assert(CPT * NT == CK && (CPT == 1 || CPT == 2), "one or two offsets per thread in the cross round");
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    ulonglong2 *tw = reinterpret_cast<ulonglong2 *>(smem_raw);
-    u64 *sm = reinterpret_cast<u64 *>(smem_raw + sizeof(ulonglong2) * Gm::TWN);
-
-    const int tile = (int)cl_rank();  // the chunk this CTA holds
-    const int gidx = blockIdx.x / kCl;
-    if (P.count && gidx >= *P.count) return idle_exit();  // the whole cluster leaves
-    const NttGroup &G = P.groups[gidx];
-    const int nl = (int)G.nl;
-    const DevPrime pr = P.primes[G.prime];
-    const u64 nq = 0ull - pr.q;
-    constexpr int s0 = 3;
-    const ulonglong2 *twg = INV ? pr.iw : pr.w;
-    // the local rounds' staged twiddles (stages s0 + l, l < LS, of this tile)
-#pragma unroll
-    for (int l = 0; l < Gm::LS; l++) {
-        const int n = 1 << l;
-        if (s0 + l < P.ts) {
-            const ulonglong2 *g = twg + (1 << (s0 + l)) + (size_t)tile * n;
-            for (int f = threadIdx.x; f < n; f += NT) __pipeline_memcpy_async(&tw[n - 1 + f], &g[f], 16);
+// Set `si` (of 2^(E-R)) of this thread in the round of stages [L0, L0 + R):
+// element v of the set is in-group index k = (khi << (LOGM - L0)) |
+// (v << LO) | klo of group (or column) grp, LO = LOGM - L0 - R.  The lowest
+// thread bits walk the words that are consecutive in memory.
+template <class P, int L0, int R>
+struct RoundSet {
+    static constexpr int LO = P::LOGM - L0 - R, SPT = 1 << (P::E - R);
+    int grp, khi, klo;
+    __device__ __forceinline__ explicit RoundSet(int si)
+    {
+        const int s = threadIdx.x + si * P::NT;
+        if (P::STRIDED) {
+            grp = s % P::NG;
+            klo = (s / P::NG) & ((1 << LO) - 1);
+            khi = (s / P::NG) >> LO;
         } else {
-            for (int f = threadIdx.x; f < n; f += NT)
-                __pipeline_memcpy_async(&tw[n - 1 + f], &twg[tw_pos(s0 + l, P.ts, (size_t)tile * n + f)], 16);
+            klo = s & ((1 << LO) - 1);
+            khi = (s >> LO) & ((1 << L0) - 1);
+            grp = s >> (LO + L0);
         }
+    }
+    __device__ __forceinline__ int k() const { return (khi << (P::LOGM - L0)) | klo; }
+    // tile-linear index of element 0, and the step to element v
+    __device__ __forceinline__ int lin() const { return P::STRIDED ? k() * P::NG + grp : grp * P::M + k(); }
+    static __device__ __forceinline__ constexpr int step(int v) { return (v << LO) * (P::STRIDED ? P::NG : 1); }
+    // word of the limb
+    __device__ __forceinline__ size_t word(int tile) const
+    {
+        return P::STRIDED ? ((size_t)k() << (P::LOGN - P::LOGM)) + (size_t)(tile * P::NG + grp)
+                          : (size_t)tile * P::TE + lin();
+    }
+    static __device__ __forceinline__ constexpr size_t wstep(int v)
+    {
+        return P::STRIDED ? (size_t)(v << LO) << (P::LOGN - P::LOGM) : (size_t)step(v);
+    }
+};
+
+// Shared-memory words of a set: one pad word per 16.  Element v's offset has
+// no bit in common with element 0's index, so the padding of the sum splits
+// into the base's and a compile-time one.
+template <class P, int L0, int R>
+__device__ __forceinline__ void smem_put(u64 *sm, const u64 (&a)[1 << P::E])
+{
+    using S = RoundSet<P, L0, R>;
+#pragma unroll
+    for (int si = 0; si < S::SPT; si++) {
+        u64 *b = sm + padi(S(si).lin());
+#pragma unroll
+        for (int v = 0; v < (1 << R); v++) b[S::step(v) + (S::step(v) >> 4)] = a[(si << R) + v];
+    }
+}
+template <class P, int L0, int R>
+__device__ __forceinline__ void smem_get(const u64 *sm, u64 (&a)[1 << P::E])
+{
+    using S = RoundSet<P, L0, R>;
+#pragma unroll
+    for (int si = 0; si < S::SPT; si++) {
+        const u64 *b = sm + padi(S(si).lin());
+#pragma unroll
+        for (int v = 0; v < (1 << R); v++) a[(si << R) + v] = b[S::step(v) + (S::step(v) >> 4)];
+    }
+}
+template <class P, int L0, int R>
+__device__ __forceinline__ void mem_get(const u64 *src, int tile, u64 (&a)[1 << P::E])
+{
+    using S = RoundSet<P, L0, R>;
+#pragma unroll
+    for (int si = 0; si < S::SPT; si++) {
+        const u64 *b = src + S(si).word(tile);
+#pragma unroll
+        for (int v = 0; v < (1 << R); v++) a[(si << R) + v] = b[S::wstep(v)];
+    }
+}
+
+// Base and step (per j) of the twiddles of local stage l = L0 + lp for the
+// sets with T0 = (G << L0) + khi: twiddle j of the stage is entry
+// t = (T0 << lp) + j of the run of stage sigma.  The runs of stages
+// sigma >= TS are stored transposed (with d = sigma - TS, entry t at
+// (t mod 2^d) 2^TS + floor(t / 2^d)), so that a warp whose sets are
+// consecutive reads consecutive entries per j.
+template <class P, int L0>
+__device__ __forceinline__ const ulonglong2 *tw_entry(const ulonglong2 *twg, int T0, int lp, int j)
+{
+    const int sigma = P::S0 + L0 + lp, d = sigma - P::TS;
+    const ulonglong2 *run = twg + ((size_t)1 << sigma);
+    if (d <= 0) return run + ((size_t)T0 << lp) + j;
+    if (d <= lp) return run + ((size_t)(j & ((1 << d) - 1)) << P::TS) + ((size_t)T0 << (lp - d)) + (j >> d);
+    const int e = d - lp;
+    return run + ((size_t)(((T0 & ((1 << e) - 1)) << lp) + j) << P::TS) + (T0 >> e);
+}
+
+// Staged twiddles (shared memory): the strided pass keeps TB_W[1, M), which
+// every tile uses; the contiguous pass the runs of its tile for the stages
+// before the last round, stage l of group grp at NG (2^l - 1) + (grp << l).
+template <class P>
+__device__ __forceinline__ void stage_twiddles(ulonglong2 *tw, const ulonglong2 *twg, int tile)
+{
+    if constexpr (P::STRIDED) {
+        for (int f = threadIdx.x; f < P::TWN; f += P::NT) __pipeline_memcpy_async(&tw[f], &twg[1 + f], 16);
+    } else {
+#pragma unroll
+        for (int l = 0; l < P::LOGM - P::RL; l++)
+            for (int f = threadIdx.x; f < (P::NG << l); f += P::NT)
+                __pipeline_memcpy_async(&tw[P::NG * ((1 << l) - 1) + f],
+                                        tw_entry<P, 0>(twg, 0, l, tile * (P::NG << l) + f), 16);
     }
     __pipeline_commit();
-    prefetch_direct_tw<LOGM, TE, RL, NT>(twg, tile, s0, P.ts);
-    // this thread's cross-round offsets and their words in every CTA's shared memory
-    const int k0 = tile * CK + CPT * threadIdx.x;
-    uint32_t ko[CPT];
-#pragma unroll
-    for (int c = 0; c < CPT; c++) ko[c] = 8u * (uint32_t)padi(k0 + c);
-    uint32_t rb[kCl];
-#pragma unroll
-    for (int v = 0; v < kCl; v++) rb[v] = cl_map(sm, (unsigned)v);
-    // the chunk's thread walk (as the contiguous pass with one tile per limb)
-    const size_t g2 = (size_t)tile * TE + 2 * threadIdx.x, gs2 = 2 * NT;
+}
 
-    constexpr int SPT = (TE >> RL) / NT;
-    const int te = s0 + L0 - P.ts;
-    auto load_direct = [&](TwReg<RL, SPT> &T) {
+// Where a round's twiddles come from: the staged ones, or registers loaded
+// ahead (the contiguous pass's last round, whose twiddles one thread uses
+// once: entry 2^lp - 1 + j of stage L0 + lp).
+template <class P, int L0>
+struct TwSmem {
+    const ulonglong2 *tw;
+    int grp, khi;
+    __device__ __forceinline__ ulonglong2 get(int lp, int j) const
+    {
+        const int l = L0 + lp;
+        return P::STRIDED ? tw[(1 << l) - 1 + (khi << lp) + j]
+                          : tw[P::NG * ((1 << l) - 1) + (grp << l) + (khi << lp) + j];
+    }
+};
+template <int R>
+struct TwRegs {
+    ulonglong2 w[(1 << R) - 1];
+    __device__ __forceinline__ ulonglong2 get(int lp, int j) const { return w[(1 << lp) - 1 + j]; }
+};
+// Stages [LP0, LP1) of the last round's twiddles of set si -> registers.
+template <class P, int LP0, int LP1>
+__device__ __forceinline__ void load_last(TwRegs<P::RL> &t, const ulonglong2 *twg, int tile, int si)
+{
+    constexpr int L0 = P::LOGM - P::RL;
+    const RoundSet<P, L0, P::RL> st(si);
+    const int T0 = ((tile * P::NG + st.grp) << L0) + st.khi;
 #pragma unroll
-        for (int si = 0; si < SPT; si++) {
-            const int s = threadIdx.x + si * NT;
-            const int Tn = ((tile + (s >> L0)) << L0) + (s & ((1 << L0) - 1));
+    for (int lp = LP0; lp < LP1; lp++)
 #pragma unroll
-            for (int lp = 0; lp < RL; lp++) {
-                const ulonglong2 *g = direct_base(twg, s0 + L0 + lp, P.ts, te, lp, Tn);
+        for (int j = 0; j < (1 << lp); j++) t.w[(1 << lp) - 1 + j] = ld_tw(tw_entry<P, L0>(twg, T0, lp, j));
+}
+
+// Stage L0 + LP of a round on one set of the thread's registers.
+template <int R, int LP, bool INV, class TW>
+__device__ __forceinline__ void stage_regs(u64 *x, const TW &tw, const NttMod &km)
+{
+    constexpr int H = 1 << (R - 1 - LP);
 #pragma unroll
-                for (int j = 0; j < (1 << lp); j++) T.t[si][(1 << lp) - 1 + j] = ld_tw(g + ((size_t)j << P.ts));
-            }
+    for (int j = 0; j < (1 << LP); j++) {
+        const ulonglong2 w = tw.get(LP, j);
+#pragma unroll
+        for (int v = 0; v < H; v++) {
+            const int i = (j << (R - LP)) + v;
+            if (INV) gs_bfly(x[i], x[i + H], w, km);
+            else ct_bfly(x[i], x[i + H], w, km);
         }
-    };
+    }
+    if (!INV && R > 2 && LP == 1 && (km.flags & kFwdFoldSecond)) {
+#pragma unroll
+        for (int v = 0; v < (1 << R); v++) x[v] = fold_tw(x[v], km);
+    }
+    if (INV && R > 2 && LP == R - 2 && (km.flags & kInvFoldSecond)) {
+#pragma unroll
+        for (int v = 0; v < (1 << R); v++)
+            if (!(v & H)) x[v] = fold_tw(x[v], km);
+    }
+}
 
-    griddep_wait(P.pdl >= 2);  // the limbs come from the previous kernels
+template <int R, bool INV, class TW, int... LP>
+__device__ __forceinline__ void stages_regs(std::integer_sequence<int, LP...>, u64 *x, const TW &tw, const NttMod &km)
+{
+    (stage_regs<R, INV ? R - 1 - LP : LP, INV>(x, tw, km), ...);
+}
+
+// All stages of a round on one set.
+template <int R, bool INV, class TW>
+__device__ __forceinline__ void set_stages(u64 *x, const TW &tw, const NttMod &km)
+{
+    stages_regs<R, INV>(std::make_integer_sequence<int, R>(), x, tw, km);
+    if (!INV && (km.flags & kFwdFoldRound)) {
+#pragma unroll
+        for (int v = 0; v < (1 << R); v++) x[v] = fold_tw(x[v], km);
+    }
+    if (INV) {
+        // the sums of the last stage; the products only where the prime needs it
+#pragma unroll
+        for (int v = 0; v < (1 << R) / 2; v++) x[v] = fold_tw(x[v], km);
+        if (km.flags & kInvFoldAll) {
+#pragma unroll
+            for (int v = (1 << R) / 2; v < (1 << R); v++) x[v] = fold_tw(x[v], km);
+        }
+    }
+}
+
+// The stages [L0, L0 + R) on the thread's registers, twiddles staged.
+template <class P, int L0, int R, bool INV>
+__device__ __forceinline__ void round_regs(u64 (&a)[1 << P::E], const ulonglong2 *tw, const NttMod &km)
+{
+    using S = RoundSet<P, L0, R>;
+#pragma unroll
+    for (int si = 0; si < S::SPT; si++) {
+        const S st(si);
+        const TwSmem<P, L0> t = {tw, st.grp, st.khi};
+        set_stages<R, INV>(a + (si << R), t, km);
+    }
+}
+
+// L2 prefetch of the lines the contiguous pass's last round will read (one
+// thread per 128-byte line); issued when a CTA starts, before it waits for the
+// previous kernel.
+template <class P>
+__device__ __forceinline__ void prefetch_last_round(const ulonglong2 *twg, int tile)
+{
+    constexpr int L0 = P::LOGM - P::RL;
+    using S = RoundSet<P, L0, P::RL>;
+    constexpr int e = P::S0 + L0 - P::TS;  // consecutive entries: the sets whose floor(T0 / 2^e) differ
+#pragma unroll
+    for (int si = 0; si < S::SPT; si++) {
+        const S st(si);
+        const int T0 = ((tile * P::NG + st.grp) << L0) + st.khi;
+        if ((T0 >> (e > 0 ? e : 0)) & 7) continue;
+#pragma unroll
+        for (int lp = 0; lp < P::RL; lp++)
+#pragma unroll
+            for (int j = 0; j < (1 << lp); j++)
+                asm volatile("prefetch.global.L2::evict_last [%0];" ::"l"(tw_entry<P, L0>(twg, T0, lp, j)));
+    }
+}
+
+// Resident CTAs per SM the register allocation is bounded for.
+__host__ __device__ constexpr int ntt_min_blocks(int nt) { return nt >= 512 ? 1 : nt >= 256 ? 4 : nt >= 128 ? 5 : 8; }
+
+template <class P, int R0, int R1, int R2, int R3, bool INV, int FUSE>
+__global__ void __launch_bounds__(P::NT, ntt_min_blocks(P::NT)) k_ntt_pass(const NttArgs A)
+{
+    constexpr bool STRIDED = P::STRIDED, COMBINE = FUSE == kFuseCombine;
+    constexpr bool COMPUTED = FUSE == kFuseTensor || FUSE == kFuseIp;  // the tile load computes its words
+    constexpr bool FIRST = P::WHOLE || STRIDED != INV, LAST = P::WHOLE || STRIDED == INV;
+    static_assert(!COMBINE || (LAST && !INV && !STRIDED), "the combine follows a forward contiguous last pass");
+    static_assert(!COMPUTED || (FIRST && INV && !STRIDED), "computed tiles feed an inverse contiguous first pass");
+    constexpr int TE = P::TE, NT = P::NT, RL = P::RL, LL = P::LOGM - RL;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ulonglong2 *tw = reinterpret_cast<ulonglong2 *>(smem_raw);
+    u64 *sm = reinterpret_cast<u64 *>(tw + P::TWN);
+
+    const int gidx = blockIdx.x / P::TILES, tile = blockIdx.x % P::TILES;
+    if (A.count && gidx >= *A.count) return idle_exit();
+    const NttGroup &G = A.groups[gidx];
+    const int nl = (int)G.nl;
+    const DevPrime pr = A.primes[G.prime];
+    const NttMod &km = pr.nt;
+    const u64 nq = 0ull - pr.q;
+    const ulonglong2 *twg = INV ? pr.iw : pr.w;
+    // the tables are static: staged, and the last round's lines brought to L2,
+    // while the previous kernel still runs
+    stage_twiddles<P>(tw, twg, tile);
+    if (!STRIDED) prefetch_last_round<P>(twg, tile);
+    // the limbs come from the previous kernels; the pass that streams the key
+    // (kFuseIp) does not launch its successor early, whose waiting CTAs would
+    // hold SM slots its last loads need (measured: 2^17 985 against 992 us)
+    griddep_wait(A.pdl >= 2 && FUSE != kFuseIp);
+    const size_t g2 = (size_t)tile * TE + 2 * threadIdx.x, gs2 = 2 * NT;  // coalesced pairs of a contiguous tile
+
+    using SL = RoundSet<P, LL, RL>;
     for (int i = 0; i < nl; i++) {
-        TwReg<RL, SPT> TR;
-        ulonglong2 cw[7];
-#pragma unroll
-        for (int t = 0; t < 7; t++) cw[t] = ld_tw(twg + 1 + t);
-        if (!INV) {
-            const u64 *src = P.src + ((size_t)G.src[i] << P.logN);
-            u64 a[CPT][8];
-#pragma unroll
-            for (int v = 0; v < 8; v++) {
-                if constexpr (CPT == 2) {
-                    const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(src + (size_t)v * TE + k0);
-                    a[0][v] = x.x;
-                    a[CPT - 1][v] = x.y;
-                } else {
-                    a[0][v] = src[(size_t)v * TE + k0];
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < CPT; c++) cross_fwd(a[c], cw, nq, pr.q4);
-            cl_sync();  // every CTA of the cluster runs and is done with its previous chunk
-#pragma unroll
-            for (int v = 0; v < 8; v++)
-#pragma unroll
-                for (int c = 0; c < CPT; c++) cl_st(rb[v] + ko[c], a[c][v]);
-            __pipeline_wait_prior(0);  // this thread's staged twiddles
-            cl_sync();                 // every chunk complete, the twiddles visible
-            ntt_round<LOGM, TE, R0, false, false, NT, false>(sm, tw, TR, 0, nq, pr.q4);
-            __syncthreads();
-            ntt_round<LOGM, TE, R1, false, false, NT, false>(sm, tw, TR, R0, nq, pr.q4);
-            __syncthreads();
-            ntt_round<LOGM, TE, R2, false, false, NT, false>(sm, tw, TR, R0 + R1, nq, pr.q4);
-            if constexpr (R4 != 0) {
+        const u64 *src = FIRST ? A.src + ((size_t)G.src[i] << P::LOGN) : A.dst + ((size_t)G.dst[i] << P::LOGN);
+        u64 *dst = A.dst + ((size_t)G.dst[i] << P::LOGN);
+        u64 a[1 << P::E];
+        if constexpr (!INV) {
+            mem_get<P, 0, R0>(src, tile, a);
+            if (i == 0) __pipeline_wait_prior(0);
+            __syncthreads();  // the staged twiddles; the previous limb's words have been read
+            round_regs<P, 0, R0, false>(a, tw, km);
+            smem_put<P, 0, R0>(sm, a);
+            if constexpr (P::ROUNDS > 2) {
                 __syncthreads();
-                ntt_round<LOGM, TE, R3, false, false, NT, false>(sm, tw, TR, R0 + R1 + R2, nq, pr.q4);
+                smem_get<P, R0, R1>(sm, a);
+                round_regs<P, R0, R1, false>(a, tw, km);
+                smem_put<P, R0, R1>(sm, a);  // the words this thread read
             }
-            load_direct(TR);
-            __syncthreads();
-            ntt_round<LOGM, TE, RL, false, false, NT, true>(sm, tw, TR, L0, nq, pr.q4);
-            __syncthreads();
-            if (COMBINE) combine_store<TE, NT>(P, G, i, sm, g2, gs2, pr, nq);
-            else final_store<TE, NT, true, false>(P, G, i, sm, g2, gs2, pr, nq);
-        } else {
-            if (i > 0) cl_sync();  // the peers are done reading this CTA's previous chunk
-            if constexpr (TENSOR) {
-                tensor_tile<TE, NT>(P, G, i, tile, pr, sm);
+            if constexpr (P::ROUNDS > 3) {
+                __syncthreads();
+                smem_get<P, R0 + R1, R2>(sm, a);
+                round_regs<P, R0 + R1, R2, false>(a, tw, km);
+                smem_put<P, R0 + R1, R2>(sm, a);
+            }
+            if constexpr (STRIDED) {
+                __syncthreads();
+                smem_get<P, LL, RL>(sm, a);
+                round_regs<P, LL, RL, false>(a, tw, km);
+                const bool mid = (km.flags & kFwdFoldPass) != 0;
+#pragma unroll
+                for (int si = 0; si < SL::SPT; si++) {
+                    u64 *d = dst + SL(si).word(tile);
+#pragma unroll
+                    for (int v = 0; v < (1 << RL); v++) {
+                        u64 x = a[(si << RL) + v];
+                        if (mid) x = fold_tw(x, km);
+                        d[SL::wstep(v)] = x;
+                    }
+                }
             } else {
-                const u64 *src = P.src + ((size_t)G.src[i] << P.logN) + (size_t)tile * TE + threadIdx.x;
-                u64 *d = sm + padi(threadIdx.x);
+                // the last round's twiddles but its last stage's travel while the
+                // words are exchanged, the last stage's during the stages before it
+                TwRegs<RL> t;
+                load_last<P, 0, RL - 1>(t, twg, tile, 0);
+                __syncthreads();
+                smem_get<P, LL, RL>(sm, a);
 #pragma unroll
-                for (int k = 0; k < TE / NT; k++) {
-                    __pipeline_memcpy_async(d, src, 8);
-                    d += NT + NT / 16;
-                    src += NT;
+                for (int si = 0; si < SL::SPT; si++) {
+                    if (si) load_last<P, 0, RL - 1>(t, twg, tile, si);
+                    load_last<P, RL - 1, RL>(t, twg, tile, si);
+                    set_stages<RL, false>(a + (si << RL), t, km);
                 }
-                __pipeline_commit();
+                smem_put<P, LL, RL>(sm, a);
+                __syncthreads();
+                if constexpr (COMBINE) combine_store<TE, NT>(A, G, i, sm, g2, gs2, pr, nq);
+                else final_store<TE, NT>(A, G, i, sm, g2, gs2, pr);
             }
-            load_direct(TR);
-            __pipeline_wait_prior(0);
+        } else {
+            if constexpr (STRIDED) {
+                mem_get<P, LL, RL>(src, tile, a);
+                if (i == 0) __pipeline_wait_prior(0);
+                __syncthreads();  // as above
+                round_regs<P, LL, RL, true>(a, tw, km);
+            } else {
+                TwRegs<RL> t;
+                if constexpr (!COMPUTED) load_last<P, RL - 1, RL>(t, twg, tile, 0);
+                if (i) __syncthreads();  // the previous limb's words have been read
+                if constexpr (FUSE == kFuseTensor) {
+                    tensor_tile<TE, NT>(A, G, i, tile, pr, sm);
+                } else if constexpr (FUSE == kFuseIp) {
+                    ip_tile<TE, NT>(A, G, i, tile, pr, sm);
+                } else {
+                    const u64 *p = src + (size_t)tile * TE + threadIdx.x;
+                    u64 *d = sm + padi(threadIdx.x);
+#pragma unroll
+                    for (int k = 0; k < TE / NT; k++) __pipeline_memcpy_async(d + k * (NT + NT / 16), p + k * NT, 8);
+                    __pipeline_commit();
+                }
+                if constexpr (COMPUTED) load_last<P, RL - 1, RL>(t, twg, tile, 0);
+                __pipeline_wait_prior(0);
+                __syncthreads();
+                smem_get<P, LL, RL>(sm, a);
+#pragma unroll
+                for (int si = 0; si < SL::SPT; si++) {
+                    if (si) load_last<P, RL - 1, RL>(t, twg, tile, si);
+                    load_last<P, 0, RL - 1>(t, twg, tile, si);
+                    set_stages<RL, true>(a + (si << RL), t, km);
+                }
+            }
+            smem_put<P, LL, RL>(sm, a);
             __syncthreads();
-            ntt_round<LOGM, TE, RL, false, true, NT, true>(sm, tw, TR, L0, nq, pr.q4);
-            __syncthreads();
-            if constexpr (R4 != 0) {
-                ntt_round<LOGM, TE, R3, false, true, NT, false>(sm, tw, TR, R0 + R1 + R2, nq, pr.q4);
+            if constexpr (P::ROUNDS > 3) {
+                smem_get<P, R0 + R1, R2>(sm, a);
+                round_regs<P, R0 + R1, R2, true>(a, tw, km);
+                smem_put<P, R0 + R1, R2>(sm, a);
                 __syncthreads();
             }
-            ntt_round<LOGM, TE, R2, false, true, NT, false>(sm, tw, TR, R0 + R1, nq, pr.q4);
-            __syncthreads();
-            ntt_round<LOGM, TE, R1, false, true, NT, false>(sm, tw, TR, R0, nq, pr.q4);
-            __syncthreads();
-            ntt_round<LOGM, TE, R0, false, true, NT, false>(sm, tw, TR, 0, nq, pr.q4);
-            cl_sync();  // every chunk transformed
-            u64 a[CPT][8];
-#pragma unroll
-            for (int v = 0; v < 8; v++)
-#pragma unroll
-                for (int c = 0; c < CPT; c++) a[c][v] = cl_ld(rb[v] + ko[c]);
-#pragma unroll
-            for (int c = 0; c < CPT; c++) cross_inv(a[c], cw, nq, pr.q4);
-            u64 *dst = P.dst + ((size_t)G.dst[i] << P.logN) + k0;
+            if constexpr (P::ROUNDS > 2) {
+                smem_get<P, R0, R1>(sm, a);
+                round_regs<P, R0, R1, true>(a, tw, km);
+                smem_put<P, R0, R1>(sm, a);
+                __syncthreads();
+            }
+            smem_get<P, 0, R0>(sm, a);
+            round_regs<P, 0, R0, true>(a, tw, km);
             const u64 sc = G.scale[i], scs = G.scale_sh[i];
+            using S = RoundSet<P, 0, R0>;
 #pragma unroll
-            for (int v = 0; v < 8; v++) {
-                if constexpr (CPT == 2)
-                    *reinterpret_cast<ulonglong2 *>(dst + (size_t)v * TE) = make_ulonglong2(
-                        shoup_canon(a[0][v], sc, scs, pr.q, nq), shoup_canon(a[CPT - 1][v], sc, scs, pr.q, nq));
-                else
-                    dst[(size_t)v * TE] = shoup_canon(a[0][v], sc, scs, pr.q, nq);
+            for (int si = 0; si < S::SPT; si++) {
+                u64 *d = dst + S(si).word(tile);
+#pragma unroll
+                for (int v = 0; v < (1 << R0); v++) {
+                    const u64 x = a[(si << R0) + v];
+                    d[S::wstep(v)] = LAST ? shoup_canon(x, sc, scs, pr.q, nq) : x;
+                }
             }
         }
     }
-    if (INV) cl_sync();  // no CTA leaves while a peer still reads its shared memory
 }
 
 // ngroups == 0 only sets the kernel's shared-memory limit (no launch).
-template <int R0, int R1, int R2, int R3, int R4, bool INV, int FUSE = kFuseNone>
-cudaError_t run_cluster(const NttArgs &a, int ngroups, cudaStream_t st)
+template <int LOGN, bool STRIDED, bool INV, int FUSE, int TE, int R0, int R1, int R2 = 0, int R3 = 0>
+cudaError_t run_pass(const NttArgs &a, int ngroups, cudaStream_t st)
 {
-    using CG = ClGeom<R0, R1, R2, R3, R4>;
-    auto kern = k_ntt_cluster<R0, R1, R2, R3, R4, INV, FUSE>;
+    using P = Pass<LOGN, STRIDED, R0, R1, R2, R3, TE>;
+    auto kern = k_ntt_pass<P, R0, R1, R2, R3, INV, FUSE>;
     static bool configured = false;  // once per instantiation
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CG::SMEM);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::SMEM);
         if (e != cudaSuccess) return e;
         configured = true;
     }
     if (ngroups == 0) return cudaSuccess;
-    launch_k(a.pdl != 0, kern, dim3(ngroups * kCl), dim3(CG::NT), CG::SMEM, st, a);
+    launch_k(a.pdl != 0, kern, dim3(ngroups * P::TILES), dim3(P::NT), P::SMEM, st, a);
     return cudaGetLastError();
 }
 
-// Pass plans per ring size: the strided pass covers the first S1 stages
-// (rounds A1, B1, C1), the contiguous pass the last S2 (rounds A2, B2, C2).
-// N = 2^12 is one contiguous pass of rounds 4, 4, 4.
-template <int LOGN> struct Plan;
-template <> struct Plan<13> { static constexpr int S1 = 7, A1 = 4, B1 = 3, C1 = 0, S2 = 6, A2 = 3, B2 = 3, C2 = 0; };
-template <> struct Plan<14> { static constexpr int S1 = 7, A1 = 4, B1 = 3, C1 = 0, S2 = 7, A2 = 4, B2 = 3, C2 = 0; };
-template <> struct Plan<15> { static constexpr int S1 = 8, A1 = 4, B1 = 4, C1 = 0, S2 = 7, A2 = 4, B2 = 3, C2 = 0; };
-template <> struct Plan<16> { static constexpr int S1 = 8, A1 = 4, B1 = 4, C1 = 0, S2 = 8, A2 = 4, B2 = 4, C2 = 0; };
-template <> struct Plan<17> { static constexpr int S1 = 9, A1 = 3, B1 = 3, C1 = 3, S2 = 8, A2 = 4, B2 = 4, C2 = 0; };
-template <int LOGN> constexpr int plan_direct() { return Plan<LOGN>::C2 ? Plan<LOGN>::C2 : Plan<LOGN>::B2; }
-
-// Radix-8 plans: every round of at most three stages, so a tile has 256
-// threads (twice the radix-16 plans' threads per limb: launches over few
-// limbs fill more of the GPU).  The direct round (the contiguous pass's last
-// two or three stages) lies inside the transposed region of the table the
-// radix-16 plan lays out (plan_direct stages), so both plans share one table.
-template <int LOGN> struct Plan8;
-// The round orders are the ones whose shared-memory accesses are free of
-// bank conflicts with the one-word-per-16 padding (a warp's 32 8-byte words
-// in two wavefronts), checked exhaustively on the CPU.
-template <> struct Plan8<13> { static constexpr int S1 = 7, A1 = 3, B1 = 2, C1 = 2, S2 = 6, A2 = 3, B2 = 3, C2 = 0; };
-template <> struct Plan8<14> { static constexpr int S1 = 7, A1 = 3, B1 = 2, C1 = 2, S2 = 7, A2 = 2, B2 = 3, C2 = 2; };
-template <> struct Plan8<15> { static constexpr int S1 = 8, A1 = 2, B1 = 3, C1 = 3, S2 = 7, A2 = 2, B2 = 3, C2 = 2; };
-template <> struct Plan8<16> { static constexpr int S1 = 8, A1 = 2, B1 = 3, C1 = 3, S2 = 8, A2 = 2, B2 = 3, C2 = 3; };
-template <> struct Plan8<17> { static constexpr int S1 = 9, A1 = 3, B1 = 3, C1 = 3, S2 = 8, A2 = 2, B2 = 3, C2 = 3; };
-template <int LOGN> constexpr bool plan8_fits()
+// The two passes of each ring size: the strided one covers the first stages
+// (forward order), the contiguous one the rest.  N = 2^12 is a single
+// contiguous pass.  Rounds of four stages (sixteen elements per thread) where
+// the multiply pipe bounds the pass; rounds of at most three (eight elements,
+// twice the warps) where memory latency does, in the passes that compute
+// their tile from many streams, and for the nine stages of 2^17.
+template <bool STRIDED, bool INV, int FUSE>
+cudaError_t pass(int logN, const NttArgs &a, int ng, cudaStream_t st)
 {
-    return (Plan8<LOGN>::C2 ? Plan8<LOGN>::C2 : Plan8<LOGN>::B2) <= plan_direct<LOGN>();
-}
-static_assert(plan8_fits<13>() && plan8_fits<14>() && plan8_fits<15>() && plan8_fits<16>() && plan8_fits<17>(),
-              "the radix-8 direct round must lie in the transposed region");
-
-// Pass splits (the launch shape's ntt_split): SPLIT 1 moves one stage from
-// the strided pass to the contiguous one, SPLIT 2 the other way (2^16:
-// 7 + 9 and 9 + 7 stages; 2^17: 8 + 9 and 10 + 7), each in a radix-16 and a
-// radix-8 form (R8).  Every plan's direct round lies in the transposed
-// region of the one twiddle table, and every round's shared-memory index map
-// was checked on the CPU (each tile element touched once, the padding of
-// e0 + c equal to padi(e0) plus the compile-time offset, addresses inside
-// the padded buffer).  Other ring sizes keep their default plans.
-template <int LOGN, int SPLIT, bool R8> struct PlanV : std::conditional_t<R8, Plan8<LOGN>, Plan<LOGN>> {};
-template <> struct PlanV<16, 1, false> { static constexpr int S1 = 7, A1 = 4, B1 = 3, C1 = 0, S2 = 9, A2 = 4, B2 = 2, C2 = 3; };
-template <> struct PlanV<16, 1, true> { static constexpr int S1 = 7, A1 = 3, B1 = 2, C1 = 2, S2 = 9, A2 = 3, B2 = 3, C2 = 3; };
-template <> struct PlanV<16, 2, false> { static constexpr int S1 = 9, A1 = 4, B1 = 3, C1 = 2, S2 = 7, A2 = 4, B2 = 3, C2 = 0; };
-template <> struct PlanV<16, 2, true> { static constexpr int S1 = 9, A1 = 3, B1 = 3, C1 = 3, S2 = 7, A2 = 2, B2 = 3, C2 = 2; };
-template <> struct PlanV<17, 1, false> { static constexpr int S1 = 8, A1 = 4, B1 = 4, C1 = 0, S2 = 9, A2 = 4, B2 = 2, C2 = 3; };
-template <> struct PlanV<17, 1, true> { static constexpr int S1 = 8, A1 = 2, B1 = 3, C1 = 3, S2 = 9, A2 = 3, B2 = 3, C2 = 3; };
-template <> struct PlanV<17, 2, false> { static constexpr int S1 = 10, A1 = 4, B1 = 3, C1 = 3, S2 = 7, A2 = 4, B2 = 3, C2 = 0; };
-template <> struct PlanV<17, 2, true> { static constexpr int S1 = 10, A1 = 4, B1 = 3, C1 = 3, S2 = 7, A2 = 2, B2 = 3, C2 = 2; };
-template <int LOGN, int SPLIT, bool R8> constexpr bool planv_fits()
-{
-    using P = PlanV<LOGN, SPLIT, R8>;
-    return P::S1 + P::S2 == LOGN && P::A1 + P::B1 + P::C1 == P::S1 && P::A2 + P::B2 + P::C2 == P::S2 &&
-           (P::C2 ? P::C2 : P::B2) <= plan_direct<LOGN>() && P::S1 <= LOGN - plan_direct<LOGN>();
-}
-static_assert(planv_fits<16, 1, false>() && planv_fits<16, 1, true>() && planv_fits<16, 2, false>() &&
-                  planv_fits<16, 2, true>() && planv_fits<17, 1, false>() && planv_fits<17, 1, true>() &&
-                  planv_fits<17, 2, false>() && planv_fits<17, 2, true>(),
-              "split plans: stages, rounds and the transposed region");
-
-// plan id: bit 0 the radix-8 form, bits 1-2 the split (0, 1, 2), bit 3
-// 1024-element tiles (twice the CTAs, each half the work, for launches with
-// few limbs; every round's index map at that tile size was checked on the
-// CPU as for 2048)
-// bit 4: the one-pass transform over a cluster (N = 2^16; other sizes
-// ignore it)
-constexpr int kPlanOnePass = 16;
-constexpr int kNttPlans = 32;
-// 1024-element tiles of a plan: a strided pass of 2^10 stages would be one
-// column wide, so that plan keeps 2048
-template <class P> constexpr int small_te() { return P::S1 >= 10 ? 2048 : 1024; }
-
-// Two-pass transform: the strided pass covers the first S1 stages (forward
-// order), the contiguous pass the last S2.
-template <int S1, int A1, int B1, int C1, int S2, int A2, int B2, int C2, int TE>
-cudaError_t two_pass(const he_ctx *c, NttArgs a, int ngroups, bool inverse, cudaStream_t st, const char *tag)
-{
-    a.tiles = (1 << (S1 + S2)) / TE;
-    cudaError_t e;
-    const char *t1 = inverse ? ".inv_pass1" : ".fwd_pass1";
-    const char *t2 = inverse ? ".inv_pass2" : ".fwd_pass2";
-    if (ngroups == 0) {  // configure only
-        e = run_pass<S1, A1, B1, C1, true, false, true, false, TE>(a, 0, st);
-        if (e == cudaSuccess) e = run_pass<S2, A2, B2, C2, false, false, false, true, TE>(a, 0, st);
-        if (e == cudaSuccess) e = run_pass<S2, A2, B2, C2, false, true, true, false, TE>(a, 0, st);
-        if (e == cudaSuccess) e = run_pass<S1, A1, B1, C1, true, true, false, true, TE>(a, 0, st);
-        return e;
-    }
-    if (!inverse) {
-        e = run_pass<S1, A1, B1, C1, true, false, true, false, TE>(a, ngroups, st);
-        if (e != cudaSuccess) return e;
-        prof_mark(c, st, tag, t1);
-        e = run_pass<S2, A2, B2, C2, false, false, false, true, TE>(a, ngroups, st);
-        prof_mark(c, st, tag, t2);
-        return e;
-    }
-    e = run_pass<S2, A2, B2, C2, false, true, true, false, TE>(a, ngroups, st);
-    if (e != cudaSuccess) return e;
-    prof_mark(c, st, tag, t1);
-    e = run_pass<S1, A1, B1, C1, true, true, false, true, TE>(a, ngroups, st);
-    prof_mark(c, st, tag, t2);
-    return e;
-}
-
-// One-pass transforms over a cluster.  Local rounds (3, 3, 3, 4), 512
-// threads, free of shared-memory bank conflicts with the one-word-per-16
-// padding; with the plan's radix-8 bit, (3, 3, 2, 2, 3), 1024 threads at most
-// 64 registers (a 2-way conflict in the fourth round).  Both keep the direct
-// round inside the table's transposed region.
-#define HE_CL16 3, 3, 3, 4, 0
-#define HE_CL8 3, 3, 2, 2, 3
-cudaError_t onepass(const he_ctx *c, const NttArgs &a, int ngroups, bool inverse, cudaStream_t st, const char *tag,
-                    int plan)
-{
-    if (ngroups == 0) {  // configure only
-        cudaError_t e = run_cluster<HE_CL16, false>(a, 0, st);
-        if (e == cudaSuccess) e = run_cluster<HE_CL16, true>(a, 0, st);
-        if (e == cudaSuccess) e = run_cluster<HE_CL8, false>(a, 0, st);
-        return e == cudaSuccess ? run_cluster<HE_CL8, true>(a, 0, st) : e;
-    }
-    cudaError_t e;
-    if (plan & 1) e = inverse ? run_cluster<HE_CL8, true>(a, ngroups, st) : run_cluster<HE_CL8, false>(a, ngroups, st);
-    else e = inverse ? run_cluster<HE_CL16, true>(a, ngroups, st) : run_cluster<HE_CL16, false>(a, ngroups, st);
-    prof_mark(c, st, tag, inverse ? ".inv_onepass" : ".fwd_onepass");
-    return e;
-}
-
-cudaError_t onepass_combine(const he_ctx *c, const NttArgs &a, int ngroups, cudaStream_t st, const char *tag,
-                            int plan)
-{
-    if (ngroups == 0) {
-        const cudaError_t e = run_cluster<HE_CL16, false, kFuseCombine>(a, 0, st);
-        return e == cudaSuccess ? run_cluster<HE_CL8, false, kFuseCombine>(a, 0, st) : e;
-    }
-    const cudaError_t e = (plan & 1) ? run_cluster<HE_CL8, false, kFuseCombine>(a, ngroups, st)
-                                     : run_cluster<HE_CL16, false, kFuseCombine>(a, ngroups, st);
-    prof_mark(c, st, tag, ".fwd_onepass_combine");
-    return e;
-}
-
-cudaError_t onepass_tensor(const he_ctx *c, const NttArgs &a, int ngroups, cudaStream_t st, const char *tag,
-                           int plan)
-{
-    if (ngroups == 0) {
-        const cudaError_t e = run_cluster<HE_CL16, true, kFuseTensor>(a, 0, st);
-        return e == cudaSuccess ? run_cluster<HE_CL8, true, kFuseTensor>(a, 0, st) : e;
-    }
-    const cudaError_t e = (plan & 1) ? run_cluster<HE_CL8, true, kFuseTensor>(a, ngroups, st)
-                                     : run_cluster<HE_CL16, true, kFuseTensor>(a, ngroups, st);
-    prof_mark(c, st, tag, ".tensor_inv_onepass");
-    return e;
-}
-#undef HE_CL16
-#undef HE_CL8
-
-template <int LOGN, class P = Plan<LOGN>, int TE = 2048>
-cudaError_t two_pass_plan(const he_ctx *c, NttArgs a, int ngroups, bool inverse, cudaStream_t st, const char *tag)
-{
-    return two_pass<P::S1, P::A1, P::B1, P::C1, P::S2, P::A2, P::B2, P::C2, TE>(c, a, ngroups, inverse, st, tag);
-}
-
-template <int LOGN>
-cudaError_t two_pass_any(const he_ctx *c, NttArgs a, int ngroups, bool inverse, cudaStream_t st, const char *tag, int plan)
-{
-    if (LOGN == kClLogN && (plan & kPlanOnePass)) return onepass(c, a, ngroups, inverse, st, tag, plan);
-    // bit 3: 1024-element tiles (2^16 and 2^17; a pass over 2^10 stages keeps 2048)
-    constexpr bool SMALL_OK = LOGN == 16 || LOGN == 17;
-    if (SMALL_OK && (plan & 8)) {
-        switch (plan & 7) {
-        case 1: return two_pass_plan<LOGN, Plan8<LOGN>, SMALL_OK ? 1024 : 2048>(c, a, ngroups, inverse, st, tag);
-        case 2: return two_pass_plan<LOGN, PlanV<LOGN, 1, false>, SMALL_OK ? 1024 : 2048>(c, a, ngroups, inverse, st, tag);
-        case 3: return two_pass_plan<LOGN, PlanV<LOGN, 1, true>, SMALL_OK ? 1024 : 2048>(c, a, ngroups, inverse, st, tag);
-        case 4: return two_pass_plan<LOGN, PlanV<LOGN, 2, false>, small_te<PlanV<LOGN, 2, false>>()>(c, a, ngroups, inverse, st, tag);
-        case 5: return two_pass_plan<LOGN, PlanV<LOGN, 2, true>, small_te<PlanV<LOGN, 2, true>>()>(c, a, ngroups, inverse, st, tag);
-        default: return two_pass_plan<LOGN, Plan<LOGN>, SMALL_OK ? 1024 : 2048>(c, a, ngroups, inverse, st, tag);
+    constexpr bool COMPUTED = FUSE == kFuseTensor || FUSE == kFuseIp;
+#define HE_PASS(...) run_pass<__VA_ARGS__>(a, ng, st)
+    if constexpr (STRIDED) {
+        switch (logN) {
+        case 13: return HE_PASS(13, true, INV, FUSE, 2048, 4, 3);
+        case 14: return HE_PASS(14, true, INV, FUSE, 2048, 4, 3);
+        case 15: return HE_PASS(15, true, INV, FUSE, 2048, 4, 4);
+        case 16: return HE_PASS(16, true, INV, FUSE, 2048, 4, 4);
+        case 17: return HE_PASS(17, true, INV, FUSE, 2048, 3, 3, 3);
+        default: return cudaErrorInvalidValue;
+        }
+    } else if constexpr (COMPUTED) {
+        switch (logN) {
+        case 12: return HE_PASS(12, false, INV, FUSE, 4096, 3, 3, 3, 3);
+        case 13: return HE_PASS(13, false, INV, FUSE, 2048, 3, 3);
+        case 14: return HE_PASS(14, false, INV, FUSE, 2048, 2, 3, 2);
+        case 15: return HE_PASS(15, false, INV, FUSE, 2048, 2, 3, 2);
+        case 16: return HE_PASS(16, false, INV, FUSE, 2048, 2, 3, 3);
+        case 17: return HE_PASS(17, false, INV, FUSE, 2048, 2, 3, 3);
+        default: return cudaErrorInvalidValue;
+        }
+    } else {
+        switch (logN) {
+        case 12: return HE_PASS(12, false, INV, FUSE, 4096, 3, 3, 3, 3);
+        case 13: return HE_PASS(13, false, INV, FUSE, 2048, 3, 3);
+        case 14: return HE_PASS(14, false, INV, FUSE, 2048, 4, 3);
+        case 15: return HE_PASS(15, false, INV, FUSE, 2048, 4, 3);
+        case 16: return HE_PASS(16, false, INV, FUSE, 2048, 4, 4);
+        case 17: return HE_PASS(17, false, INV, FUSE, 2048, 4, 4);
+        default: return cudaErrorInvalidValue;
         }
     }
-    switch (plan & 7) {
-    case 1: return two_pass_plan<LOGN, Plan8<LOGN>>(c, a, ngroups, inverse, st, tag);
-    case 2: return two_pass_plan<LOGN, PlanV<LOGN, 1, false>>(c, a, ngroups, inverse, st, tag);
-    case 3: return two_pass_plan<LOGN, PlanV<LOGN, 1, true>>(c, a, ngroups, inverse, st, tag);
-    case 4: return two_pass_plan<LOGN, PlanV<LOGN, 2, false>>(c, a, ngroups, inverse, st, tag);
-    case 5: return two_pass_plan<LOGN, PlanV<LOGN, 2, true>>(c, a, ngroups, inverse, st, tag);
-    default: return two_pass_plan<LOGN, Plan<LOGN>>(c, a, ngroups, inverse, st, tag);
-    }
+#undef HE_PASS
 }
 
-// Forward transform whose last pass also applies the final combine.
-template <int LOGN, class P, int TE = 2048>
-cudaError_t combine_plan(const he_ctx *c, NttArgs a, int ngroups, cudaStream_t st, const char *tag)
+// The whole transform; ngroups == 0 configures its kernels.
+template <bool INV, int FUSE>
+cudaError_t transform(const he_ctx *c, const NttArgs &a, int ng, cudaStream_t st, const char *tag)
 {
-    a.tiles = (1 << LOGN) / TE;
-    if (ngroups == 0) return run_pass<P::S2, P::A2, P::B2, P::C2, false, false, false, true, TE, kFuseCombine>(a, 0, st);
-    cudaError_t e = run_pass<P::S1, P::A1, P::B1, P::C1, true, false, true, false, TE>(a, ngroups, st);
+    static const char *const kMark[4] = {"", "_combine", ".tensor_inv", ".ip_inv"};
+    const int lg = c->logN;
+    if (lg == 12) {
+        const cudaError_t e = pass<false, INV, FUSE>(lg, a, ng, st);
+        if (ng) {
+            if (FUSE == kFuseTensor || FUSE == kFuseIp) prof_mark(c, st, tag, kMark[FUSE]);
+            else prof_mark(c, st, tag, INV ? ".inv" : FUSE == kFuseCombine ? ".fwd_combine" : ".fwd");
+        }
+        return e;
+    }
+    cudaError_t e = INV ? pass<false, true, INV ? FUSE : kFuseNone>(lg, a, ng, st)
+                        : pass<true, false, kFuseNone>(lg, a, ng, st);
     if (e != cudaSuccess) return e;
-    prof_mark(c, st, tag, ".fwd_pass1");
-    e = run_pass<P::S2, P::A2, P::B2, P::C2, false, false, false, true, TE, kFuseCombine>(a, ngroups, st);
-    prof_mark(c, st, tag, ".fwd_pass2_combine");
+    if (ng)
+        prof_mark(c, st, tag, !INV ? ".fwd_pass1" : FUSE == kFuseTensor ? ".tensor_inv_pass1" : FUSE == kFuseIp ? ".ip_inv_pass1" : ".inv_pass1");
+    e = INV ? pass<true, true, kFuseNone>(lg, a, ng, st) : pass<false, false, INV ? kFuseNone : FUSE>(lg, a, ng, st);
+    if (ng) prof_mark(c, st, tag, INV ? ".inv_pass2" : FUSE == kFuseCombine ? ".fwd_pass2_combine" : ".fwd_pass2");
     return e;
 }
 
-template <int LOGN>
-cudaError_t combine_any(const he_ctx *c, NttArgs a, int ngroups, cudaStream_t st, const char *tag, int plan)
+NttArgs ntt_args(const he_ctx *c, const u64 *src, u64 *dst, const NttGroup *groups, const int *dev_count)
 {
-    if (LOGN == kClLogN && (plan & kPlanOnePass)) return onepass_combine(c, a, ngroups, st, tag, plan);
-    // bit 3: 1024-element tiles (2^16 and 2^17; a pass over 2^10 stages keeps 2048)
-    constexpr bool SMALL_OK = LOGN == 16 || LOGN == 17;
-    if (SMALL_OK && (plan & 8)) {
-        switch (plan & 7) {
-        case 1: return combine_plan<LOGN, Plan8<LOGN>, SMALL_OK ? 1024 : 2048>(c, a, ngroups, st, tag);
-        case 2: return combine_plan<LOGN, PlanV<LOGN, 1, false>, SMALL_OK ? 1024 : 2048>(c, a, ngroups, st, tag);
-        case 3: return combine_plan<LOGN, PlanV<LOGN, 1, true>, SMALL_OK ? 1024 : 2048>(c, a, ngroups, st, tag);
-        case 4: return combine_plan<LOGN, PlanV<LOGN, 2, false>, small_te<PlanV<LOGN, 2, false>>()>(c, a, ngroups, st, tag);
-        case 5: return combine_plan<LOGN, PlanV<LOGN, 2, true>, small_te<PlanV<LOGN, 2, true>>()>(c, a, ngroups, st, tag);
-        default: return combine_plan<LOGN, Plan<LOGN>, SMALL_OK ? 1024 : 2048>(c, a, ngroups, st, tag);
-        }
-    }
-    switch (plan & 7) {
-    case 1: return combine_plan<LOGN, Plan8<LOGN>>(c, a, ngroups, st, tag);
-    case 2: return combine_plan<LOGN, PlanV<LOGN, 1, false>>(c, a, ngroups, st, tag);
-    case 3: return combine_plan<LOGN, PlanV<LOGN, 1, true>>(c, a, ngroups, st, tag);
-    case 4: return combine_plan<LOGN, PlanV<LOGN, 2, false>>(c, a, ngroups, st, tag);
-    case 5: return combine_plan<LOGN, PlanV<LOGN, 2, true>>(c, a, ngroups, st, tag);
-    default: return combine_plan<LOGN, Plan<LOGN>>(c, a, ngroups, st, tag);
-    }
-}
-
-// Inverse transform whose first pass computes its input: the tensor
-// product (kFuseTensor) or the key-switch sums (kFuseIp).
-template <int LOGN, class P, int FUSE, int TE = 2048>
-cudaError_t computed_plan(const he_ctx *c, NttArgs a, int ngroups, cudaStream_t st, const char *tag)
-{
-    a.tiles = (1 << LOGN) / TE;
-    if (ngroups == 0) return run_pass<P::S2, P::A2, P::B2, P::C2, false, true, true, false, TE, FUSE>(a, 0, st);
-    cudaError_t e = run_pass<P::S2, P::A2, P::B2, P::C2, false, true, true, false, TE, FUSE>(a, ngroups, st);
-    if (e != cudaSuccess) return e;
-    prof_mark(c, st, tag, FUSE == kFuseTensor ? ".tensor_inv_pass1" : ".ip_inv_pass1");
-    e = run_pass<P::S1, P::A1, P::B1, P::C1, true, true, false, true, TE>(a, ngroups, st);
-    prof_mark(c, st, tag, ".inv_pass2");
-    return e;
-}
-
-// The plans of computed_plan (the one-pass cluster transform takes the
-// tensor product only; with the key-switch sums that bit is ignored).
-template <int LOGN, int FUSE>
-cudaError_t computed_any(const he_ctx *c, NttArgs a, int ngroups, cudaStream_t st, const char *tag, int plan)
-{
-    if (FUSE == kFuseTensor && LOGN == kClLogN && (plan & kPlanOnePass)) return onepass_tensor(c, a, ngroups, st, tag, plan);
-    // bit 3: 1024-element tiles (2^16 and 2^17; a pass over 2^10 stages keeps 2048)
-    constexpr bool SMALL_OK = LOGN == 16 || LOGN == 17;
-    constexpr int TS = SMALL_OK ? 1024 : 2048;
-    if (SMALL_OK && (plan & 8)) {
-        switch (plan & 7) {
-        case 1: return computed_plan<LOGN, Plan8<LOGN>, FUSE, TS>(c, a, ngroups, st, tag);
-        case 2: return computed_plan<LOGN, PlanV<LOGN, 1, false>, FUSE, TS>(c, a, ngroups, st, tag);
-        case 3: return computed_plan<LOGN, PlanV<LOGN, 1, true>, FUSE, TS>(c, a, ngroups, st, tag);
-        case 4: return computed_plan<LOGN, PlanV<LOGN, 2, false>, FUSE, small_te<PlanV<LOGN, 2, false>>()>(c, a, ngroups, st, tag);
-        case 5: return computed_plan<LOGN, PlanV<LOGN, 2, true>, FUSE, small_te<PlanV<LOGN, 2, true>>()>(c, a, ngroups, st, tag);
-        default: return computed_plan<LOGN, Plan<LOGN>, FUSE, TS>(c, a, ngroups, st, tag);
-        }
-    }
-    switch (plan & 7) {
-    case 1: return computed_plan<LOGN, Plan8<LOGN>, FUSE>(c, a, ngroups, st, tag);
-    case 2: return computed_plan<LOGN, PlanV<LOGN, 1, false>, FUSE>(c, a, ngroups, st, tag);
-    case 3: return computed_plan<LOGN, PlanV<LOGN, 1, true>, FUSE>(c, a, ngroups, st, tag);
-    case 4: return computed_plan<LOGN, PlanV<LOGN, 2, false>, FUSE>(c, a, ngroups, st, tag);
-    case 5: return computed_plan<LOGN, PlanV<LOGN, 2, true>, FUSE>(c, a, ngroups, st, tag);
-    default: return computed_plan<LOGN, Plan<LOGN>, FUSE>(c, a, ngroups, st, tag);
-    }
-}
-
-// An inverse transform with a computed first pass, at the context's ring size.
-cudaError_t launch_computed(const he_ctx *c, const NttArgs &a, int ngroups, cudaStream_t st, const char *tag, int plan,
-                            bool ip)
-{
-    switch (c->logN) {
-    case 12: {
-        cudaError_t e = ip ? run_pass<12, 4, 4, 4, false, true, true, true, 4096, kFuseIp>(a, ngroups, st)
-                           : run_pass<12, 4, 4, 4, false, true, true, true, 4096, kFuseTensor>(a, ngroups, st);
-        if (ngroups) prof_mark(c, st, tag, ip ? ".ip_inv" : ".tensor_inv");
-        return e;
-    }
-    case 13: return ip ? computed_any<13, kFuseIp>(c, a, ngroups, st, tag, plan) : computed_any<13, kFuseTensor>(c, a, ngroups, st, tag, plan);
-    case 14: return ip ? computed_any<14, kFuseIp>(c, a, ngroups, st, tag, plan) : computed_any<14, kFuseTensor>(c, a, ngroups, st, tag, plan);
-    case 15: return ip ? computed_any<15, kFuseIp>(c, a, ngroups, st, tag, plan) : computed_any<15, kFuseTensor>(c, a, ngroups, st, tag, plan);
-    case 16: return ip ? computed_any<16, kFuseIp>(c, a, ngroups, st, tag, plan) : computed_any<16, kFuseTensor>(c, a, ngroups, st, tag, plan);
-    case 17: return ip ? computed_any<17, kFuseIp>(c, a, ngroups, st, tag, plan) : computed_any<17, kFuseTensor>(c, a, ngroups, st, tag, plan);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
-}  // namespace
-
-cudaError_t launch_ntt_tensor(const he_ctx *c, u64 *base, const NttGroup *groups, int ngroups, const JobRef &R,
-                              cudaStream_t st, const char *tag, const int *dev_count, int plan)
-{
-    if (ngroups < 0) return cudaSuccess;  // ngroups == 0: configure the kernels only
-    NttArgs a;
-    memset(&a, 0, sizeof(a));
-    a.src = base;
-    a.dst = base;
-    a.groups = groups;
-    a.primes = c->d_primes;
-    a.logN = c->logN;
-    a.ts = c->logN - ntt_direct_stages(c->logN);
-    a.tiles = 1;
-    a.count = dev_count;
-    a.pdl = c->pdl;
-    a.R = R;
-    a.levels = c->d_levels;
-    a.pinv = c->d_pinv;
-    return launch_computed(c, a, ngroups, st, tag, plan, false);
-}
-
-cudaError_t launch_ntt_ip(const he_ctx *c, u64 *base, const NttGroup *groups, int ngroups, const JobRef &R,
-                          const u64 *evk, cudaStream_t st, const char *tag, const int *dev_count, int plan)
-{
-    if (ngroups < 0) return cudaSuccess;  // ngroups == 0: configure the kernels only
-    NttArgs a;
-    memset(&a, 0, sizeof(a));
-    a.src = base;
-    a.dst = base;
-    a.groups = groups;
-    a.primes = c->d_primes;
-    a.logN = c->logN;
-    a.ts = c->logN - ntt_direct_stages(c->logN);
-    a.tiles = 1;
-    a.count = dev_count;
-    a.pdl = c->pdl;
-    a.R = R;
-    a.levels = c->d_levels;
-    a.evk = evk;
-    a.EL = c->K + c->L;
-    return launch_computed(c, a, ngroups, st, tag, plan, true);
-}
-
-cudaError_t launch_ntt_combine(const he_ctx *c, u64 *base, const NttGroup *groups, int ngroups, const JobRef &R,
-                               cudaStream_t st, const char *tag, const int *dev_count, int plan)
-{
-    if (ngroups < 0) return cudaSuccess;  // ngroups == 0: configure the kernels only
-    NttArgs a;
-    memset(&a, 0, sizeof(a));
-    a.src = base;
-    a.dst = base;
-    a.groups = groups;
-    a.primes = c->d_primes;
-    a.logN = c->logN;
-    a.ts = c->logN - ntt_direct_stages(c->logN);
-    a.tiles = 1;
-    a.count = dev_count;
-    a.pdl = c->pdl;
-    a.R = R;
-    a.levels = c->d_levels;
-    a.pinv = c->d_pinv;
-    switch (c->logN) {
-    case 12: {
-        cudaError_t e = run_pass<12, 4, 4, 4, false, false, true, true, 4096, kFuseCombine>(a, ngroups, st);
-        if (ngroups) prof_mark(c, st, tag, ".fwd_combine");
-        return e;
-    }
-    case 13: return combine_any<13>(c, a, ngroups, st, tag, plan);
-    case 14: return combine_any<14>(c, a, ngroups, st, tag, plan);
-    case 15: return combine_any<15>(c, a, ngroups, st, tag, plan);
-    case 16: return combine_any<16>(c, a, ngroups, st, tag, plan);
-    case 17: return combine_any<17>(c, a, ngroups, st, tag, plan);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
-cudaError_t launch_ntt2(const he_ctx *c, const u64 *src, u64 *dst, const NttGroup *groups, int ngroups, bool inverse,
-                        cudaStream_t st, const char *tag, const int *dev_count, int plan)
-{
-    if (ngroups < 0) return cudaSuccess;  // ngroups == 0: configure the kernels only
     NttArgs a;
     memset(&a, 0, sizeof(a));
     a.src = src;
@@ -1282,66 +782,75 @@ cudaError_t launch_ntt2(const he_ctx *c, const u64 *src, u64 *dst, const NttGrou
     a.groups = groups;
     a.primes = c->d_primes;
     a.logN = c->logN;
-    a.ts = c->logN - ntt_direct_stages(c->logN);
-    a.tiles = 1;
     a.count = dev_count;
     a.pdl = c->pdl;
-    switch (c->logN) {
-    case 12: {
-        if (ngroups == 0) {
-            cudaError_t e = run_pass<12, 4, 4, 4, false, true, true, true, 4096>(a, 0, st);
-            return e == cudaSuccess ? run_pass<12, 4, 4, 4, false, false, true, true, 4096>(a, 0, st) : e;
-        }
-        cudaError_t e = inverse ? run_pass<12, 4, 4, 4, false, true, true, true, 4096>(a, ngroups, st)
-                                : run_pass<12, 4, 4, 4, false, false, true, true, 4096>(a, ngroups, st);
-        prof_mark(c, st, tag, inverse ? ".inv" : ".fwd");
-        return e;
-    }
-    case 13: return two_pass_any<13>(c, a, ngroups, inverse, st, tag, plan);
-    case 14: return two_pass_any<14>(c, a, ngroups, inverse, st, tag, plan);
-    case 15: return two_pass_any<15>(c, a, ngroups, inverse, st, tag, plan);
-    case 16: return two_pass_any<16>(c, a, ngroups, inverse, st, tag, plan);
-    case 17: return two_pass_any<17>(c, a, ngroups, inverse, st, tag, plan);
-    default: return cudaErrorInvalidValue;
-    }
+    return a;
 }
 
-int ntt_direct_stages(int logN)
+}  // namespace
+
+cudaError_t launch_ntt_tensor(const he_ctx *c, u64 *base, const NttGroup *groups, int ngroups, const JobRef &R,
+                              cudaStream_t st, const char *tag, const int *dev_count)
 {
-    switch (logN) {
-    case 12: return 4;  // the single pass's third round
-    case 13: return plan_direct<13>();
-    case 14: return plan_direct<14>();
-    case 15: return plan_direct<15>();
-    case 16: return plan_direct<16>();
-    case 17: return plan_direct<17>();
-    default: return 0;
-    }
+    if (ngroups < 0) return cudaSuccess;  // ngroups == 0: configure the kernels only
+    NttArgs a = ntt_args(c, base, base, groups, dev_count);
+    a.R = R;
+    a.levels = c->d_levels;
+    return transform<true, kFuseTensor>(c, a, ngroups, st, tag);
 }
+
+cudaError_t launch_ntt_ip(const he_ctx *c, u64 *base, const NttGroup *groups, int ngroups, const JobRef &R,
+                          const u64 *evk, cudaStream_t st, const char *tag, const int *dev_count)
+{
+    if (ngroups < 0) return cudaSuccess;
+    NttArgs a = ntt_args(c, base, base, groups, dev_count);
+    a.R = R;
+    a.levels = c->d_levels;
+    a.evk = evk;
+    a.EL = c->K + c->L;
+    return transform<true, kFuseIp>(c, a, ngroups, st, tag);
+}
+
+cudaError_t launch_ntt_combine(const he_ctx *c, u64 *base, const NttGroup *groups, int ngroups, const JobRef &R,
+                               cudaStream_t st, const char *tag, const int *dev_count)
+{
+    if (ngroups < 0) return cudaSuccess;
+    NttArgs a = ntt_args(c, base, base, groups, dev_count);
+    a.R = R;
+    a.levels = c->d_levels;
+    a.pinv = c->d_pinv;
+    return transform<false, kFuseCombine>(c, a, ngroups, st, tag);
+}
+
+cudaError_t launch_ntt2(const he_ctx *c, const u64 *src, u64 *dst, const NttGroup *groups, int ngroups, bool inverse,
+                        cudaStream_t st, const char *tag, const int *dev_count)
+{
+    if (ngroups < 0) return cudaSuccess;
+    const NttArgs a = ntt_args(c, src, dst, groups, dev_count);
+    return inverse ? transform<true, kFuseNone>(c, a, ngroups, st, tag)
+                   : transform<false, kFuseNone>(c, a, ngroups, st, tag);
+}
+
+int ntt_direct_stages(int logN) { return logN >= 12 && logN <= 17 ? direct_stages(logN) : 0; }
 
 cudaError_t launch_ntt(const he_ctx *c, u64 *base, const NttGroup *groups, int ngroups, bool inverse, cudaStream_t st,
-                       const char *tag, const int *dev_count, int plan)
+                       const char *tag, const int *dev_count)
 {
-    return launch_ntt2(c, base, base, groups, ngroups, inverse, st, tag, dev_count, plan);
+    return launch_ntt2(c, base, base, groups, ngroups, inverse, st, tag, dev_count);
 }
 
 // Set the dynamic shared-memory limit of every NTT pass this ring size uses,
-// in every plan (done once per context, before any launch or stream capture).
+// (done once per context, before any launch or stream capture).
 cudaError_t configure_ntt(const he_ctx *c)
 {
     JobRef R;
     memset(&R, 0, sizeof(R));
-    for (int plan = 0; plan < kNttPlans; plan++) {
-        cudaError_t e = launch_ntt2(c, nullptr, nullptr, nullptr, 0, false, nullptr, nullptr, nullptr, plan);
-        if (e != cudaSuccess) return e;
-        e = launch_ntt_combine(c, nullptr, nullptr, 0, R, nullptr, nullptr, nullptr, plan);
-        if (e != cudaSuccess) return e;
-        e = launch_ntt_tensor(c, nullptr, nullptr, 0, R, nullptr, nullptr, nullptr, plan);
-        if (e != cudaSuccess) return e;
-        e = launch_ntt_ip(c, nullptr, nullptr, 0, R, nullptr, nullptr, nullptr, nullptr, plan);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    cudaError_t e = launch_ntt2(c, nullptr, nullptr, nullptr, 0, false, nullptr);
+    if (e == cudaSuccess) e = launch_ntt2(c, nullptr, nullptr, nullptr, 0, true, nullptr);
+    if (e == cudaSuccess) e = launch_ntt_combine(c, nullptr, nullptr, 0, R, nullptr);
+    if (e == cudaSuccess) e = launch_ntt_tensor(c, nullptr, nullptr, 0, R, nullptr);
+    if (e == cudaSuccess) e = launch_ntt_ip(c, nullptr, nullptr, 0, R, nullptr, nullptr, nullptr, nullptr);
+    return e;
 }
 
 }  // namespace he

@@ -8,8 +8,8 @@
 // GPU at the clocks of the run:
 //
 //  * butterflies: ct_bfly (modarith.cuh), the forward butterfly every NTT
-//    pass issues (the paper's modified Shoup product of Sec. 5.2 plus the
-//    lazy additions of Algo 4), eight independent chains per thread.  The
+//    pass issues (the split twiddle product plus the lazy additions of
+//    Algo 4), eight independent chains per thread.  The
 //    values are not kept reduced (they wrap), which changes no instruction.
 //  * base conversion: the inner loop of k_modup / k_moddown_conv (Sec. 7's
 //    mod up / mod down as fast base conversion, with the delayed-modulo
@@ -26,10 +26,8 @@ namespace {
 
 constexpr int kChains = 8;
 
-__global__ void __launch_bounds__(256) k_probe_bfly(u64 *out, u64 q, u64 w, u64 wp, int iters)
+__global__ void __launch_bounds__(256) k_probe_bfly(u64 *out, u64 q, ulonglong2 tw, const NttMod km, int iters)
 {
-    const u64 q4 = 4 * q, nq = 0ull - q;
-    const ulonglong2 tw = make_ulonglong2(w, wp);
     u64 x[kChains], y[kChains];
 #pragma unroll
     for (int c = 0; c < kChains; c++) {
@@ -38,7 +36,7 @@ __global__ void __launch_bounds__(256) k_probe_bfly(u64 *out, u64 q, u64 w, u64 
     }
     for (int it = 0; it < iters; it++) {
 #pragma unroll
-        for (int c = 0; c < kChains; c++) ct_bfly(x[c], y[c], tw, nq, q4);
+        for (int c = 0; c < kChains; c++) ct_bfly(x[c], y[c], tw, km);
     }
     u64 acc = 0;
 #pragma unroll
@@ -161,10 +159,13 @@ extern "C" int he_probe_butterfly_rate(int blocks, int iters, double *bfly_per_s
     if (cudaMallocAsync((void **)&out, sizeof(u64) * blocks * 256, st) != cudaSuccess) return HE_ECUDA;
     const u64 q = kProbeQ;
     const u64 w = 1234567890123ull % q;
-    const u64 wp = (u64)(((unsigned __int128)w << 64) / q);
+    NttMod km;
+    if (!he::ntt_mod(q, 16, &km)) return HE_EINVAL;
+    const u64 w2 = (u64)(((unsigned __int128)w << 32) % q), m = (1ull << km.s) - 1;
+    const ulonglong2 tw = make_ulonglong2((w & m) | ((w >> km.s) << 32), (w2 & m) | ((w2 >> km.s) << 32));
     float ms = 0;
     const int rc = time_launch(st, [&](bool warm) {
-        k_probe_bfly<<<blocks, 256, 0, st>>>(out, q, w, wp, warm ? iters / 10 + 1 : iters);
+        k_probe_bfly<<<blocks, 256, 0, st>>>(out, q, tw, km, warm ? iters / 10 + 1 : iters);
     }, &ms);
     cudaFreeAsync(out, st);
     if (rc != HE_OK) return rc;
