@@ -68,7 +68,7 @@ __device__ __forceinline__ uint32_t chunk28(const u64 (&w)[WI], int k)
 // y over polys, z over prime groups of kCP.
 template <int WI>
 __global__ void __launch_bounds__(kT)
-k_nr_crt(const u64 *__restrict__ in, int wi, size_t stride, u64 *__restrict__ out, int np,
+k_nr_crt(const u64 *in, int wi, size_t stride, u64 *out, int np,
          const u64 *__restrict__ tab, int tab_stride, const DevPrime *__restrict__ primes, int K, int N)
 {
     constexpr int CH = (64 * WI + 27) / 28;
@@ -111,7 +111,7 @@ k_nr_crt(const u64 *__restrict__ in, int wi, size_t stride, u64 *__restrict__ ou
 // [D0 | D1 | D2 | -] with d0 = b1 b2, d1 = a1 b2 + a2 b1, d2 = a1 a2 mod p_i.
 // grid: x over N / 2 / kT, y over primes.
 __global__ void __launch_bounds__(kT)
-k_nr_tensor(u64 *__restrict__ r, int np, const DevPrime *__restrict__ primes, int K, int N)
+k_nr_tensor(u64 *r, int np, const DevPrime *__restrict__ primes, int K, int N)
 {
     const int i = blockIdx.y;
     const DevPrime pr = primes[K + i];
@@ -130,7 +130,7 @@ k_nr_tensor(u64 *__restrict__ r, int np, const DevPrime *__restrict__ primes, in
 // Region 2 products: r[0] (d2 residues) -> KS_b in place, r[1] = KS_a, with
 // the prepared key ek = [b | a][np][N].  grid: x over N / 2 / kT, y over primes.
 __global__ void __launch_bounds__(kT)
-k_nr_ks_mult(u64 *__restrict__ r, const u64 *__restrict__ ek, int np, const DevPrime *__restrict__ primes, int K,
+k_nr_ks_mult(u64 *r, const u64 *ek, int np, const DevPrime *__restrict__ primes, int K,
              int N)
 {
     const int i = blockIdx.y;
@@ -157,9 +157,9 @@ k_nr_ks_mult(u64 *__restrict__ r, const u64 *__restrict__ ek, int np, const DevP
 // ([np][W]) and NEG ([np + 1][W]).
 template <int W, bool KS>
 __global__ void __launch_bounds__(kIT)
-k_nr_icrt(const u64 *__restrict__ y, int np, const u64 *__restrict__ M, const u64 *__restrict__ NEG,
-          const double *__restrict__ inv, u64 *__restrict__ out, int ostride, int wo, int kout,
-          const u64 *__restrict__ d, int s, int N)
+k_nr_icrt(const u64 *y, int np, const u64 *__restrict__ M, const u64 *__restrict__ NEG,
+          const double *__restrict__ inv, u64 *out, int ostride, int wo, int kout,
+          const u64 *d, int s, int N)
 {
     extern __shared__ __align__(16) u64 sh[];
     u64 *sM = sh;                         // [np][W]
@@ -253,7 +253,7 @@ k_nr_icrt(const u64 *__restrict__ y, int np, const u64 *__restrict__ M, const u6
 // Rescale by 2^s with rounding: out = floor((a + 2^(s-1)) / 2^s) mod 2^kout.
 // grid: x over N / kT, y over the two halves.
 __global__ void __launch_bounds__(kT)
-k_nr_rescale(const u64 *__restrict__ in, int wi, u64 *__restrict__ out, int wo, int kout, int s, int N)
+k_nr_rescale(const u64 *in, int wi, u64 *out, int wo, int kout, int s, int N)
 {
     const int n = blockIdx.x * kT + threadIdx.x;
     const u64 *a = in + (size_t)blockIdx.y * wi * N + n;

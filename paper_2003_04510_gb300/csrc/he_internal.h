@@ -243,6 +243,8 @@ inline void launch_k(bool dep, void (*k)(KArgs...), dim3 grid, dim3 block, size_
 // idle and run their prologue; they wait in their own griddep_wait for this
 // grid's completion and memory flush before touching its data.  Without it
 // the next kernel is launched as this grid's CTAs exit.
+// No pointer to data of an earlier kernel is declared __restrict__ or read with
+// __ldg: either lets the compiler move the loads above this wait.
 __device__ __forceinline__ void griddep_wait(bool trigger = false)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

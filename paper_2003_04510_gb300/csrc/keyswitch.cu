@@ -533,7 +533,7 @@ k_combine_plain(const JobRef R, const ulonglong2 *__restrict__ pinv, const DevLe
 
 // Rescale on its own: out[h][i] = (c_h[i] - Z[h][i]) q_{l-1}^-1, i < l-1
 __global__ void __launch_bounds__(kThreads)
-k_rescale_combine(const u64 *__restrict__ ct, const u64 *__restrict__ Z, u64 *__restrict__ out,
+k_rescale_combine(const u64 *ct, const u64 *Z, u64 *out,
                   const DevLevel *__restrict__ lv_arr, const DevPrime *__restrict__ primes, int K, int l, int N)
 {
     const int i = blockIdx.y, h = blockIdx.z;
@@ -554,7 +554,7 @@ k_rescale_combine(const u64 *__restrict__ ct, const u64 *__restrict__ Z, u64 *__
 // switching inputs into the workspace: d0 = kappa(b), d1 = 0,
 // d2 = -kappa(a) mod q_i.  grid: x over N/2/kThreads, y over limbs.
 __global__ void __launch_bounds__(kThreads)
-k_automorph(const u64 *__restrict__ ct, u64 *__restrict__ ws, const DevLevel *__restrict__ lv_arr,
+k_automorph(const u64 *ct, u64 *ws, const DevLevel *__restrict__ lv_arr,
             const DevPrime *__restrict__ primes, int K, int l, int N, int logN, unsigned long long g)
 {
     const int i = blockIdx.y;

@@ -236,8 +236,8 @@ __device__ __forceinline__ void combine_store(const NttArgs &P, const NttGroup &
         ulonglong2 dv[B4], kv[B4];
 #pragma unroll
         for (int k = 0; k < B4; k++) {
-            dv[k] = __ldg(reinterpret_cast<const ulonglong2 *>(dd + (b0 + k) * gs2));
-            kv[k] = __ldg(reinterpret_cast<const ulonglong2 *>(kk + (b0 + k) * gs2));
+            dv[k] = *reinterpret_cast<const ulonglong2 *>(dd + (b0 + k) * gs2);
+            kv[k] = *reinterpret_cast<const ulonglong2 *>(kk + (b0 + k) * gs2);
         }
 #pragma unroll
         for (int k = 0; k < B4; k++) {
