@@ -634,12 +634,6 @@ def run_ours(args):
     torch.cuda.synchronize()
     lat = np.array([a.elapsed_time(b) for a, b in ev])
     value = job_rate(args.steps, wsz, elapsed_ms * 1e-3)
-    # the final combine runs inside the last NTT pass; with fuse bit 0 the
-    # tensor product runs inside the first one (bit 1 moves the q rows of the
-    # inner product into the ModDown launch: the launch count stays; bit 2
-    # with it moves the other rows into the special limbs' iNTT: one fewer)
-    fz = g.he_get_shape(ctx)[5]
-    launches_per_step = (12 if prm.logN > 12 else 8) - (1 if fz & 1 else 0) - (1 if (fz & 6) == 6 else 0)
 
     # ---- end to end: host buffers through he_mul_rescale_host ----
     hws = torch.empty(g.he_host_workspace_bytes(ctx, level) // 8, dtype=torch.int64, device=dev)
@@ -712,6 +706,7 @@ def run_ours(args):
         step(k)
     prof = g.he_profile_read(ctx)
     g.he_profile(ctx, False)
+    launches_per_step = sum(v[1] for v in prof.values()) // prof_steps  # one mark per kernel
     per_kernel = {}
     split = 0  # the passes' stages follow the ring size alone (he_shape's ntt_split has no effect)
     for k, v in prof.items():
@@ -885,8 +880,9 @@ def run_ours(args):
         plan.close()
         del nws, prep, nevk, nct, nout
 
-    # ALU ceilings: the NTT's butterfly and the conversions' inner loop,
-    # register-resident, measured in this run at its clocks
+    # ALU ceilings: the NTT's butterfly and the CUDA-core conversions' inner loop,
+    # register-resident, measured in this run at its clocks (conversions on the
+    # tensor cores, for primes of 52 to 55 bits, run above the latter)
     bfly_peak = g.he_probe_butterfly_rate(152 * 8, 4096, stream)
     conv_width = {"modup": kernel_width(prm.alpha), "moddown_conv": kernel_width(prm.K)}
     conv_peak = {k: g.he_probe_conversion_rate(w, 152 * 8, max(64, 4096 // w), stream) for k, w in conv_width.items()}

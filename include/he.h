@@ -459,17 +459,20 @@ int he_nr_rescale(he_nr_plan *plan, const uint64_t *ct, int logq, uint64_t *out,
 
 /* Launch shape of the path: the most NTT limbs of one prime that a CTA of a
  * batch takes one after another (they share the staged twiddles; 1..4; a single
- * HE Mul always runs one limb per CTA), ModUp targets per CTA (4, 8 or 16),
+ * HE Mul always runs one limb per CTA), ModUp targets per CTA (4, 8 or 16;
+ * contexts whose base conversions run on the CUDA cores, below),
  * whether the path's kernels use programmatic dependent launch (1: a kernel's
  * CTAs may be scheduled while its predecessor drains; each waits for it in
- * hardware before touching its data; 2: as 1, and a kernel allows its successor
- * to be launched as soon as its own last wave runs, so the successor's CTAs fill
- * the SMs its tail leaves idle; 0: off).  Speed only: every shape gives
+ * hardware before touching its data; the NTT passes and launches of many CTAs
+ * allow it as soon as their own last wave runs, so the successor's CTAs fill
+ * the SMs their tail leaves idle; 2: as 1, and every kernel does; 0: off).  Speed only: every shape gives
  * bit-identical results.  Default {4, 8, 1, 0, 8, 7, 0, 0, 0}.  A batch graph
  * keeps the shape it was captured with, except the limb-group cap.
  * ntt_r8, ntt_split, ntt_small and ntt_onepass are checked, kept and returned,
  * and have no effect: the NTT passes choose their rounds and tiles by ring size
- * and role. */
+ * and role.  Contexts whose primes have 52 to 55 bits convert bases on the tensor
+ * cores (and form every key-switch sum in the inner product); there modup_chunk
+ * and fuse's bits 1 and 2 have no effect either. */
 typedef struct {
     int group_cap;
     int modup_chunk;

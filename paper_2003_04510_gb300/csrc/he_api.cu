@@ -267,6 +267,7 @@ static int create(he_ctx **out, const he_params *p, bool device)
     int rc = build_context(c, p, device);
     if (rc != HE_OK) {
         if (c->arena) cudaFree(c->arena);
+        if (c->flag) cudaFreeHost(c->flag);
         delete c;
         return rc;
     }
@@ -288,6 +289,7 @@ int he_ctx_destroy(he_ctx *c)
     if (c->io_h2d2) cudaStreamDestroy(c->io_h2d2);
     if (c->io_d2h) cudaStreamDestroy(c->io_d2h);
     if (c->arena) cudaFree(c->arena);
+    if (c->flag) cudaFreeHost(c->flag);
     delete c;
     return HE_OK;
 }
@@ -725,6 +727,7 @@ int he_autotune(he_ctx *c, const he_job *jobs, int count, const uint64_t *evk, v
         float ms = 0;
         if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)
             return HE_ECUDA;
+        if ((r = device_waits(c)) != HE_OK) return r;
         sh.ms = ms / reps;
         if (tried && n < max_tried) tried[n] = sh;
         n++;
@@ -820,6 +823,7 @@ int he_autotune(he_ctx *c, const he_job *jobs, int count, const uint64_t *evk, v
                 if (rc == HE_OK &&
                     (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
                     rc = HE_ECUDA;
+                if (rc == HE_OK) rc = device_waits(c);
                 t[k].push_back(ms / (2 * reps));
             }
         if (rc == HE_OK) {
@@ -848,6 +852,7 @@ int he_profile_read(he_ctx *c, int max, char *names, double *total_ms, int *call
 {
     if (check_dev(c) || max < 1 || !names || !total_ms || !calls || !count) return HE_EINVAL;
     if (c->prof_used > 0 && cudaEventSynchronize(c->prof_pool[c->prof_used - 1]) != cudaSuccess) return HE_ECUDA;
+    if (int rc = device_waits(c)) return rc;
     std::vector<std::string> keys;
     std::vector<double> ms;
     std::vector<int> n;
@@ -901,7 +906,7 @@ int he_mul_rescale_host(he_ctx *c, const uint64_t *ct1, const uint64_t *ct2, con
     if (rc) return rc;
     HE_TRY(cudaMemcpyAsync(out, dout, 2 * (size_t)(level - 1) * limb, cudaMemcpyDeviceToHost, st));
     HE_TRY(cudaStreamSynchronize(st));
-    return HE_OK;
+    return device_waits(c);
 }
 
 size_t he_host_stream_workspace_bytes(const he_ctx *c, int max_level, int slots)
@@ -973,7 +978,7 @@ int he_mul_rescale_host_stream(he_ctx *c, int count, const uint64_t *const *ct1,
     }
     HE_TRY(cudaStreamSynchronize(down));
     HE_TRY(cudaStreamSynchronize(st));
-    return HE_OK;
+    return device_waits(c);
 }
 
 }  // extern "C"
@@ -1257,7 +1262,10 @@ int he_batch_graph_launch(he_batch_graph *g, int count, const he_job *jobs, void
     }
     // the launch that last read this pinned header must have finished
     const int b = g->memcpy_node ? (int)(g->nlaunch & 1u) : 0;
-    if (g->launched[b] && cudaEventSynchronize(g->done[b]) != cudaSuccess) return HE_ECUDA;
+    if (g->launched[b]) {
+        if (cudaEventSynchronize(g->done[b]) != cudaSuccess) return HE_ECUDA;
+        if (int rc = device_waits(c)) return rc;
+    }
     unsigned char *pin = g->pinned[b];
     const size_t N = (size_t)c->N;
     u64 *data = (u64 *)(g->ws + g->hdr);

@@ -56,6 +56,13 @@ struct NttGroup {
 // within a prime is kept); the groups come out sorted by prime.
 std::vector<NttGroup> group_jobs(const std::vector<NttJob> &jobs, int cap = kGroupMax);
 
+// One target of a tensor-core base conversion (tc.cuh): the constant added to
+// its recombined planes, 2^b - q and b - 36, b = bitlen(q).
+struct TcTarget {
+    u64 base;
+    uint32_t delta, shift;
+};
+
 // Per-level constants on the device.
 struct DevLevel {
     int l, beta, E, A;             // level, digits, K+l, alpha padded for the kernels
@@ -66,6 +73,11 @@ struct DevLevel {
     const ulonglong2 *qinv_last;   // [l-1]: q_{l-1}^-1 mod q_i (value, Shoup)
     const ulonglong2 *pinv_qinv;   // [l-1]: P^-1 * q_{l-1}^-1 mod q_i
     const u64 *pbpq;               // [l-1][KP]: [Phat_k P^-1 q_{l-1}]_{q_i} (one division by P q_{l-1})
+    // tensor-core conversions (he_ctx::tc): ModUp images and targets
+    // [beta][up_nch][up_tp], up_tc targets per chunk; pbpq's images [chunk]
+    const unsigned char *tc_up, *tc_pq;
+    const TcTarget *tc_up_t, *tc_pq_t;
+    int up_nch, up_tc, up_tp, up_bytes;
 };
 
 // One HE Mul of a launch: its operands, output, workspace base and level.
@@ -81,7 +93,7 @@ struct JobRef {
     BatchItem one;
     int B;                   // number of jobs
     int lmax;                // largest level among them
-    int trigger;             // early dependent launch (the shape's pdl = 2): see griddep_wait
+    int trigger;             // let the next launch start early (early_launch): see griddep_wait
 };
 #ifdef __CUDACC__
 __device__ __forceinline__ BatchItem job_item(const JobRef &R, int z) { return R.items ? R.items[z] : R.one; }
@@ -124,6 +136,9 @@ struct HostLevel {
     WsLayout ws;
     std::vector<NttJob> intt1, intt1f, ntt_up, intt2, intt2f, ntt_conv, ntt_z, rs_intt, rs_ntt, intt2pq;
     std::vector<u64> modupB;
+    std::vector<unsigned char> tc_up, tc_pq;
+    std::vector<TcTarget> tc_up_t, tc_pq_t;
+    int up_nch = 0, up_tc = 0, up_tp = 0, up_bytes = 0;
     std::vector<u64> pbpq;  // [l-1][KP]: [Phat_k P^-1 q_{l-1}]_{q_i}, split at bit 28 (one division by P q_{l-1})
     std::vector<ulonglong2> qinv_last, pinv_qinv;
 };
@@ -140,12 +155,13 @@ struct he_ctx {
     int group_cap = he::kGroupMax;
     int modup_chunk = 8;
     int pdl = 1;                         // programmatic dependent launch between the path's kernels:
-                                         // 0 off, 1 on, 2 on with early dependent launch (griddep_wait)
+                                         // 0 off, 1 on, 2 on with every early start (early_launch)
     int ntt_r8 = 0, ntt_split = 0, ntt_small = 0, ntt_onepass = 0;  // kept for he_get_shape; no effect
     int ip_jobs = he::kIpJobsMax;        // batches: jobs sharing one CTA's key words in the inner product (1: none)
     int fuse = 7;                        // bit 0: the tensor product inside the first inverse NTT pass of d2;
                                          // bit 1: the q limbs' key-switch sums beside the ModDown conversion;
                                          // bit 2: the special limbs' sums inside their iNTT's first pass
+                                         // (bits 1 and 2, modup_chunk: CUDA-core conversions only)
     std::vector<u64> ext;                // moduli, ext order
     std::vector<NttMod> nt;              // the NTT's constants of each modulus
     std::vector<u64> psi;                // smallest primitive 2N-th roots, ext order
@@ -158,6 +174,17 @@ struct he_ctx {
     std::vector<ulonglong2> pinv;        // [L]: P^-1 mod q_i
     std::vector<ulonglong2> phat_inv;    // [K]: Phat_k^-1 mod p_k
     std::vector<he::HostLevel> host_levels;  // index l (1..L)
+    // base conversions on the tensor cores: primes of 52 to 55 bits whose
+    // constants keep every plane exact (tc_image); else the CUDA-core kernels
+    bool tc = false;
+    unsigned *flag = nullptr, *d_flag = nullptr;  // mapped host word a bounded device wait sets when it gives up
+    uint32_t up_off5 = 0, dn_off5 = 0;   // top digits' offsets of ModUp's and ModDown's sources
+    int up_smem = 0, dn_smem = 0;        // shared memory of a CTA
+    int dn_nch = 0, dn_tc = 0, dn_tp = 0, dn_bytes = 0, dn_last_bytes = 0;  // ModDown: chunks of targets
+    std::vector<unsigned char> tc_PB, tc_PBP, tc_last;  // [dn_nch] images; [L] images of one target
+    std::vector<he::TcTarget> tc_PB_t, tc_PBP_t;        // [L]
+    const unsigned char *d_tc_PB = nullptr, *d_tc_PBP = nullptr, *d_tc_last = nullptr;
+    const he::TcTarget *d_tc_PB_t = nullptr, *d_tc_PBP_t = nullptr;
     // device
     int device_id = -1;
     void *arena = nullptr;               // one allocation holding every device table
@@ -194,6 +221,19 @@ struct he_ctx {
 namespace he {
 // host_params.cpp
 int build_context(he_ctx *ctx, const he_params *p, bool device);
+// After a synchronisation: HE_ETIMEOUT if a bounded device wait has given up
+// since the last check, else HE_OK.
+inline int device_waits(const he_ctx *c)
+{
+    return c->flag && __atomic_exchange_n(c->flag, 0u, __ATOMIC_RELAXED) ? HE_ETIMEOUT : HE_OK;
+}
+// tc_tables.cpp
+int tc_groups(int nsrc);  // groups of four source limbs
+bool tc_source_ok(u64 p);
+uint32_t tc_off5(const std::vector<u64> &src);
+bool tc_image(const std::vector<u64> &c, const std::vector<u64> &q, int T, const std::vector<u64> &src, int tp,
+              unsigned char *image, TcTarget *targets);
+cudaError_t configure_conversions(const he_ctx *c);  // shared-memory limits of the tensor-core conversions
 // kernels (ntt.cu, keyswitch.cu); return cudaError_t
 // Record a profiling mark named after the kernel that just finished (no-op
 // unless profiling is enabled on the context).
@@ -216,6 +256,17 @@ enum LaunchTag {
 };
 extern thread_local std::vector<int> *capture_log;
 extern thread_local int capture_tag;
+
+// Whether a launch of `ctas` CTAs, other than an NTT pass, lets its successor
+// start early (griddep_wait).  NTT passes always do at pdl >= 1: their successor's
+// CTAs load twiddles meanwhile (measured, pass by pass off against on: 2^12 L = 3
+// 41.4 -> 39.4 us, 2^17 L = 44 815 -> 804, the 2^16 weighted sum 62.2 -> 59.4).
+// The other kernels do it only from 8 CTAs per SM.  Below that the waiting CTAs
+// take the room of the running kernel's late CTAs, and a conversion's persistent
+// CTAs wait behind them: 2^15 L = 9 takes 83.2 us with the early start in every
+// kernel, 71.9 with it above 152 CTAs and 69.8 above 1216; larger rings do not
+// tell the limits apart (2^16 198.4 each time, 2^17 803.7 and 805.9).
+inline int early_launch(int pdl, long long ctas) { return pdl >= 2 || (pdl == 1 && ctas >= 8 * 152); }
 
 template <typename... KArgs, typename... Args>
 inline void launch_k(bool dep, void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,

@@ -225,6 +225,114 @@ static WsLayout layout_for(int l, int K, int alpha)
     return w;
 }
 
+// Images and targets of the tensor-core conversions (tc.cuh); false where the
+// context's primes or sizes do not allow them, and the CUDA-core kernels run.  The
+// line is where the six planes are exact: primes of at most 55 bits fill six digits
+// (a 56-bit target's last plane passes its 22 bits), targets of 52 or more fold in
+// one step, and some 14 limbs' worth of digits stay below the planes' offsets, for
+// the constants at hand (tc_image counts).  Inside it this form is the faster one at
+// every size measured: one HE Mul + rescale 212 -> 198 us at 2^16 (level 24), 952 ->
+// 804 at 2^17 (level 44), 71.9 -> 69.8 at 2^15 (level 9).
+static bool build_tc(he_ctx *c)
+{
+    const int K = c->K, L = c->L;
+    const std::vector<u64> ps(c->ext.begin(), c->ext.begin() + K), qs(c->ext.begin() + K, c->ext.end());
+    for (u64 x : c->ext)
+        if (!tc_source_ok(x)) return false;
+    auto round8 = [](int v) { return (v + 7) & ~7; };
+    auto k_pad = [](int g) { return (24 * g + 1 + 15) / 16 * 16; };  // tc::k_pad
+    auto rows = [](int tp) { return (6 * tp + 15) / 16 * 16; };
+    // [prod_{i2 != skip} m[i2]]_t over m[lo, hi)
+    auto hat = [&](const std::vector<u64> &m, int lo, int hi, int skip, u64 t) {
+        u64 v = 1;
+        for (int i = lo; i < hi; i++)
+            if (i != skip) v = mul(v, m[i] % t, t);
+        return v;
+    };
+    c->up_off5 = tc_off5(qs);
+    c->dn_off5 = tc_off5(ps);
+    // ModDown: chunks of at most 24 targets (tc::kTargets)
+    const int kd = k_pad(tc_groups(K));
+    c->dn_nch = (L + 23) / 24;
+    c->dn_tc = (L + c->dn_nch - 1) / c->dn_nch;
+    c->dn_tp = round8(c->dn_tc);
+    c->dn_bytes = rows(c->dn_tp) * kd * 2;
+    c->dn_last_bytes = 16 * kd * 2;
+    c->dn_smem = 3 * 128 * kd * 2 + c->dn_bytes + c->dn_last_bytes;  // three teams
+    c->tc_PB.assign((size_t)c->dn_nch * c->dn_bytes, 0);
+    c->tc_PBP.assign((size_t)c->dn_nch * c->dn_bytes, 0);
+    c->tc_last.assign((size_t)L * c->dn_last_bytes, 0);
+    c->tc_PB_t.resize((size_t)c->dn_nch * c->dn_tp);
+    c->tc_PBP_t.resize((size_t)c->dn_nch * c->dn_tp);
+    std::vector<u64> pb((size_t)L * K), pbp((size_t)L * K);
+    for (int i = 0; i < L; i++)
+        for (int k = 0; k < K; k++) {
+            pb[(size_t)i * K + k] = hat(ps, 0, K, k, qs[i]);
+            pbp[(size_t)i * K + k] = mul(pb[(size_t)i * K + k], c->pinv[i].x, qs[i]);
+        }
+    auto slice = [&](const std::vector<u64> &m, int i0, int n) {
+        return std::vector<u64>(m.begin() + (size_t)i0 * K, m.begin() + (size_t)(i0 + n) * K);
+    };
+    for (int ch = 0; ch < c->dn_nch; ch++) {
+        const int i0 = ch * c->dn_tc, n = std::min(c->dn_tc, L - i0);
+        const std::vector<u64> t(qs.begin() + i0, qs.begin() + i0 + n);
+        if (!tc_image(slice(pb, i0, n), t, n, ps, c->dn_tp, &c->tc_PB[(size_t)ch * c->dn_bytes],
+                      &c->tc_PB_t[(size_t)ch * c->dn_tp]) ||
+            !tc_image(slice(pbp, i0, n), t, n, ps, c->dn_tp, &c->tc_PBP[(size_t)ch * c->dn_bytes],
+                      &c->tc_PBP_t[(size_t)ch * c->dn_tp]))
+            return false;
+    }
+    for (int i = 0; i < L; i++) {
+        TcTarget t1;
+        if (!tc_image(slice(pbp, i, 1), {qs[i]}, 1, ps, 1, &c->tc_last[(size_t)i * c->dn_last_bytes], &t1)) return false;
+    }
+    // per level: ModUp images of every digit, and the one-division ModDown's
+    const int ku = k_pad(tc_groups(c->alpha));
+    for (int l = 1; l <= L; l++) {
+        HostLevel &H = c->host_levels[l];
+        const int beta = (l + c->alpha - 1) / c->alpha, El = K + l;
+        const int nlast = l - (beta - 1) * c->alpha, tmax = El - nlast;  // the last digit has the most targets
+        H.up_nch = (tmax + 23) / 24;
+        H.up_tc = (tmax + H.up_nch - 1) / H.up_nch;
+        H.up_tp = round8(H.up_tc);
+        H.up_bytes = rows(H.up_tp) * ku * 2;
+        c->up_smem = std::max(c->up_smem, 3 * 128 * ku * 2 + H.up_bytes);  // three teams
+        H.tc_up.assign((size_t)beta * H.up_nch * H.up_bytes, 0);
+        H.tc_up_t.resize((size_t)beta * H.up_nch * H.up_tp);
+        for (int j = 0; j < beta; j++) {
+            const int lo = j * c->alpha, hi = std::min((j + 1) * c->alpha, l), nj = hi - lo;
+            std::vector<u64> src(c->alpha, qs[lo]);  // every digit runs with alpha limbs; unused ones have no constant
+            for (int i = lo; i < hi; i++) src[i - lo] = qs[i];
+            for (int ch = 0; ch < H.up_nch; ch++) {
+                std::vector<u64> cst, t;
+                for (int u = ch * H.up_tc; u < std::min((ch + 1) * H.up_tc, El - nj); u++) {
+                    const int e = u < K + lo ? u : u + nj;
+                    t.push_back(c->ext[e]);
+                    for (int i = 0; i < c->alpha; i++)
+                        cst.push_back(i < nj ? hat(qs, lo, hi, lo + i, c->ext[e]) : 0);
+                }
+                const size_t at = (size_t)j * H.up_nch + ch;
+                if (!tc_image(cst, t, (int)t.size(), src, H.up_tp, &H.tc_up[at * H.up_bytes], &H.tc_up_t[at * H.up_tp]))
+                    return false;
+            }
+        }
+        H.tc_pq.assign((size_t)c->dn_nch * c->dn_bytes, 0);
+        H.tc_pq_t.resize((size_t)c->dn_nch * c->dn_tp);
+        const u64 ql = qs[l - 1];
+        for (int ch = 0; ch < c->dn_nch; ch++) {
+            std::vector<u64> cst, t;
+            for (int i = ch * c->dn_tc; i < std::min((ch + 1) * c->dn_tc, l - 1); i++) {
+                t.push_back(qs[i]);
+                for (int k = 0; k < K; k++) cst.push_back(mul(pbp[(size_t)i * K + k], ql % qs[i], qs[i]));
+            }
+            if (!tc_image(cst, t, (int)t.size(), ps, c->dn_tp, &H.tc_pq[(size_t)ch * c->dn_bytes],
+                          &H.tc_pq_t[(size_t)ch * c->dn_tp]))
+                return false;
+        }
+    }
+    return true;
+}
+
 int build_context(he_ctx *c, const he_params *p, bool device)
 {
     // q_bits, p_bits <= 57 keep every base-conversion accumulator (at most 16
@@ -424,6 +532,12 @@ int build_context(he_ctx *c, const he_params *p, bool device)
         }
     }
     if (!device) return HE_OK;
+    c->tc = build_tc(c);
+    if (c->tc) {
+        if (cudaHostAlloc((void **)&c->flag, sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess) return HE_ECUDA;
+        *c->flag = 0;
+        if (cudaHostGetDevicePointer((void **)&c->d_flag, c->flag, 0) != cudaSuccess) return HE_ECUDA;
+    }
 
     // ---- device arena -------------------------------------------------------
     size_t off = 0;
@@ -440,6 +554,9 @@ int build_context(he_ctx *c, const he_params *p, bool device)
     }
     const size_t o_PB = take(sizeof(u64) * c->PB.size());
     const size_t o_PBP = take(sizeof(u64) * c->PBP.size());
+    const size_t o_tPB = take(c->tc_PB.size()), o_tPBP = take(c->tc_PBP.size()), o_tlast = take(c->tc_last.size()),
+                 o_tPBt = take(sizeof(TcTarget) * c->tc_PB_t.size()),
+                 o_tPBPt = take(sizeof(TcTarget) * c->tc_PBP_t.size());
     const size_t o_pinv = take(sizeof(ulonglong2) * L);
     const size_t o_levels = take(sizeof(DevLevel) * (L + 1));
     // per level: the NTT lists of one job, one limb per group (a group's limbs
@@ -447,7 +564,7 @@ int build_context(he_ctx *c, const he_params *p, bool device)
     // to give up CTAs for it; at N = 2^16, level 24, 211 us against 236 with
     // two limbs per group and 264 with four)
     constexpr int NL = 10;  // job lists per level
-    struct LvlOff { size_t modupB, qinv, pq, pbpq, j[NL]; };
+    struct LvlOff { size_t modupB, qinv, pq, pbpq, tc[4], j[NL]; };
     std::vector<LvlOff> lo(L + 1);
     std::vector<std::vector<std::vector<NttGroup>>> gl(L + 1, std::vector<std::vector<NttGroup>>(NL));
     for (int l = 1; l <= L; l++) {
@@ -456,6 +573,10 @@ int build_context(he_ctx *c, const he_params *p, bool device)
         lo[l].qinv = take(sizeof(ulonglong2) * H.qinv_last.size());
         lo[l].pq = take(sizeof(ulonglong2) * H.pinv_qinv.size());
         lo[l].pbpq = take(sizeof(u64) * H.pbpq.size());
+        lo[l].tc[0] = take(H.tc_up.size());
+        lo[l].tc[1] = take(sizeof(TcTarget) * H.tc_up_t.size());
+        lo[l].tc[2] = take(H.tc_pq.size());
+        lo[l].tc[3] = take(sizeof(TcTarget) * H.tc_pq_t.size());
         const std::vector<NttJob> *lists[NL] = {&H.intt1, &H.intt1f, &H.ntt_up, &H.intt2, &H.intt2f,
                                                 &H.ntt_conv, &H.ntt_z, &H.rs_intt, &H.rs_ntt, &H.intt2pq};
         for (int t = 0; t < NL; t++) {
@@ -507,6 +628,13 @@ int build_context(he_ctx *c, const he_params *p, bool device)
     memcpy(img.data() + o_PB, c->PB.data(), sizeof(u64) * c->PB.size());
     memcpy(img.data() + o_PBP, c->PBP.data(), sizeof(u64) * c->PBP.size());
     memcpy(img.data() + o_pinv, c->pinv.data(), sizeof(ulonglong2) * L);
+    if (c->tc) {
+        memcpy(img.data() + o_tPB, c->tc_PB.data(), c->tc_PB.size());
+        memcpy(img.data() + o_tPBP, c->tc_PBP.data(), c->tc_PBP.size());
+        memcpy(img.data() + o_tlast, c->tc_last.data(), c->tc_last.size());
+        memcpy(img.data() + o_tPBt, c->tc_PB_t.data(), sizeof(TcTarget) * c->tc_PB_t.size());
+        memcpy(img.data() + o_tPBPt, c->tc_PBP_t.data(), sizeof(TcTarget) * c->tc_PBP_t.size());
+    }
     c->dev_levels.assign(L + 1, DevLevel());
     c->jobs.assign(L + 1, LevelJobs());
     for (int l = 1; l <= L; l++) {
@@ -533,6 +661,20 @@ int build_context(he_ctx *c, const he_params *p, bool device)
         D.qinv_last = (const ulonglong2 *)(base + lo[l].qinv);
         D.pinv_qinv = (const ulonglong2 *)(base + lo[l].pq);
         D.pbpq = (const u64 *)(base + lo[l].pbpq);
+        if (c->tc) {
+            memcpy(img.data() + lo[l].tc[0], H.tc_up.data(), H.tc_up.size());
+            memcpy(img.data() + lo[l].tc[1], H.tc_up_t.data(), sizeof(TcTarget) * H.tc_up_t.size());
+            memcpy(img.data() + lo[l].tc[2], H.tc_pq.data(), H.tc_pq.size());
+            memcpy(img.data() + lo[l].tc[3], H.tc_pq_t.data(), sizeof(TcTarget) * H.tc_pq_t.size());
+            D.tc_up = (const unsigned char *)(base + lo[l].tc[0]);
+            D.tc_up_t = (const TcTarget *)(base + lo[l].tc[1]);
+            D.tc_pq = (const unsigned char *)(base + lo[l].tc[2]);
+            D.tc_pq_t = (const TcTarget *)(base + lo[l].tc[3]);
+            D.up_nch = H.up_nch;
+            D.up_tc = H.up_tc;
+            D.up_tp = H.up_tp;
+            D.up_bytes = H.up_bytes;
+        }
         const NttGroup *dptr[NL];
         int cnt[NL];
         for (int t = 0; t < NL; t++) {
@@ -558,9 +700,15 @@ int build_context(he_ctx *c, const he_params *p, bool device)
     c->d_primes = (DevPrime *)(base + o_primes);
     c->d_PB = (const u64 *)(base + o_PB);
     c->d_PBP = (const u64 *)(base + o_PBP);
+    c->d_tc_PB = (const unsigned char *)(base + o_tPB);
+    c->d_tc_PBP = (const unsigned char *)(base + o_tPBP);
+    c->d_tc_last = (const unsigned char *)(base + o_tlast);
+    c->d_tc_PB_t = (const TcTarget *)(base + o_tPBt);
+    c->d_tc_PBP_t = (const TcTarget *)(base + o_tPBPt);
     c->d_pinv = (const ulonglong2 *)(base + o_pinv);
     c->d_levels = (DevLevel *)(base + o_levels);
     if (configure_ntt(c) != cudaSuccess) return HE_ECUDA;
+    if (c->tc && configure_conversions(c) != cudaSuccess) return HE_ECUDA;
     return HE_OK;
 }
 

@@ -28,12 +28,14 @@
 
 #include "he_internal.h"
 #include "modarith.cuh"
+#include "tc.cuh"
 
 namespace he {
 
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kSMs = 152;
 // Base conversions: two targets per loop trip, so one target's reduction
 // overlaps the next target's multiply-adds.
 constexpr int kConvUnroll = 2;
@@ -137,6 +139,82 @@ k_modup(const JobRef R, const DevLevel *__restrict__ lv_arr, const DevPrime *__r
         else
             st2(Uj + (size_t)se[u] * N + n, acc3k_reduce_lazy(ax, q, mu, sh), acc3k_reduce_lazy(ay, q, mu, sh));
     }
+}
+
+// ModUp on the tensor cores (tc.cuh).  grid: x over CTAs of three teams, which
+// share the tiles of (digit, chunk of at most 24 targets) y of job z; the outputs
+// are those of k_modup, lazily below 3q, or canonical.
+constexpr int kTeams = 3;
+
+template <int G>
+struct UpJob {
+    const u64 *y;  // the digit's first limb
+    u64 *U;        // the digit's outputs
+    const u64 *q;  // CANON: the targets' moduli
+    int N, nj;
+    bool canon;
+    u64 v[(G + 1) / 2][4];
+    u64 *o;
+    __device__ __forceinline__ void load(size_t n, int half)
+    {
+#pragma unroll
+        for (int k = 0; k < (G + 1) / 2; k++)
+            if (2 * k + half < G) {
+#pragma unroll
+                for (int i = 0; i < 4; i++) v[k][i] = y[(size_t)min(4 * (2 * k + half) + i, nj - 1) * N + n];
+            }
+    }
+    __device__ __forceinline__ u64 value(int k, int i) const { return v[k][i]; }
+    __device__ __forceinline__ void start(size_t n) { o = U + n; }
+    __device__ __forceinline__ void extra(const uint32_t *) {}
+    __device__ __forceinline__ void put(int u, u64 x, const tc::Row &t)
+    {
+        if (canon) x = csub(csub(x, 2 * q[u]), q[u]);
+        o[t.off] = x;
+    }
+};
+
+template <int G, bool CANON>
+__global__ void __launch_bounds__(kTeams *tc::kTeam, 1)
+k_modup_tc(const JobRef R, const DevLevel *__restrict__ lv_arr, const DevPrime *__restrict__ primes, int K, int N,
+           int nchmax, uint32_t off5, unsigned *flag)
+{
+    const BatchItem it = job_of(R, blockIdx.z);
+    const DevLevel &lv = lv_arr[it.level];
+    const int j = blockIdx.y / nchmax, ch = blockIdx.y - j * nchmax;
+    if (j >= lv.beta || ch >= lv.up_nch) return idle_exit();
+    const int lo = lv.dig_lo[j], nj = lv.dig_n[j], u0 = ch * lv.up_tc;
+    const int cnt = min(lv.up_tc, lv.E - nj - u0);
+    if (cnt <= 0) return idle_exit();
+    extern __shared__ __align__(128) unsigned char sm[];
+    __shared__ tc::Row st[tc::kTargets + 1];
+    __shared__ u64 sq[tc::kTargets];
+    __shared__ tc::Shared<kTeams> ts;
+    constexpr int ABYTES = tc::k_pad(G) * tc::kRows * 2;
+    unsigned char *B = sm + kTeams * ABYTES;
+    tc::begin(ts);
+    const size_t at = (size_t)j * lv.up_nch + ch;
+    tc::copy_image(B, lv.tc_up + at * lv.up_bytes, lv.up_bytes);
+    if (threadIdx.x < cnt) {
+        const int u = u0 + threadIdx.x;
+        const int e = u < K + lo ? u : u + nj;
+        st[threadIdx.x] = tc::make_row(lv.tc_up_t[at * lv.up_tp + threadIdx.x], (uint32_t)e * (uint32_t)N);
+        sq[threadIdx.x] = primes[e].q;
+    }
+    const uint32_t tmem = tc::ready(ts);
+    griddep_wait(R.trigger);
+    const int team = threadIdx.x / tc::kTeam;
+    UpJob<G> job;
+    job.y = it.ws + ((size_t)lv.o_y + lo) * N;
+    job.U = it.ws + ((size_t)lv.o_u + (size_t)j * lv.E) * N;
+    job.q = sq;
+    job.N = N;
+    job.nj = nj;
+    job.canon = CANON;
+    tc::team_tiles<G, false>(job, sm + team * ABYTES, B, B, (uint32_t)lv.up_bytes / (2 * tc::k_pad(G)),
+                             tmem + team * tc::kCols, &ts.bar[team], team, blockIdx.x * kTeams + team,
+                             gridDim.x * kTeams, N / tc::kRows, cnt, st, off5, flag);
+    tc::end(ts);
 }
 
 // grid: x over N/2/kThreads, y over ext limbs (up to K + lmax), z over jobs.
@@ -506,6 +584,103 @@ k_moddown_ipq(const JobRef R, const u64 *__restrict__ PB, const ulonglong2 *__re
     ip_body<BM, SEEDED>(R, it, lv_arr[it.level], e, evk, primes, K, L, N, seeds);
 }
 
+// The ModDown conversion on the tensor cores (tc.cuh): the outputs of
+// moddown_body.  The row of q_{l-1} that the rescaling tail needs first is the
+// extra target.
+struct DnArgs {
+    const unsigned char *img, *last;  // images [chunk]; of one target [L]
+    const TcTarget *tgt;              // [chunk][tp]
+    const ulonglong2 *pinv;
+    const DevLevel *levels;
+    const DevPrime *primes;
+    unsigned *flag;
+    int K, N, nch, tc, tp, bytes, last_bytes;
+    uint32_t off5;
+};
+
+template <int G, int MODE>
+struct DnJob {
+    const u64 *ys, *rr;
+    u64 *z;
+    const tc::Row *last;  // q_{l-1}'s
+    ulonglong2 pv;  // P^-1 mod q_{l-1}
+    u64 q;          // q_{l-1}
+    int N, K, h;
+    u64 v[(G + 1) / 2][4], r0, r1, r;
+    u64 *o;
+    __device__ __forceinline__ void load(size_t n, int half)
+    {
+#pragma unroll
+        for (int k = 0; k < (G + 1) / 2; k++)
+            if (2 * k + half < G) {
+#pragma unroll
+                for (int i = 0; i < 4; i++) v[k][i] = ys[(size_t)min(4 * (2 * k + half) + i, K - 1) * N + n];
+            }
+        if (MODE != kTailPlain) {
+            r0 = rr[(size_t)h * N + n];
+            r1 = rr[(size_t)(2 + h) * N + n];
+        }
+    }
+    __device__ __forceinline__ u64 value(int k, int i) const { return v[k][i]; }
+    __device__ __forceinline__ void start(size_t n)
+    {
+        o = z + n;
+        // kTailRescalePQ: y_last; kTailRescale: conv_{l-1} P^-1 still to subtract
+        r = MODE != kTailPlain ? add_mod(r0, shoup(r1, pv.x, pv.y, q), q) : 0;
+    }
+    __device__ __forceinline__ void extra(const uint32_t *P)
+    {
+        const u64 c = tc::recombine(P[0], P[1], P[2], P[3], P[4], P[5], *last);
+        r = sub_mod(r, csub(csub(c, 2 * q), q), q);
+    }
+    // z feeds a forward NTT, which takes inputs below 4q: the conversion (below
+    // 3q) and r (below q_{l-1} < q_i) are added without a reduction
+    __device__ __forceinline__ void put(int, u64 x, const tc::Row &t) { o[t.off] = x + r; }
+};
+
+// grid: x over CTAs of three teams, y over (half, chunk), z over jobs.
+template <int G, int MODE>
+__global__ void __launch_bounds__(kTeams *tc::kTeam, 1) k_moddown_tc(const JobRef R, const DnArgs D)
+{
+    const int h = blockIdx.y / D.nch, ch = blockIdx.y - h * D.nch;
+    constexpr bool FUSED = MODE == kTailRescale, PQ = MODE == kTailRescalePQ;
+    const BatchItem it = job_of(R, blockIdx.z);
+    const int l = it.level, N = D.N, K = D.K;
+    const DevLevel &lv = D.levels[l];
+    const int nout = MODE != kTailPlain ? l - 1 : l, i0 = ch * D.tc, cnt = min(D.tc, nout - i0);
+    if (cnt <= 0) return idle_exit();
+    extern __shared__ __align__(128) unsigned char sm[];
+    __shared__ tc::Row st[tc::kTargets + 1];
+    __shared__ tc::Shared<kTeams> ts;
+    constexpr int ABYTES = tc::k_pad(G) * tc::kRows * 2;
+    unsigned char *B = sm + kTeams * ABYTES, *B1 = B + D.bytes;
+    tc::begin(ts);
+    const TcTarget *tgt = PQ ? lv.tc_pq_t : D.tgt;
+    tc::copy_image(B, (PQ ? lv.tc_pq : D.img) + (size_t)ch * D.bytes, D.bytes);
+    if (FUSED) tc::copy_image(B1, D.last + (size_t)(l - 1) * D.last_bytes, D.last_bytes);
+    if (threadIdx.x < cnt)
+        st[threadIdx.x] = tc::make_row(tgt[(size_t)ch * D.tp + threadIdx.x], (uint32_t)threadIdx.x * (uint32_t)N);
+    DnJob<G, MODE> job;
+    if (FUSED && threadIdx.x == 64)
+        st[tc::kTargets] = tc::make_row(tgt[(size_t)((l - 1) / D.tc) * D.tp + (l - 1) % D.tc], 0);
+    job.last = &st[tc::kTargets];
+    job.q = D.primes[K + l - 1].q;
+    job.pv = D.pinv[l - 1];
+    job.ys = it.ws + ((size_t)lv.o_ys + (size_t)h * K) * N;
+    job.rr = it.ws + (size_t)lv.o_r * N;
+    job.z = it.ws + ((size_t)lv.o_z + (size_t)h * nout + i0) * N;
+    job.N = N;
+    job.K = K;
+    job.h = h;
+    const uint32_t tmem = tc::ready(ts);
+    griddep_wait(R.trigger);
+    const int team = threadIdx.x / tc::kTeam;
+    tc::team_tiles<G, FUSED>(job, sm + team * ABYTES, B, B1, (uint32_t)D.bytes / (2 * tc::k_pad(G)),
+                             tmem + team * tc::kCols, &ts.bar[team], team, blockIdx.x * kTeams + team,
+                             gridDim.x * kTeams, N / tc::kRows, cnt, st, D.off5, D.flag);
+    tc::end(ts);
+}
+
 // grid: x over N/2/kThreads, y over limbs, z over 2 * jobs (h = z & 1).
 // out[h][i] = d_h[i] + (KS_h[K+i] - C[h][i]) P^-1 mod q_i, i < l
 __global__ void __launch_bounds__(kThreads)
@@ -614,6 +789,13 @@ k_elementwise(const u64 *x, const u64 *y, u64 *out, const DevPrime *__restrict__
     st2(out + o, r0, r1);
 }
 
+// The launch's job reference, with early dependent launch as its size asks.
+inline JobRef sized(const he_ctx *c, JobRef R, dim3 g)
+{
+    R.trigger = early_launch(c->pdl, (long long)g.x * g.y * g.z);
+    return R;
+}
+
 inline dim3 grid_x(int N) { return dim3((unsigned)(N / 2 / kThreads)); }
 
 }  // namespace
@@ -623,7 +805,7 @@ cudaError_t run_tensor(const he_ctx *c, const JobRef &R, cudaStream_t st)
     dim3 g = grid_x(c->N);
     g.y = R.lmax;
     g.z = R.B;
-    launch_k(c->pdl, k_tensor, g, dim3(kThreads), 0, st, R, c->d_primes, c->d_levels, c->K, c->N);
+    launch_k(c->pdl, k_tensor, g, dim3(kThreads), 0, st, sized(c, R, g), c->d_primes, c->d_levels, c->K, c->N);
     return cudaGetLastError();
 }
 
@@ -661,7 +843,7 @@ cudaError_t launch_modup(const he_ctx *c, const JobRef &R, cudaStream_t st)
     g.z = R.B;
     const int a = c->AP;
 #define HE_MODUP(AA) \
-    launch_k(c->pdl, k_modup<AA, CH, CANON>, g, dim3(kThreads), 0, st, R, c->d_levels, c->d_primes, c->K, c->N, chunks)
+    launch_k(c->pdl, k_modup<AA, CH, CANON>, g, dim3(kThreads), 0, st, sized(c, R, g), c->d_levels, c->d_primes, c->K, c->N, chunks)
     if (a == 1) HE_MODUP(1);
     else if (a == 2) HE_MODUP(2);
     else if (a == 4) HE_MODUP(4);
@@ -672,8 +854,96 @@ cudaError_t launch_modup(const he_ctx *c, const JobRef &R, cudaStream_t st)
     return cudaGetLastError();
 }
 
+// CTAs that share the tiles of one of `lists` lists (digit or half, chunk, job):
+// one CTA per SM runs at a time, so a launch of few lists gives each an equal
+// part of the SMs, and one of many lists a quarter of the tiles' teams (a list's
+// constants are copied by each of its CTAs, so fewer CTAs take more tiles each).
+int tc_ctas(const he_ctx *c, int lists)
+{
+    const int tiles = c->N / tc::kRows, most = (tiles + kTeams - 1) / kTeams;
+    return std::max(1, std::min(most, std::max(kSMs / lists, (tiles + 4 * kTeams - 1) / (4 * kTeams) * (lists > kSMs / 4))));
+}
+
+template <bool CANON>
+cudaError_t launch_modup_tc(const he_ctx *c, const JobRef &R, cudaStream_t st)
+{
+    // chunks of any level up to lmax: K + (beta - 1) alpha targets at most
+    const int beta = (R.lmax + c->alpha - 1) / c->alpha,
+              nch = (c->K + (beta - 1) * c->alpha + tc::kTargets - 1) / tc::kTargets;
+    const dim3 g((unsigned)tc_ctas(c, beta * nch * R.B), (unsigned)(beta * nch), (unsigned)R.B);
+#define HE_UP(GG)                                                                                                   \
+    launch_k(c->pdl, k_modup_tc<GG, CANON>, g, dim3(kTeams *tc::kTeam), (size_t)c->up_smem, st, sized(c, R, g), c->d_levels,     \
+             c->d_primes, c->K, c->N, nch, c->up_off5, c->d_flag)
+    switch (tc_groups(c->alpha)) {
+    case 1: HE_UP(1); break;
+    case 2: HE_UP(2); break;
+    case 3: HE_UP(3); break;
+    default: HE_UP(4); break;
+    }
+#undef HE_UP
+    return cudaGetLastError();
+}
+
+DnArgs dn_args(const he_ctx *c, int mode, int lmax)
+{
+    DnArgs D;
+    D.img = mode == kTailRescale ? c->d_tc_PBP : c->d_tc_PB;
+    D.last = c->d_tc_last;
+    D.tgt = mode == kTailRescale ? c->d_tc_PBP_t : c->d_tc_PB_t;
+    D.pinv = c->d_pinv;
+    D.levels = c->d_levels;
+    D.primes = c->d_primes;
+    D.flag = c->d_flag;
+    D.K = c->K;
+    D.N = c->N;
+    D.tc = c->dn_tc;
+    D.nch = (lmax + c->dn_tc - 1) / c->dn_tc;
+    D.tp = c->dn_tp;
+    D.bytes = c->dn_bytes;
+    D.last_bytes = c->dn_last_bytes;
+    D.off5 = c->dn_off5;
+    return D;
+}
+
+template <int GU>
+cudaError_t configure_up()
+{
+    const int most = 200 * 1024;
+    cudaError_t e = cudaFuncSetAttribute(k_modup_tc<GU, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_modup_tc<GU, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    return e;
+}
+template <int GD>
+cudaError_t configure_dn()
+{
+    const int most = 200 * 1024;
+    cudaError_t e = cudaFuncSetAttribute(k_moddown_tc<GD, kTailPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_moddown_tc<GD, kTailRescale>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_moddown_tc<GD, kTailRescalePQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    return e;
+}
+
+cudaError_t configure_conversions(const he_ctx *c)
+{
+    cudaError_t e;
+    switch (tc_groups(c->alpha)) {
+    case 1: e = configure_up<1>(); break;
+    case 2: e = configure_up<2>(); break;
+    case 3: e = configure_up<3>(); break;
+    default: e = configure_up<4>(); break;
+    }
+    if (e != cudaSuccess) return e;
+    switch (tc_groups(c->K)) {
+    case 1: return configure_dn<1>();
+    case 2: return configure_dn<2>();
+    case 3: return configure_dn<3>();
+    default: return configure_dn<4>();
+    }
+}
+
 cudaError_t run_modup(const he_ctx *c, const JobRef &R, cudaStream_t st, bool canonical)
 {
+    if (c->tc) return canonical ? launch_modup_tc<true>(c, R, st) : launch_modup_tc<false>(c, R, st);
     if (canonical) return launch_modup<8, true>(c, R, st);
     if (c->modup_chunk == 4) return launch_modup<4, false>(c, R, st);
     if (c->modup_chunk == 16) return launch_modup<16, false>(c, R, st);
@@ -711,10 +981,10 @@ cudaError_t run_inner_product(const he_ctx *c, const JobRef &R, const u64 *evk, 
 #define HE_IP(B)                                                                                                     \
     do {                                                                                                             \
         if (seeded)                                                                                                  \
-            launch_k(c->pdl, k_inner_product<B, true>, g, dim3(kThreads), 0, st, R, evk, c->d_levels, c->d_primes,   \
+            launch_k(c->pdl, k_inner_product<B, true>, g, dim3(kThreads), 0, st, sized(c, R, g), evk, c->d_levels, c->d_primes,   \
                      c->K, c->L, c->N, ss, rows);                                                                    \
         else                                                                                                         \
-            launch_k(c->pdl, k_inner_product<B, false>, g, dim3(kThreads), 0, st, R, evk, c->d_levels, c->d_primes,  \
+            launch_k(c->pdl, k_inner_product<B, false>, g, dim3(kThreads), 0, st, sized(c, R, g), evk, c->d_levels, c->d_primes,  \
                      c->K, c->L, c->N, ss, rows);                                                                    \
     } while (0)
     // three digits get their own width: 64 registers, four CTAs per SM
@@ -749,10 +1019,10 @@ cudaError_t run_inner_product_shared(const he_ctx *c, const JobRef &R, const IpG
 #define HE_IPS(B)                                                                                                  \
     do {                                                                                                           \
         if (seeded)                                                                                                \
-            launch_k(c->pdl, k_inner_product_shared<B, true>, g, dim3(kThreads), 0, st, R, groups, dev_count, evk, \
+            launch_k(c->pdl, k_inner_product_shared<B, true>, g, dim3(kThreads), 0, st, sized(c, R, g), groups, dev_count, evk, \
                      c->d_levels, c->d_primes, c->K, c->L, c->N, ss);                                              \
         else                                                                                                       \
-            launch_k(c->pdl, k_inner_product_shared<B, false>, g, dim3(kThreads), 0, st, R, groups, dev_count,     \
+            launch_k(c->pdl, k_inner_product_shared<B, false>, g, dim3(kThreads), 0, st, sized(c, R, g), groups, dev_count,     \
                      evk, c->d_levels, c->d_primes, c->K, c->L, c->N, ss);                                         \
     } while (0)
     if (bm <= 2) HE_IPS(2);
@@ -762,8 +1032,29 @@ cudaError_t run_inner_product_shared(const he_ctx *c, const JobRef &R, const IpG
     return cudaGetLastError();
 }
 
+template <int G>
+cudaError_t launch_moddown_tc(const he_ctx *c, const JobRef &R, int mode, cudaStream_t st)
+{
+    const DnArgs D = dn_args(c, mode, R.lmax);
+    const dim3 g((unsigned)tc_ctas(c, 2 * D.nch * R.B), (unsigned)(2 * D.nch), (unsigned)R.B);
+    const dim3 b(kTeams * tc::kTeam);
+    const size_t sm = (size_t)c->dn_smem;
+    if (mode == kTailRescale) launch_k(c->pdl, k_moddown_tc<G, kTailRescale>, g, b, sm, st, sized(c, R, g), D);
+    else if (mode == kTailRescalePQ) launch_k(c->pdl, k_moddown_tc<G, kTailRescalePQ>, g, b, sm, st, sized(c, R, g), D);
+    else launch_k(c->pdl, k_moddown_tc<G, kTailPlain>, g, b, sm, st, sized(c, R, g), D);
+    return cudaGetLastError();
+}
+
 cudaError_t run_moddown_conv(const he_ctx *c, const JobRef &R, int mode, cudaStream_t st)
 {
+    if (c->tc) {
+        switch (tc_groups(c->K)) {
+        case 1: return launch_moddown_tc<1>(c, R, mode, st);
+        case 2: return launch_moddown_tc<2>(c, R, mode, st);
+        case 3: return launch_moddown_tc<3>(c, R, mode, st);
+        default: return launch_moddown_tc<4>(c, R, mode, st);
+        }
+    }
     const int chunks = (R.lmax + kModdownChunk - 1) / kModdownChunk;
     dim3 g = grid_x(c->N);
     g.y = 2 * chunks;
@@ -772,13 +1063,13 @@ cudaError_t run_moddown_conv(const he_ctx *c, const JobRef &R, int mode, cudaStr
 #define HE_MD(KK)                                                                                                   \
     do {                                                                                                            \
         if (mode == kTailRescale)                                                                                   \
-            launch_k(c->pdl, k_moddown_conv<KK, kTailRescale>, g, dim3(kThreads), 0, st, R, c->d_PBP, c->d_pinv,    \
+            launch_k(c->pdl, k_moddown_conv<KK, kTailRescale>, g, dim3(kThreads), 0, st, sized(c, R, g), c->d_PBP, c->d_pinv,    \
                      c->d_levels, c->d_primes, K, c->N, chunks);                                                    \
         else if (mode == kTailRescalePQ)                                                                            \
-            launch_k(c->pdl, k_moddown_conv<KK, kTailRescalePQ>, g, dim3(kThreads), 0, st, R, c->d_PB, c->d_pinv,   \
+            launch_k(c->pdl, k_moddown_conv<KK, kTailRescalePQ>, g, dim3(kThreads), 0, st, sized(c, R, g), c->d_PB, c->d_pinv,   \
                      c->d_levels, c->d_primes, K, c->N, chunks);                                                    \
         else                                                                                                        \
-            launch_k(c->pdl, k_moddown_conv<KK, kTailPlain>, g, dim3(kThreads), 0, st, R, c->d_PB, c->d_pinv,       \
+            launch_k(c->pdl, k_moddown_conv<KK, kTailPlain>, g, dim3(kThreads), 0, st, sized(c, R, g), c->d_PB, c->d_pinv,       \
                      c->d_levels, c->d_primes, K, c->N, chunks);                                                    \
     } while (0)
     const int kp = c->KP;
@@ -794,7 +1085,7 @@ cudaError_t run_moddown_conv(const he_ctx *c, const JobRef &R, int mode, cudaStr
 
 bool moddown_ipq_fits(const he_ctx *c)
 {
-    return (c->L + c->alpha - 1) / c->alpha <= 4 && (c->KP == 1 || c->KP == 8 || c->KP == 12);
+    return (c->L + c->alpha - 1) / c->alpha <= 4 && !c->tc && (c->KP == 1 || c->KP == 8 || c->KP == 12);
 }
 
 cudaError_t run_moddown_ipq(const he_ctx *c, const JobRef &R, int mode, const u64 *evk, cudaStream_t st)
@@ -809,7 +1100,7 @@ cudaError_t run_moddown_ipq(const he_ctx *c, const JobRef &R, int mode, const u6
     const SeedStates ss = seed_states(c, evk, &seeded);
     const u64 *PB = mode == kTailRescale ? c->d_PBP : c->d_PB;
 #define HE_MDQ(KK, MM, BB, SS)                                                                                       \
-    launch_k(c->pdl, k_moddown_ipq<KK, MM, BB, SS>, g, dim3(kThreads), 0, st, R, PB, c->d_pinv, c->d_levels,         \
+    launch_k(c->pdl, k_moddown_ipq<KK, MM, BB, SS>, g, dim3(kThreads), 0, st, sized(c, R, g), PB, c->d_pinv, c->d_levels,         \
              c->d_primes, K, c->N, chunks, evk, c->L, ss)
 #define HE_MDQ_B(KK, MM)                                                                                             \
     do {                                                                                                             \
@@ -837,7 +1128,7 @@ cudaError_t run_combine_plain(const he_ctx *c, const JobRef &R, cudaStream_t st)
     dim3 g = grid_x(c->N);
     g.y = R.lmax;
     g.z = 2 * R.B;
-    launch_k(c->pdl, k_combine_plain, g, dim3(kThreads), 0, st, R, c->d_pinv, c->d_levels, c->d_primes, c->K, c->N);
+    launch_k(c->pdl, k_combine_plain, g, dim3(kThreads), 0, st, sized(c, R, g), c->d_pinv, c->d_levels, c->d_primes, c->K, c->N);
     return cudaGetLastError();
 }
 

@@ -65,7 +65,7 @@ struct NttArgs {
     const DevPrime *primes;
     int logN;
     const int *count;  // optional device-side group count (grids sized for a maximum)
-    int pdl;           // programmatic dependent launch: 0 off, 1 on, 2 with early dependent launch
+    int pdl;           // programmatic dependent launch: 0 off, 1, 2
     // fused final combine (COMBINE passes only)
     JobRef R;
     const DevLevel *levels;
@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(P::NT, ntt_min_blocks(P::NT)) k_ntt_pass(const
     // the limbs come from the previous kernels; the pass that streams the key
     // (kFuseIp) does not launch its successor early, whose waiting CTAs would
     // hold SM slots its last loads need (measured: 2^17 985 against 992 us)
-    griddep_wait(A.pdl >= 2 && FUSE != kFuseIp);
+    griddep_wait(A.pdl >= 1 && FUSE != kFuseIp);
     const size_t g2 = (size_t)tile * TE + 2 * threadIdx.x, gs2 = 2 * NT;  // coalesced pairs of a contiguous tile
 
     using SL = RoundSet<P, LL, RL>;

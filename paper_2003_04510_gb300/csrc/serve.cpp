@@ -88,6 +88,7 @@ struct Flight {
     std::vector<uint64_t> tickets;
     std::vector<clk::time_point> t_submit;
     size_t ws_off = 0, ws_bytes = 0;
+    he_ctx *ctx = nullptr;  // of the batch in flight
     int rc = HE_OK;
 };
 
@@ -133,6 +134,7 @@ bool step(he_server *s)
         if (!f.busy) continue;
         cudaError_t q = cudaEventQuery(f.done);
         if (q == cudaErrorNotReady) continue;
+        if (q == cudaSuccess && f.rc == HE_OK) f.rc = he::device_waits(f.ctx);
         const auto now = clk::now();
         std::lock_guard<std::mutex> lk(s->mu);
         const int st = (q == cudaSuccess && f.rc == HE_OK) ? 1 : -(f.rc == HE_OK ? HE_ECUDA : f.rc);
@@ -207,6 +209,7 @@ bool step(he_server *s)
                                                (char *)s->arena_mem + off, bytes, f.stream);
         cudaEventRecord(f.done, f.stream);
         f.busy = true;
+        f.ctx = c;
         f.ws_off = off;
         f.ws_bytes = bytes;
         for (const Req &q : take) {
