@@ -12,11 +12,11 @@
 //          d2 = a1 a2 mod p_i; k_nr_ks_mult: d2 times the evaluation key)
 //   iNTT   with N^-1 [Phat_i^-1]_{p_i} folded into its scaling, so its
 //          outputs are y_i = [x_i Phat_i^-1]_{p_i}
-//   iCRT   (k_nr_icrt: Algo 6's matrix form) C = sum_i y_i Phat_i - u P with
-//          u = round(sum_i y_i / p_i), which is exact because P exceeds four
-//          times the product's magnitude (the fraction is never near 1/2);
-//          C mod 2^(64 W) column by column, u P taken from a table of
-//          (2^(64 W) - u P) rows.
+//   iCRT   (k_icrt, icrt.cuh: Algo 6's matrix form) C = sum_i y_i Phat_i - u P
+//          with u = round(sum_i y_i / p_i), which is exact because P exceeds
+//          four times the product's magnitude (the fraction is never near
+//          1/2); the sums mod 2^(64 W) on the tensor cores, u P taken from a
+//          table of (2^(64 W) - u P) rows.
 // Region 2 (the evaluation key, coefficients mod Q^2) folds the division by
 // Q with rounding and the final addition into its iCRT.
 #include <algorithm>
@@ -26,6 +26,8 @@
 #include <vector>
 
 #include "he_internal.h"
+#include "host_math.h"
+#include "icrt.cuh"
 #include "modarith.cuh"
 
 struct he_nr_plan {
@@ -34,8 +36,9 @@ struct he_nr_plan {
     int chunks_ct = 0, chunks_evk = 0;
     void *dev = nullptr;  // one allocation: tables and NTT group lists
     const u64 *crt = nullptr;           // [np2][chunks_evk]: 2^(28k) mod p_i, split at bit 28
-    const u64 *m1 = nullptr, *neg1 = nullptr, *m2 = nullptr, *neg2 = nullptr;
-    const double *inv1 = nullptr, *inv2 = nullptr;
+    const unsigned char *image1 = nullptr, *image2 = nullptr;  // iCRT constants (icrt.cuh)
+    const u64 *neg1 = nullptr, *neg2 = nullptr;
+    const he::icrt::Prime *prime = nullptr;                    // [np2]
     const he::NttGroup *gF1 = nullptr, *gI1 = nullptr, *gF2 = nullptr, *gI2 = nullptr, *gFe = nullptr;
     int nF1 = 0, nI1 = 0, nF2 = 0, nI2 = 0, nFe = 0;
 };
@@ -45,9 +48,9 @@ namespace he {
 namespace {
 
 constexpr int kT = 256;     // one coefficient per thread (CRT, products, rescale)
-constexpr int kIT = 128;    // iCRT threads per CTA
 constexpr int kCP = 8;      // primes per CTA in the CRT
-constexpr int kMaxNp = 64;  // primes of a plan (the context's ciphertext primes)
+constexpr int kMaxNp = icrt::kMaxNp;  // primes of a plan (the context's ciphertext primes)
+constexpr int kSMs = 152;
 constexpr int kChunkBlock = 40;  // 28-bit chunks accumulated before a reduction
 
 __device__ __forceinline__ ulonglong2 ld2(const u64 *p) { return *reinterpret_cast<const ulonglong2 *>(p); }
@@ -141,113 +144,6 @@ k_nr_ks_mult(u64 *r, const u64 *ek, int np, const DevPrime *__restrict__ primes,
     const ulonglong2 d = ld2(r + o), kb = ld2(ek + o), ka = ld2(ek + L + o);
     st2(r + o, mul_mod(d.x, kb.x, pr.q, pr.mu, pr.s), mul_mod(d.y, kb.y, pr.q, pr.mu, pr.s));
     st2(r + L + o, mul_mod(d.x, ka.x, pr.q, pr.mu, pr.s), mul_mod(d.y, ka.y, pr.q, pr.mu, pr.s));
-}
-
-// iCRT of polys y[poly][np][N] (y_i = [x_i Phat_i^-1]_{p_i}) into BigInts.
-// T = sum_i y_i M_i + NEG_u (mod 2^(64 W)), M_i = Phat_i mod 2^(64 W),
-// NEG_u = (2^(64 W) - u P + rnd) mod 2^(64 W), u = round(sum_i y_i / p_i).
-// Each thread keeps one accumulator per column in registers (column w
-// collects the low words of y_i M_i[w] and the high words of y_i M_i[w-1]),
-// in passes over at most 19 columns, reading the y_i once per pass; the
-// carries run after each pass's sums.
-// KS = false: out[poly] = T mod 2^kout (wo words; polys ostride * N words apart).
-// KS = true: out[poly] = d[poly] + floor((T + 2^(s-1)) / 2^s) mod 2^kout, the
-// rounding term being part of NEG_u (s = logQ).
-// grid: x over N / kIT, y over polys; dynamic shared memory holds M
-// ([np][W]) and NEG ([np + 1][W]).
-template <int W, bool KS>
-__global__ void __launch_bounds__(kIT)
-k_nr_icrt(const u64 *y, int np, const u64 *__restrict__ M, const u64 *__restrict__ NEG,
-          const double *__restrict__ inv, u64 *out, int ostride, int wo, int kout,
-          const u64 *d, int s, int N)
-{
-    extern __shared__ __align__(16) u64 sh[];
-    u64 *sM = sh;                         // [np][W]
-    u64 *sN = sM + (size_t)np * W;        // [np + 1][W]
-    for (int t = threadIdx.x; t < np * W; t += kIT) sM[t] = M[t];
-    for (int t = threadIdx.x; t < (np + 1) * W; t += kIT) sN[t] = NEG[t];
-    const int n = blockIdx.x * kIT + threadIdx.x;
-    const u64 *yp = y + (size_t)blockIdx.y * np * N + n;
-    __syncthreads();
-    griddep_wait();
-    // columns in passes of CW (one pass for W <= 24): fewer live accumulators;
-    // the high words of a pass's last column seed the next pass's first one
-    constexpr int CW = W > 24 ? (W + 1) / 2 : W;
-    constexpr int NPASS = (W + CW - 1) / CW;
-    u64 *o = out + (size_t)blockIdx.y * ostride * N + n;
-    const u64 *dp = KS ? d + (size_t)blockIdx.y * ostride * N + n : nullptr;
-    const int q0 = s >> 6, r = s & 63;
-    u64 carry = 0, prev = 0, dc = 0, ov_lo = 0;
-    uint32_t ov_hi = 0;
-    int u = 0;
-#pragma unroll
-    for (int ps = 0; ps < NPASS; ps++) {
-        const int w0 = ps * CW;
-        u64 lo[CW + 1];
-        uint32_t hi[CW + 1];  // carries out of the low words: at most 2 np per column
-#pragma unroll
-        for (int w = 0; w <= CW; w++) {
-            lo[w] = 0;
-            hi[w] = 0;
-        }
-        lo[0] = ov_lo;
-        hi[0] = ov_hi;
-        double f = 0;
-        u64 ynext = yp[0];
-        for (int i = 0; i < np; i++) {
-            const u64 a = ynext;
-            if (i + 1 < np) ynext = yp[(size_t)(i + 1) * N];
-            if (ps == 0) f = fma((double)a, inv[i], f);
-            const u64 *m = sM + (size_t)i * W + w0;
-#pragma unroll
-            for (int w = 0; w < CW; w++) {
-                if (w0 + w < W) {
-                    const u64 mw = m[w];
-                    const u64 pl = a * mw, ph = __umul64hi(a, mw);
-                    lo[w] += pl;
-                    hi[w] += lo[w] < pl ? 1u : 0u;
-                    lo[w + 1] += ph;
-                    hi[w + 1] += lo[w + 1] < ph ? 1u : 0u;
-                }
-            }
-        }
-        if (ps == 0) u = (int)llrint(f);
-        ov_lo = lo[CW];
-        ov_hi = hi[CW];
-        const u64 *neg = sN + (size_t)u * W;
-#pragma unroll
-        for (int k = 0; k < CW; k++) {
-            const int w = w0 + k;
-            if (w >= W) break;
-            u64 col = lo[k] + carry;
-            u64 c = (u64)hi[k] + (col < carry ? 1ull : 0ull);
-            const u64 ng = neg[w];
-            col += ng;
-            c += col < ng ? 1ull : 0ull;
-            carry = c;
-            if (!KS) {
-                if (w < wo) {
-                    u64 v = col;
-                    if (w == wo - 1 && (kout & 63)) v &= (1ull << (kout & 63)) - 1;
-                    o[(size_t)w * N] = v;
-                }
-            } else {
-                // output word j = bits [s + 64 j, s + 64 j + 64) of T: columns q0 + j and q0 + j + 1
-                const int j = w - q0 - 1;
-                if (j >= 0 && j < wo) {
-                    const u64 v = r ? (prev >> r) | (col << (64 - r)) : prev;
-                    const u64 dv = dp[(size_t)j * N];
-                    u64 sum = v + dv;
-                    const u64 c1 = sum < v ? 1ull : 0ull;
-                    sum += dc;
-                    dc = c1 + (sum < dc ? 1ull : 0ull);
-                    if (j == wo - 1 && (kout & 63)) sum &= (1ull << (kout & 63)) - 1;
-                    o[(size_t)j * N] = sum;
-                }
-                prev = col;
-            }
-        }
-    }
 }
 
 // Rescale by 2^s with rounding: out = floor((a + 2^(s-1)) / 2^s) mod 2^kout.
@@ -385,22 +281,81 @@ void launch_crt(const he_nr_plan *pl, const u64 *in, int wi, int polys, u64 *out
              (const DevPrime *)c->d_primes, c->K, c->N);
 }
 
-template <int W, bool KS>
-cudaError_t launch_icrt(const he_nr_plan *pl, const u64 *y, int np, const u64 *M, const u64 *NEG, const double *inv,
-                        u64 *out, int ostride, int wo, int kout, const u64 *d, int s, int polys, cudaStream_t st)
+// Constants of an iCRT: the image of M_i = Phat_i mod 2^(64 W) (balanced bytes)
+// and the rows NEG_u, to which the products of the digits' offsets and the
+// accumulators' offsets are added.
+void icrt_tables(const he_ctx *c, int np, int W, int add_bit, std::vector<u64> &phinv, std::vector<uint16_t> &image,
+                 std::vector<u64> &neg)
+{
+    const int chunks = (W + icrt::kWords - 1) / icrt::kWords, npad = icrt::padded(np);
+    std::vector<u64> M, P;
+    crt_tables(c, np, W, M, P, phinv);
+    image.assign((size_t)chunks * npad * icrt::kCols * 8, 0);
+    std::vector<int> m(8 * W);
+    MW fix(W, 0);  // sum_i H M_i - sum_c kOff 2^(8c)
+    for (int i = 0; i < np; i++) {
+        int carry = 0;
+        for (int e = 0; e < 8 * W; e++) {
+            int v = (int)((M[(size_t)i * W + e / 8] >> (8 * (e % 8))) & 255) + carry;
+            carry = v >= 128;
+            m[e] = v - 256 * carry;
+        }
+        for (int ct = 0; ct < 8 * W; ct++)
+            for (int d = 0; d < 8 && d <= ct; d++)
+                image[(((size_t)(ct / icrt::kCols) * npad + i) * icrt::kCols + ct % icrt::kCols) * 8 + d] =
+                    half_of(m[ct - d]);
+        MW h(M.begin() + (size_t)i * W, M.begin() + (size_t)(i + 1) * W);
+        mw_mul_small(h, 0x0080808080808080ull);
+        mw_add(fix, h);
+    }
+    MW off(W, 0);
+    for (int w = 0; w < W; w++) {
+        unsigned __int128 v = 0;
+        for (int b = 0; b < 8; b++) v += (unsigned __int128)icrt::kOff << (8 * b);
+        MW x(W, 0);
+        x[w] = (u64)v;
+        if (w + 1 < W) x[w + 1] = (u64)(v >> 64);
+        mw_add(off, x);
+    }
+    for (auto &x : off) x = ~x;  // minus off
+    MW one(1, 1);
+    mw_add(off, one);
+    mw_add(fix, off);
+    neg = neg_rows(P, np, W, add_bit);
+    for (int u = 0; u <= np; u++) {
+        MW row(neg.begin() + (size_t)u * W, neg.begin() + (size_t)(u + 1) * W);
+        mw_add(row, fix);
+        std::copy(row.begin(), row.end(), neg.begin() + (size_t)u * W);
+    }
+}
+
+// out[poly] (out_stride words apart): T mod 2^kout, or (d) d[poly] (d_stride words
+// apart) plus T / 2^s rounded, mod 2^kout.
+cudaError_t launch_icrt(const he_nr_plan *pl, const u64 *y, int np, int W, const unsigned char *image, const u64 *neg,
+                        u64 *out, int out_stride, int kout, const u64 *d, int d_stride, int s, int polys, cudaStream_t st)
 {
     const he_ctx *c = pl->c;
-    const size_t smem = sizeof(u64) * ((size_t)np * W + (size_t)(np + 1) * W);
-    auto kern = k_nr_icrt<W, KS>;
-    static bool configured = false;
-    if (!configured) {
-        const size_t most = sizeof(u64) * ((size_t)kMaxNp * W + (size_t)(kMaxNp + 1) * W);
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
-    dim3 g((unsigned)(c->N / kIT), (unsigned)polys);
-    launch_k(c->pdl, kern, g, dim3(kIT), smem, st, y, np, M, NEG, inv, out, ostride, wo, kout, d, s, c->N);
+    icrt::Args P;
+    P.y = y;
+    P.image = image;
+    P.neg = neg;
+    P.prime = pl->prime;
+    P.out = out;
+    P.d = d;
+    P.flag = c->d_flag;
+    P.np = np;
+    P.W = W;
+    P.chunks = (W + icrt::kWords - 1) / icrt::kWords;
+    P.polys = polys;
+    P.out_stride = out_stride;
+    P.d_stride = d_stride;
+    P.wo = (kout + 63) / 64;
+    P.kout = kout;
+    P.s = s;
+    P.N = c->N;
+    dim3 g((unsigned)std::min(kSMs, polys * (c->N / tc::kRows)));
+    launch_k(c->pdl, d ? icrt::k_icrt<true> : icrt::k_icrt<false>, g, dim3(icrt::kThreads), (size_t)icrt::smem_bytes(np, W),
+             st, P);
     return cudaGetLastError();
 }
 
@@ -453,8 +408,8 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
     pl->logp = logp;
     pl->np1 = np1;
     pl->np2 = np2;
-    pl->W1 = kW1;
-    pl->W2 = kW2;
+    pl->W1 = nwords(logQ);
+    pl->W2 = nwords(2 * logQ);
     pl->chunks_ct = (64 * kW1 + 27) / 28;
     pl->chunks_evk = (64 * kW2 + 27) / 28;
     const int N = c->N, K = c->K;
@@ -467,13 +422,17 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
             crt[(size_t)i * pl->chunks_evk + k] = (v & 0xFFFFFFFull) | ((v >> 28) << 32);
         }
     }
-    std::vector<u64> M1, P1, phinv1, M2, P2, phinv2;
-    crt_tables(c, np1, kW1, M1, P1, phinv1);
-    crt_tables(c, np2, kW2, M2, P2, phinv2);
-    std::vector<u64> neg1 = neg_rows(P1, np1, kW1, -1), neg2 = neg_rows(P2, np2, kW2, logQ - 1);
-    std::vector<double> inv1(np1), inv2(np2);
-    for (int i = 0; i < np1; i++) inv1[i] = 1.0 / (double)c->ext[K + i];
-    for (int i = 0; i < np2; i++) inv2[i] = 1.0 / (double)c->ext[K + i];
+    std::vector<u64> phinv1, phinv2, neg1, neg2;
+    std::vector<uint16_t> image1, image2;
+    icrt_tables(c, np1, pl->W1, -1, phinv1, image1, neg1);
+    icrt_tables(c, np2, pl->W2, logQ - 1, phinv2, image2, neg2);
+    std::vector<icrt::Prime> prime(np2);
+    for (int i = 0; i < np2; i++) {
+        const u64 p = c->ext[K + i];
+        const int b = hm::bitlen(p);
+        prime[i].inv = (uint32_t)(((unsigned __int128)1 << (25 + b)) / p);
+        prime[i].shift = (uint32_t)(b - 32);
+    }
     // NTT job lists (offsets in limbs from the workspace, or from the prepared key)
     const unsigned d_limbs = (unsigned)(3 * kW1);  // the d0, d1, d2 words, in units of N words
     const unsigned r2 = (unsigned)(4 * np1) + d_limbs;
@@ -514,24 +473,28 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
         off += (b + 255) & ~(size_t)255;
         return o;
     };
-    const size_t o_crt = take(crt.size() * 8), o_m1 = take(M1.size() * 8), o_n1 = take(neg1.size() * 8),
-                 o_i1 = take(inv1.size() * 8), o_m2 = take(M2.size() * 8), o_n2 = take(neg2.size() * 8),
-                 o_i2 = take(inv2.size() * 8), o_g1 = take(gF1.size() * sizeof(NttGroup)),
+    const size_t o_crt = take(crt.size() * 8), o_m1 = take(image1.size() * 2), o_n1 = take(neg1.size() * 8),
+                 o_m2 = take(image2.size() * 2), o_n2 = take(neg2.size() * 8),
+                 o_p = take(prime.size() * sizeof(icrt::Prime)), o_g1 = take(gF1.size() * sizeof(NttGroup)),
                  o_g2 = take(gI1.size() * sizeof(NttGroup)), o_g3 = take(gF2.size() * sizeof(NttGroup)),
                  o_g4 = take(gI2.size() * sizeof(NttGroup)), o_g5 = take(gFe.size() * sizeof(NttGroup));
-    if (cudaMalloc(&pl->dev, off) != cudaSuccess) {
+    // the iCRTs' operands and ring
+    if (cudaFuncSetAttribute(icrt::k_icrt<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             icrt::smem_bytes(kMaxNp, kW2)) != cudaSuccess ||
+        cudaFuncSetAttribute(icrt::k_icrt<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             icrt::smem_bytes(kMaxNp, kW2)) != cudaSuccess ||
+        cudaMalloc(&pl->dev, off) != cudaSuccess) {
         delete pl;
         return HE_ECUDA;
     }
     std::vector<unsigned char> img(off, 0);
     auto put = [&](size_t o, const void *p, size_t b) { memcpy(img.data() + o, p, b); };
     put(o_crt, crt.data(), crt.size() * 8);
-    put(o_m1, M1.data(), M1.size() * 8);
+    put(o_m1, image1.data(), image1.size() * 2);
     put(o_n1, neg1.data(), neg1.size() * 8);
-    put(o_i1, inv1.data(), inv1.size() * 8);
-    put(o_m2, M2.data(), M2.size() * 8);
+    put(o_m2, image2.data(), image2.size() * 2);
     put(o_n2, neg2.data(), neg2.size() * 8);
-    put(o_i2, inv2.data(), inv2.size() * 8);
+    put(o_p, prime.data(), prime.size() * sizeof(icrt::Prime));
     put(o_g1, gF1.data(), gF1.size() * sizeof(NttGroup));
     put(o_g2, gI1.data(), gI1.size() * sizeof(NttGroup));
     put(o_g3, gF2.data(), gF2.size() * sizeof(NttGroup));
@@ -544,12 +507,11 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
     }
     char *b = (char *)pl->dev;
     pl->crt = (const u64 *)(b + o_crt);
-    pl->m1 = (const u64 *)(b + o_m1);
+    pl->image1 = (const unsigned char *)(b + o_m1);
     pl->neg1 = (const u64 *)(b + o_n1);
-    pl->inv1 = (const double *)(b + o_i1);
-    pl->m2 = (const u64 *)(b + o_m2);
+    pl->image2 = (const unsigned char *)(b + o_m2);
     pl->neg2 = (const u64 *)(b + o_n2);
-    pl->inv2 = (const double *)(b + o_i2);
+    pl->prime = (const icrt::Prime *)(b + o_p);
     pl->gF1 = (const NttGroup *)(b + o_g1);
     pl->gI1 = (const NttGroup *)(b + o_g2);
     pl->gF2 = (const NttGroup *)(b + o_g3);
@@ -622,8 +584,7 @@ int he_nr_mul(he_nr_plan *pl, const uint64_t *ct1, const uint64_t *ct2, const ui
     prof_mark(c, st, "nr_tensor");
     if (launch_ntt(cm, w, pl->gI1, pl->nI1, true, st, "nr_intt1") != cudaSuccess) return HE_ECUDA;
     // d0, d1, d2 mod q (word-major, wq words each, stride kW1 words)
-    if (launch_icrt<kW1, false>(pl, R1, np1, pl->m1, pl->neg1, pl->inv1, D, kW1, wq, logq, nullptr, 0, 3, st) !=
-        cudaSuccess)
+    if (launch_icrt(pl, R1, np1, pl->W1, pl->image1, pl->neg1, D, kW1, logq, nullptr, 0, 0, 3, st) != cudaSuccess)
         return HE_ECUDA;
     prof_mark(c, st, "nr_icrt1");
     // region 2: CRT of d2, NTT, products with the prepared key, iNTT, iCRT + shift + add
@@ -637,11 +598,8 @@ int he_nr_mul(he_nr_plan *pl, const uint64_t *ct1, const uint64_t *ct2, const ui
     prof_mark(c, st, "nr_ks_mult");
     if (launch_ntt(cm, w, pl->gI2, pl->nI2, true, st, "nr_intt2") != cudaSuccess) return HE_ECUDA;
     // out[h] = d_h + round(KS_h / Q) mod q; the d's sit kW1 words apart, out wq words apart
-    for (int h = 0; h < 2; h++)
-        if (launch_icrt<kW2, true>(pl, R2 + (size_t)h * np2 * N, np2, pl->m2, pl->neg2, pl->inv2,
-                                   out + (size_t)h * wq * N, 0, wq, logq, D + (size_t)h * kW1 * N, pl->logQ, 1, st) !=
-            cudaSuccess)
-            return HE_ECUDA;
+    if (launch_icrt(pl, R2, np2, pl->W2, pl->image2, pl->neg2, out, wq, logq, D, kW1, pl->logQ, 2, st) != cudaSuccess)
+        return HE_ECUDA;
     prof_mark(c, st, "nr_icrt2");
     return HE_OK;
 }

@@ -228,6 +228,7 @@ inline int device_waits(const he_ctx *c)
     return c->flag && __atomic_exchange_n(c->flag, 0u, __ATOMIC_RELAXED) ? HE_ETIMEOUT : HE_OK;
 }
 // tc_tables.cpp
+uint16_t half_of(int v);  // f16 bits of an integer that f16 holds exactly
 int tc_groups(int nsrc);  // groups of four source limbs
 bool tc_source_ok(u64 p);
 uint32_t tc_off5(const std::vector<u64> &src);

@@ -533,11 +533,9 @@ int build_context(he_ctx *c, const he_params *p, bool device)
     }
     if (!device) return HE_OK;
     c->tc = build_tc(c);
-    if (c->tc) {
-        if (cudaHostAlloc((void **)&c->flag, sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess) return HE_ECUDA;
-        *c->flag = 0;
-        if (cudaHostGetDevicePointer((void **)&c->d_flag, c->flag, 0) != cudaSuccess) return HE_ECUDA;
-    }
+    if (cudaHostAlloc((void **)&c->flag, sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess) return HE_ECUDA;
+    *c->flag = 0;
+    if (cudaHostGetDevicePointer((void **)&c->d_flag, c->flag, 0) != cudaSuccess) return HE_ECUDA;
 
     // ---- device arena -------------------------------------------------------
     size_t off = 0;

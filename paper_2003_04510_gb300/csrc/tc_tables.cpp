@@ -23,7 +23,8 @@ static_assert(kTcPair < 0 && kTcMass <= kTcOff && kTcOff + kTcMass < (1 << 23) &
               "pairs of planes");
 static_assert(2 * kTcOffTop < (1 << 23) && 512ll * 2 * kTcOffTop + (1 << 23) < (1ll << 32), "the last pair");
 
-// f16 bits of an integer that f16 holds exactly
+}  // namespace
+
 uint16_t half_of(int v)
 {
     if (v == 0) return 0;
@@ -33,8 +34,6 @@ uint16_t half_of(int v)
     while ((m >> e) > 1) e++;
     return (uint16_t)(sign | ((e + 15) << 10) | ((e <= 10 ? m << (10 - e) : m >> (e - 10)) & 0x3ff));
 }
-
-}  // namespace
 
 int tc_groups(int nsrc) { return (nsrc + 3) / 4; }
 

@@ -1,0 +1,51 @@
+"""BigInt HE Mul at the edges of the tensor-core iCRT: word counts around its
+chunks of ten, prime counts around its stages of eight and both accumulators,
+moduli at and off word boundaries, the smallest and largest; coefficients at zero,
+at the modulus less one and random.  Word for word against the oracle.
+"""
+import numpy as np
+import pytest
+
+import oracle
+
+
+@pytest.fixture(scope="module")
+def g():
+    from paper_2003_04510_gb300 import build
+    build.build()
+    import paper_2003_04510_gb300 as pkg
+    return pkg
+
+
+def words(k, N, seed):
+    rng = np.random.default_rng(seed)
+    a = rng.integers(0, 1 << 63, size=(oracle.nwords(k), N), dtype=np.uint64) * np.uint64(2) + \
+        rng.integers(0, 2, size=(oracle.nwords(k), N), dtype=np.uint64)
+    a[:, :100] = np.uint64(2**64 - 1)
+    a[:, 100:130] = 0
+    if k % 64:
+        a[-1] &= np.uint64((1 << (k % 64)) - 1)
+    return a
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("logN,logQ,logqs", [(12, 64, (64, 31)), (12, 65, (65,)), (13, 129, (129, 128)), (12, 200, (137,)),
+                                             (12, 320, (320, 319)), (12, 321, (321, 65)), (12, 640, (640, 600)),
+                                             (12, 700, (700,)), (12, 1001, (1001, 2 * 64)), (12, 1205, (1205, 1000))])
+def test_he_mul_at_icrt_edges(g, logN, logQ, logqs):
+    import torch
+    prm = oracle.nr_params(logN, logQ, 20)
+    ctx = g.Context(g.Params(logN, prm.np2, 1, 16, 57, 57, 64), device=True)
+    assert np.array_equal(ctx.q[: prm.np2], prm.primes)
+    plan = g.NrPlan(ctx, logQ, 20)
+    assert (plan.np1, plan.np2) == (prm.np1, prm.np2)
+    evk = np.stack([words(2 * logQ, prm.N, 5), words(2 * logQ, prm.N, 6)])
+    prep, ws = plan.prepare_evk(g.to_device(evk)), plan.workspace()
+    for logq in logqs:
+        c1, c2 = (np.stack([words(logq, prm.N, 10 * c + h) for h in range(2)]) for c in (1, 2))
+        out = torch.zeros((2, oracle.nwords(logq), prm.N), dtype=torch.int64, device="cuda")
+        plan.mul(g.to_device(c1), g.to_device(c2), prep, logq, out, ws)
+        torch.cuda.synchronize()
+        assert np.array_equal(g.to_host(out), oracle.nr_he_mul(prm, c1, c2, evk, logq)), logq
+    plan.close()
+    ctx.close()
