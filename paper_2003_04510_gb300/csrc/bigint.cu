@@ -374,7 +374,7 @@ constexpr int kW1 = 19, kW2 = 38;
 size_t ws_words(const he_nr_plan *pl)
 {
     const size_t N = (size_t)pl->c->N;
-    return (size_t)4 * pl->np1 * N + (size_t)3 * pl->W1 * N + (size_t)2 * pl->np2 * N;
+    return (size_t)4 * pl->np1 * N + (size_t)3 * kW1 * N + (size_t)2 * pl->np2 * N;
 }
 
 int dev_try(cudaError_t e) { return e == cudaSuccess ? HE_OK : HE_ECUDA; }

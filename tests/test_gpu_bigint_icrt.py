@@ -40,12 +40,15 @@ def test_he_mul_at_icrt_edges(g, logN, logQ, logqs):
     plan = g.NrPlan(ctx, logQ, 20)
     assert (plan.np1, plan.np2) == (prm.np1, prm.np2)
     evk = np.stack([words(2 * logQ, prm.N, 5), words(2 * logQ, prm.N, 6)])
-    prep, ws = plan.prepare_evk(g.to_device(evk)), plan.workspace()
+    prep, n = plan.prepare_evk(g.to_device(evk)), plan.workspace().numel()
+    guarded = torch.full((n + 64 * prm.N,), 0x5A5A5A5A, dtype=torch.int64, device="cuda")
+    ws = guarded[:n]  # nothing is written behind the workspace
     for logq in logqs:
         c1, c2 = (np.stack([words(logq, prm.N, 10 * c + h) for h in range(2)]) for c in (1, 2))
         out = torch.zeros((2, oracle.nwords(logq), prm.N), dtype=torch.int64, device="cuda")
         plan.mul(g.to_device(c1), g.to_device(c2), prep, logq, out, ws)
         torch.cuda.synchronize()
         assert np.array_equal(g.to_host(out), oracle.nr_he_mul(prm, c1, c2, evk, logq)), logq
+    assert bool((guarded[n:] == 0x5A5A5A5A).all())
     plan.close()
     ctx.close()
