@@ -4,9 +4,10 @@
 // paper's Table 3: q = 2^logq, Q = 2^logQ, p = 2^logp), stored word-major:
 // word w of coefficient n at a[w * N + n], little-endian, ceil(k / 64) words.
 // Each polynomial product follows the paper's five steps (Fig. 2, Sec. 4):
-//   CRT    BigInt -> residues mod np NTT primes (k_nr_crt: 28-bit chunks
-//          times 2^(28k) mod p_i, lazy 32x32->64 multiply-adds, one Barrett
-//          reduction -- Algo 1's accumulate-then-reduce, without BigInt carries)
+//   CRT    BigInt -> residues mod np NTT primes (k_crt, crt.cuh: bytes times
+//          2^(8k) mod p_i on the tensor cores, one Barrett reduction -- Algo
+//          1's accumulate-then-reduce, without BigInt carries; the evaluation
+//          key's, once per key: k_nr_crt, 28-bit chunks times 2^(28k) mod p_i)
 //   NTT    the RNS path's k_ntt_pass over the context's primes
 //   mul    element-wise (k_nr_tensor: d0 = b1 b2, d1 = a1 b2 + a2 b1,
 //          d2 = a1 a2 mod p_i; k_nr_ks_mult: d2 times the evaluation key)
@@ -25,6 +26,7 @@
 #include <new>
 #include <vector>
 
+#include "crt.cuh"
 #include "he_internal.h"
 #include "host_math.h"
 #include "icrt.cuh"
@@ -33,9 +35,12 @@
 struct he_nr_plan {
     he_ctx *c = nullptr;
     int logQ = 0, logp = 0, np1 = 0, np2 = 0, W1 = 0, W2 = 0;
-    int chunks_ct = 0, chunks_evk = 0;
+    int chunks_evk = 0;
+    bool crt_folds = false;  // every prime reduces by folding (crt.cuh)
     void *dev = nullptr;  // one allocation: tables and NTT group lists
     const u64 *crt = nullptr;           // [np2][chunks_evk]: 2^(28k) mod p_i, split at bit 28
+    const unsigned char *crt1 = nullptr, *crt2 = nullptr;      // CRT constants over np1 and np2 primes (crt.cuh)
+    const he::crt::Prime *crt_prime = nullptr;                 // [np2]
     const unsigned char *image1 = nullptr, *image2 = nullptr;  // iCRT constants (icrt.cuh)
     const u64 *neg1 = nullptr, *neg2 = nullptr;
     const he::icrt::Prime *prime = nullptr;                    // [np2]
@@ -272,13 +277,72 @@ std::vector<u64> neg_rows(const std::vector<u64> &P, int np, int W, int add_bit)
     return out;
 }
 
-template <int WI>
-void launch_crt(const he_nr_plan *pl, const u64 *in, int wi, int polys, u64 *out, int np, cudaStream_t st)
+// The evaluation key's CRT.
+void launch_crt_evk(const he_nr_plan *pl, const u64 *in, int wi, int polys, u64 *out, int np, cudaStream_t st)
 {
     const he_ctx *c = pl->c;
     dim3 g((unsigned)(c->N / kT), (unsigned)polys, (unsigned)((np + kCP - 1) / kCP));
-    launch_k(c->pdl, k_nr_crt<WI>, g, dim3(kT), 0, st, in, wi, (size_t)wi * c->N, out, np, pl->crt, pl->chunks_evk,
-             (const DevPrime *)c->d_primes, c->K, c->N);
+    launch_k(c->pdl, k_nr_crt<2 * crt::kMaxWords>, g, dim3(kT), 0, st, in, wi, (size_t)wi * c->N, out, np, pl->crt,
+             pl->chunks_evk, (const DevPrime *)c->d_primes, c->K, c->N);
+}
+
+// CRT of polys polynomials of wi <= W1 words over np primes.
+cudaError_t launch_crt(const he_nr_plan *pl, const u64 *const *in, int polys, int wi, u64 *out, int np,
+                       const unsigned char *image, cudaStream_t st)
+{
+    const he_ctx *c = pl->c;
+    crt::Args P;
+    for (int k = 0; k < 4; k++) P.in[k] = in[k < polys ? k : 0];
+    P.out = out;
+    P.image = image;
+    P.prime = pl->crt_prime;
+    P.flag = c->d_flag;
+    P.wi = wi;
+    P.W = pl->W1;
+    P.np = np;
+    P.pc = crt::chunk_primes(np);
+    P.polys = polys;
+    P.N = c->N;
+    const int nch = (np + P.pc - 1) / P.pc;
+    dim3 g((unsigned)std::min(kSMs / nch, polys * (c->N / tc::kRows)), (unsigned)nch);
+    launch_k(c->pdl, pl->crt_folds ? crt::k_crt<true> : crt::k_crt<false>, g, dim3(crt::kThreads), (size_t)crt::smem_bytes(P.W, P.pc), st, P);
+    return cudaGetLastError();
+}
+
+// Image of 2^(8k) mod p_i, k < 8 W, over np primes, and each prime's constants.
+void crt_image(const he_ctx *c, int np, int W, std::vector<uint16_t> &image, std::vector<crt::Prime> &prime)
+{
+    const int pc = crt::chunk_primes(np), nch = (np + pc - 1) / pc;
+    image.assign((size_t)nch * crt::image_bytes(W, pc) / 2, 0);
+    prime.resize(np);
+    for (int i = 0; i < np; i++) {
+        const u64 p = c->ext[c->K + i];
+        uint16_t *im = image.data() + (size_t)(i / pc) * crt::image_bytes(W, pc) / 2;
+        auto at = [&](int k, int col) -> uint16_t & { return im[((size_t)(k / 8) * 8 * pc + 8 * (i % pc) + col) * 8 + k % 8]; };
+        u64 v = 1 % p, sum = 0;  // sum of the bytes' offsets
+        for (int k = 0; k < 8 * W; k++) {
+            long long x = v > p / 2 ? (long long)v - (long long)p : (long long)v;
+            for (int col = 0; col < 8; col++) {
+                const long long r = ((x + 128) & 255) - 128;
+                at(k, col) = half_of((int)r);
+                x = (x - r) / 256;
+            }
+            sum = hm::add(sum, v, p);
+            v = hm::mul(v, 256, p);
+        }
+        u64 off = 0, w = 1 % p;
+        for (int col = 0; col < 8; col++) {
+            at(8 * W, col) = half_of(6144);  // times the digits' 2048
+            if (col % 2 == 0) off = hm::add(off, hm::mul(crt::kPair % p, w, p), p);
+            w = hm::mul(w, 256, p);
+        }
+        prime[i].q = p;
+        prime[i].s = (uint32_t)hm::bitlen(p) - 2;
+        prime[i].mu = (u64)(((unsigned __int128)1 << (64 + prime[i].s)) / p);
+        prime[i].base = hm::sub(hm::mul(sum, 128, p), off, p);
+        const u64 delta = (1ull << hm::bitlen(p)) - p;
+        prime[i].delta = delta >> 31 ? 0 : (uint32_t)delta;
+    }
 }
 
 // Constants of an iCRT: the image of M_i = Phat_i mod 2^(64 W) (balanced bytes)
@@ -410,7 +474,6 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
     pl->np2 = np2;
     pl->W1 = nwords(logQ);
     pl->W2 = nwords(2 * logQ);
-    pl->chunks_ct = (64 * kW1 + 27) / 28;
     pl->chunks_evk = (64 * kW2 + 27) / 28;
     const int N = c->N, K = c->K;
     // host tables
@@ -424,6 +487,12 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
     }
     std::vector<u64> phinv1, phinv2, neg1, neg2;
     std::vector<uint16_t> image1, image2;
+    std::vector<uint16_t> crt1, crt2;
+    std::vector<crt::Prime> crt_prime;
+    crt_image(c, np1, pl->W1, crt1, crt_prime);
+    crt_image(c, np2, pl->W1, crt2, crt_prime);
+    pl->crt_folds = true;
+    for (const crt::Prime &p : crt_prime) pl->crt_folds = pl->crt_folds && crt::folds(p);
     icrt_tables(c, np1, pl->W1, -1, phinv1, image1, neg1);
     icrt_tables(c, np2, pl->W2, logQ - 1, phinv2, image2, neg2);
     std::vector<icrt::Prime> prime(np2);
@@ -475,11 +544,16 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
     };
     const size_t o_crt = take(crt.size() * 8), o_m1 = take(image1.size() * 2), o_n1 = take(neg1.size() * 8),
                  o_m2 = take(image2.size() * 2), o_n2 = take(neg2.size() * 8),
-                 o_p = take(prime.size() * sizeof(icrt::Prime)), o_g1 = take(gF1.size() * sizeof(NttGroup)),
+                 o_p = take(prime.size() * sizeof(icrt::Prime)), o_c1 = take(crt1.size() * 2),
+                 o_c2 = take(crt2.size() * 2), o_cp = take(crt_prime.size() * sizeof(crt::Prime)), o_g1 = take(gF1.size() * sizeof(NttGroup)),
                  o_g2 = take(gI1.size() * sizeof(NttGroup)), o_g3 = take(gF2.size() * sizeof(NttGroup)),
                  o_g4 = take(gI2.size() * sizeof(NttGroup)), o_g5 = take(gFe.size() * sizeof(NttGroup));
     // the iCRTs' operands and ring
-    if (cudaFuncSetAttribute(icrt::k_icrt<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(crt::k_crt<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             crt::smem_bytes(crt::kMaxWords, crt::kPrimes)) != cudaSuccess ||
+        cudaFuncSetAttribute(crt::k_crt<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             crt::smem_bytes(crt::kMaxWords, crt::kPrimes)) != cudaSuccess ||
+        cudaFuncSetAttribute(icrt::k_icrt<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              icrt::smem_bytes(kMaxNp, kW2)) != cudaSuccess ||
         cudaFuncSetAttribute(icrt::k_icrt<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              icrt::smem_bytes(kMaxNp, kW2)) != cudaSuccess ||
@@ -495,6 +569,9 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
     put(o_m2, image2.data(), image2.size() * 2);
     put(o_n2, neg2.data(), neg2.size() * 8);
     put(o_p, prime.data(), prime.size() * sizeof(icrt::Prime));
+    put(o_c1, crt1.data(), crt1.size() * 2);
+    put(o_c2, crt2.data(), crt2.size() * 2);
+    put(o_cp, crt_prime.data(), crt_prime.size() * sizeof(crt::Prime));
     put(o_g1, gF1.data(), gF1.size() * sizeof(NttGroup));
     put(o_g2, gI1.data(), gI1.size() * sizeof(NttGroup));
     put(o_g3, gF2.data(), gF2.size() * sizeof(NttGroup));
@@ -512,6 +589,9 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
     pl->image2 = (const unsigned char *)(b + o_m2);
     pl->neg2 = (const u64 *)(b + o_n2);
     pl->prime = (const icrt::Prime *)(b + o_p);
+    pl->crt1 = (const unsigned char *)(b + o_c1);
+    pl->crt2 = (const unsigned char *)(b + o_c2);
+    pl->crt_prime = (const crt::Prime *)(b + o_cp);
     pl->gF1 = (const NttGroup *)(b + o_g1);
     pl->gI1 = (const NttGroup *)(b + o_g2);
     pl->gF2 = (const NttGroup *)(b + o_g3);
@@ -551,7 +631,7 @@ int he_nr_evk_prepare(he_nr_plan *pl, const uint64_t *evk, uint64_t *prep, void 
 {
     if (!pl || !evk || !prep) return HE_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    launch_crt<kW2>(pl, evk, nwords(2 * pl->logQ), 2, prep, pl->np2, st);
+    launch_crt_evk(pl, evk, nwords(2 * pl->logQ), 2, prep, pl->np2, st);
     if (cudaGetLastError() != cudaSuccess) return HE_ECUDA;
     return dev_try(launch_ntt(pl->c, prep, pl->gFe, pl->nFe, false, st, "nr_evk"));
 }
@@ -571,11 +651,8 @@ int he_nr_mul(he_nr_plan *pl, const uint64_t *ct1, const uint64_t *ct2, const ui
     u64 *R1 = w, *D = w + (size_t)4 * np1 * N, *R2 = D + (size_t)3 * kW1 * N;
     prof_mark(c, st, "");
     // region 1: CRT of a1, b1, a2, b2 (ct = [b | a], word-major)
-    launch_crt<kW1>(pl, ct1 + (size_t)wq * N, wq, 1, R1, np1, st);
-    launch_crt<kW1>(pl, ct1, wq, 1, R1 + (size_t)np1 * N, np1, st);
-    launch_crt<kW1>(pl, ct2 + (size_t)wq * N, wq, 1, R1 + (size_t)2 * np1 * N, np1, st);
-    launch_crt<kW1>(pl, ct2, wq, 1, R1 + (size_t)3 * np1 * N, np1, st);
-    if (cudaGetLastError() != cudaSuccess) return HE_ECUDA;
+    const u64 *in1[4] = {ct1 + (size_t)wq * N, ct1, ct2 + (size_t)wq * N, ct2};
+    if (launch_crt(pl, in1, 4, wq, R1, np1, pl->crt1, st) != cudaSuccess) return HE_ECUDA;
     prof_mark(c, st, "nr_crt1");
     if (launch_ntt(cm, w, pl->gF1, pl->nF1, false, st, "nr_ntt1") != cudaSuccess) return HE_ECUDA;
     launch_k(c->pdl, k_nr_tensor, dim3((unsigned)(N / 2 / kT), (unsigned)np1), dim3(kT), 0, st, R1, np1,
@@ -588,8 +665,8 @@ int he_nr_mul(he_nr_plan *pl, const uint64_t *ct1, const uint64_t *ct2, const ui
         return HE_ECUDA;
     prof_mark(c, st, "nr_icrt1");
     // region 2: CRT of d2, NTT, products with the prepared key, iNTT, iCRT + shift + add
-    launch_crt<kW1>(pl, D + (size_t)2 * kW1 * N, wq, 1, R2, np2, st);
-    if (cudaGetLastError() != cudaSuccess) return HE_ECUDA;
+    const u64 *d2 = D + (size_t)2 * kW1 * N;
+    if (launch_crt(pl, &d2, 1, wq, R2, np2, pl->crt2, st) != cudaSuccess) return HE_ECUDA;
     prof_mark(c, st, "nr_crt2");
     if (launch_ntt(cm, w, pl->gF2, pl->nF2, false, st, "nr_ntt2") != cudaSuccess) return HE_ECUDA;
     launch_k(c->pdl, k_nr_ks_mult, dim3((unsigned)(N / 2 / kT), (unsigned)np2), dim3(kT), 0, st, R2, prep, np2,

@@ -97,11 +97,13 @@ __device__ __forceinline__ void bulk_copy(void *dst, const void *src, uint32_t b
                  : "memory");
 }
 
-// The eight digits of y as f16.
+// The eight digits of y as f16; o7: minus the offsets of the last two, 1024 each and 128
+// where the byte is not small.
+template <uint32_t o7>
 __device__ __forceinline__ uint4 digits(u64 y)
 {
     const uint32_t lo = (uint32_t)y, hi = (uint32_t)(y >> 32), e = 0x64646464u;  // f16 1024 + byte
-    const uint32_t o = 0xE480E480u, o7 = 0xE400E480u;                             // -1152 twice; -1024 | -1152
+    const uint32_t o = 0xE480E480u;                                               // -1152 twice
     uint4 r;
     asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r.x) : "r"(__byte_perm(lo, e, 0x4140)), "r"(o));
     asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r.y) : "r"(__byte_perm(lo, e, 0x4342)), "r"(o));
@@ -266,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_icrt(const Args P)
                 if (i < P.np) {
                     const Prime pr = S.prime[i];
                     f += __umulhi((uint32_t)(v[k] >> pr.shift), pr.inv);
-                    reinterpret_cast<uint4 *>(A)[i * tc::kRows + row] = digits(v[k]);
+                    reinterpret_cast<uint4 *>(A)[i * tc::kRows + row] = digits<0xE400E480u>(v[k]);  // -1024 | -1152
                 }
                 constexpr int per = kStagePrimes / 2;
                 if (k % per == per - 1 && k / per < stages) {  // the stage's primes: its MMAs may start
@@ -339,6 +341,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_icrt(const Args P)
                 }
             }
         }
+        // the last arrival lands before the CTA ends
+        if (it && ok) ok = __all_sync(~0u, tc::bar_wait(&S.a_free, (it - 1) & 1));
     }
     if (!ok) *(volatile unsigned *)P.flag = 1;
     tc::fence_before_sync();

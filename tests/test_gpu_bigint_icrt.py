@@ -1,5 +1,6 @@
-"""BigInt HE Mul at the edges of the tensor-core iCRT: word counts around its
-chunks of ten, prime counts around its stages of eight and both accumulators,
+"""BigInt HE Mul at the edges of the tensor-core CRT and iCRT: word counts around
+the iCRT's chunks of ten, prime counts around its stages of eight and both
+accumulators and around the CRT's 32 per CTA, primes that fold and that do not,
 moduli at and off word boundaries, the smallest and largest; coefficients at zero,
 at the modulus less one and random.  Word for word against the oracle.
 """
@@ -29,13 +30,15 @@ def words(k, N, seed):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("logN,logQ,logqs", [(12, 64, (64, 31)), (12, 65, (65,)), (13, 129, (129, 128)), (12, 200, (137,)),
-                                             (12, 320, (320, 319)), (12, 321, (321, 65)), (12, 640, (640, 600)),
-                                             (12, 700, (700,)), (12, 1001, (1001, 2 * 64)), (12, 1205, (1205, 1000))])
-def test_he_mul_at_icrt_edges(g, logN, logQ, logqs):
+@pytest.mark.parametrize("bits,logN,logQ,logqs", [
+    (57, 12, 64, (64, 31)), (57, 12, 65, (65,)), (57, 12, 66, (66,)), (57, 13, 129, (129, 128)), (57, 12, 200, (137,)),
+    (57, 12, 320, (320, 319)), (57, 12, 321, (321, 65)), (57, 12, 640, (640, 600)), (57, 12, 700, (700,)),
+    (57, 12, 1001, (1001, 2 * 64)), (57, 12, 1205, (1205, 1000)), (57, 15, 130, (130,)),
+    (41, 12, 260, (260,)), (54, 12, 600, (600, 599)), (55, 12, 600, (600,)), (56, 13, 330, (330,))])
+def test_he_mul_at_icrt_edges(g, bits, logN, logQ, logqs):
     import torch
-    prm = oracle.nr_params(logN, logQ, 20)
-    ctx = g.Context(g.Params(logN, prm.np2, 1, 16, 57, 57, 64), device=True)
+    prm = oracle.nr_params(logN, logQ, 20, bits)
+    ctx = g.Context(g.Params(logN, prm.np2, 1, 16, bits, bits, 64), device=True)
     assert np.array_equal(ctx.q[: prm.np2], prm.primes)
     plan = g.NrPlan(ctx, logQ, 20)
     assert (plan.np1, plan.np2) == (prm.np1, prm.np2)
