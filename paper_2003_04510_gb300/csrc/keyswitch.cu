@@ -263,6 +263,18 @@ __device__ __forceinline__ int ip_row(int rows, int y, int K, int l)
     }
 }
 
+// A key-switch sum's products in the split form of the base conversions (mac28k:
+// three multiply-adds each, no carries; words below 2^57, at most 16 digits).  In
+// 64 x 64-bit products the sums were bound by the multiplier, about 22 instructions
+// a product against 5: one HE Mul's sums 38.9 -> 34.8 us at 2^16 (level 24), 169 ->
+// 140 at 2^17 (level 44), a batch of 64 at 2^16 883 -> 764.  What is left is HBM:
+// 5.1 to 5.9 TB/s of reads and writes.
+__device__ __forceinline__ u64 pack28(u64 x) { return (x & 0xFFFFFFFull) | ((x >> 28) << 32); }
+__device__ __forceinline__ u64 ip_reduce(const Acc3 &s, const DevPrime &pr)
+{
+    return csub(csub(acc3k_reduce_lazy(s, pr.q, pr.mu, pr.s), 2 * pr.q), pr.q);
+}
+
 template <int BM, bool SEEDED>
 __device__ __forceinline__ void ip_body(const JobRef &R, const BatchItem &it, const DevLevel &lv, int e,
                                         const u64 *__restrict__ evk, const DevPrime *__restrict__ primes, int K,
@@ -294,24 +306,27 @@ __device__ __forceinline__ void ip_body(const JobRef &R, const BatchItem &it, co
             }
         }
     }
-    U128 bx = {0, 0}, by = {0, 0}, ax = {0, 0}, ay = {0, 0};
+    Acc3 bx = {0, 0, 0}, by = {0, 0, 0}, ax = {0, 0, 0}, ay = {0, 0, 0};
 #pragma unroll
     for (int j = 0; j < BM; j++) {
         if (j < beta) {
-            mac(bx, u[j].x, kb[j].x);
-            mac(by, u[j].y, kb[j].y);
-            mac(ax, u[j].x, ka[j].x);
-            mac(ay, u[j].y, ka[j].y);
+            uint32_t x0, x1, y0, y1;
+            split28(u[j].x, x0, x1);
+            split28(u[j].y, y0, y1);
+            mac28k(bx, x0, x1, x0 + x1, pack28(kb[j].x));
+            mac28k(ax, x0, x1, x0 + x1, pack28(ka[j].x));
+            mac28k(by, y0, y1, y0 + y1, pack28(kb[j].y));
+            mac28k(ay, y0, y1, y0 + y1, pack28(ka[j].y));
         }
     }
     u64 *KS = it.ws + (size_t)lv.o_ks * N;
-    st2(KS + (size_t)e * N + n, barrett128(bx, pr.q, pr.mu, pr.s), barrett128(by, pr.q, pr.mu, pr.s));
-    st2(KS + ((size_t)E + e) * N + n, barrett128(ax, pr.q, pr.mu, pr.s), barrett128(ay, pr.q, pr.mu, pr.s));
+    st2(KS + (size_t)e * N + n, ip_reduce(bx, pr), ip_reduce(by, pr));
+    st2(KS + ((size_t)E + e) * N + n, ip_reduce(ax, pr), ip_reduce(ay, pr));
 }
 
 // grid: x over N/2/kThreads, y over the rows selected (IpRows), z over jobs.
 template <int BM, bool SEEDED>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, BM == 3 ? 4 : 1)
 k_inner_product(const JobRef R, const u64 *__restrict__ evk, const DevLevel *__restrict__ lv_arr,
                 const DevPrime *__restrict__ primes, int K, int L, int N, const SeedStates seeds, int rows)
 {
@@ -331,13 +346,13 @@ k_inner_product(const JobRef R, const u64 *__restrict__ evk, const DevLevel *__r
 // k_inner_product: the key limbs and digits do not depend on the level (one
 // full-level key serves every level), only U, d2, KS and beta do.  The jobs'
 // row addresses are gathered into shared memory before the wait for the
-// previous kernel (they come from host-written tables); after it, the U words
-// of a chunk of jobs (four; two at four digits, for registers) are loaded
-// together with the key words, so a thread has every load of a chunk in
-// flight before its first product.
+// previous kernel (they come from host-written tables); after it, a job's U words
+// are loaded while the job before it is summed.  The registers allow three CTAs per
+// SM (two at four digits): 64 jobs at 2^16 (levels 4 to 24) take 764 us, 895 with
+// the words of two jobs at once and 120 registers, 833 with five CTAs and spills.
 
 template <int BM, bool SEEDED>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, BM <= 3 ? 3 : 2)
 k_inner_product_shared(const JobRef R, const IpGroup *__restrict__ groups, const int *count,
                        const u64 *__restrict__ evk, const DevLevel *__restrict__ lv_arr,
                        const DevPrime *__restrict__ primes, int K, int L, int N, const SeedStates seeds)
@@ -395,37 +410,43 @@ k_inner_product_shared(const JobRef R, const IpGroup *__restrict__ groups, const
             }
         }
     }
-    constexpr int CJ = BM >= 4 ? 2 : 4;
-    for (int c0 = 0; c0 < njobs; c0 += CJ) {
-        ulonglong2 u[CJ][BM];
 #pragma unroll
-        for (int g = 0; g < CJ; g++) {
-            const int gg = c0 + g;
-            if (gg < njobs) {
+    for (int j = 0; j < BM; j++) {
+        kb[j] = make_ulonglong2(pack28(kb[j].x), pack28(kb[j].y));
+        ka[j] = make_ulonglong2(pack28(ka[j].x), pack28(ka[j].y));
+    }
+    ulonglong2 u[2][BM];
+    auto load = [&](ulonglong2 *w, int g) {
 #pragma unroll
-                for (int j = 0; j < BM; j++)
-                    if (j < s_beta[gg]) u[g][j] = ld2_hint(s_row[gg][j] + n, pol);
+        for (int j = 0; j < BM; j++)
+            if (j < s_beta[g]) w[j] = ld2_hint(s_row[g][j] + n, pol);
+    };
+    auto sums = [&](const ulonglong2 *w, int g) {
+        Acc3 bx = {0, 0, 0}, by = {0, 0, 0}, ax = {0, 0, 0}, ay = {0, 0, 0};
+        const int b = s_beta[g];
+#pragma unroll
+        for (int j = 0; j < BM; j++) {
+            if (j < b) {
+                uint32_t x0, x1, y0, y1;
+                split28(w[j].x, x0, x1);
+                split28(w[j].y, y0, y1);
+                mac28k(bx, x0, x1, x0 + x1, kb[j].x);
+                mac28k(ax, x0, x1, x0 + x1, ka[j].x);
+                mac28k(by, y0, y1, y0 + y1, kb[j].y);
+                mac28k(ay, y0, y1, y0 + y1, ka[j].y);
             }
         }
-#pragma unroll
-        for (int g = 0; g < CJ; g++) {
-            const int gg = c0 + g;
-            if (gg < njobs) {
-                U128 bx = {0, 0}, by = {0, 0}, ax = {0, 0}, ay = {0, 0};
-                const int b = s_beta[gg];
-#pragma unroll
-                for (int j = 0; j < BM; j++) {
-                    if (j < b) {
-                        mac(bx, u[g][j].x, kb[j].x);
-                        mac(by, u[g][j].y, kb[j].y);
-                        mac(ax, u[g][j].x, ka[j].x);
-                        mac(ay, u[g][j].y, ka[j].y);
-                    }
-                }
-                st2(s_ks[gg][0] + n, barrett128(bx, pr.q, pr.mu, pr.s), barrett128(by, pr.q, pr.mu, pr.s));
-                st2(s_ks[gg][1] + n, barrett128(ax, pr.q, pr.mu, pr.s), barrett128(ay, pr.q, pr.mu, pr.s));
-            }
-        }
+        st2(s_ks[g][0] + n, ip_reduce(bx, pr), ip_reduce(by, pr));
+        st2(s_ks[g][1] + n, ip_reduce(ax, pr), ip_reduce(ay, pr));
+    };
+    if (njobs > 0) load(u[0], 0);
+#pragma unroll 1
+    for (int g = 0; g < njobs; g += 2) {
+        if (g + 1 < njobs) load(u[1], g + 1);
+        sums(u[0], g);
+        if (g + 1 >= njobs) break;
+        if (g + 2 < njobs) load(u[0], g + 2);
+        sums(u[1], g + 1);
     }
 }
 
@@ -988,7 +1009,7 @@ cudaError_t run_inner_product(const he_ctx *c, const JobRef &R, const u64 *evk, 
                      c->K, c->L, c->N, ss, rows);                                                                    \
     } while (0)
     // three digits get their own width: 64 registers, four CTAs per SM
-    // (the four-digit width takes 78 and fits three)
+    // (the four-digit width takes 80 and fits three)
     if (bm <= 2) HE_IP(2);
     else if (bm == 3) HE_IP(3);
     else if (bm <= 4) HE_IP(4);
