@@ -458,8 +458,9 @@ int he_nr_rescale(he_nr_plan *plan, const uint64_t *ct, int logq, uint64_t *out,
 /* ---- launch shapes and autotuning (no paper counterpart) ------------------ */
 
 /* Launch shape of the path: the most NTT limbs of one prime that a CTA of a
- * batch takes one after another (they share the staged twiddles; 1..4; a single
- * HE Mul always runs one limb per CTA), ModUp targets per CTA (4, 8 or 16;
+ * batch takes one after another (they share the staged twiddles; 1..4; fewer where
+ * the batch would not fill the GPU in such groups, at most 2 above N = 2^12; a
+ * single HE Mul always runs one limb per CTA), ModUp targets per CTA (4, 8 or 16;
  * contexts whose base conversions run on the CUDA cores, below),
  * whether the path's kernels use programmatic dependent launch (1: a kernel's
  * CTAs may be scheduled while its predecessor drains; each waits for it in

@@ -96,6 +96,21 @@ struct Stages {
 int run_keyswitch(he_ctx *c, const JobRef &R, u64 *ntt_base, const Stages &S, const u64 *evk, int mode,
                   cudaStream_t st, bool tensor_fused = false);
 
+// Limbs of one prime that a CTA of a batch takes one after another, for an NTT list
+// of `limbs` limbs; the shape's group_cap is the most.  Sharing staged twiddles pays
+// while the grid stays full.  Two-pass rings: pairs from six waves of single limbs
+// (five CTAs per SM), where two-limb groups take over: 16 jobs at 2^15 590 against
+// 598 us, 16 at 2^16 1543 against 1573; four jobs at 2^16 427 against 418, eight at
+// 2^15 316 against 306.  Larger groups gain nothing there (64 jobs at 2^16: 5888,
+// 5890 and 5921 us in twos, threes and fours).  2^12, whose CTAs each stage the
+// ring's whole table and fill an SM: as many as keep one wave (128 jobs 385, 323,
+// 301 and 293 us in ones to fours; 16 jobs 79, 92, 117 and 142).
+int limb_group(const he_ctx *c, size_t limbs)
+{
+    const size_t n = c->logN == 12 ? (limbs + 151) / 152 : limbs * (size_t)(c->N / 2048) >= 6 * 5 * 152 ? 2 : 1;
+    return (int)std::min((size_t)c->group_cap, std::max<size_t>(n, 1));
+}
+
 int run_pipeline(he_ctx *c, const JobRef &R, u64 *ntt_base, const Stages &S, const u64 *evk, int mode,
                  cudaStream_t st)
 {
@@ -563,9 +578,8 @@ int he_mul_batch(he_ctx *c, int count, const he_job *jobs, const uint64_t *evk, 
     }
     if (off * N >= ((size_t)1 << 32) * N) return HE_EINVAL;  // offsets are 32-bit limb counts
     // regroup by prime across jobs: limbs of different jobs share a twiddle tile
-    const int cap = c->group_cap;
-    std::vector<NttGroup> g1 = group_jobs(l1, cap), g2 = group_jobs(l2, cap), g3 = group_jobs(l3, cap),
-                          g4 = group_jobs(l4, cap);
+    auto group = [&](const std::vector<NttJob> &l) { return group_jobs(l, limb_group(c, l.size())); };
+    std::vector<NttGroup> g1 = group(l1), g2 = group(l2), g3 = group(l3), g4 = group(l4);
     std::vector<unsigned char> head(hdr, 0);
     const size_t items_bytes = round_up(sizeof(BatchItem) * count);
     memcpy(head.data(), items.data(), sizeof(BatchItem) * count);
@@ -1000,8 +1014,8 @@ struct he_batch_graph {
     size_t hdr = 0, slot_limbs = 0;
     size_t items_bytes = 0, counts_off = 0, lists_off[4] = {0, 0, 0, 0}, ipg_off = 0;
     size_t hdr_copy = 0;  // header bytes the graph's first node copies (up to the last list's end)
-    int list_max[4] = {0, 0, 0, 0};  // groups each NTT list may hold (and its launch's grid) at `cap`
-    int cap = 1;                     // limb-group cap at capture
+    int list_max[4] = {0, 0, 0, 0};  // groups each NTT list may hold (and its launch's grid)
+    int cap[4] = {1, 1, 1, 1};       // limbs per group its bound was taken for
     int ip_jobs = 0;  // jobs per inner-product group captured (0: one job per CTA)
     // kernel nodes resized at every launch to the batch it runs (NTT nodes to
     // its limb groups, per-job nodes to its jobs); empty if the captured
@@ -1047,11 +1061,10 @@ int graph_list_bound(const he_ctx *c, int max_jobs, int t, int cap)
 }
 
 // Header layout: [items | counts | inner-product groups | four NTT lists at
-// the capture cap's bounds | room up to the bounds at cap 1], then the jobs'
+// the bounds of a full batch's groups | room up to the bounds at cap 1], then the jobs'
 // workspaces; the workspace size does not depend on the cap.
-void graph_layout(const he_ctx *c, int max_jobs, he_batch_graph *g, int cap)
+void graph_layout(const he_ctx *c, int max_jobs, he_batch_graph *g)
 {
-    g->cap = cap;
     g->items_bytes = round_up(sizeof(BatchItem) * max_jobs);
     g->counts_off = g->items_bytes;
     size_t off = g->counts_off + 256;
@@ -1059,10 +1072,12 @@ void graph_layout(const he_ctx *c, int max_jobs, he_batch_graph *g, int cap)
     off += round_up(sizeof(IpGroup) * (size_t)max_jobs);
     size_t room = off;
     for (int t = 0; t < 4; t++) {
-        g->list_max[t] = graph_list_bound(c, max_jobs, t, cap);
+        const int limbs = graph_list_bound(c, max_jobs, t, 1);
+        g->cap[t] = limb_group(c, (size_t)limbs);
+        g->list_max[t] = graph_list_bound(c, max_jobs, t, g->cap[t]);
         g->lists_off[t] = off;
         off += round_up(sizeof(NttGroup) * (size_t)g->list_max[t]);
-        room += round_up(sizeof(NttGroup) * (size_t)graph_list_bound(c, max_jobs, t, 1));
+        room += round_up(sizeof(NttGroup) * (size_t)limbs);
     }
     g->hdr_copy = off;
     g->hdr = std::max(off, room);
@@ -1159,7 +1174,7 @@ size_t he_batch_graph_workspace_bytes(const he_ctx *c, int max_jobs)
 {
     if (!c || max_jobs < 1 || max_jobs > 65535 || c->L < 2) return 0;
     he_batch_graph g;
-    graph_layout(c, max_jobs, &g, 1);
+    graph_layout(c, max_jobs, &g);
     return g.hdr + (size_t)max_jobs * g.slot_limbs * c->N * sizeof(u64);
 }
 
@@ -1175,7 +1190,7 @@ int he_batch_graph_create(he_ctx *c, int max_jobs, const uint64_t *evk, void *ws
     g->max_jobs = max_jobs;
     g->evk = evk;
     g->ws = (char *)ws;
-    graph_layout(c, max_jobs, g, c->group_cap);
+    graph_layout(c, max_jobs, g);
     // capture runs nothing, so it uses a private stream: capture is not
     // permitted on the legacy default stream the caller may be using
     (void)stream;
@@ -1293,7 +1308,10 @@ int he_batch_graph_launch(he_batch_graph *g, int count, const he_job *jobs, void
     }
     int *counts = (int *)(pin + g->counts_off);
     for (int t = 0; t < 4; t++) {
-        std::vector<NttGroup> grp = group_jobs(lists[t], std::max(c->group_cap, g->cap));
+        // the list holds a full batch in groups of cap[t]; fewer jobs in smaller groups may fit
+        const int want = std::min(limb_group(c, lists[t].size()), g->cap[t]);
+        std::vector<NttGroup> grp = group_jobs(lists[t], want);
+        if ((int)grp.size() > g->list_max[t]) grp = group_jobs(lists[t], g->cap[t]);
         if ((int)grp.size() > g->list_max[t]) return HE_EINVAL;  // cannot happen: bounded at capture
         memcpy(pin + g->lists_off[t], grp.data(), sizeof(NttGroup) * grp.size());
         counts[t] = (int)grp.size();
