@@ -176,15 +176,9 @@ int run_keyswitch(he_ctx *c, const JobRef &R, u64 *ntt_base, const Stages &S, co
         prof_mark(c, st, "moddown_conv");
     }
     capture_tag = kTagNtt0 + 3;
-    if (mode != kTailPlain) {
-        // the final combine runs in the last NTT pass (writes each job's output)
-        HE_TRY(launch_ntt_combine(c, ntt_base, S.ntt_last, S.n_ntt_last, R, st, "ntt_moddown", cnt ? cnt + 3 : nullptr));
-    } else {
-        HE_TRY(launch_ntt(c, ntt_base, S.ntt_last, S.n_ntt_last, false, st, "ntt_moddown", cnt ? cnt + 3 : nullptr));
-        capture_tag = kTagFixed;
-        HE_TRY(run_combine_plain(c, R, st));
-        prof_mark(c, st, "combine");
-    }
+    // the final combine runs in the last NTT pass (writes each job's output)
+    HE_TRY(launch_ntt_combine(c, ntt_base, S.ntt_last, S.n_ntt_last, R, mode == kTailPlain, st, "ntt_moddown",
+                              cnt ? cnt + 3 : nullptr));
     capture_tag = kTagFixed;
     return HE_OK;
 }
@@ -510,8 +504,7 @@ int he_step_moddown(he_ctx *c, const uint64_t *X, int level, uint64_t *out, void
     HE_TRY(launch_ntt(c, w, J.intt2, J.n_intt2, true, st));
     const JobRef R = single_job(c, nullptr, nullptr, w + W.y * N, w, level);  // both halves land at y, u
     HE_TRY(run_moddown_conv(c, R, false, st));
-    HE_TRY(launch_ntt(c, w, J.ntt_conv, J.n_ntt_conv, false, st));
-    HE_TRY(run_combine_plain(c, R, st));
+    HE_TRY(launch_ntt_combine(c, w, J.ntt_conv, J.n_ntt_conv, R, true, st));
     HE_TRY(cudaMemcpyAsync(out, w + W.y * N, (size_t)level * N * sizeof(u64), cudaMemcpyDeviceToDevice, st));
     return HE_OK;
 }

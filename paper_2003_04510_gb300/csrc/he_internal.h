@@ -345,9 +345,10 @@ cudaError_t launch_ntt2(const he_ctx *ctx, const u64 *src, u64 *dst, const NttGr
 cudaError_t configure_ntt(const he_ctx *ctx);
 // Forward NTT of the fused ModDown + rescale limbs with the final combine in
 // its last pass: out[h][i] = (d_h[i] + KS_h[K+i] P^-1 - NTT(z)) q_{l-1}^-1,
-// written to each job's output (groups carry the combine fields).
+// written to each job's output (groups carry the combine fields).  plain: the
+// limbs of a plain ModDown, out[h][i] = d_h[i] + (KS_h[K+i] - NTT(z)) P^-1.
 cudaError_t launch_ntt_combine(const he_ctx *ctx, u64 *base, const NttGroup *groups, int ngroups, const JobRef &R,
-                               cudaStream_t st, const char *tag = nullptr, const int *dev_count = nullptr);
+                               bool plain, cudaStream_t st, const char *tag = nullptr, const int *dev_count = nullptr);
 // Inverse NTT of d2 (and the rescale limbs of d0, d1) whose first pass forms
 // its input tiles with the tensor product from each job's ciphertexts and
 // stores d0, d1, d2 to the job's workspace (groups carry job and ci = limb |
@@ -390,6 +391,5 @@ cudaError_t run_inner_product_shared(const he_ctx *c, const JobRef &R, const IpG
 // bit-identical to he_mul then he_rescale), or one division by P q_{l-1}.
 enum TailMode { kTailPlain = 0, kTailRescale = 1, kTailRescalePQ = 2 };
 cudaError_t run_moddown_conv(const he_ctx *c, const JobRef &R, int mode, cudaStream_t st);
-cudaError_t run_combine_plain(const he_ctx *c, const JobRef &R, cudaStream_t st);
 cudaError_t run_rescale_combine(const he_ctx *c, const u64 *ct, const u64 *Z, u64 *out, int l, cudaStream_t st);
 }  // namespace he

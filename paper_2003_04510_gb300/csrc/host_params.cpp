@@ -507,7 +507,8 @@ int build_context(he_ctx *c, const he_params *p, bool device)
         for (int h = 0; h < 2; h++)
             for (int i = 0; i < l; i++)
                 H.ntt_conv.push_back(NttJob{(unsigned)(W.z + (size_t)h * l + i), (unsigned)(W.z + (size_t)h * l + i),
-                                            (unsigned)(K + i), 0, 0, 0});
+                                            (unsigned)(K + i), 0, 0, 0, 0, ((unsigned)h << 31) | (unsigned)i,
+                                            (unsigned)((h ? W.d1 : W.d0) + i), (unsigned)(W.ks + (size_t)h * El + K + i)});
         for (int h = 0; h < 2; h++)
             for (int i = 0; i + 1 < l; i++)
                 H.ntt_z.push_back(NttJob{(unsigned)(W.z + (size_t)h * (l - 1) + i),

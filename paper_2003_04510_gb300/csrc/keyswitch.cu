@@ -14,8 +14,7 @@
 //  k_moddown_conv  mod down (Sec. 7): conv_i = sum_k y_k [Phat_k]_{q_i} mod q_i;
 //                  the fused variant uses constants [Phat_k P^-1]_{q_i}, giving
 //                  conv_i P^-1 directly, and folds in the rescale residue.
-//  k_combine_plain the final additions (Fig. 2) after a plain ModDown; with
-//                  rescale, the same combine runs in the last NTT pass of the
+//                  The final additions (Fig. 2) run in the last NTT pass of the
 //                  ModDown limbs (ntt.cu).
 //
 // Every kernel handles two consecutive coefficients per thread with 16-byte
@@ -702,31 +701,6 @@ __global__ void __launch_bounds__(kTeams *tc::kTeam, 1) k_moddown_tc(const JobRe
     tc::end(ts);
 }
 
-// grid: x over N/2/kThreads, y over limbs, z over 2 * jobs (h = z & 1).
-// out[h][i] = d_h[i] + (KS_h[K+i] - C[h][i]) P^-1 mod q_i, i < l
-__global__ void __launch_bounds__(kThreads)
-k_combine_plain(const JobRef R, const ulonglong2 *__restrict__ pinv, const DevLevel *__restrict__ lv_arr,
-                const DevPrime *__restrict__ primes, int K, int N)
-{
-    const BatchItem it = job_of(R, blockIdx.z >> 1);
-    const int h = blockIdx.z & 1, l = it.level, i = blockIdx.y;
-    if (i >= l) return idle_exit();
-    const DevLevel &lv = lv_arr[l];
-    const int E = K + l;
-    const size_t n = 2 * ((size_t)blockIdx.x * kThreads + threadIdx.x);
-    const DevPrime pr = primes[K + i];
-    const ulonglong2 pv = pinv[i];
-    const u64 *d = it.ws + (size_t)(h ? lv.o_d1 : lv.o_d0) * N;
-    const u64 *KS = it.ws + (size_t)lv.o_ks * N, *C = it.ws + (size_t)lv.o_z * N;
-    griddep_wait(R.trigger);
-    const ulonglong2 dv = ld2(d + (size_t)i * N + n);
-    const ulonglong2 ks = ld2(KS + ((size_t)h * E + K + i) * N + n);
-    const ulonglong2 c = ld2(C + ((size_t)h * l + i) * N + n);
-    const u64 x = add_mod(dv.x, shoup(sub_mod(ks.x, c.x, pr.q), pv.x, pv.y, pr.q), pr.q);
-    const u64 y = add_mod(dv.y, shoup(sub_mod(ks.y, c.y, pr.q), pv.x, pv.y, pr.q), pr.q);
-    st2(it.out + ((size_t)h * l + i) * N + n, x, y);
-}
-
 // Rescale on its own: out[h][i] = (c_h[i] - Z[h][i]) q_{l-1}^-1, i < l-1
 __global__ void __launch_bounds__(kThreads)
 k_rescale_combine(const u64 *ct, const u64 *Z, u64 *out,
@@ -1141,15 +1115,6 @@ cudaError_t run_moddown_ipq(const he_ctx *c, const JobRef &R, int mode, const u6
 #undef HE_MDQ_M
 #undef HE_MDQ_B
 #undef HE_MDQ
-    return cudaGetLastError();
-}
-
-cudaError_t run_combine_plain(const he_ctx *c, const JobRef &R, cudaStream_t st)
-{
-    dim3 g = grid_x(c->N);
-    g.y = R.lmax;
-    g.z = 2 * R.B;
-    launch_k(c->pdl, k_combine_plain, g, dim3(kThreads), 0, st, sized(c, R, g), c->d_pinv, c->d_levels, c->d_primes, c->K, c->N);
     return cudaGetLastError();
 }
 

@@ -214,19 +214,21 @@ __device__ __forceinline__ void ip_tile(const NttArgs &P, const NttGroup &G, int
 // group (ModDown output (h, ci) of job G.job[i]),
 // out[h][ci] = (d_h[ci] + KS_h[K+ci] P^-1 - z) q_{l-1}^-1 with z the
 // transform in shared memory (thread pairs 2 t, +1 at g2 + k gs2 and shared
-// word padi(2 t) + k (2 NT + NT / 8)).
-template <int TE, int NT>
+// word padi(2 t) + k (2 NT + NT / 8)).  PLAIN: out[h][ci] = d_h[ci] +
+// (KS_h[K+ci] - z) P^-1, which was a kernel of its own (a rotation at 2^16, level
+// 13: 125.4 -> 123.5 us).
+template <int TE, int NT, bool PLAIN>
 __device__ __forceinline__ void combine_store(const NttArgs &P, const NttGroup &G, int i, const u64 *sm, size_t g2,
                                               size_t gs2, const DevPrime &pr, u64 nq)
 {
     const BatchItem it = job_item(P.R, (int)G.job[i]);
     const int ci = (int)(G.ci[i] & 0x7fffffffu), hh = (int)(G.ci[i] >> 31);
-    const ulonglong2 pv = P.pinv[ci], qv = P.levels[it.level].qinv_last[ci];
+    const ulonglong2 pv = P.pinv[ci], qv = PLAIN ? pv : P.levels[it.level].qinv_last[ci];
     // at least any forward-NTT output: d + KS P^-1 (lazy, < 4q) + Cz - z
     // stays positive and below Cz + 5q < 2^64 (ntt_mod leaves 8q of room),
     // and one Shoup product by q_{l-1}^-1 reduces it
     const u64 Cz = pr.nt.cz;
-    u64 *o = it.out + ((((size_t)hh * (it.level - 1) + ci)) << P.logN) + g2;
+    u64 *o = it.out + ((((size_t)hh * (PLAIN ? it.level : it.level - 1) + ci)) << P.logN) + g2;
     const u64 *dd = P.dst + ((size_t)G.cd[i] << P.logN) + g2, *kk = P.dst + ((size_t)G.cks[i] << P.logN) + g2;
     const u64 *sp = sm + padi(2 * threadIdx.x);
     // four pairs per step: their d and KS loads are all in flight before the first product
@@ -243,6 +245,12 @@ __device__ __forceinline__ void combine_store(const NttArgs &P, const NttGroup &
         for (int k = 0; k < B4; k++) {
             // KS P^-1 lazily in [0, 4q)
             const u64 *z = sp + (b0 + k) * (2 * NT + NT / 8);
+            if (PLAIN) {
+                *reinterpret_cast<ulonglong2 *>(o + (b0 + k) * gs2) =
+                    make_ulonglong2(add_mod(dv[k].x, shoup_canon(kv[k].x + Cz - z[0], pv.x, pv.y, pr.q, nq), pr.q),
+                                    add_mod(dv[k].y, shoup_canon(kv[k].y + Cz - z[1], pv.x, pv.y, pr.q, nq), pr.q));
+                continue;
+            }
             const u64 x = dv[k].x + shoup_approx_nq(kv[k].x, pv.x, pv.y, nq) + Cz - z[0];
             const u64 y = dv[k].y + shoup_approx_nq(kv[k].y, pv.x, pv.y, nq) + Cz - z[1];
             *reinterpret_cast<ulonglong2 *>(o + (b0 + k) * gs2) =
@@ -282,12 +290,12 @@ __device__ __forceinline__ void final_store(const NttArgs &P, const NttGroup &G,
 // inverse runs them in reverse) on tiles of TE elements of a ring of 2^LOGN,
 // each thread holding 2^E of them (E the longest round).  FUSE: kFuseNone;
 // kFuseCombine, the final combine in the store loop of the forward contiguous
-// last pass (ModDown + rescale limbs); kFuseTensor, the tensor product computed
+// last pass (ModDown + rescale limbs), kFusePlain the same after a plain ModDown; kFuseTensor, the tensor product computed
 // in place of the inverse contiguous first pass's tile load (d2 limbs and the
 // rescale limbs of d0, d1); kFuseIp, the key-switch sums of Fig. 2 region 2
 // computed in place of the tile load of the special limbs' inverse contiguous
 // first pass.
-enum { kFuseNone = 0, kFuseCombine = 1, kFuseTensor = 2, kFuseIp = 3 };
+enum { kFuseNone = 0, kFuseCombine = 1, kFuseTensor = 2, kFuseIp = 3, kFusePlain = 4 };
 
 template <int LOGN_, bool STRIDED_, int R0, int R1, int R2, int R3, int TE_>
 struct Pass {
@@ -541,7 +549,7 @@ __host__ __device__ constexpr int ntt_min_blocks(int nt) { return nt >= 512 ? 1 
 template <class P, int R0, int R1, int R2, int R3, bool INV, int FUSE>
 __global__ void __launch_bounds__(P::NT, ntt_min_blocks(P::NT)) k_ntt_pass(const NttArgs A)
 {
-    constexpr bool STRIDED = P::STRIDED, COMBINE = FUSE == kFuseCombine;
+    constexpr bool STRIDED = P::STRIDED, COMBINE = FUSE == kFuseCombine || FUSE == kFusePlain;
     constexpr bool COMPUTED = FUSE == kFuseTensor || FUSE == kFuseIp;  // the tile load computes its words
     constexpr bool FIRST = P::WHOLE || STRIDED != INV, LAST = P::WHOLE || STRIDED == INV;
     static_assert(!COMBINE || (LAST && !INV && !STRIDED), "the combine follows a forward contiguous last pass");
@@ -622,7 +630,7 @@ __global__ void __launch_bounds__(P::NT, ntt_min_blocks(P::NT)) k_ntt_pass(const
                 }
                 smem_put<P, LL, RL>(sm, a);
                 __syncthreads();
-                if constexpr (COMBINE) combine_store<TE, NT>(A, G, i, sm, g2, gs2, pr, nq);
+                if constexpr (COMBINE) combine_store<TE, NT, FUSE == kFusePlain>(A, G, i, sm, g2, gs2, pr, nq);
                 else final_store<TE, NT>(A, G, i, sm, g2, gs2, pr);
             }
         } else {
@@ -753,13 +761,13 @@ cudaError_t pass(int logN, const NttArgs &a, int ng, cudaStream_t st)
 template <bool INV, int FUSE>
 cudaError_t transform(const he_ctx *c, const NttArgs &a, int ng, cudaStream_t st, const char *tag)
 {
-    static const char *const kMark[4] = {"", "_combine", ".tensor_inv", ".ip_inv"};
+    static const char *const kMark[4] = {"", "", ".tensor_inv", ".ip_inv"};
     const int lg = c->logN;
     if (lg == 12) {
         const cudaError_t e = pass<false, INV, FUSE>(lg, a, ng, st);
         if (ng) {
             if (FUSE == kFuseTensor || FUSE == kFuseIp) prof_mark(c, st, tag, kMark[FUSE]);
-            else prof_mark(c, st, tag, INV ? ".inv" : FUSE == kFuseCombine ? ".fwd_combine" : ".fwd");
+            else prof_mark(c, st, tag, INV ? ".inv" : FUSE == kFuseNone ? ".fwd" : ".fwd_combine");
         }
         return e;
     }
@@ -769,7 +777,7 @@ cudaError_t transform(const he_ctx *c, const NttArgs &a, int ng, cudaStream_t st
     if (ng)
         prof_mark(c, st, tag, !INV ? ".fwd_pass1" : FUSE == kFuseTensor ? ".tensor_inv_pass1" : FUSE == kFuseIp ? ".ip_inv_pass1" : ".inv_pass1");
     e = INV ? pass<true, true, kFuseNone>(lg, a, ng, st) : pass<false, false, INV ? kFuseNone : FUSE>(lg, a, ng, st);
-    if (ng) prof_mark(c, st, tag, INV ? ".inv_pass2" : FUSE == kFuseCombine ? ".fwd_pass2_combine" : ".fwd_pass2");
+    if (ng) prof_mark(c, st, tag, INV ? ".inv_pass2" : FUSE == kFuseNone ? ".fwd_pass2" : ".fwd_pass2_combine");
     return e;
 }
 
@@ -812,14 +820,15 @@ cudaError_t launch_ntt_ip(const he_ctx *c, u64 *base, const NttGroup *groups, in
 }
 
 cudaError_t launch_ntt_combine(const he_ctx *c, u64 *base, const NttGroup *groups, int ngroups, const JobRef &R,
-                               cudaStream_t st, const char *tag, const int *dev_count)
+                               bool plain, cudaStream_t st, const char *tag, const int *dev_count)
 {
     if (ngroups < 0) return cudaSuccess;
     NttArgs a = ntt_args(c, base, base, groups, dev_count);
     a.R = R;
     a.levels = c->d_levels;
     a.pinv = c->d_pinv;
-    return transform<false, kFuseCombine>(c, a, ngroups, st, tag);
+    return plain ? transform<false, kFusePlain>(c, a, ngroups, st, tag)
+                 : transform<false, kFuseCombine>(c, a, ngroups, st, tag);
 }
 
 cudaError_t launch_ntt2(const he_ctx *c, const u64 *src, u64 *dst, const NttGroup *groups, int ngroups, bool inverse,
@@ -847,7 +856,8 @@ cudaError_t configure_ntt(const he_ctx *c)
     memset(&R, 0, sizeof(R));
     cudaError_t e = launch_ntt2(c, nullptr, nullptr, nullptr, 0, false, nullptr);
     if (e == cudaSuccess) e = launch_ntt2(c, nullptr, nullptr, nullptr, 0, true, nullptr);
-    if (e == cudaSuccess) e = launch_ntt_combine(c, nullptr, nullptr, 0, R, nullptr);
+    if (e == cudaSuccess) e = launch_ntt_combine(c, nullptr, nullptr, 0, R, false, nullptr);
+    if (e == cudaSuccess) e = launch_ntt_combine(c, nullptr, nullptr, 0, R, true, nullptr);
     if (e == cudaSuccess) e = launch_ntt_tensor(c, nullptr, nullptr, 0, R, nullptr);
     if (e == cudaSuccess) e = launch_ntt_ip(c, nullptr, nullptr, 0, R, nullptr, nullptr, nullptr, nullptr);
     return e;
