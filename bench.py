@@ -882,7 +882,7 @@ def run_ours(args):
 
     # ALU ceilings: the NTT's butterfly and the CUDA-core conversions' inner loop,
     # register-resident, measured in this run at its clocks (conversions on the
-    # tensor cores, for primes of 52 to 55 bits, run above the latter)
+    # tensor cores, for primes of 52 to 55 bits, are not bound by the latter)
     bfly_peak = g.he_probe_butterfly_rate(152 * 8, 4096, stream)
     conv_width = {"modup": kernel_width(prm.alpha), "moddown_conv": kernel_width(prm.K)}
     conv_peak = {k: g.he_probe_conversion_rate(w, 152 * 8, max(64, 4096 // w), stream) for k, w in conv_width.items()}

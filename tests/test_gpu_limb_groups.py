@@ -8,20 +8,19 @@ import pytest
 
 import oracle
 
-from test_gpu_parity import ctx_for, dev, g, host, rand_ct, rand_evk  # noqa: F401
+from test_gpu_parity import dev, g, host, rand_ct, rand_evk  # noqa: F401
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("name,lmax,counts", [("n12", 3, (200, 45, 77, 1, 200)), ("n13", 6, (150, 20, 3))])
+@pytest.mark.parametrize("logN,L,K,bits,counts", [(12, 3, 2, 50, (200, 45, 77, 1, 200)), (13, 6, 2, 54, (150, 20, 3))])
 @pytest.mark.parametrize("cap", [4, 3, 1])
-def test_batches_across_group_sizes(g, name, lmax, counts, cap):
+def test_batches_across_group_sizes(g, logN, L, K, bits, counts, cap):
     import torch
-    ctx = ctx_for(g, name)
-    op = oracle.preset(name)
+    ctx = g.Context(g.Params(logN, L, K, 2, bits, bits, 64), device=True)
+    op = oracle.make_params(logN, L, K, 2, bits, bits)
     evk = rand_evk(op, 77)
     evk_t = dev(g, evk)
-    lmax = min(lmax, op.L)
-    levels = [2 + k % (lmax - 1) for k in range(max(counts))]
+    levels = [2 + k % (L - 1) for k in range(max(counts))]
     base = {lv: (rand_ct(op, lv, 10 + lv), rand_ct(op, lv, 30 + lv)) for lv in set(levels)}
     ops, want = {}, {}
     for lv, (a, b) in base.items():
@@ -29,18 +28,16 @@ def test_batches_across_group_sizes(g, name, lmax, counts, cap):
         want[lv] = oracle.rescale(op, oracle.he_mul(op, a, b, evk, lv), lv)
     outs = [torch.empty((2, lv - 1, op.N), dtype=torch.int64, device="cuda") for lv in levels]
     jobs = [(*ops[lv], out, lv) for lv, out in zip(levels, outs)]
-    try:
-        g.he_set_shape(ctx, cap, 8, 1)
-        graph = g.BatchGraph(ctx, max(counts), evk_t)
-        ws = torch.empty(g.he_batch_workspace_bytes(ctx, levels) // 8, dtype=torch.int64, device="cuda")
-        for n in counts:
-            for run in (lambda: graph.launch(jobs[:n]), lambda: g.he_mul_batch(ctx, jobs[:n], evk_t, ws)):
-                for o in outs[:n]:
-                    o.fill_(-1)
-                run()
-                torch.cuda.synchronize()
-                for lv, o in zip(levels[:n], outs):
-                    assert np.array_equal(host(g, o), want[lv]), (n, lv)
-        graph.close()
-    finally:
-        g.he_set_shape(ctx, 4, 8, 1)
+    g.he_set_shape(ctx, cap, 8, 1)
+    graph = g.BatchGraph(ctx, max(counts), evk_t)
+    ws = torch.empty(g.he_batch_workspace_bytes(ctx, levels) // 8, dtype=torch.int64, device="cuda")
+    for n in counts:
+        for run in (lambda: graph.launch(jobs[:n]), lambda: g.he_mul_batch(ctx, jobs[:n], evk_t, ws)):
+            for o in outs[:n]:
+                o.fill_(-1)
+            run()
+            torch.cuda.synchronize()
+            for lv, o in zip(levels[:n], outs):
+                assert np.array_equal(host(g, o), want[lv]), (n, lv)
+    graph.close()
+    ctx.close()
