@@ -485,7 +485,8 @@ typedef struct {
                     while the context has at most four digits (dnum <= 4), else 1. */
     int fuse;    /* bit 0: the tensor product (Fig. 2 region 1) is formed inside the first inverse-NTT pass
                     of d2, which loads the ciphertexts instead of d2 and also stores d0, d1, d2 (one launch
-                    and one read of d2 fewer); else its own kernel.  bit 1 (single HE Mul with rescale):
+                    and one read of d2 fewer), where that pass has three CTAs per SM or more; else its
+                    own kernel.  bit 1 (single HE Mul with rescale, above N = 2^12):
                     the key-switch sums of Fig. 2 region 2 are split: those of the special primes and of
                     q_{level-1} (the next iNTT's inputs) first, those of the other q primes (read only by
                     the final additions) in the same launch as the ModDown conversion, so the key stream

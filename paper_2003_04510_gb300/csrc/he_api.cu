@@ -116,7 +116,12 @@ int run_pipeline(he_ctx *c, const JobRef &R, u64 *ntt_base, const Stages &S, con
 {
     prof_mark(c, st, "");
     // Region 1: tensor product, on its own or inside the first iNTT pass of d2
-    const bool fused = (c->fuse & 1) != 0;
+    // the fused pass forms the products on its own CTAs: below three per SM that is
+    // slower than a kernel over all SMs (2^12 L = 3 39.2 against 36.8 us, 2^15 L = 16
+    // 94.9 against 89.3, 2^16 L = 8 95.4 against 91.6), from there on it saves a launch
+    // and a read of d2 (2^16 L = 12 123.7 and 123.6, L = 24 194.6 against 198.2)
+    const int tiles = c->logN == 12 ? 1 : c->N / 2048;
+    const bool fused = (c->fuse & 1) && (long long)S.n_intt1 * tiles >= 3 * 152;
     if (!fused) {
         capture_tag = kTagJobs;
         HE_TRY(run_tensor(c, R, st));
@@ -145,7 +150,8 @@ int run_keyswitch(he_ctx *c, const JobRef &R, u64 *ntt_base, const Stages &S, co
     // a single job's q-limb sums (read only by the final combine) may run
     // beside the ModDown conversion: the sums of the special limbs and the
     // last q limb (the next iNTT's inputs) come first
-    const bool split = (c->fuse & 2) && !S.ipg && !R.items && moddown_ipq_fits(c);
+    // (at 2^12 a limb's CTA does its whole row of sums alone: 36.8 us split, 35.0 not)
+    const bool split = (c->fuse & 2) && !S.ipg && !R.items && moddown_ipq_fits(c) && c->logN > 12;
     // with the split, the sums of the special limbs and the last q limb may
     // instead be formed by the first pass of their own iNTT (unseeded keys)
     bool seeded = false;
