@@ -560,6 +560,15 @@ int he_probe_conversion_rate(int width, int blocks, int iters, double *mac_per_s
  * 2^18. */
 int he_probe_recombine_rate(int blocks, int iters, double *out_per_s, void *stream);
 
+/* Test helper: the bounded waits of a tensor-core conversion's team of 256
+ * threads around products that never complete (no paper counterpart).  Every
+ * thread gives up after `tries` (1 .. 2^18, the path's own limit); with
+ * `partial` the products complete and only one thread of the team has given
+ * up.  passes (host, 256): the tiles each thread has begun, equal when the
+ * team ends together; ms: how long it took.  The context's wait then counts as
+ * given up (HE_ETIMEOUT). */
+int he_probe_wait(he_ctx *ctx, int tries, int partial, int *passes, double *ms, void *stream);
+
 const char *he_strerror(int code);
 /* Name of the CUDA error behind the calling thread's last HE_ECUDA. */
 const char *he_last_cuda_error(void);

@@ -128,6 +128,8 @@ _SIGS = {
     "he_probe_butterfly_rate": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p]),
     "he_probe_conversion_rate": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_void_p,
                                                 ctypes.c_void_p]),
+    "he_probe_wait": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p,
+                                     ctypes.c_void_p]),
     "he_probe_recombine_rate": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p]),
     "he_galois_elt": (ctypes.c_uint64, [ctypes.c_void_p, ctypes.c_int]),
     "he_conj_elt": (ctypes.c_uint64, [ctypes.c_void_p]),
@@ -642,6 +644,16 @@ def he_probe_recombine_rate(blocks: int, iters: int, stream=None) -> float:
     _check(lib().he_probe_recombine_rate(blocks, iters, ctypes.byref(r), _stream_ptr(stream)),
            "he_probe_recombine_rate")
     return r.value
+
+
+def he_probe_wait(ctx, tries: int, partial: bool, stream=None) -> tuple[np.ndarray, float]:
+    """(tiles each of the team's 256 threads has begun, ms) of waits that give up;
+    the context answers HE_ETIMEOUT afterwards."""
+    passes = np.zeros(256, dtype=np.int32)
+    ms = ctypes.c_double()
+    _check(lib().he_probe_wait(ctx.ptr, tries, int(partial), _np_ptr(passes), ctypes.byref(ms), _stream_ptr(stream)),
+           "he_probe_wait")
+    return passes, ms.value
 
 
 class BatchGraph:

@@ -56,7 +56,7 @@ struct Args {
 };
 
 struct Shared {
-    uint64_t a_full[2], a_free[2], d_full[2], d_free[2];
+    uint64_t a_full[2], a_free[2], d_full[2], d_free[2], drain;
     uint32_t tmem;
     Prime prime[kPrimes];
 };
@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_crt(const Args P)
             icrt::bar_init(&S.d_full[i], 1);
             icrt::bar_init(&S.d_free[i], kEpilogue);
         }
+        icrt::bar_init(&S.drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc::copy_image(B, P.image + (size_t)blockIdx.y * bbytes, bbytes);
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_crt(const Args P)
             const int poly = x / per_poly, buf = it & 1;
             u64 *o = P.out + ((size_t)poly * P.np + i0 + u0) * P.N + (size_t)(x - poly * per_poly) * tc::kRows + row;
             const uint32_t lane = tmem + ((uint32_t)(warp & 3) << 21) + buf * 256;
-            if (!(ok = __all_sync(~0u, tc::bar_wait(&S.d_full[buf], (it >> 1) & 1)))) break;
+            if (!(ok = tc::warp_wait(&S.d_full[buf], (it >> 1) & 1))) break;
             tc::fence_after_sync();
             uint32_t c[2][8];
             auto put = [&](const uint32_t *p, int u) {
@@ -188,13 +189,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_crt(const Args P)
         }
     } else {
         // ---- MMAs: the warp keeps together and one lane issues ----
+        griddep_wait();  // as the roles it waits for: their time alone counts against its limits
         const uint64_t b = tc::smem_desc(tc::smem_u32(B), cols * 16);
         const uint32_t idesc = tc::mma_idesc(cols);
         int it = 0;
         for (int x = blockIdx.x; x < tiles; x += gridDim.x, it++) {
             const int buf = it & 1;
-            if (it >= 2 && !(ok = __all_sync(~0u, tc::bar_wait(&S.d_free[buf], ((it >> 1) - 1) & 1)))) break;
-            if (!(ok = __all_sync(~0u, tc::bar_wait(&S.a_full[buf], (it >> 1) & 1)))) break;
+            if (it >= 2 && !(ok = tc::warp_wait(&S.d_free[buf], ((it >> 1) - 1) & 1))) break;
+            if (!(ok = tc::warp_wait(&S.a_full[buf], (it >> 1) & 1))) break;
             tc::fence_after_sync();
             if (tc::elect_one()) {
                 uint64_t as = tc::smem_desc(tc::smem_u32(A + buf * abytes), tc::kRows * 16), bs = b;
@@ -209,7 +211,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_crt(const Args P)
         }
         // the last arrivals land before the CTA ends
         for (int k = it > 2 ? it - 2 : 0; k < it && ok; k++)
-            ok = __all_sync(~0u, tc::bar_wait(&S.a_free[k & 1], (k >> 1) & 1));
+            ok = tc::warp_wait(&S.a_free[k & 1], (k >> 1) & 1);
+        if (!ok) {  // products still under way read the operands: a second wait
+            if (tc::elect_one()) tc::mma_commit(&S.drain);
+            tc::warp_wait(&S.drain, 0);
+        }
     }
     if (!ok) *(volatile unsigned *)P.flag = 1;
     tc::fence_before_sync();

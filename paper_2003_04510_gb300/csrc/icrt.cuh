@@ -63,7 +63,7 @@ struct Args {
 };
 
 struct Shared {
-    uint64_t a_full[kMaxNp / kStagePrimes], a_free, b_full[kStages], b_free[kStages], d_full[2], d_free[2];
+    uint64_t a_full[kMaxNp / kStagePrimes], a_free, b_full[kStages], b_free[kStages], d_full[2], d_free[2], drain;
     uint32_t tmem;
     Prime prime[kMaxNp];
     uint32_t usum[kUBuf][2][tc::kRows];
@@ -138,6 +138,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_icrt(const Args P)
             bar_init(&S.d_full[i], 2);  // the MMAs, and their thread (which has seen the tile's u sums)
             bar_init(&S.d_free[i], kEpilogue);
         }
+        bar_init(&S.drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int i = t; i < P.np; i += kThreads) S.prime[i] = P.prime[i];
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_icrt(const Args P)
                     dv[k] = dn[k];
                     dn[k] = dload(w0 + kWords + k);
                 }
-                if (!(ok = __all_sync(~0u, tc::bar_wait(&S.d_full[buf], (g >> 1) & 1)))) break;
+                if (!(ok = tc::warp_wait(&S.d_full[buf], (g >> 1) & 1))) break;
                 tc::fence_after_sync();
                 if (ch == 0) {
                     const uint32_t u = (S.usum[it % kUBuf][0][t] + S.usum[it % kUBuf][1][t] + (1u << 24)) >> 25;
@@ -287,6 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_icrt(const Args P)
             for (int x = blockIdx.x; x < tiles && ok; x += gridDim.x)
                 for (int k = 0; k < P.chunks * stages; k++, c++) {
                     const int slot = c % kStages;
+                    if (c == kStages) griddep_wait();  // as the roles it waits for from here on
                     if (c >= kStages && !(ok = tc::bar_wait(&S.b_free[slot], (c / kStages - 1) & 1))) break;
                     bulk_copy(B + slot * kStageBytes, P.image + (size_t)k * kStageBytes, kStageBytes, &S.b_full[slot]);
                 }
@@ -296,6 +298,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_icrt(const Args P)
         }
     } else {
         // ---- MMAs ----
+        griddep_wait();  // as the roles it waits for: their time alone counts against its limits
         // the warp keeps together and one lane issues: descriptors stay in
         // uniform registers (issued by a lane of a diverged warp, an MMA took
         // about 115 cycles)
@@ -307,7 +310,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_icrt(const Args P)
         for (int x = blockIdx.x; x < tiles && ok; x += gridDim.x, it++) {
             for (int ch = 0; ch < P.chunks && ok; ch++, g++) {
                 const int buf = g & 1;
-                if (g >= 2 && !(ok = __all_sync(~0u, tc::bar_wait(&S.d_free[buf], ((g >> 1) - 1) & 1)))) break;
+                if (g >= 2 && !(ok = tc::warp_wait(&S.d_free[buf], ((g >> 1) - 1) & 1))) break;
                 tc::fence_after_sync();
                 const uint32_t d0 = tmem + buf * 2 * kCols;
                 if (tc::elect_one()) {
@@ -316,8 +319,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_icrt(const Args P)
                 }
                 uint64_t as = a;
                 for (int st = 0; st < stages; st++) {
-                    if (ch == 0 && !(ok = __all_sync(~0u, tc::bar_wait(&S.a_full[st], it & 1)))) break;
-                    if (!(ok = __all_sync(~0u, tc::bar_wait(&S.b_full[slot], turn & 1)))) break;
+                    if (ch == 0 && !(ok = tc::warp_wait(&S.a_full[st], it & 1))) break;
+                    if (!(ok = tc::warp_wait(&S.b_full[slot], turn & 1))) break;
                     tc::fence_after_sync();
                     if (tc::elect_one()) {
                         const uint32_t d = st < first ? d0 : d0 + kCols;
@@ -342,7 +345,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_icrt(const Args P)
             }
         }
         // the last arrival lands before the CTA ends
-        if (it && ok) ok = __all_sync(~0u, tc::bar_wait(&S.a_free, (it - 1) & 1));
+        if (it && ok) ok = tc::warp_wait(&S.a_free, (it - 1) & 1);
+        if (!ok) {  // products still under way read the operands: a second wait
+            if (tc::elect_one()) tc::mma_commit(&S.drain);
+            tc::warp_wait(&S.drain, 0);
+        }
     }
     if (!ok) *(volatile unsigned *)P.flag = 1;
     tc::fence_before_sync();

@@ -20,7 +20,9 @@
 //    inputs in registers, as the kernels do, and walks a table of constant
 //    rows; the outputs are folded into a checksum instead of stored.
 #include "he_internal.h"
+#include "icrt.cuh"
 #include "modarith.cuh"
+#include "tc.cuh"
 
 namespace {
 
@@ -123,6 +125,32 @@ __global__ void __launch_bounds__(256) k_probe_recombine(u64 *out, u64 q, u64 mu
         }
     }
     out[blockIdx.x * blockDim.x + threadIdx.x] = acc;
+}
+
+// The waits of a tensor-core conversion's team (tc.cuh) around products that do not
+// complete, without the products: five tiles, of which the third's barrier nothing
+// arrives at, so every thread gives up after `tries`; or (partial) one that completes
+// but which one thread of the fourth warp has no tries for.  passes[t]: tiles thread t
+// has begun.
+constexpr int kProbeTiles = 5, kProbeStop = 2;
+
+__global__ void __launch_bounds__(he::tc::kTeam) k_probe_wait(int tries, bool partial, int *passes, unsigned *flag)
+{
+    __shared__ uint64_t bar;
+    const int t = threadIdx.x;
+    if (t == 0) he::tc::bar_init(&bar);
+    __syncthreads();
+    bool ok = true;
+    int n = 0;
+    uint32_t phase = 0;
+    for (int x = 0; x < kProbeTiles; x++, phase ^= 1) {
+        if (he::tc::team_sync_any<he::tc::kTeam>(1, !ok)) break;
+        n++;
+        if (t == 0 && (x != kProbeStop || partial)) he::icrt::bar_arrive(&bar);
+        ok = he::tc::warp_wait(&bar, phase, x == kProbeStop && partial && t == 127 ? 0 : tries);
+    }
+    if (!ok && (t & 31) == 0) *(volatile unsigned *)flag = 1;
+    passes[t] = n;
 }
 
 // q_0 of the N = 2^16 chain (54 bits) and its Barrett constants as the
@@ -234,5 +262,29 @@ extern "C" int he_probe_recombine_rate(int blocks, int iters, double *out_per_s,
     cudaFreeAsync(out, st);
     if (rc != HE_OK) return rc;
     *out_per_s = (double)blocks * 256.0 * kRows * (double)iters / (ms * 1e-3);
+    return HE_OK;
+}
+
+extern "C" int he_probe_wait(he_ctx *c, int tries, int partial, int *passes, double *ms, void *stream)
+{
+    if (!c || !c->device || tries < 1 || tries > he::tc::kTries || !passes || !ms) return HE_EINVAL;
+    cudaStream_t st = (cudaStream_t)stream;
+    int *out = nullptr;
+    cudaEvent_t a = nullptr, b = nullptr;
+    if (cudaMallocAsync((void **)&out, sizeof(int) * he::tc::kTeam, st) != cudaSuccess) return HE_ECUDA;
+    float t = 0;
+    bool ok = cudaEventCreate(&a) == cudaSuccess && cudaEventCreate(&b) == cudaSuccess;
+    if (ok) {
+        cudaEventRecord(a, st);
+        k_probe_wait<<<1, he::tc::kTeam, 0, st>>>(tries, partial != 0, out, c->d_flag);
+        cudaEventRecord(b, st);
+        ok = cudaMemcpyAsync(passes, out, sizeof(int) * he::tc::kTeam, cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+             cudaStreamSynchronize(st) == cudaSuccess && cudaEventElapsedTime(&t, a, b) == cudaSuccess;
+    }
+    if (a) cudaEventDestroy(a);
+    if (b) cudaEventDestroy(b);
+    cudaFreeAsync(out, st);
+    if (!ok) return HE_ECUDA;
+    *ms = t;
     return HE_OK;
 }

@@ -85,10 +85,11 @@ __device__ __forceinline__ void bar_init(uint64_t *bar)
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
-// Wait for the phase; false after the limit (about a second).
-__device__ __forceinline__ bool bar_wait(const uint64_t *bar, uint32_t parity)
+// Wait for the phase; false after the limit.
+constexpr int kTries = 1 << 18;  // about a second: a try that fails takes 3.8 us
+__device__ __forceinline__ bool bar_wait(const uint64_t *bar, uint32_t parity, int tries = kTries)
 {
-    for (int it = 0; it < (1 << 22); it++) {
+    for (int it = 0; it < tries; it++) {
         uint32_t ok;
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
                      "selp.u32 %0, 1, 0, p;\n\t}"
@@ -98,6 +99,27 @@ __device__ __forceinline__ bool bar_wait(const uint64_t *bar, uint32_t parity)
         if (ok) return true;
     }
     return false;
+}
+
+// A wait may give up in some threads and not in others.  What must not split does
+// not: a warp waits as one (tcgen05.ld takes whole warps), and the warps of a team
+// learn at their next barrier whether one of them has lost its tile, so that no
+// warp is left waiting there for one that returned.
+__device__ __forceinline__ bool warp_wait(const uint64_t *bar, uint32_t parity, int tries = kTries)
+{
+    return __all_sync(~0u, bar_wait(bar, parity, tries));
+}
+// Barrier `id` of the team's `threads`; true to all of them if `lost` is to any.
+template <int threads>
+__device__ __forceinline__ bool team_sync_any(int id, bool lost)
+{
+    uint32_t any;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbar.red.or.pred q, %2, %3, p;\n\t"
+                 "selp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(any)
+                 : "r"((uint32_t)lost), "r"(id), "n"(threads)
+                 : "memory");
+    return any != 0;
 }
 
 // Consecutive columns of this thread's TMEM lane.
@@ -291,11 +313,12 @@ __device__ __forceinline__ void team_tiles(J &job, unsigned char *A, const unsig
     const int per = ((cnt + 1) / 2 + 1) & ~1, u0 = half * per, u1 = min(cnt, u0 + per);
     if (half) put_padding<G>(A, row);
     uint32_t phase = 0;
+    bool ok = true;
     if (x < tiles) job.load((size_t)x * kRows + row, half);
     for (; x < tiles; x += step) {
 #pragma unroll
         for (int k = 0; k < (G + 1) / 2; k++)
-            if (2 * k + half < G) {
+            if (ok && 2 * k + half < G) {  // operands of products still under way stay
                 u64 v[4];
 #pragma unroll
                 for (int i = 0; i < 4; i++) v[i] = job.value(k, i);
@@ -304,7 +327,7 @@ __device__ __forceinline__ void team_tiles(J &job, unsigned char *A, const unsig
         job.start((size_t)x * kRows + row);
         fence_smem();
         fence_before_sync();  // the team's reads of the tile before, and these writes, precede the MMAs
-        asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kTeam) : "memory");
+        if (team_sync_any<kTeam>(team + 1, !ok)) break;
         if (t == 0) {
             fence_after_sync();
             issue<G>(tmem, A, B, rows);
@@ -312,14 +335,10 @@ __device__ __forceinline__ void team_tiles(J &job, unsigned char *A, const unsig
             mma_commit(bar);
         }
         if (x + step < tiles) job.load((size_t)(x + step) * kRows + row, half);
-        const bool ok = bar_wait(bar, phase);
-        __syncwarp();
+        ok = warp_wait(bar, phase);
         fence_after_sync();
         phase ^= 1;
-        if (!ok) {  // the products never completed: nothing more is issued
-            if (t == 0) *(volatile unsigned *)flag = 1;
-            return;
-        }
+        if (!ok) continue;  // to the barrier, where the team ends together
         if (EXTRA) {
             uint32_t P[8];
             tmem_ld8(P, lane + rows);
@@ -349,6 +368,10 @@ __device__ __forceinline__ void team_tiles(J &job, unsigned char *A, const unsig
                 put2(P[1], u + 2);
             }
         }
+    }
+    if (!ok) {  // the products never completed: nothing more is issued, and the operands and TMEM outlive a second wait
+        if ((t & 31) == 0) *(volatile unsigned *)flag = 1;
+        warp_wait(bar, phase ^ 1);
     }
 }
 
