@@ -325,7 +325,7 @@ __device__ __forceinline__ void ip_body(const JobRef &R, const BatchItem &it, co
 
 // grid: x over N/2/kThreads, y over the rows selected (IpRows), z over jobs.
 template <int BM, bool SEEDED>
-__global__ void __launch_bounds__(kThreads, BM == 3 ? 4 : 1)
+__global__ void __launch_bounds__(kThreads, BM <= 3 ? 4 : 1)
 k_inner_product(const JobRef R, const u64 *__restrict__ evk, const DevLevel *__restrict__ lv_arr,
                 const DevPrime *__restrict__ primes, int K, int L, int N, const SeedStates seeds, int rows)
 {
@@ -982,8 +982,9 @@ cudaError_t run_inner_product(const he_ctx *c, const JobRef &R, const u64 *evk, 
             launch_k(c->pdl, k_inner_product<B, false>, g, dim3(kThreads), 0, st, sized(c, R, g), evk, c->d_levels, c->d_primes,  \
                      c->K, c->L, c->N, ss, rows);                                                                    \
     } while (0)
-    // three digits get their own width: 64 registers, four CTAs per SM
-    // (the four-digit width takes 80 and fits three)
+    // at most three digits run at 64 registers, four CTAs per SM (the two-digit width
+    // takes 66 and fits three if left alone: he_step_inner_product at 2^15, level
+    // 16, 26.4 us against 24.7)
     if (bm <= 2) HE_IP(2);
     else if (bm == 3) HE_IP(3);
     else if (bm <= 4) HE_IP(4);
