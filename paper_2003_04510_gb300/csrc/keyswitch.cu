@@ -241,8 +241,7 @@ __device__ __forceinline__ u64 seeded_a(u64 state, u64 idx, u64 t)
 
 // U: [beta][E][N] (own-digit rows read from d2), evk: [dnum][2][K+L][N]
 // (SEEDED: [dnum][K+L][N], b halves only, a halves regenerated), KS: [2][E][N].
-// The digit loop is unrolled to BM >= beta with guards, so every operand
-// load of a thread is issued before the first product.
+// The digit loop is unrolled to BM >= beta with guards.
 //
 // Rows: the key-switch sum of ext limb e of one job.  Which limb a CTA takes
 // (IpRows): every limb (grid.y over K + lmax); the special limbs and, for the
@@ -287,35 +286,46 @@ __device__ __forceinline__ void ip_body(const JobRef &R, const BatchItem &it, co
     // the key and the ModUp outputs are read once: evict-first keeps them from
     // displacing the twiddle tables in L2
     const u64 pol = l2_policy_stream();
-    ulonglong2 u[BM], kb[BM], ka[BM];
+    // every load of C digits is issued before their first product.  The sixteen-digit
+    // width of a seeded key takes its digits in two halves: all at once, the words
+    // regenerated for one thread's a halves waited in registers beside its loads
+    // (2^16, 15 digits, 32 limbs: 375 us against 249 for the carry chains before; one
+    // HE Mul + rescale 807 us, 686 in halves, 677 in quarters, which lose
+    // at 6 digits used: 173.6 against 170.9)
+    constexpr int C = SEEDED && BM > 8 ? 8 : BM;
+    Acc3 bx = {0, 0, 0}, by = {0, 0, 0}, ax = {0, 0, 0}, ay = {0, 0, 0};
+#pragma unroll 1
+    for (int j0 = 0; j0 < BM; j0 += C) {
+        ulonglong2 u[C], kb[C], ka[C];
 #pragma unroll
-    for (int j = 0; j < BM; j++) {
-        if (j < beta) {
-            const int lo = lv.dig_lo[j], nj = lv.dig_n[j];
-            const bool own = e >= K && e - K >= lo && e - K < lo + nj;
-            const u64 *up = own ? d2 + (size_t)(e - K) * N : U + ((size_t)j * E + e) * N;
-            u[j] = own ? ld2(up + n) : ld2_hint(up + n, pol);
-            if (SEEDED) {
-                kb[j] = ld2_hint(evk + ((size_t)j * EL + e) * N + n, pol);
-                const u64 idx = (u64)e * (u64)N + n;
-                ka[j] = make_ulonglong2(seeded_a(seeds.s[j], idx, pr.q), seeded_a(seeds.s[j], idx + 1, pr.q));
-            } else {
-                kb[j] = ld2_hint(evk + ((size_t)(2 * j) * EL + e) * N + n, pol);
-                ka[j] = ld2_hint(evk + ((size_t)(2 * j + 1) * EL + e) * N + n, pol);
+        for (int k = 0; k < C; k++) {
+            const int j = j0 + k;
+            if (j < beta) {
+                const int lo = lv.dig_lo[j], nj = lv.dig_n[j];
+                const bool own = e >= K && e - K >= lo && e - K < lo + nj;
+                const u64 *up = own ? d2 + (size_t)(e - K) * N : U + ((size_t)j * E + e) * N;
+                u[k] = own ? ld2(up + n) : ld2_hint(up + n, pol);
+                if (SEEDED) {
+                    kb[k] = ld2_hint(evk + ((size_t)j * EL + e) * N + n, pol);
+                    const u64 idx = (u64)e * (u64)N + n;
+                    ka[k] = make_ulonglong2(seeded_a(seeds.s[j], idx, pr.q), seeded_a(seeds.s[j], idx + 1, pr.q));
+                } else {
+                    kb[k] = ld2_hint(evk + ((size_t)(2 * j) * EL + e) * N + n, pol);
+                    ka[k] = ld2_hint(evk + ((size_t)(2 * j + 1) * EL + e) * N + n, pol);
+                }
             }
         }
-    }
-    Acc3 bx = {0, 0, 0}, by = {0, 0, 0}, ax = {0, 0, 0}, ay = {0, 0, 0};
 #pragma unroll
-    for (int j = 0; j < BM; j++) {
-        if (j < beta) {
-            uint32_t x0, x1, y0, y1;
-            split28(u[j].x, x0, x1);
-            split28(u[j].y, y0, y1);
-            mac28k(bx, x0, x1, x0 + x1, pack28(kb[j].x));
-            mac28k(ax, x0, x1, x0 + x1, pack28(ka[j].x));
-            mac28k(by, y0, y1, y0 + y1, pack28(kb[j].y));
-            mac28k(ay, y0, y1, y0 + y1, pack28(ka[j].y));
+        for (int k = 0; k < C; k++) {
+            if (j0 + k < beta) {
+                uint32_t x0, x1, y0, y1;
+                split28(u[k].x, x0, x1);
+                split28(u[k].y, y0, y1);
+                mac28k(bx, x0, x1, x0 + x1, pack28(kb[k].x));
+                mac28k(ax, x0, x1, x0 + x1, pack28(ka[k].x));
+                mac28k(by, y0, y1, y0 + y1, pack28(kb[k].y));
+                mac28k(ay, y0, y1, y0 + y1, pack28(ka[k].y));
+            }
         }
     }
     u64 *KS = it.ws + (size_t)lv.o_ks * N;
