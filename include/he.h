@@ -31,9 +31,15 @@
  *
  * Errors: every call returns an int status (HE_OK on success).  Argument
  * errors are detected on the host before anything is enqueued.  A CUDA launch
- * failure returns HE_ECUDA.  Bounded device waits (batched and served
- * execution) that give up surface as HE_ETIMEOUT at the next synchronising
- * call.  he_strerror() names a code.
+ * failure returns HE_ECUDA.  The tensor-core kernels wait on the device for a
+ * bounded time (about a second; base conversions of 52- to 55-bit primes, the
+ * BigInt CRT and iCRT).  If such a wait gives up, results of the context's
+ * calls then in flight may be wrong: from then on every call that enqueues or
+ * synchronises work of that context, he_ctx_info, and every request of a server
+ * that finishes on it returns HE_ETIMEOUT, until the context is destroyed (the
+ * destroy functions themselves do not).  A
+ * caller that synchronises its own stream asks he_ctx_info afterwards.
+ * he_strerror() names a code.
  */
 #ifndef HE_GB300_H
 #define HE_GB300_H
@@ -86,7 +92,8 @@ int he_ctx_create_host(he_ctx **out, const he_params *p);
 int he_ctx_destroy(he_ctx *ctx);
 
 /* Query: N, dnum, and the moduli in ext order (K specials then L ciphertext
- * primes; `moduli` must hold K+L words). */
+ * primes; `moduli` must hold K+L words).  Any output may be NULL.  HE_ETIMEOUT,
+ * with the outputs filled, once a device wait of the context has given up. */
 int he_ctx_info(const he_ctx *ctx, int *N, int *dnum, uint64_t *moduli);
 
 /* ---- host side (plain C buffers, caller-owned) --------------------------- */

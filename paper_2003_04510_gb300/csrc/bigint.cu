@@ -630,6 +630,7 @@ size_t he_nr_evk_bytes(const he_nr_plan *pl) { return pl ? (size_t)2 * pl->np2 *
 int he_nr_evk_prepare(he_nr_plan *pl, const uint64_t *evk, uint64_t *prep, void *stream)
 {
     if (!pl || !evk || !prep) return HE_EINVAL;
+    if (int w = device_waits(pl->c)) return w;
     cudaStream_t st = (cudaStream_t)stream;
     launch_crt_evk(pl, evk, nwords(2 * pl->logQ), 2, prep, pl->np2, st);
     if (cudaGetLastError() != cudaSuccess) return HE_ECUDA;
@@ -642,6 +643,7 @@ int he_nr_mul(he_nr_plan *pl, const uint64_t *ct1, const uint64_t *ct2, const ui
     if (!pl || !ct1 || !ct2 || !prep || !out || !ws) return HE_EINVAL;
     if (logq < pl->logp + 1 || logq > pl->logQ) return HE_ELEVEL;
     if (ws_bytes < ws_words(pl) * sizeof(u64)) return HE_ENOMEM;
+    if (int w = device_waits(pl->c)) return w;
     const he_ctx *c = pl->c;
     he_ctx *cm = pl->c;
     const size_t N = (size_t)c->N;
@@ -685,6 +687,7 @@ int he_nr_rescale(he_nr_plan *pl, const uint64_t *ct, int logq, uint64_t *out, v
 {
     if (!pl || !ct || !out) return HE_EINVAL;
     if (logq <= pl->logp || logq > pl->logQ) return HE_ELEVEL;
+    if (int w = device_waits(pl->c)) return w;
     const he_ctx *c = pl->c;
     const int wi = nwords(logq), wo = nwords(logq - pl->logp);
     launch_k(c->pdl, k_nr_rescale, dim3((unsigned)(c->N / kT), 2u), dim3(kT), 0, (cudaStream_t)stream, ct, wi, out,

@@ -65,6 +65,12 @@ bool aligned(const void *p) { return ((uintptr_t)p & 255) == 0; }
 
 size_t ws_bytes_for(const he_ctx *c, int l) { return c->host_levels[l].ws.total * (size_t)c->N * sizeof(u64); }
 
+// A call about to enqueue work: HE_ETIMEOUT if a device wait of the context has given up.
+#define HE_WAITS(c)                             \
+    do {                                        \
+        if (int w_ = device_waits(c)) return w_; \
+    } while (0)
+
 int check_dev(const he_ctx *c) { return (c && c->device) ? HE_OK : HE_EINVAL; }
 
 // Upload a small job list for the per-step entry points (test helpers).
@@ -315,12 +321,13 @@ int he_ctx_info(const he_ctx *c, int *N, int *dnum, uint64_t *moduli)
     if (N) *N = c->N;
     if (dnum) *dnum = c->dnum;
     if (moduli) memcpy(moduli, c->ext.data(), sizeof(u64) * c->E);
-    return HE_OK;
+    return device_waits(c);
 }
 
 int he_evk_upload(he_ctx *c, const uint64_t *evk_host, uint64_t *evk_dev, void *stream)
 {
     if (check_dev(c) || !evk_host || !evk_dev) return HE_EINVAL;
+    HE_WAITS(c);
     size_t bytes = (size_t)c->dnum * 2 * c->E * c->N * sizeof(u64);
     HE_TRY(cudaMemcpyAsync(evk_dev, evk_host, bytes, cudaMemcpyHostToDevice, S(stream)));
     return HE_OK;
@@ -339,6 +346,7 @@ int he_mul(he_ctx *c, const uint64_t *ct1, const uint64_t *ct2, const uint64_t *
     if (level < 1 || level > c->L) return HE_ELEVEL;
     if (!aligned(ct1) || !aligned(ct2) || !aligned(out) || !aligned(ws) || !aligned(evk)) return HE_EINVAL;
     if (ws_bytes < ws_bytes_for(c, level)) return HE_ENOMEM;
+    HE_WAITS(c);
     return hemul_pipeline(c, ct1, ct2, evk, level, out, (u64 *)ws, kTailPlain, S(stream));
 }
 
@@ -349,6 +357,7 @@ int he_mul_rescale(he_ctx *c, const uint64_t *ct1, const uint64_t *ct2, const ui
     if (level < 2 || level > c->L) return HE_ELEVEL;
     if (!aligned(ct1) || !aligned(ct2) || !aligned(out) || !aligned(ws) || !aligned(evk)) return HE_EINVAL;
     if (ws_bytes < ws_bytes_for(c, level)) return HE_ENOMEM;
+    HE_WAITS(c);
     return hemul_pipeline(c, ct1, ct2, evk, level, out, (u64 *)ws, kTailRescale, S(stream));
 }
 
@@ -359,6 +368,7 @@ int he_mul_rescale_pq(he_ctx *c, const uint64_t *ct1, const uint64_t *ct2, const
     if (level < 2 || level > c->L) return HE_ELEVEL;
     if (!aligned(ct1) || !aligned(ct2) || !aligned(out) || !aligned(ws) || !aligned(evk)) return HE_EINVAL;
     if (ws_bytes < ws_bytes_for(c, level)) return HE_ENOMEM;
+    HE_WAITS(c);
     return hemul_pipeline(c, ct1, ct2, evk, level, out, (u64 *)ws, kTailRescalePQ, S(stream));
 }
 
@@ -368,6 +378,7 @@ int elementwise(he_ctx *c, int op, const uint64_t *x, const uint64_t *y, int lev
     if (check_dev(c) || !x || !y || !out) return HE_EINVAL;
     if (level < 1 || level > c->L) return HE_ELEVEL;
     if (!aligned(x) || !aligned(y) || !aligned(out)) return HE_EINVAL;
+    HE_WAITS(c);
     HE_TRY(run_elementwise(c, op, x, y, out, level, S(stream)));
     return HE_OK;
 }
@@ -401,6 +412,7 @@ int he_rotate(he_ctx *c, const uint64_t *ct, const uint64_t *rk, int level, uint
     if (level < 1 || level > c->L) return HE_ELEVEL;
     if (!aligned(ct) || !aligned(out) || !aligned(ws) || !aligned(rk)) return HE_EINVAL;
     if (ws_bytes < ws_bytes_for(c, level)) return HE_ENOMEM;
+    HE_WAITS(c);
     cudaStream_t st = S(stream);
     u64 *w = (u64 *)ws;
     prof_mark(c, st, "");
@@ -416,6 +428,7 @@ int he_rescale(he_ctx *c, const uint64_t *ct, int level, uint64_t *out, void *ws
     if (level < 2 || level > c->L) return HE_ELEVEL;
     if (!aligned(ct) || !aligned(out) || !aligned(ws)) return HE_EINVAL;
     if (ws_bytes < ws_bytes_for(c, level)) return HE_ENOMEM;
+    HE_WAITS(c);
     const WsLayout &W = c->host_levels[level].ws;
     const LevelJobs &J = c->jobs[level];
     const size_t N = (size_t)c->N;
@@ -436,6 +449,7 @@ int he_step_ntt(he_ctx *c, uint64_t *data, const int *prime_idx, int count, int 
         int e = prime_idx[i];
         jobs[i] = NttJob{(unsigned)i, (unsigned)i, (unsigned)e, 0, c->ninv[e], c->ninv_sh[e]};
     }
+    HE_WAITS(c);
     cudaStream_t st = S(stream);
     std::vector<NttGroup> groups = group_jobs(jobs, 1);
     NttGroup *dj = nullptr;
@@ -450,6 +464,7 @@ int he_step_tensor(he_ctx *c, const uint64_t *ct1, const uint64_t *ct2, int leve
 {
     if (check_dev(c) || !ct1 || !ct2 || !d) return HE_EINVAL;
     if (level < 1 || level > c->L) return HE_ELEVEL;
+    HE_WAITS(c);
     // d0, d1, d2 sit at limb offsets 0, l, 2l of a workspace: d serves as one
     HE_TRY(run_tensor(c, single_job(c, ct1, ct2, nullptr, (u64 *)d, level), S(stream)));
     return HE_OK;
@@ -460,6 +475,7 @@ int he_step_modup(he_ctx *c, const uint64_t *d2, int level, uint64_t *U, void *w
     if (check_dev(c) || !d2 || !U || !ws) return HE_EINVAL;
     if (level < 1 || level > c->L) return HE_ELEVEL;
     if (ws_bytes < ws_bytes_for(c, level)) return HE_ENOMEM;
+    HE_WAITS(c);
     const WsLayout &W = c->host_levels[level].ws;
     const LevelJobs &J = c->jobs[level];
     const size_t N = (size_t)c->N;
@@ -480,6 +496,7 @@ int he_step_inner_product(he_ctx *c, const uint64_t *U, const uint64_t *d2, cons
     if (check_dev(c) || !U || !d2 || !evk || !KS || !ws) return HE_EINVAL;
     if (level < 1 || level > c->L) return HE_ELEVEL;
     if (ws_bytes < ws_bytes_for(c, level)) return HE_ENOMEM;
+    HE_WAITS(c);
     const WsLayout &W = c->host_levels[level].ws;
     const size_t N = (size_t)c->N;
     const size_t E = (size_t)c->K + level, beta = (size_t)(level + c->alpha - 1) / c->alpha;
@@ -497,6 +514,7 @@ int he_step_moddown(he_ctx *c, const uint64_t *X, int level, uint64_t *out, void
     if (check_dev(c) || !X || !out || !ws) return HE_EINVAL;
     if (level < 1 || level > c->L) return HE_ELEVEL;
     if (ws_bytes < ws_bytes_for(c, level)) return HE_ENOMEM;
+    HE_WAITS(c);
     const WsLayout &W = c->host_levels[level].ws;
     const LevelJobs &J = c->jobs[level];
     const size_t N = (size_t)c->N;
@@ -543,6 +561,7 @@ int he_mul_batch(he_ctx *c, int count, const he_job *jobs, const uint64_t *evk, 
         lmax = std::max(lmax, j.level);
     }
     if (ws_bytes < batch_bytes(c, count, levels.data())) return HE_ENOMEM;
+    HE_WAITS(c);
     const size_t N = (size_t)c->N;
     const size_t hdr = batch_header_bytes(c, count, levels.data());
     char *wsb = (char *)ws;
@@ -906,6 +925,7 @@ int he_mul_rescale_host(he_ctx *c, const uint64_t *ct1, const uint64_t *ct2, con
     if (level < 2 || level > c->L) return HE_ELEVEL;
     if (!aligned(ws) || !aligned(evk)) return HE_EINVAL;
     if (ws_bytes < he_host_workspace_bytes(c, level)) return HE_ENOMEM;
+    HE_WAITS(c);
     const size_t limb = (size_t)c->N * sizeof(u64);
     char *base = (char *)ws;
     u64 *w = (u64 *)base;
@@ -946,6 +966,7 @@ int he_mul_rescale_host_stream(he_ctx *c, int count, const uint64_t *const *ct1,
         ml = std::max(ml, levels[k]);
     }
     if (ws_bytes < he_host_stream_workspace_bytes(c, ml, slots)) return HE_ENOMEM;
+    HE_WAITS(c);
     {
         std::lock_guard<std::mutex> lk(c->io_mu);
         if (!c->io_h2d && cudaStreamCreateWithFlags(&c->io_h2d, cudaStreamNonBlocking) != cudaSuccess) return HE_ECUDA;
@@ -1183,6 +1204,7 @@ int he_batch_graph_create(he_ctx *c, int max_jobs, const uint64_t *evk, void *ws
     if (check_dev(c) || !evk || !ws || !out || !aligned(ws) || !aligned(evk)) return HE_EINVAL;
     if (max_jobs < 1 || max_jobs > 65535 || c->L < 2) return HE_EINVAL;
     if (ws_bytes < he_batch_graph_workspace_bytes(c, max_jobs)) return HE_ENOMEM;
+    HE_WAITS(c);
     he_batch_graph *g = new (std::nothrow) he_batch_graph();
     if (!g) return HE_ENOMEM;
     g->c = c;
@@ -1274,6 +1296,7 @@ int he_batch_graph_launch(he_batch_graph *g, int count, const he_job *jobs, void
         if (!j.ct1 || !j.ct2 || !j.out || !aligned(j.ct1) || !aligned(j.ct2) || !aligned(j.out)) return HE_EINVAL;
         if (j.level < 2 || j.level > c->L) return HE_ELEVEL;
     }
+    HE_WAITS(c);
     // the launch that last read this pinned header must have finished
     const int b = g->memcpy_node ? (int)(g->nlaunch & 1u) : 0;
     if (g->launched[b]) {

@@ -177,7 +177,7 @@ struct he_ctx {
     // base conversions on the tensor cores: primes of 52 to 55 bits whose
     // constants keep every plane exact (tc_image); else the CUDA-core kernels
     bool tc = false;
-    unsigned *flag = nullptr, *d_flag = nullptr;  // mapped host word a bounded device wait sets when it gives up
+    unsigned *flag = nullptr, *d_flag = nullptr;  // mapped host word a bounded device wait sets when it gives up, for good
     uint32_t up_off5 = 0, dn_off5 = 0;   // top digits' offsets of ModUp's and ModDown's sources
     int up_smem = 0, dn_smem = 0;        // shared memory of a CTA
     int dn_nch = 0, dn_tc = 0, dn_tp = 0, dn_bytes = 0, dn_last_bytes = 0;  // ModDown: chunks of targets
@@ -221,11 +221,13 @@ struct he_ctx {
 namespace he {
 // host_params.cpp
 int build_context(he_ctx *ctx, const he_params *p, bool device);
-// After a synchronisation: HE_ETIMEOUT if a bounded device wait has given up
-// since the last check, else HE_OK.
+// HE_ETIMEOUT once a bounded device wait of the context has given up, else HE_OK.
+// The word stays set: several calls may be in flight on several streams, and the one
+// whose results are wrong is not told from the others, so every call that ends or
+// begins afterwards reports it.
 inline int device_waits(const he_ctx *c)
 {
-    return c->flag && __atomic_exchange_n(c->flag, 0u, __ATOMIC_RELAXED) ? HE_ETIMEOUT : HE_OK;
+    return c->flag && __atomic_load_n(c->flag, __ATOMIC_RELAXED) ? HE_ETIMEOUT : HE_OK;
 }
 // tc_tables.cpp
 uint16_t half_of(int v);  // f16 bits of an integer that f16 holds exactly
