@@ -32,8 +32,8 @@
  * Errors: every call returns an int status (HE_OK on success).  Argument
  * errors are detected on the host before anything is enqueued.  A CUDA launch
  * failure returns HE_ECUDA.  The tensor-core kernels wait on the device for a
- * bounded time (about a second; base conversions of 52- to 55-bit primes, the
- * BigInt CRT and iCRT).  If such a wait gives up, results of the context's
+ * bounded time (base conversions of 52- to 55-bit primes 62 ms a wait, the BigInt
+ * CRT and iCRT about a second).  If such a wait gives up, results of the context's
  * calls then in flight may be wrong: from then on every call that enqueues or
  * synchronises work of that context, he_ctx_info, and every request of a server
  * that finishes on it returns HE_ETIMEOUT, until the context is destroyed (the
@@ -569,11 +569,11 @@ int he_probe_recombine_rate(int blocks, int iters, double *out_per_s, void *stre
 
 /* Test helper: the bounded waits of a tensor-core conversion's team of 256
  * threads around products that never complete (no paper counterpart).  Every
- * thread gives up after `tries` (1 .. 2^18, the path's own limit); with
- * `partial` the products complete and only one thread of the team has given
- * up.  passes (host, 256): the tiles each thread has begun, equal when the
- * team ends together; ms: how long it took.  The context's wait then counts as
- * given up (HE_ETIMEOUT). */
+ * thread gives up after `tries` (1 .. 2^14, the path's own limit); with
+ * `partial` the products complete and only one thread gives up.  passes
+ * (host, 256): the tiles of five that each thread has done, which is all of them
+ * (a team goes on together); ms: how long it took.  The context's wait then
+ * counts as given up (HE_ETIMEOUT). */
 int he_probe_wait(he_ctx *ctx, int tries, int partial, int *passes, double *ms, void *stream);
 
 const char *he_strerror(int code);

@@ -647,7 +647,7 @@ def he_probe_recombine_rate(blocks: int, iters: int, stream=None) -> float:
 
 
 def he_probe_wait(ctx, tries: int, partial: bool, stream=None) -> tuple[np.ndarray, float]:
-    """(tiles each of the team's 256 threads has begun, ms) of waits that give up;
+    """(tiles each of the team's 256 threads has done, ms) of waits that give up;
     the context answers HE_ETIMEOUT afterwards."""
     passes = np.zeros(256, dtype=np.int32)
     ms = ctypes.c_double()

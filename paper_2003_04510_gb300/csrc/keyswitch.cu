@@ -212,8 +212,8 @@ k_modup_tc(const JobRef R, const DevLevel *__restrict__ lv_arr, const DevPrime *
     job.canon = CANON;
     tc::team_tiles<G, false>(job, sm + team * ABYTES, B, B, (uint32_t)lv.up_bytes / (2 * tc::k_pad(G)),
                              tmem + team * tc::kCols, &ts.bar[team], team, blockIdx.x * kTeams + team,
-                             gridDim.x * kTeams, N / tc::kRows, cnt, st, off5, flag);
-    tc::end(ts);
+                             gridDim.x * kTeams, N / tc::kRows, cnt, st, off5, &ts.lost);
+    tc::end(ts, flag);
 }
 
 // grid: x over N/2/kThreads, y over ext limbs (up to K + lmax), z over jobs.
@@ -707,8 +707,8 @@ __global__ void __launch_bounds__(kTeams *tc::kTeam, 1) k_moddown_tc(const JobRe
     const int team = threadIdx.x / tc::kTeam;
     tc::team_tiles<G, FUSED>(job, sm + team * ABYTES, B, B1, (uint32_t)D.bytes / (2 * tc::k_pad(G)),
                              tmem + team * tc::kCols, &ts.bar[team], team, blockIdx.x * kTeams + team,
-                             gridDim.x * kTeams, N / tc::kRows, cnt, st, D.off5, D.flag);
-    tc::end(ts);
+                             gridDim.x * kTeams, N / tc::kRows, cnt, st, D.off5, &ts.lost);
+    tc::end(ts, D.flag);
 }
 
 // Rescale on its own: out[h][i] = (c_h[i] - Z[h][i]) q_{l-1}^-1, i < l-1

@@ -130,26 +130,27 @@ __global__ void __launch_bounds__(256) k_probe_recombine(u64 *out, u64 q, u64 mu
 // The waits of a tensor-core conversion's team (tc.cuh) around products that do not
 // complete, without the products: five tiles, of which the third's barrier nothing
 // arrives at, so every thread gives up after `tries`; or (partial) one that completes
-// but which one thread of the fourth warp has no tries for.  passes[t]: tiles thread t
-// has begun.
+// but which one thread has no tries for.  passes[t]: tiles thread t has done.
 constexpr int kProbeTiles = 5, kProbeStop = 2;
 
 __global__ void __launch_bounds__(he::tc::kTeam) k_probe_wait(int tries, bool partial, int *passes, unsigned *flag)
 {
     __shared__ uint64_t bar;
+    __shared__ uint32_t lost;
     const int t = threadIdx.x;
     if (t == 0) he::tc::bar_init(&bar);
+    if (t == 32) lost = 0;
     __syncthreads();
-    bool ok = true;
     int n = 0;
     uint32_t phase = 0;
     for (int x = 0; x < kProbeTiles; x++, phase ^= 1) {
-        if (he::tc::team_sync_any<he::tc::kTeam>(1, !ok)) break;
-        n++;
+        asm volatile("bar.sync 1, %0;" ::"n"(he::tc::kTeam) : "memory");
         if (t == 0 && (x != kProbeStop || partial)) he::icrt::bar_arrive(&bar);
-        ok = he::tc::warp_wait(&bar, phase, x == kProbeStop && partial && t == 127 ? 0 : tries);
+        he::tc::team_wait(&bar, phase, &lost, x == kProbeStop && partial && t == 127 ? 0 : tries);
+        n++;
     }
-    if (!ok && (t & 31) == 0) *(volatile unsigned *)flag = 1;
+    __syncthreads();
+    if (t == 0 && lost) *(volatile unsigned *)flag = 1;
     passes[t] = n;
 }
 
@@ -267,7 +268,7 @@ extern "C" int he_probe_recombine_rate(int blocks, int iters, double *out_per_s,
 
 extern "C" int he_probe_wait(he_ctx *c, int tries, int partial, int *passes, double *ms, void *stream)
 {
-    if (!c || !c->device || tries < 1 || tries > he::tc::kTries || !passes || !ms) return HE_EINVAL;
+    if (!c || !c->device || tries < 1 || tries > he::tc::kTeamTries || !passes || !ms) return HE_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     int *out = nullptr;
     cudaEvent_t a = nullptr, b = nullptr;

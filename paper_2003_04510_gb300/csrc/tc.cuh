@@ -100,26 +100,25 @@ __device__ __forceinline__ bool bar_wait(const uint64_t *bar, uint32_t parity, i
     }
     return false;
 }
-
-// A wait may give up in some threads and not in others.  What must not split does
-// not: a warp waits as one (tcgen05.ld takes whole warps), and the warps of a team
-// learn at their next barrier whether one of them has lost its tile, so that no
-// warp is left waiting there for one that returned.
-__device__ __forceinline__ bool warp_wait(const uint64_t *bar, uint32_t parity, int tries = kTries)
+// The same for a warp that acts on the answer as one.
+__device__ __forceinline__ bool warp_wait(const uint64_t *bar, uint32_t parity)
 {
-    return __all_sync(~0u, bar_wait(bar, parity, tries));
+    return __all_sync(~0u, bar_wait(bar, parity));
 }
-// Barrier `id` of the team's `threads`; true to all of them if `lost` is to any.
-template <int threads>
-__device__ __forceinline__ bool team_sync_any(int id, bool lost)
+// The wait of a team's thread (team_tiles) for a tile's products, which take a
+// microsecond.  Some threads may give up and others not; what must not split does not: a
+// thread that gives up marks its CTA (end() reports it) and goes on with its team,
+// barriers and whole-warp instructions included.  Its outputs are as wrong as the report
+// says.  A team has up to 86 tiles, hence a shorter limit (62 ms).  The code around
+// the wait is kept this short because the tiles' chain runs through it: an answer shared
+// by the warp or the team, or a report from here, cost up to 10 us of a 78 us launch of
+// short tiles.
+constexpr int kTeamTries = 1 << 14;
+__device__ __forceinline__ void team_wait(const uint64_t *bar, uint32_t parity, uint32_t *lost, int tries = kTeamTries)
 {
-    uint32_t any;
-    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbar.red.or.pred q, %2, %3, p;\n\t"
-                 "selp.u32 %0, 1, 0, q;\n\t}"
-                 : "=r"(any)
-                 : "r"((uint32_t)lost), "r"(id), "n"(threads)
-                 : "memory");
-    return any != 0;
+    const bool ok = bar_wait(bar, parity, tries);
+    __syncwarp();
+    if (!ok) *(volatile uint32_t *)lost = 1;
 }
 
 // Consecutive columns of this thread's TMEM lane.
@@ -261,7 +260,7 @@ __device__ __forceinline__ u64 recombine(uint32_t w0, uint32_t w1, uint32_t w2, 
 template <int NT>
 struct Shared {
     uint64_t bar[NT];
-    uint32_t tmem;
+    uint32_t tmem, lost;  // lost: a thread of the CTA has given up a wait
 };
 template <int NT>
 __host__ __device__ constexpr uint32_t alloc_cols() { return NT * kCols <= 256 ? 256 : 512; }
@@ -273,6 +272,7 @@ __device__ __forceinline__ void begin(Shared<NT> &s)
 {
     static_assert(NT * kCols <= 512, "TMEM");
     if (threadIdx.x / 32 == 0) tmem_alloc(&s.tmem, alloc_cols<NT>());
+    if (threadIdx.x == 32) s.lost = 0;
     if (threadIdx.x >= 32 && threadIdx.x < 32 + NT) bar_init(&s.bar[threadIdx.x - 32]);
 }
 template <int NT>
@@ -287,11 +287,19 @@ __device__ __forceinline__ uint32_t ready(Shared<NT> &s)
     return s.tmem;
 }
 template <int NT>
-__device__ __forceinline__ void end(Shared<NT> &s)
+__device__ __forceinline__ void end(Shared<NT> &s, unsigned *flag)
 {
     fence_before_sync();
     __syncthreads();
-    if (threadIdx.x / 32 == 0) tmem_free(s.tmem, alloc_cols<NT>());
+    if (threadIdx.x / 32 == 0) {
+        if (s.lost) {
+            *(volatile unsigned *)flag = 1;
+            // products may be under way: operands and TMEM outlive a second wait, for either phase
+            for (int i = 0; i < 2 * NT; i++) bar_wait(&s.bar[i / 2], i & 1, kTeamTries);
+        }
+        __syncwarp();
+        tmem_free(s.tmem, alloc_cols<NT>());
+    }
 }
 
 // One team's tiles x, x + step, ... < tiles.  A: the team's operand buffer; B, B1:
@@ -306,19 +314,18 @@ template <int G, bool EXTRA, class J>
 __device__ __forceinline__ void team_tiles(J &job, unsigned char *A, const unsigned char *B, const unsigned char *B1,
                                            uint32_t rows, uint32_t tmem, const uint64_t *bar, int team, int x,
                                            int step, int tiles, int cnt, const Row *st, uint32_t off5,
-                                           unsigned *flag)
+                                           uint32_t *lost)
 {
     const int t = threadIdx.x - team * kTeam, row = t & 127, half = t >> 7;
     const uint32_t lane = tmem + (((threadIdx.x / 32) & 3u) << 21);  // warp w reads lanes 32 (w mod 4) + its lane
     const int per = ((cnt + 1) / 2 + 1) & ~1, u0 = half * per, u1 = min(cnt, u0 + per);
     if (half) put_padding<G>(A, row);
     uint32_t phase = 0;
-    bool ok = true;
     if (x < tiles) job.load((size_t)x * kRows + row, half);
     for (; x < tiles; x += step) {
 #pragma unroll
         for (int k = 0; k < (G + 1) / 2; k++)
-            if (ok && 2 * k + half < G) {  // operands of products still under way stay
+            if (2 * k + half < G) {
                 u64 v[4];
 #pragma unroll
                 for (int i = 0; i < 4; i++) v[i] = job.value(k, i);
@@ -327,7 +334,7 @@ __device__ __forceinline__ void team_tiles(J &job, unsigned char *A, const unsig
         job.start((size_t)x * kRows + row);
         fence_smem();
         fence_before_sync();  // the team's reads of the tile before, and these writes, precede the MMAs
-        if (team_sync_any<kTeam>(team + 1, !ok)) break;
+        asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kTeam) : "memory");
         if (t == 0) {
             fence_after_sync();
             issue<G>(tmem, A, B, rows);
@@ -335,10 +342,9 @@ __device__ __forceinline__ void team_tiles(J &job, unsigned char *A, const unsig
             mma_commit(bar);
         }
         if (x + step < tiles) job.load((size_t)(x + step) * kRows + row, half);
-        ok = warp_wait(bar, phase);
+        team_wait(bar, phase, lost);
         fence_after_sync();
         phase ^= 1;
-        if (!ok) continue;  // to the barrier, where the team ends together
         if (EXTRA) {
             uint32_t P[8];
             tmem_ld8(P, lane + rows);
@@ -368,10 +374,6 @@ __device__ __forceinline__ void team_tiles(J &job, unsigned char *A, const unsig
                 put2(P[1], u + 2);
             }
         }
-    }
-    if (!ok) {  // the products never completed: nothing more is issued, and the operands and TMEM outlive a second wait
-        if ((t & 31) == 0) *(volatile unsigned *)flag = 1;
-        warp_wait(bar, phase ^ 1);
     }
 }
 

@@ -1,6 +1,6 @@
-"""Bounded device waits that give up: a team of a tensor-core conversion ends
-together, whether all of its threads give up or one does, and after about a second at
-the path's own limit; and every call of the context reports it from then on, however
+"""Bounded device waits that give up: a team of a tensor-core conversion comes to its
+end, whether all of its threads give up or one does, and soon at the path's own
+limit; and every call of the context reports it from then on, however
 many are in flight, while other contexts work on.
 """
 import numpy as np
@@ -20,26 +20,23 @@ def ctx(g):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("partial", [False, True])
-@pytest.mark.parametrize("tries", [1, 1000, 1 << 16])
-def test_team_ends_together(g, ctx, tries, partial):
+@pytest.mark.parametrize("tries", [1, 1000])
+def test_team_goes_on_together(g, ctx, tries, partial):
     passes, _ = g.he_probe_wait(ctx, tries, partial)
-    # the third tile is lost; nobody begins the fourth, and nobody stays behind
-    if tries > 1:
-        assert np.array_equal(passes, np.full(256, 3)), passes
-    else:  # a wait of one try may be lost earlier
-        assert passes.min() == passes.max() <= 3, passes
+    assert np.array_equal(passes, np.full(256, 5)), passes
+    assert g.lib().he_ctx_info(ctx.ptr, None, None, None) == g.HE_ETIMEOUT
 
 
 @pytest.mark.gpu
 def test_limit_is_short(g, ctx):
-    passes, ms = g.he_probe_wait(ctx, 1 << 18, False)
-    assert np.array_equal(passes, np.full(256, 3))
-    assert 500 < ms < 4_000, ms
+    passes, ms = g.he_probe_wait(ctx, 1 << 14, False)
+    assert np.array_equal(passes, np.full(256, 5))
+    assert ms < 1_000, ms  # a wait is 62 ms, and the rest may each be as long
 
 
 @pytest.mark.gpu
 def test_bad_arguments(g, ctx):
-    for tries in (0, -1, (1 << 18) + 1):
+    for tries in (0, -1, (1 << 14) + 1):
         with pytest.raises(g.HeError):
             g.he_probe_wait(ctx, tries, False)
 
