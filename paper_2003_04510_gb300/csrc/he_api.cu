@@ -148,7 +148,7 @@ int run_keyswitch(he_ctx *c, const JobRef &R, u64 *ntt_base, const Stages &S, co
         HE_TRY(launch_ntt_tensor(c, ntt_base, S.intt1, S.n_intt1, R, st, "intt_d2", cnt ? cnt + 0 : nullptr));
     else
         HE_TRY(launch_ntt(c, ntt_base, S.intt1, S.n_intt1, true, st, "intt_d2", cnt ? cnt + 0 : nullptr));
-    capture_tag = kTagJobs;
+    capture_tag = kTagUp;
     HE_TRY(run_modup(c, R, st));
     prof_mark(c, st, "modup");
     capture_tag = kTagNtt0 + 1;
@@ -179,7 +179,7 @@ int run_keyswitch(he_ctx *c, const JobRef &R, u64 *ntt_base, const Stages &S, co
         HE_TRY(launch_ntt_ip(c, ntt_base, S.intt2, S.n_intt2, R, evk, st, "intt_special", cnt ? cnt + 2 : nullptr));
     else
         HE_TRY(launch_ntt(c, ntt_base, S.intt2, S.n_intt2, true, st, "intt_special", cnt ? cnt + 2 : nullptr));
-    capture_tag = kTagJobs;
+    capture_tag = kTagDown;
     if (split) {
         HE_TRY(run_moddown_ipq(c, R, mode, evk, st));
         prof_mark(c, st, "moddown_conv_ipq");
@@ -1345,6 +1345,8 @@ int he_batch_graph_launch(he_batch_graph *g, int count, const he_job *jobs, void
         memcpy(pin + g->ipg_off, ipg.data(), sizeof(IpGroup) * ipg.size());
         counts[4] = (int)ipg.size();
     }
+    int lmax = 0;
+    for (int i = 0; i < count; i++) lmax = std::max(lmax, jobs[i].level);
     // the header copy reads this launch's pinned buffer; every kernel node is
     // sized to this batch (the updates apply to this launch, not to one that
     // is still running)
@@ -1356,12 +1358,15 @@ int he_batch_graph_launch(he_batch_graph *g, int count, const he_job *jobs, void
         cudaKernelNodeParams p = f.p;
         if (f.tag >= kTagNtt0 && f.tag < kTagNtt0 + 4)
             p.gridDim.x = (unsigned)std::max(1, counts[f.tag - kTagNtt0]) * f.tiles;
-        else if (f.tag == kTagJobs)
+        else if (f.tag == kTagJobs || f.tag == kTagUp || f.tag == kTagDown)
             p.gridDim.z = (unsigned)count;
         else if (f.tag == kTagIpGroups)
             p.gridDim.z = (unsigned)std::max(1, counts[4]);
         else
             continue;
+        // few jobs' conversions take the SMs that a full batch's would have used: one
+        // job on a graph captured for 16 at 2^15, level 16, 188 -> 101 us; 2^16, level 24, 337 -> 214
+        if (f.tag == kTagUp || f.tag == kTagDown) p.gridDim.x = conversion_ctas(c, f.tag, lmax, count);
         if (cudaGraphExecKernelNodeSetParams(g->exec, f.node, &p) != cudaSuccess) return HE_ECUDA;
     }
     cudaStream_t st = S(stream);

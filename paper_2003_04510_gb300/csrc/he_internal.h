@@ -254,6 +254,7 @@ void prof_mark(const he_ctx *ctx, cudaStream_t st, const char *tag, const char *
 enum LaunchTag {
     kTagNtt0 = 0,   // NTT launches over group list t (0..3): grid.x = groups x tiles
     kTagJobs = 8,   // per-job kernels: grid.z = jobs
+    kTagUp, kTagDown,  // base conversions: also grid.x, the CTAs that share a list of tiles (conversion_ctas)
     kTagIpGroups,   // the shared-key inner product: grid.z = its job groups
     kTagFixed       // not resized
 };
@@ -393,5 +394,7 @@ cudaError_t run_inner_product_shared(const he_ctx *c, const JobRef &R, const IpG
 // bit-identical to he_mul then he_rescale), or one division by P q_{l-1}.
 enum TailMode { kTailPlain = 0, kTailRescale = 1, kTailRescalePQ = 2 };
 cudaError_t run_moddown_conv(const he_ctx *c, const JobRef &R, int mode, cudaStream_t st);
+// grid.x of ModUp (kTagUp) or of a ModDown conversion (kTagDown) for `jobs` jobs up to level lmax
+unsigned conversion_ctas(const he_ctx *c, int tag, int lmax, int jobs);
 cudaError_t run_rescale_combine(const he_ctx *c, const u64 *ct, const u64 *Z, u64 *out, int l, cudaStream_t st);
 }  // namespace he

@@ -869,13 +869,28 @@ int tc_ctas(const he_ctx *c, int lists)
     return std::max(1, std::min(most, std::max(kSMs / lists, (tiles + 4 * kTeams - 1) / (4 * kTeams) * (lists > kSMs / 4))));
 }
 
+// Digits of a level up to lmax, and chunks of their targets: K + (beta - 1) alpha at most.
+void modup_lists(const he_ctx *c, int lmax, int &beta, int &nch)
+{
+    beta = (lmax + c->alpha - 1) / c->alpha;
+    nch = (c->K + (beta - 1) * c->alpha + tc::kTargets - 1) / tc::kTargets;
+}
+
+unsigned conversion_ctas(const he_ctx *c, int tag, int lmax, int jobs)
+{
+    if (!c->tc) return grid_x(c->N).x;
+    if (tag == kTagDown) return (unsigned)tc_ctas(c, 2 * ((lmax + c->dn_tc - 1) / c->dn_tc) * jobs);
+    int beta, nch;
+    modup_lists(c, lmax, beta, nch);
+    return (unsigned)tc_ctas(c, beta * nch * jobs);
+}
+
 template <bool CANON>
 cudaError_t launch_modup_tc(const he_ctx *c, const JobRef &R, cudaStream_t st)
 {
-    // chunks of any level up to lmax: K + (beta - 1) alpha targets at most
-    const int beta = (R.lmax + c->alpha - 1) / c->alpha,
-              nch = (c->K + (beta - 1) * c->alpha + tc::kTargets - 1) / tc::kTargets;
-    const dim3 g((unsigned)tc_ctas(c, beta * nch * R.B), (unsigned)(beta * nch), (unsigned)R.B);
+    int beta, nch;
+    modup_lists(c, R.lmax, beta, nch);
+    const dim3 g(conversion_ctas(c, kTagUp, R.lmax, R.B), (unsigned)(beta * nch), (unsigned)R.B);
 #define HE_UP(GG)                                                                                                   \
     launch_k(c->pdl, k_modup_tc<GG, CANON>, g, dim3(kTeams *tc::kTeam), (size_t)c->up_smem, st, sized(c, R, g), c->d_levels,     \
              c->d_primes, c->K, c->N, nch, c->up_off5, c->d_flag)
@@ -1042,7 +1057,7 @@ template <int G>
 cudaError_t launch_moddown_tc(const he_ctx *c, const JobRef &R, int mode, cudaStream_t st)
 {
     const DnArgs D = dn_args(c, mode, R.lmax);
-    const dim3 g((unsigned)tc_ctas(c, 2 * D.nch * R.B), (unsigned)(2 * D.nch), (unsigned)R.B);
+    const dim3 g(conversion_ctas(c, kTagDown, R.lmax, R.B), (unsigned)(2 * D.nch), (unsigned)R.B);
     const dim3 b(kTeams * tc::kTeam);
     const size_t sm = (size_t)c->dn_smem;
     if (mode == kTailRescale) launch_k(c->pdl, k_moddown_tc<G, kTailRescale>, g, b, sm, st, sized(c, R, g), D);
