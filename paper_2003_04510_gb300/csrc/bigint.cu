@@ -309,30 +309,55 @@ cudaError_t launch_crt(const he_nr_plan *pl, const u64 *const *in, int polys, in
     return cudaGetLastError();
 }
 
-// Image of 2^(8k) mod p_i, k < 8 W, over np primes, and each prime's constants.
-void crt_image(const he_ctx *c, int np, int W, std::vector<uint16_t> &image, std::vector<crt::Prime> &prime)
+// f16 of the balanced bytes, which the images hold by the hundred thousand.
+const uint16_t *byte_halves()
 {
-    const int pc = crt::chunk_primes(np), nch = (np + pc - 1) / pc;
-    image.assign((size_t)nch * crt::image_bytes(W, pc) / 2, 0);
-    prime.resize(np);
-    for (int i = 0; i < np; i++) {
+    static const std::vector<uint16_t> t = [] {
+        std::vector<uint16_t> h(256);
+        for (int v = -128; v < 128; v++) h[v + 128] = half_of(v);
+        return h;
+    }();
+    return t.data() + 128;
+}
+
+// Images of 2^(8k) mod p_i, k < 8 W, over the first np1 and over all np2 >= np1 primes,
+// and each prime's constants.
+void crt_images(const he_ctx *c, int np1, int np2, int W, std::vector<uint16_t> &image1, std::vector<uint16_t> &image2,
+                std::vector<crt::Prime> &prime)
+{
+    const uint16_t *half = byte_halves(), offset = half_of(6144);  // times the digits' 2048
+    std::vector<uint16_t> *image[2] = {&image1, &image2};
+    const int np[2] = {np1, np2};
+    int pc[2];
+    for (int t = 0; t < 2; t++) {
+        pc[t] = crt::chunk_primes(np[t]);
+        image[t]->assign((size_t)((np[t] + pc[t] - 1) / pc[t]) * crt::image_bytes(W, pc[t]) / 2, 0);
+    }
+    prime.resize(np2);
+    for (int i = 0; i < np2; i++) {
         const u64 p = c->ext[c->K + i];
-        uint16_t *im = image.data() + (size_t)(i / pc) * crt::image_bytes(W, pc) / 2;
-        auto at = [&](int k, int col) -> uint16_t & { return im[((size_t)(k / 8) * 8 * pc + 8 * (i % pc) + col) * 8 + k % 8]; };
+        const u64 two8 = shoup_c(256, p);  // 256 < p
+        uint16_t *im[2];  // the prime's first row: rows of eight digits, 8 pc rows to a core column
+        for (int t = 0; t < 2; t++)
+            im[t] = i < np[t] ? image[t]->data() + (size_t)(i / pc[t]) * crt::image_bytes(W, pc[t]) / 2 + (size_t)(i % pc[t]) * 64
+                              : nullptr;
         u64 v = 1 % p, sum = 0;  // sum of the bytes' offsets
         for (int k = 0; k < 8 * W; k++) {
             long long x = v > p / 2 ? (long long)v - (long long)p : (long long)v;
             for (int col = 0; col < 8; col++) {
-                const long long r = ((x + 128) & 255) - 128;
-                at(k, col) = half_of((int)r);
-                x = (x - r) / 256;
+                const int r = (int)((x + 128) & 255) - 128;
+                for (int t = 0; t < 2; t++)
+                    if (im[t]) im[t][((size_t)(k / 8) * 8 * pc[t] + col) * 8 + k % 8] = half[r];
+                x = (x - r) >> 8;  // exact
             }
             sum = hm::add(sum, v, p);
-            v = hm::mul(v, 256, p);
+            v = v * 256 - (u64)(((unsigned __int128)v * two8) >> 64) * p;  // Shoup: below 2 p
+            v = v >= p ? v - p : v;
         }
         u64 off = 0, w = 1 % p;
         for (int col = 0; col < 8; col++) {
-            at(8 * W, col) = half_of(6144);  // times the digits' 2048
+            for (int t = 0; t < 2; t++)
+                if (im[t]) im[t][((size_t)W * 8 * pc[t] + col) * 8] = offset;
             if (col % 2 == 0) off = hm::add(off, hm::mul(crt::kPair % p, w, p), p);
             w = hm::mul(w, 256, p);
         }
@@ -355,6 +380,7 @@ void icrt_tables(const he_ctx *c, int np, int W, int add_bit, std::vector<u64> &
     std::vector<u64> M, P;
     crt_tables(c, np, W, M, P, phinv);
     image.assign((size_t)chunks * npad * icrt::kCols * 8, 0);
+    const uint16_t *half = byte_halves();
     std::vector<int> m(8 * W);
     MW fix(W, 0);  // sum_i H M_i - sum_c kOff 2^(8c)
     for (int i = 0; i < np; i++) {
@@ -364,10 +390,10 @@ void icrt_tables(const he_ctx *c, int np, int W, int add_bit, std::vector<u64> &
             carry = v >= 128;
             m[e] = v - 256 * carry;
         }
-        for (int ct = 0; ct < 8 * W; ct++)
-            for (int d = 0; d < 8 && d <= ct; d++)
-                image[(((size_t)(ct / icrt::kCols) * npad + i) * icrt::kCols + ct % icrt::kCols) * 8 + d] =
-                    half_of(m[ct - d]);
+        for (int ct = 0; ct < 8 * W; ct++) {
+            uint16_t *row = &image[(((size_t)(ct / icrt::kCols) * npad + i) * icrt::kCols + ct % icrt::kCols) * 8];
+            for (int d = 0; d < 8 && d <= ct; d++) row[d] = half[m[ct - d]];
+        }
         MW h(M.begin() + (size_t)i * W, M.begin() + (size_t)(i + 1) * W);
         mw_mul_small(h, 0x0080808080808080ull);
         mw_add(fix, h);
@@ -480,8 +506,8 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
     std::vector<u64> crt((size_t)np2 * pl->chunks_evk);
     for (int i = 0; i < np2; i++) {
         const u64 p = c->ext[K + i];
-        for (int k = 0; k < pl->chunks_evk; k++) {
-            const u64 v = powmod(2, 28ull * (u64)k, p);
+        u64 v = 1;
+        for (int k = 0; k < pl->chunks_evk; k++, v = hm::mul(v, 1ull << 28, p)) {
             crt[(size_t)i * pl->chunks_evk + k] = (v & 0xFFFFFFFull) | ((v >> 28) << 32);
         }
     }
@@ -489,8 +515,7 @@ int he_nr_plan_create(he_ctx *c, int logQ, int logp, he_nr_plan **out)
     std::vector<uint16_t> image1, image2;
     std::vector<uint16_t> crt1, crt2;
     std::vector<crt::Prime> crt_prime;
-    crt_image(c, np1, pl->W1, crt1, crt_prime);
-    crt_image(c, np2, pl->W1, crt2, crt_prime);
+    crt_images(c, np1, np2, pl->W1, crt1, crt2, crt_prime);
     pl->crt_folds = true;
     for (const crt::Prime &p : crt_prime) pl->crt_folds = pl->crt_folds && crt::folds(p);
     icrt_tables(c, np1, pl->W1, -1, phinv1, image1, neg1);
