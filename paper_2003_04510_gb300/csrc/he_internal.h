@@ -299,7 +299,8 @@ inline void launch_k(bool dep, void (*k)(KArgs...), dim3 grid, dim3 block, size_
 // grid's completion and memory flush before touching its data.  Without it
 // the next kernel is launched as this grid's CTAs exit.
 // No pointer to data of an earlier kernel is declared __restrict__ or read with
-// __ldg: either lets the compiler move the loads above this wait.
+// __ldg: either lets the compiler move the loads above this wait.  Nor is it read with
+// a non-coherent load (ld2_hint, ld2_static).
 __device__ __forceinline__ void griddep_wait(bool trigger = false)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -331,8 +332,18 @@ __device__ __forceinline__ u64 l2_policy_keep()
     asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
-// 16-byte read-only load with an L2 policy, no L1 allocation.
+// 16-byte loads with an L2 policy, no L1 allocation.  ld2_hint: data, which an
+// earlier kernel may still be writing while this one is resident (a non-coherent load
+// is allowed only for what no one writes during the kernel).  ld2_static: tables
+// that only the host writes, before any kernel of the context.
 __device__ __forceinline__ ulonglong2 ld2_hint(const void *p, u64 pol)
+{
+    ulonglong2 v;
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;"
+                 : "=l"(v.x), "=l"(v.y) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ ulonglong2 ld2_static(const void *p, u64 pol)
 {
     ulonglong2 v;
     asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;"

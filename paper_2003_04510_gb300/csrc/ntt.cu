@@ -78,7 +78,7 @@ struct NttArgs {
 
 // 16-byte read-only load that does not allocate in L1 (twiddles read once).
 // The table's lines are kept in L2 (evict-last): every HE Mul rereads them.
-__device__ __forceinline__ ulonglong2 ld_tw(const ulonglong2 *p) { return ld2_hint(p, l2_policy_keep()); }
+__device__ __forceinline__ ulonglong2 ld_tw(const ulonglong2 *p) { return ld2_static(p, l2_policy_keep()); }
 
 __host__ __device__ constexpr int cmax(int a, int b) { return a > b ? a : b; }
 
