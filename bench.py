@@ -279,6 +279,27 @@ def shape_dict(t) -> dict:
     return d
 
 
+def tune_report(best, tried) -> dict:
+    """The autotuner's choice for the result line: the kept shape and how many it timed (the hundreds of
+    timed shapes themselves would be most of the line)."""
+    return dict(shape_dict(best), shapes_timed=len(tried))
+
+
+def short(o):
+    """Floats of a result to six significant digits."""
+    if isinstance(o, dict):
+        return {k: short(v) for k, v in o.items()}
+    if isinstance(o, (list, tuple)):
+        return [short(v) for v in o]
+    return float(f"{o:.6g}") if isinstance(o, float) else o
+
+
+def tensor_conversions(moduli) -> bool:
+    """Whether a context of these primes converts bases on the tensor cores (which the CUDA-core conversion
+    probe does not bound)."""
+    return all(52 <= int(q).bit_length() <= 55 for q in moduli)
+
+
 def committed_traffic(kernel: str):
     """Per-launch DRAM bytes of `kernel` (a name of the bench's event profile)
     from a committed ncu summary under profiles/ that names it ("bench kernel:
@@ -396,7 +417,7 @@ def run_batched(g, ctx, evk_t, dev, stream, wsz, count=64, reps=20):
         ms = float(np.median(totals))
         lat = np.array(lat)
         res[name] = {"HE_Mul_per_s": wsz * count * reps / (ms * 1e-3), "ms_per_batch": ms / reps,
-                     "loops_ms": totals, "batch_latency_ms_p50": float(np.percentile(lat, 50)),
+                     "batch_latency_ms_p50": float(np.percentile(lat, 50)),
                      "batch_latency_ms_p99": float(np.percentile(lat, 99))}
     graph.close()
     # per-kernel device time of one batch (CUDA events between the launches)
@@ -410,7 +431,7 @@ def run_batched(g, ctx, evk_t, dev, stream, wsz, count=64, reps=20):
         ip_bytes = sum(kernel_work("inner_product", ctx.prm, lv)[1] for lv in levels)
         res["inner_product_gbs"] = ip_bytes / (res["kernels_us"]["inner_product"] * 1e-6) / 1e9
     g.he_set_shape(ctx, *shape_before)
-    res["autotune"] = dict(shape_dict(best), ms_per_batch=best[9], tried=[shape_dict(t) for t in tried])
+    res["autotune"] = tune_report(best, tried)
     res["config"] = {"jobs": count, "N": N, "levels": "uniform 4..24 (seed 1604)", "mean_level": float(np.mean(levels)),
                      "operands": "uniform residues"}
     return res
@@ -708,9 +729,9 @@ def run_ours(args):
     g.he_profile(ctx, False)
     launches_per_step = sum(v[1] for v in prof.values()) // prof_steps  # one mark per kernel
     per_kernel = {}
-    split = 0  # the passes' stages follow the ring size alone (he_shape's ntt_split has no effect)
+    tc = tensor_conversions(ctx.moduli)
     for k, v in prof.items():
-        kind, work = kernel_work(k, ctx.prm, level, split)
+        kind, work = kernel_work(k, ctx.prm, level)
         d = {"ms_total": v[0], "calls": v[1], "ms_avg": v[0] / v[1], "kind": kind}
         if kind == "alu":
             d["Gbutterfly_s"] = work / (d["ms_avg"] * 1e-3) / 1e9
@@ -720,8 +741,8 @@ def run_ours(args):
             d["GMAC_s"] = work / (d["ms_avg"] * 1e-3) / 1e9
         per_kernel[k] = d
     # the dominant kernel with one roofline (a launch mixing a compute-bound and
-    # a memory-bound part has neither)
-    graded = [k for k in per_kernel if per_kernel[k]["kind"] in ("alu", "mac", "hbm")]
+    # a memory-bound part has neither, nor has a conversion on the tensor cores)
+    graded = [k for k in per_kernel if per_kernel[k]["kind"] in (("alu", "hbm") if tc else ("alu", "mac", "hbm"))]
     dom = max(graded, key=lambda k: per_kernel[k]["ms_total"]) if graded else None
 
     # ---- seeded evaluation key: b halves on the device, a halves regenerated ----
@@ -881,33 +902,33 @@ def run_ours(args):
         del nws, prep, nevk, nct, nout
 
     # ALU ceilings: the NTT's butterfly and the CUDA-core conversions' inner loop,
-    # register-resident, measured in this run at its clocks (conversions on the
-    # tensor cores, for primes of 52 to 55 bits, are not bound by the latter)
+    # register-resident, measured in this run at its clocks (the latter bounds no
+    # conversion on the tensor cores, for primes of 52 to 55 bits: those have no frac_of_probe)
     bfly_peak = g.he_probe_butterfly_rate(152 * 8, 4096, stream)
     conv_width = {"modup": kernel_width(prm.alpha), "moddown_conv": kernel_width(prm.K)}
     conv_peak = {k: g.he_probe_conversion_rate(w, 152 * 8, max(64, 4096 // w), stream) for k, w in conv_width.items()}
     probe = {"butterfly_per_s": bfly_peak, "conversion_mac_per_s": conv_peak, "conversion_width": conv_width}
-    # the CUDA-core remainder of a byte-split tensor-core conversion (planes ->
-    # 128 bits -> reduction) against the whole CUDA-core conversion, per output
+    # the CUDA-core remainder of a 13-plane byte-split tensor-core conversion (planes ->
+    # 128 bits -> reduction) against the whole CUDA-core conversion, per output; the
+    # tensor-core conversions built have six planes and another recombination
     recomb = g.he_probe_recombine_rate(152 * 8, 1024, stream)
     probe["byte_split_tensor_conversion"] = {
         "recombine_outputs_per_s": recomb,
         "cuda_core_outputs_per_s": {k: conv_peak[k] / w for k, w in conv_width.items()},
-        "what": "outputs/s of the CUDA-core work left per output by a byte-split tensor-core conversion (13 fp32 "
-                "planes to 128 bits, lazy Barrett; MMA not counted) beside the outputs/s of the whole CUDA-core "
-                "conversion at the kernels' widths: below 1 means the tensor-core form cannot be faster"}
+        "what": "a 13-plane form's CUDA-core remainder beside the CUDA-core conversion, outputs/s (the form built "
+                "has 6 planes)"}
     probe["byte_split_tensor_conversion"]["ratio"] = {
         k: recomb / v for k, v in probe["byte_split_tensor_conversion"]["cuda_core_outputs_per_s"].items()}
     for k, d in per_kernel.items():
         if d["kind"] == "alu":
             d["frac_of_probe"] = d["Gbutterfly_s"] * 1e9 / bfly_peak
-        elif d["kind"] == "mac" and k.split(".")[0] in conv_peak:
+        elif d["kind"] == "mac" and not tc and k.split(".")[0] in conv_peak:
             d["frac_of_probe"] = d["GMAC_s"] * 1e9 / conv_peak[k.split(".")[0]]
         elif d["kind"] == "mixed":
             # the ModDown conversion (ALU) and the q rows' key-switch sums (HBM)
             # in one launch: each part's rate, and the launch against the two
             # ideal times added (the bound if the parts did not overlap)
-            macs = kernel_work(k, ctx.prm, level, split)[1]
+            macs = kernel_work(k, ctx.prm, level)[1]
             beta = -(-level // ctx.prm.alpha)
             qbytes = (3 * beta + 2) * (level - 1) * ctx.N * 8
             t = d["ms_avg"] * 1e-3
@@ -922,7 +943,7 @@ def run_ours(args):
     hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
     roof = None
     if dom:
-        kind, work = kernel_work(dom, ctx.prm, level, split)
+        kind, work = kernel_work(dom, ctx.prm, level)
         avg_s = per_kernel[dom]["ms_avg"] * 1e-3
         if kind == "alu":
             ach = work / avg_s / 1e9
@@ -992,8 +1013,7 @@ def run_ours(args):
                            f"median of {len(e2e_runs)} runs",
                     "runs": e2e_runs,
                     "link": {"value": link_val, "unit": "HE Mul/s",
-                             "what": "the same bytes per step as plain pinned-host copies (the two uploads and the "
-                                     "download each on its own stream), no kernels"},
+                             "what": "the same bytes as plain pinned-host copies on three streams, no kernels"},
                     "decrypt_max_err": e2e_err,
                     "single_call": {"value": single_val, "unit": "HE Mul/s", "api": "he_mul_rescale_host",
                                     "steps": single_steps}},
@@ -1002,7 +1022,7 @@ def run_ours(args):
             "inner_product_hbm": ip,
             "probe": probe,
             "kernels": per_kernel,
-            "autotune": dict(shape_dict(tune_best), tried=[shape_dict(t) for t in tune_tried]),
+            "autotune": tune_report(tune_best, tune_tried),
             "n17_single": n17,
             "rescale_pq": pq,
             "seeded_evk": seeded,
@@ -1015,7 +1035,9 @@ def run_ours(args):
             "clocks": clk,
             "decrypt_max_err": dec_err,
         }
-        print(json.dumps(line), flush=True)
+        for d in per_kernel.values():
+            del d["ms_total"]  # ms_avg times calls
+        print(json.dumps(short(line), separators=(",", ":")), flush=True)
     if wsz > 1:
         torch.distributed.destroy_process_group()
 
