@@ -71,7 +71,6 @@ struct DevLevel {
     unsigned o_d0, o_d1, o_d2, o_y, o_u, o_ks, o_ys, o_r, o_z, o_total;
     const u64 *modupB;             // [beta][E][A]: [Qhat_{j,i}]_t split at bit 28, zero-padded
     const ulonglong2 *qinv_last;   // [l-1]: q_{l-1}^-1 mod q_i (value, Shoup)
-    const ulonglong2 *pinv_qinv;   // [l-1]: P^-1 * q_{l-1}^-1 mod q_i
     const u64 *pbpq;               // [l-1][KP]: [Phat_k P^-1 q_{l-1}]_{q_i} (one division by P q_{l-1})
     // tensor-core conversions (he_ctx::tc): ModUp images and targets
     // [beta][up_nch][up_tp], up_tc targets per chunk; pbpq's images [chunk]
@@ -140,7 +139,7 @@ struct HostLevel {
     std::vector<TcTarget> tc_up_t, tc_pq_t;
     int up_nch = 0, up_tc = 0, up_tp = 0, up_bytes = 0;
     std::vector<u64> pbpq;  // [l-1][KP]: [Phat_k P^-1 q_{l-1}]_{q_i}, split at bit 28 (one division by P q_{l-1})
-    std::vector<ulonglong2> qinv_last, pinv_qinv;
+    std::vector<ulonglong2> qinv_last;
 };
 
 }  // namespace he

@@ -527,12 +527,10 @@ int build_context(he_ctx *c, const he_params *p, bool device)
                 H.rs_ntt.push_back(NttJob{(unsigned)(W.r + h), (unsigned)(W.z + (size_t)h * (l - 1) + i), (unsigned)(K + i),
                                           0, 0, 0});
         H.qinv_last.resize(l > 1 ? l - 1 : 1);
-        H.pinv_qinv.resize(l > 1 ? l - 1 : 1);
         for (int i = 0; i + 1 < l; i++) {
             u64 qi = c->ext[K + i];
             u64 qinv = inv(ql % qi, qi);
             H.qinv_last[i] = pair(qinv, qi);
-            H.pinv_qinv[i] = pair(mul(qinv, c->pinv[i].x, qi), qi);
         }
     }
     if (!device) return HE_OK;
@@ -566,14 +564,13 @@ int build_context(he_ctx *c, const he_params *p, bool device)
     // to give up CTAs for it; at N = 2^16, level 24, 211 us against 236 with
     // two limbs per group and 264 with four)
     constexpr int NL = 10;  // job lists per level
-    struct LvlOff { size_t modupB, qinv, pq, pbpq, tc[4], j[NL]; };
+    struct LvlOff { size_t modupB, qinv, pbpq, tc[4], j[NL]; };
     std::vector<LvlOff> lo(L + 1);
     std::vector<std::vector<std::vector<NttGroup>>> gl(L + 1, std::vector<std::vector<NttGroup>>(NL));
     for (int l = 1; l <= L; l++) {
         HostLevel &H = c->host_levels[l];
         lo[l].modupB = take(sizeof(u64) * H.modupB.size());
         lo[l].qinv = take(sizeof(ulonglong2) * H.qinv_last.size());
-        lo[l].pq = take(sizeof(ulonglong2) * H.pinv_qinv.size());
         lo[l].pbpq = take(sizeof(u64) * H.pbpq.size());
         lo[l].tc[0] = take(H.tc_up.size());
         lo[l].tc[1] = take(sizeof(TcTarget) * H.tc_up_t.size());
@@ -657,11 +654,9 @@ int build_context(he_ctx *c, const he_params *p, bool device)
         }
         memcpy(img.data() + lo[l].modupB, H.modupB.data(), sizeof(u64) * H.modupB.size());
         memcpy(img.data() + lo[l].qinv, H.qinv_last.data(), sizeof(ulonglong2) * H.qinv_last.size());
-        memcpy(img.data() + lo[l].pq, H.pinv_qinv.data(), sizeof(ulonglong2) * H.pinv_qinv.size());
         memcpy(img.data() + lo[l].pbpq, H.pbpq.data(), sizeof(u64) * H.pbpq.size());
         D.modupB = (const u64 *)(base + lo[l].modupB);
         D.qinv_last = (const ulonglong2 *)(base + lo[l].qinv);
-        D.pinv_qinv = (const ulonglong2 *)(base + lo[l].pq);
         D.pbpq = (const u64 *)(base + lo[l].pbpq);
         if (c->tc) {
             memcpy(img.data() + lo[l].tc[0], H.tc_up.data(), H.tc_up.size());

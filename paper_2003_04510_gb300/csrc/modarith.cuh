@@ -185,10 +185,9 @@ __device__ __forceinline__ u64 mul_mod(u64 a, u64 b, u64 q, u64 mu, unsigned s)
 
 // Lazy dot products of a residue vector with constant vectors (base
 // conversion).  Operands are split at bit 28: x = x1*2^28 + x0, and the
-// constant is stored pre-split as b0 | (b1 << 32).  Each term is four
-// 32x32 -> 64-bit multiply-adds into three 64-bit accumulators with no carry
-// handling: for x, b < 2^57 and at most 16 terms every accumulator stays below
-// 2^63.  The 128-bit value is assembled once per output.
+// constant is stored pre-split as b0 | (b1 << 32).  Each term is three
+// 32x32 -> 64-bit multiply-adds (mac28k) into three 64-bit accumulators with no carry
+// handling.
 struct Acc3 {
     u64 a0, a1, a2;  // weights 1, 2^28, 2^56
 };
@@ -199,22 +198,12 @@ __device__ __forceinline__ void split28(u64 x, uint32_t &x0, uint32_t &x1)
     x1 = (uint32_t)(x >> 28);
 }
 
-__device__ __forceinline__ void mac28(Acc3 &s, uint32_t x0, uint32_t x1, u64 bpacked)
-{
-    const uint32_t b0 = (uint32_t)bpacked, b1 = (uint32_t)(bpacked >> 32);
-    s.a0 = mad_wide(x0, b0, s.a0);
-    s.a1 = mad_wide(x0, b1, s.a1);
-    s.a1 = mad_wide(x1, b0, s.a1);
-    s.a2 = mad_wide(x1, b1, s.a2);
-}
-
-// Karatsuba form of mac28: three multiply-adds per term, x0*b0 (into a0),
+// One term in Karatsuba's form: x0*b0 (into a0),
 // x1*b1 (into a2) and (x0+x1)*(b0+b1) (into a1, which then holds the sum of
 // all three products' middle parts plus a0 and a2; acc3k_value takes them
 // out).  xs = x0 + x1 is formed once per input.  For x, b < 2^57 and at most
 // 16 terms: a0 < 2^60, a2 < 2^62 and a1 < 16 * 9 * 2^56 < 2^64, and the
-// recovered middle sum x0*b1 + x1*b0 stays below 2^62, so acc3k_value returns
-// exactly what acc3_value returns for the four-product form.
+// recovered middle sum x0*b1 + x1*b0 stays below 2^62, so acc3k_value is exact.
 __device__ __forceinline__ void mac28k(Acc3 &s, uint32_t x0, uint32_t x1, uint32_t xs, u64 bpacked)
 {
     const uint32_t b0 = (uint32_t)bpacked, b1 = (uint32_t)(bpacked >> 32);
@@ -223,25 +212,16 @@ __device__ __forceinline__ void mac28k(Acc3 &s, uint32_t x0, uint32_t x1, uint32
     s.a1 = mad_wide(xs, b0 + b1, s.a1);
 }
 
-__device__ __forceinline__ U128 acc3_value(const Acc3 &s)
+__device__ __forceinline__ U128 acc3k_value(const Acc3 &k)
 {
     U128 v;
-    const u64 t1 = s.a1 << 28, t2 = s.a2 << 56;
-    v.lo = s.a0 + t1;
+    const u64 m = k.a1 - k.a0 - k.a2, t1 = m << 28, t2 = k.a2 << 56;
+    v.lo = k.a0 + t1;
     u64 c = v.lo < t1 ? 1ull : 0ull;
     v.lo += t2;
     c += v.lo < t2 ? 1ull : 0ull;
-    v.hi = (s.a1 >> 36) + (s.a2 >> 8) + c;
+    v.hi = (m >> 36) + (k.a2 >> 8) + c;
     return v;
-}
-
-__device__ __forceinline__ U128 acc3k_value(const Acc3 &k)
-{
-    Acc3 t;
-    t.a0 = k.a0;
-    t.a1 = k.a1 - k.a0 - k.a2;
-    t.a2 = k.a2;
-    return acc3_value(t);
 }
 
 // V mod q, lazily in [0, 3q), straight from the Karatsuba accumulators
