@@ -539,8 +539,8 @@ int he_profile(he_ctx *ctx, int enable);
 int he_profile_read(he_ctx *ctx, int max, char *names, double *total_ms, int *calls, int *count);
 
 /* Measurement helper: rate (butterflies per second) of the NTT's own lazy
- * Cooley-Tukey butterfly (Algo 4 with the modified Shoup product of Sec. 5.2;
- * the same device function the NTT passes call) on register-resident data,
+ * Cooley-Tukey butterfly (Algo 4 with the split twiddle product; the same device
+ * function the NTT passes call) on register-resident data,
  * `blocks` x 256 threads x 8 chains x `iters`.  The ALU ceiling the NTT
  * kernels are compared against.  Allocates a small output buffer with
  * cudaMallocAsync on `stream`; HE_EINVAL for a non-positive count. */
@@ -552,11 +552,12 @@ int he_probe_butterfly_rate(int blocks, int iters, double *bfly_per_s, void *str
  * of the split-28 Karatsuba multiply-accumulate with the constant read from
  * shared memory, then one reduction straight from the accumulators, on two
  * coefficients per thread held in registers; `blocks` x 256 threads x 16
- * outputs x `iters`.  The ALU ceiling the ModUp and ModDown conversions are
- * compared against.  HE_EINVAL for another width or a non-positive count. */
+ * outputs x `iters`.  The ALU ceiling the ModUp and ModDown conversions of
+ * contexts on the CUDA cores are compared against.  HE_EINVAL for another width or a non-positive count. */
 int he_probe_conversion_rate(int width, int blocks, int iters, double *mac_per_s, void *stream);
-/* Measurement helper: rate (outputs per second) of the work a byte-split
- * tensor-core base conversion would still leave on the CUDA cores per output
+/* Measurement helper: rate (outputs per second) of the work a 13-plane byte-split
+ * tensor-core base conversion (not the form built, which has six planes) would
+ * still leave on the CUDA cores per output
  * (the conversion's matrix product, Sec. 7's base conversion, cut into 8-bit
  * pieces exact in bf16 and summed in fp32): the MMA's 13 byte-diagonal planes,
  * each an exact integer below 2^23, turned into integers, shifted and added

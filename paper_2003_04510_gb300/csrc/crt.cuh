@@ -15,9 +15,9 @@
 // and store; digits and accumulators are doubled, so the three run side by side.
 // Measured against 28-bit multiply-adds on the CUDA cores, N = 2^16, log Q = 1200:
 // region 1 (four polynomials, 43 primes) 202 -> 52 us in one launch instead of
-// four, region 2 (one, 64 primes) 74 -> 23 us.  The reducing warps bound it (tensor
-// cores 22% active); the folding reduction took 61 to 52 us, eight reducing warps
-// instead of sixteen 68.
+// four, region 2 (one, 64 primes) 74 -> 23 us (51 and 21 under ncu: 55 and 46% of the
+// issue slots, tensor cores 24 and 21% active).  The reducing warps bound it;
+// the folding reduction took 61 to 52 us, eight reducing warps instead of sixteen 68.
 #pragma once
 #include "he_internal.h"
 #include "icrt.cuh"

@@ -22,7 +22,8 @@
 // while the MMAs of the next one run (two accumulator buffers); a tile's MMAs
 // start with its first eight primes' digits.  Measured against 64 x 64-bit products
 // on the CUDA cores, N = 2^16, log Q = 1200: region 1 (three products, 43 primes,
-// 19 words) 211 -> 55 us, region 2 (two, 64 primes, 38 words) 468 -> 78 us.  What
+// 19 words) 211 -> 55 us, region 2 (two, 64 primes, 38 words) 468 -> 78 us (53 and 76
+// under ncu: 33 and 29% of the issue slots, tensor cores 20 and 25% active).  What
 // bounds it is shared memory: an MMA reads 4 KB of digits and 2.5 KB of constants
 // for 80 columns, beside the copies that bring the constants.
 #pragma once

@@ -1,7 +1,7 @@
 // probe.cu -- throughput probes for the ALU rooflines of the path's
 // compute-bound kernels.
 //
-// The NTT kernels and the base conversions are bound by integer multiply
+// The NTT kernels and the CUDA-core base conversions are bound by integer multiply
 // work, not by HBM.  Each probe runs the kernels' own device functions on
 // register-resident data with no global-memory traffic inside the timed loop,
 // so its rate is the practical ceiling of that instruction sequence on this
@@ -80,8 +80,8 @@ __global__ void __launch_bounds__(256) k_probe_conv(u64 *out, const u64 *rows, u
     out[blockIdx.x * blockDim.x + threadIdx.x] = acc;
 }
 
-// The recombination a byte-split tensor-core base conversion would need per
-// output.  Such a conversion (residues and constants cut into 8-bit pieces,
+// The recombination a 13-plane byte-split tensor-core base conversion would need per
+// output (tc.cuh's form has six planes instead).  Such a conversion (residues and constants cut into 8-bit pieces,
 // exact in bf16, products summed in fp32 by the MMA) leaves, per output, 13
 // fp32 planes S_d = sum over byte pairs (a, b) with a + b = d, each an exact
 // integer below 2^23 for up to 16 terms; the output is
@@ -189,7 +189,10 @@ extern "C" int he_probe_butterfly_rate(int blocks, int iters, double *bfly_per_s
     const u64 q = kProbeQ;
     const u64 w = 1234567890123ull % q;
     NttMod km;
-    if (!he::ntt_mod(q, 16, &km)) return HE_EINVAL;
+    if (!he::ntt_mod(q, 16, &km)) {
+        cudaFreeAsync(out, st);
+        return HE_EINVAL;
+    }
     const u64 w2 = (u64)(((unsigned __int128)w << 32) % q), m = (1ull << km.s) - 1;
     const ulonglong2 tw = make_ulonglong2((w & m) | ((w >> km.s) << 32), (w2 & m) | ((w2 >> km.s) << 32));
     float ms = 0;

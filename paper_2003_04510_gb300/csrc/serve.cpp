@@ -7,8 +7,11 @@
 // one ring into a batch (he_mul_batch: every stage is one launch over the
 // whole batch) and launches it on a free stream, so batches formed while
 // earlier ones are still running overlap on the GPU.  Completion is detected
-// by polling each batch's CUDA event on the host; there are no device-side
-// waits.  Results are bit-identical to he_mul_rescale on each request alone.
+// by polling each batch's CUDA event on the host; no kernel waits for a request or
+// another batch.  (A ring's tensor-core conversions wait for their own products, for a
+// bounded time; once such a wait has given up, every batch of that ring that finishes
+// fails with HE_ETIMEOUT.)  Results are bit-identical to he_mul_rescale on each
+// request alone.
 #include <algorithm>
 #include <atomic>
 #include <chrono>

@@ -29,7 +29,7 @@
 // current one.  (A CTA per tile spent a third of its time on launch, TMEM
 // allocation and the constants' copy.)
 // Measured, CUDA cores against this: ModUp 32.7 -> 18.5 us at N = 2^16, level 24
-// (three digits of eight limbs), 174 -> 61 us at 2^17, level 44, 897 -> 496 us for
+// (three digits of eight limbs), 174 -> 63 us at 2^17, level 44, 897 -> 496 us for
 // 64 jobs at 2^16; the ModDown conversions of the 64 jobs 748 -> 483 us.  What is
 // left is the recombination's integer instructions and, below a tile or two per
 // team, the chain of one tile.
