@@ -70,23 +70,29 @@ static ulonglong2 split_tw(u64 w, u64 wsh, u64 q, unsigned s)
 // base-conversion constant stored split at bit 28 for the kernels' lazy MACs
 static u64 split28(u64 b) { return (b & 0xFFFFFFFull) | ((b >> 28) << 32); }
 
+// Groups of one prime next to each other: their CTAs run at the same time and read that
+// prime's twiddle runs from L2 instead of each from DRAM.  Every group's place follows
+// from the counts, so none is moved (a batch's thousands of groups are formed at every
+// call; sorting them took a tenth of it).
 std::vector<NttGroup> group_jobs(const std::vector<NttJob> &jobs, int cap)
 {
     cap = std::max(1, std::min(cap, kGroupMax));
-    std::vector<NttGroup> out;
-    std::vector<int> open_for_prime;  // index into out of the group being filled, per prime
+    std::vector<size_t> n, at;  // per prime: its limbs, its first group
     for (const NttJob &j : jobs) {
-        if (j.prime >= open_for_prime.size()) open_for_prime.resize(j.prime + 1, -1);
-        int g = open_for_prime[j.prime];
-        if (g < 0 || out[g].nl == (unsigned)cap) {
-            NttGroup ng;
-            memset(&ng, 0, sizeof(ng));
-            ng.prime = j.prime;
-            out.push_back(ng);
-            g = (int)out.size() - 1;
-            open_for_prime[j.prime] = g;
-        }
-        NttGroup &G = out[g];
+        if (j.prime >= n.size()) n.resize(j.prime + 1, 0);
+        n[j.prime]++;
+    }
+    size_t groups = 0;
+    for (size_t &k : n) {
+        at.push_back(groups);
+        groups += (k + cap - 1) / cap;
+        k = 0;
+    }
+    std::vector<NttGroup> out(groups);  // zeros
+    for (const NttJob &j : jobs) {
+        const size_t k = n[j.prime]++;
+        NttGroup &G = out[at[j.prime] + k / cap];
+        G.prime = j.prime;
         G.src[G.nl] = j.src;
         G.dst[G.nl] = j.dst;
         G.scale[G.nl] = j.scale;
@@ -97,9 +103,6 @@ std::vector<NttGroup> group_jobs(const std::vector<NttJob> &jobs, int cap)
         G.cks[G.nl] = j.cks;
         G.nl++;
     }
-    // groups of one prime next to each other: their CTAs run at the same time
-    // and read that prime's twiddle runs from L2 instead of each from DRAM
-    std::stable_sort(out.begin(), out.end(), [](const NttGroup &a, const NttGroup &b) { return a.prime < b.prime; });
     return out;
 }
 
