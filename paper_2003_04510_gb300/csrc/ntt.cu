@@ -56,6 +56,8 @@ namespace he {
 
 namespace {
 
+constexpr int kSMs = 152;
+
 __device__ __forceinline__ int padi(int e) { return e + (e >> 4); }
 
 struct NttArgs {
@@ -546,8 +548,8 @@ __device__ __forceinline__ void prefetch_last_round(const ulonglong2 *twg, int t
 // Resident CTAs per SM the register allocation is bounded for.
 __host__ __device__ constexpr int ntt_min_blocks(int nt) { return nt >= 512 ? 1 : nt >= 256 ? 4 : nt >= 128 ? 5 : 8; }
 
-template <class P, int R0, int R1, int R2, int R3, bool INV, int FUSE>
-__global__ void __launch_bounds__(P::NT, ntt_min_blocks(P::NT)) k_ntt_pass(const NttArgs A)
+template <class P, int R0, int R1, int R2, int R3, bool INV, int FUSE, int MIN = ntt_min_blocks(P::NT)>
+__global__ void __launch_bounds__(P::NT, MIN) k_ntt_pass(const NttArgs A)
 {
     constexpr bool STRIDED = P::STRIDED, COMBINE = FUSE == kFuseCombine || FUSE == kFusePlain;
     constexpr bool COMPUTED = FUSE == kFuseTensor || FUSE == kFuseIp;  // the tile load computes its words
@@ -697,11 +699,10 @@ __global__ void __launch_bounds__(P::NT, ntt_min_blocks(P::NT)) k_ntt_pass(const
 }
 
 // ngroups == 0 only sets the kernel's shared-memory limit (no launch).
-template <int LOGN, bool STRIDED, bool INV, int FUSE, int TE, int R0, int R1, int R2 = 0, int R3 = 0>
-cudaError_t run_pass(const NttArgs &a, int ngroups, cudaStream_t st)
+template <class P, int R0, int R1, int R2, int R3, bool INV, int FUSE, int MIN>
+cudaError_t launch_pass(const NttArgs &a, int ngroups, cudaStream_t st)
 {
-    using P = Pass<LOGN, STRIDED, R0, R1, R2, R3, TE>;
-    auto kern = k_ntt_pass<P, R0, R1, R2, R3, INV, FUSE>;
+    auto kern = k_ntt_pass<P, R0, R1, R2, R3, INV, FUSE, MIN>;
     static bool configured = false;  // once per instantiation
     if (!configured) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::SMEM);
@@ -711,6 +712,28 @@ cudaError_t run_pass(const NttArgs &a, int ngroups, cudaStream_t st)
     if (ngroups == 0) return cudaSuccess;
     launch_k(a.pdl != 0, kern, dim3(ngroups * P::TILES), dim3(P::NT), P::SMEM, st, a);
     return cudaGetLastError();
+}
+
+// The ring of one tile (2^12, 512 threads) has a second form, of two CTAs per SM at 64
+// registers, for more CTAs than SMs: 200 jobs of 8-limb digits (levels 2 to 16) 938 -> 813
+// us, 512 jobs of three limbs 818 -> 691 us of kernels.  Up to one CTA per SM the registers
+// (116 to 124) are worth more: 32 jobs of the first kind 177 us, 188 at 64 registers.  A
+// batch graph's grid is that of a full batch at the highest level (its launches are
+// smaller: 16 jobs 110 us, 119 at 64 registers), so it takes that form from two CTAs per SM.
+template <int LOGN, bool STRIDED, bool INV, int FUSE, int TE, int R0, int R1, int R2 = 0, int R3 = 0>
+cudaError_t run_pass(const NttArgs &a, int ngroups, cudaStream_t st)
+{
+    using P = Pass<LOGN, STRIDED, R0, R1, R2, R3, TE>;
+    constexpr int MIN = ntt_min_blocks(P::NT);
+    if constexpr (MIN == 1) {
+        if (ngroups == 0) {
+            const cudaError_t e = launch_pass<P, R0, R1, R2, R3, INV, FUSE, 2>(a, 0, st);
+            if (e != cudaSuccess) return e;
+        } else if (ngroups * P::TILES > (a.count ? 2 : 1) * kSMs) {
+            return launch_pass<P, R0, R1, R2, R3, INV, FUSE, 2>(a, ngroups, st);
+        }
+    }
+    return launch_pass<P, R0, R1, R2, R3, INV, FUSE, MIN>(a, ngroups, st);
 }
 
 // The two passes of each ring size: the strided one covers the first stages
