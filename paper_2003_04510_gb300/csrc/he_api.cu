@@ -109,8 +109,8 @@ int run_keyswitch(he_ctx *c, const JobRef &R, u64 *ntt_base, const Stages &S, co
 // 598 us, 16 at 2^16 1543 against 1573; four jobs at 2^16 427 against 418, eight at
 // 2^15 316 against 306.  Larger groups gain nothing there (64 jobs at 2^16: 5888,
 // 5890 and 5921 us in twos, threes and fours).  2^12, whose CTAs each stage the
-// ring's whole table and fill an SM: as many as keep one wave (128 jobs 385, 323,
-// 301 and 293 us in ones to fours; 16 jobs 79, 92, 117 and 142).
+// ring's whole table and fill an SM: as many as keep one wave (16 jobs 79, 92, 117 and
+// 142 us in ones to fours; 45 jobs of three limbs 117 us, 123 with two waves' worth).
 int limb_group(const he_ctx *c, size_t limbs)
 {
     const size_t n = c->logN == 12 ? (limbs + 151) / 152 : limbs * (size_t)(c->N / 2048) >= 6 * 5 * 152 ? 2 : 1;

@@ -248,12 +248,19 @@ static bool build_tc(he_ctx *c)
     auto round8 = [](int v) { return (v + 7) & ~7; };
     auto k_pad = [](int g) { return (24 * g + 1 + 15) / 16 * 16; };  // tc::k_pad
     auto rows = [](int tp) { return (6 * tp + 15) / 16 * 16; };
-    // [prod_{i2 != skip} m[i2]]_t over m[lo, hi)
-    auto hat = [&](const std::vector<u64> &m, int lo, int hi, int skip, u64 t) {
-        u64 v = 1;
-        for (int i = lo; i < hi; i++)
-            if (i != skip) v = mul(v, m[i] % t, t);
-        return v;
+    // [prod_{i2 != i} m[i2]]_t over m[lo, hi), for every i
+    auto hats = [&](const std::vector<u64> &m, int lo, int hi, u64 t) {
+        std::vector<u64> h(hi - lo, 1);
+        u64 below = 1, above = 1;
+        for (int i = 0; i < hi - lo; i++) {
+            h[i] = below;
+            below = mul(below, m[lo + i] % t, t);
+        }
+        for (int i = hi - lo - 1; i >= 0; i--) {
+            h[i] = mul(h[i], above, t);
+            above = mul(above, m[lo + i] % t, t);
+        }
+        return h;
     };
     c->up_off5 = tc_off5(qs);
     c->dn_off5 = tc_off5(ps);
@@ -271,11 +278,13 @@ static bool build_tc(he_ctx *c)
     c->tc_PB_t.resize((size_t)c->dn_nch * c->dn_tp);
     c->tc_PBP_t.resize((size_t)c->dn_nch * c->dn_tp);
     std::vector<u64> pb((size_t)L * K), pbp((size_t)L * K);
-    for (int i = 0; i < L; i++)
+    for (int i = 0; i < L; i++) {
+        const std::vector<u64> h = hats(ps, 0, K, qs[i]);
         for (int k = 0; k < K; k++) {
-            pb[(size_t)i * K + k] = hat(ps, 0, K, k, qs[i]);
-            pbp[(size_t)i * K + k] = mul(pb[(size_t)i * K + k], c->pinv[i].x, qs[i]);
+            pb[(size_t)i * K + k] = h[k];
+            pbp[(size_t)i * K + k] = mul(h[k], c->pinv[i].x, qs[i]);
         }
+    }
     auto slice = [&](const std::vector<u64> &m, int i0, int n) {
         return std::vector<u64>(m.begin() + (size_t)i0 * K, m.begin() + (size_t)(i0 + n) * K);
     };
@@ -314,8 +323,9 @@ static bool build_tc(he_ctx *c)
                 for (int u = ch * H.up_tc; u < std::min((ch + 1) * H.up_tc, El - nj); u++) {
                     const int e = u < K + lo ? u : u + nj;
                     t.push_back(c->ext[e]);
-                    for (int i = 0; i < c->alpha; i++)
-                        cst.push_back(i < nj ? hat(qs, lo, hi, lo + i, c->ext[e]) : 0);
+                    const std::vector<u64> h = hats(qs, lo, hi, c->ext[e]);
+                    cst.insert(cst.end(), h.begin(), h.end());
+                    cst.resize(cst.size() + c->alpha - nj, 0);
                 }
                 const size_t at = (size_t)j * H.up_nch + ch;
                 if (!tc_image(cst, t, (int)t.size(), src, H.up_tp, &H.tc_up[at * H.up_bytes], &H.tc_up_t[at * H.up_tp]))

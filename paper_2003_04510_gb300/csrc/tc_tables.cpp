@@ -65,10 +65,16 @@ bool tc_image(const std::vector<u64> &c, const std::vector<u64> &q, int T, const
     auto at = [&](int row, int k) -> uint16_t & { return img[((size_t)(k / 8) * rows + row) * 8 + k % 8]; };
     u64 H = (u64)top << 45;
     for (int d = 0; d < 5; d++) H += 256ull << (9 * d);
+    static const std::vector<uint16_t> halves = [] {  // the digits' f16, which the images hold by the hundred thousand
+        std::vector<uint16_t> h(4097);
+        for (int v = -2048; v <= 2048; v++) h[v + 2048] = half_of(v);
+        return h;
+    }();
     for (int t = 0; t < T; t++) {
         const u64 m = q[t];
         const int b = bitlen(m);
         if (b < 52 || b > 55) return false;
+        const u64 two9 = shoup(512, m);
         u64 base = 0;
         std::vector<long> mass(6, 0);  // per plane: the largest magnitude its sum can reach
         for (int i = 0; i < nsrc; i++) {
@@ -81,10 +87,11 @@ bool tc_image(const std::vector<u64> &c, const std::vector<u64> &q, int T, const
                     if (p < 5) r = ((v + 256) & 511) - 256;
                     v = (v - r) / 512;
                     if (r < -2048 || r > 2048) return false;
-                    at(6 * t + p, 24 * (i / 4) + 6 * (i % 4) + d) = half_of((int)r);
+                    at(6 * t + p, 24 * (i / 4) + 6 * (i % 4) + d) = halves[(int)r + 2048];
                     mass[p] += (long)(r < 0 ? -r : r) * (d < 5 ? 256 : top);
                 }
-                cd = mul(cd, 512, m);
+                cd = cd * 512 - (u64)(((u128)cd * two9) >> 64) * m;  // Shoup: below 2 m
+                cd = cd >= m ? cd - m : cd;
             }
         }
         for (int p = 0; p < 6; p++) {
